@@ -210,39 +210,51 @@ def _host(t):
     return None if t is None else torch.empty(t.shape, dtype=t.dtype, pin_memory=True).copy_(t)
 
 
-def prepare(case, seed):
-    c = dict(BASE, **case)
-    B, Hq, Hkv, d, T, steps = c["B"], c["Hq"], c["Hkv"], c["d"], c["T"], c["steps"]
-    torch.cuda.empty_cache()   # the layer allocates its state outside torch's pool
-    gen = torch.Generator(device="cuda").manual_seed(seed)
+def _params(c, seed):
+    """Layer parameters (or None for 1, 0, 1, 1) and the LN_q / LN_k dictionary of a case."""
     par, ln = dict(ln_w=None, ln_b=None, tau_s=None, tau_b=None), None
     if c["affine"]:
-        par = synth.make_layer_params(synth.Workload("params", B, Hq, Hkv, d, 1, c["C"], "sqrt", seed=seed), trivial=False)
+        par = synth.make_layer_params(synth.Workload("params", c["B"], c["Hq"], c["Hkv"], c["d"], 1, c["C"], "sqrt", seed=seed), trivial=False)
     if c["qk_ln"]:
         h = torch.Generator().manual_seed(seed + 1)
         ln = dict(eps=1e-5)
-        for n, heads in (("q", Hq), ("k", Hkv)):
-            ln[n + "_weight"] = 1.0 + 0.2 * torch.randn((heads, d), generator=h)
-            ln[n + "_bias"] = 0.1 * torch.randn((heads, d), generator=h)
-    layer = kvm.KVMState(
-        kvm.LayerConfig(batch=B, n_q_heads=Hq, n_kv_heads=Hkv, head_dim=d, max_block=c["C"], max_state_slots=_capacity(c),
-                        max_call_tokens=_call_tokens(c), n_bswa_chunks=c["w"], sink_len=c["S"]),
-        ln_weight=par["ln_w"], ln_bias=par["ln_b"], tau_state=par["tau_s"], tau_bswa=par["tau_b"], qk_ln=ln)
-    s = dict(c=c, layer=layer, growth=_growth(c), x=None)
-    at = 0
+        for n, heads in (("q", c["Hq"]), ("k", c["Hkv"])):
+            ln[n + "_weight"] = 1.0 + 0.2 * torch.randn((heads, c["d"]), generator=h)
+            ln[n + "_bias"] = 0.1 * torch.randn((heads, c["d"]), generator=h)
+    return par, ln
+
+
+def _inputs(c, seed, context):
+    """The tensors of a pass, in the order they are drawn; `context(q, k, v)` takes each call of the tokens before it."""
+    gen = torch.Generator(device="cuda").manual_seed(seed)
+    at, s = 0, {"x": None}
     while at < c["ctx"]:
         n = min(_call_tokens(c), c["ctx"] - at)
-        layer.prefill(*_values(c, n, gen), c["C"], s["growth"], c["r"])
+        context(*_values(c, n, gen))
         at += n
-    if T:
-        s["q"], s["k"], s["v"] = _values(c, T, gen)
-        s["out"] = torch.empty_like(s["q"])
+    if c["T"]:
+        s["q"], s["k"], s["v"] = _values(c, c["T"], gen)
         if c["d_model"]:
-            s["x"] = _rand((B, T, c["d_model"]), gen)
-            s["w_gate"] = torch.randn((Hkv, c["d_model"]), generator=gen, device="cuda") / math.sqrt(c["d_model"])
+            s["x"] = _rand((c["B"], c["T"], c["d_model"]), gen)
+            s["w_gate"] = torch.randn((c["Hkv"], c["d_model"]), generator=gen, device="cuda") / math.sqrt(c["d_model"])
     # one token per step: [step][B, heads, d], every step's tensors contiguous
-    s["tq"], s["tk"], s["tv"] = (list(t.permute(2, 0, 1, 3).contiguous()) for t in _values(c, steps, gen))
-    s["tout"] = torch.empty((steps, B, Hq, d), dtype=torch.bfloat16, device="cuda")
+    s["tq"], s["tk"], s["tv"] = (list(t.permute(2, 0, 1, 3).contiguous()) for t in _values(c, c["steps"], gen))
+    return s
+
+
+def prepare(case, seed):
+    c = dict(BASE, **case)
+    torch.cuda.empty_cache()   # the layer allocates its state outside torch's pool
+    par, ln = _params(c, seed)
+    layer = kvm.KVMState(
+        kvm.LayerConfig(batch=c["B"], n_q_heads=c["Hq"], n_kv_heads=c["Hkv"], head_dim=c["d"], max_block=c["C"],
+                        max_state_slots=_capacity(c), max_call_tokens=_call_tokens(c), n_bswa_chunks=c["w"], sink_len=c["S"]),
+        ln_weight=par["ln_w"], ln_bias=par["ln_b"], tau_state=par["tau_s"], tau_bswa=par["tau_b"], qk_ln=ln)
+    s = _inputs(c, seed, lambda q, k, v: layer.prefill(q, k, v, c["C"], _growth(c), c["r"]))
+    s.update(c=c, layer=layer, growth=_growth(c))
+    if c["T"]:
+        s["out"] = torch.empty_like(s["q"])
+    s["tout"] = torch.empty((c["steps"], c["B"], c["Hq"], c["d"]), dtype=torch.bfloat16, device="cuda")
     if c["host"]:
         for n in ("q", "k", "v", "out", "tout"):
             s[n] = _host(s[n])
@@ -273,4 +285,122 @@ def run(s):
     for i in range(c["steps"]):
         step(s["tq"][i], s["tk"][i], s["tv"][i], out=s["tout"][i])
     res["tokens"] = s["tout"]
+    return res
+
+
+def _budget(c, e):
+    if c["growth"] == "fixed":
+        return c["slots"]
+    if c["growth"] == "saturating":
+        return c["slots"] * e // (e + c["half"])
+    num, den = (1, 2) if c["growth"] == "sqrt" else (c["num"], c["den"])
+    most = c["coeff"] ** den * e ** num
+    n = int(round(most ** (1.0 / den)))
+    while n ** den > most:
+        n -= 1
+    while (n + 1) ** den <= most:
+        n += 1
+    return n
+
+
+def _norm(x, w, b, eps):
+    """LayerNorm over the channels; w, b [heads, 1, d]."""
+    x = x - x.mean(-1, keepdim=True)
+    return x / (x.square().mean(-1, keepdim=True) + eps).sqrt() * w + b
+
+
+def _exact_sequence(c, q, k, v, g, w, b, ts, tb, first, out):
+    """One batch element in 64 bits: q [Hkv, G, N, d], k, v [Hkv, N, d], g [Hkv, N] -> out [Hkv, G, N - first, d]."""
+    C, L, r, d, N, H = c["C"], c["w"] * c["C"], c["r"], c["d"], k.shape[1], k.shape[0]
+    G = q.shape[1]
+    half = r // 2
+    freq = 10000.0 ** (-torch.arange(half, dtype=torch.float64, device="cuda") / max(half, 1))
+
+    def rope(x, t0):
+        if not r:
+            return x
+        a = torch.arange(t0, t0 + x.shape[-2], dtype=torch.float64, device="cuda")[:, None] * freq
+        lo, hi = x[..., :half], x[..., half:r]
+        return torch.cat([lo * a.cos() - hi * a.sin(), lo * a.sin() + hi * a.cos(), x[..., r:]], -1)
+
+    K = V = torch.zeros((H, 0, d), dtype=torch.float64, device="cuda")
+    rho = torch.zeros((H, 0), dtype=torch.float64, device="cuda")
+    m = 0
+    for s in range(0, N, C):
+        e, z = s + C, min(s + C, N)
+        b0 = max(0, e - L)
+        kn = _norm(K, w, b, 1e-5)
+        if z > first:
+            a0 = max(s, first)
+            kw, vw = rope(k[:, b0:z].double(), b0), v[:, b0:z].double()
+            kr = V * (rho / V.norm(dim=-1).clamp_min(1e-12))[..., None]
+            qq = rope(q[:, :, a0:z].double(), a0)
+            ls = torch.matmul(qq, kn[:, None].mT) * (ts / math.sqrt(d))
+            lw = torch.matmul(qq, kw[:, None].mT) * (tb / math.sqrt(d))
+            later = torch.arange(b0, z, device="cuda")[None, :] > torch.arange(a0, z, device="cuda")[:, None]
+            lw.masked_fill_(later, -math.inf)
+            p = torch.softmax(torch.cat([ls, lw], -1), -1)
+            out[:, :, a0 - first:z - first] = torch.matmul(p, torch.cat([kr, vw], 1)[:, None])
+        if z < e or e < L:
+            continue
+        kb, vb, gb = k[:, b0:b0 + C].double().clone(), v[:, b0:b0 + C].double(), g[:, b0:b0 + C]
+        kb[..., :r] = 0.0
+        kb = _norm(kb, w, b, 1e-5)
+        na = C if m == 0 else min(max(m, min(_budget(c, e), m + C)) - m, C)
+        if na == C:
+            new = torch.arange(C, device="cuda").expand(H, C)
+        else:
+            sim = torch.matmul(kb, kn.mT)
+            new = sim.max(-1).values.sort(dim=-1, stable=True).indices[..., :na].sort(dim=-1).values
+        at = new[..., None].expand(-1, -1, d)
+        kc, vc = kb.gather(1, at), vb.gather(1, at)
+        K, V, rho = torch.cat([K, kc], 1), torch.cat([V, vc], 1), torch.cat([rho, vc.norm(dim=-1)], 1)
+        if na < C:
+            sim = torch.cat([sim, torch.matmul(kb, _norm(kc, w, b, 1e-5).mT)], -1)
+            sim[..., :c["S"]] = -math.inf
+            to = sim.argmax(-1)[..., None].expand(-1, -1, d)
+            gm = gb.scatter(1, new, 0.0)[..., None]
+            K.scatter_add_(1, to, kb * gm)
+            V.scatter_add_(1, to, vb * gm)
+        m += na
+
+
+def exact(case, seed):
+    """The layer by its definition in 64 bits.  LN_q / LN_k give bf16 tensors (as the stand-alone call does)."""
+    c = dict(BASE, **case)
+    if work(c)["flops"] > 2e13 or c["B"] * c["Hq"] * _total(c) * c["d"] > 1 << 31:
+        return None
+    B, Hq, Hkv, d = c["B"], c["Hq"], c["Hkv"], c["d"]
+    G = Hq // Hkv
+    par, ln = _params(c, seed)
+    parts = []
+    s = _inputs(c, seed, lambda *t: parts.append(t))
+    if c["T"]:
+        parts.append((s["q"], s["k"], s["v"]))
+    parts.append(tuple(torch.stack(s[n], 2) for n in ("tq", "tk", "tv")))
+    first = c["ctx"]
+
+    def dev(a, shape, default):
+        return torch.full(shape, default, dtype=torch.float64, device="cuda") if a is None else torch.as_tensor(a).to("cuda").double().reshape(shape)
+
+    w, b = dev(par["ln_w"], (Hkv, 1, d), 1.0), dev(par["ln_b"], (Hkv, 1, d), 0.0)
+    ts, tb = dev(par["tau_s"], (Hkv, G, 1, 1), 1.0), dev(par["tau_b"], (Hkv, G, 1, 1), 1.0)
+    out = torch.empty((B, Hkv, G, _total(c) - first, d), dtype=torch.float64, device="cuda")
+    gates = torch.ones((B, Hkv, _total(c)), dtype=torch.float64, device="cuda")
+    if s["x"] is not None:
+        for i in range(B):
+            z = s["x"][i].double() @ s["w_gate"].double().T
+            gates[i, :, first:first + c["T"]] = (1.0 + torch.where(z > 0, z, torch.expm1(z))).T
+    for i in range(B):
+        q, k, v = (torch.cat([t[n][i] for t in parts], 1) for n in range(3))
+        if ln:
+            q, k = (_norm(x.double(), ln[n + "_weight"].cuda().double()[:, None], ln[n + "_bias"].cuda().double()[:, None], ln["eps"]).bfloat16()
+                    for n, x in (("q", q), ("k", k)))
+        _exact_sequence(c, q.reshape(Hkv, G, -1, d), k, v, gates[i], w, b, ts, tb, first, out[i])
+    out = out.reshape(B, Hq, -1, d)
+    res = {"tokens": out[:, :, c["T"]:].permute(2, 0, 1, 3)}
+    if c["T"]:
+        res["out"] = out[:, :, :c["T"]]
+    if s["x"] is not None:
+        res["gate"] = gates[:, :, first:first + c["T"]]
     return res
