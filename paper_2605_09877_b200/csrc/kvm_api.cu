@@ -316,14 +316,6 @@ KVM_API kvm_status_t kvm_state_create(const kvm_config_t* cfg, kvm_state_t** out
   s.nsplitRoute = (int)((2 * 148 + U - 1) / U);
   if (s.nsplitRoute > kMaxSplits) s.nsplitRoute = kMaxSplits;
   if (s.nsplitRoute < 1) s.nsplitRoute = 1;
-  {
-    // decode CTAs serve up to eight query heads of a kv group; the row splits fill the GPU about four times
-    const int gq = (s.G % 8 == 0) ? 8 : (s.G % 4 == 0) ? 4 : (s.G % 2 == 0) ? 2 : 1;
-    const size_t ncta = (size_t)s.B * s.Hq / gq;
-    s.nsplitDec = (int)((4 * 148 + ncta - 1) / ncta);
-  }
-  if (s.nsplitDec > kMaxSplits) s.nsplitDec = kMaxSplits;
-  if (s.nsplitDec < 1) s.nsplitDec = 1;
 
   kvm_status_t rc = KVM_OK;
 #define A(ptr, count) if (rc == KVM_OK) rc = dev_alloc(ks, &(ptr), (count))
@@ -382,7 +374,6 @@ KVM_API kvm_status_t kvm_state_create(const kvm_config_t* cfg, kvm_state_t** out
   A(s.candV, U * (size_t)s.nsplitRoute * Cm * kTopK); A(s.candI, U * (size_t)s.nsplitRoute * Cm * kTopK);
   A(s.chunkMeta, U * (size_t)s.nsplitRoute * Cm * kChunkCap); A(s.chunkMax, U * (size_t)s.nsplitRoute * Cm * kChunkCap);
   if (rc == KVM_OK) rc = dev_alloc(ks, &s.chunkVal, U * (size_t)s.nsplitRoute * Cm * kChunkCap * 32, false);
-  A(s.decPart, (size_t)s.B * s.Hq * s.nsplitDec * (d + 2)); A(s.decQ, (size_t)s.B * s.Hq * d);
   // (tiles x splits: up to kAttnSplitTiles x kAttnMaxSplits, or 2 kAttnSplitTiles tiles of two splits)
   A(s.attnPart, (size_t)kAttnSplitTiles * kAttnMaxSplits * (d + 2) * 128); A(s.attnCnt, (size_t)2 * kAttnSplitTiles);
   if (rc == KVM_OK && cudaMemset(s.attnCnt, 0, 2 * kAttnSplitTiles * sizeof(int32_t)) != cudaSuccess) rc = KVM_ERR_CUDA;

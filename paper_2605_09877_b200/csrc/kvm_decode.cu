@@ -1,9 +1,15 @@
 // Single-token decode (Table 1 "Decode time per token"): one query per head attends over the
-// m readout rows of the state plus the window tokens [b, t].  The step is bound by HBM
-// bandwidth (it streams K_hat, V_hat and the window once), so the kernel is a streaming
-// reduction: every warp walks its share of the rows with 16-byte loads, keeps an online
-// softmax in registers, warps are merged with shuffles and shared memory, and row splits
-// (when there are too few heads to fill the GPU) are merged by a small second kernel.
+// m readout rows of the state plus the window tokens [b, t].  ONE kernel per step: every CTA rotates
+// the query heads it serves (and, where its rows end with the new token, that token's key), streams
+// its share of the rows with 16-byte loads into an online softmax, and the row splits of a head - a
+// thread-block cluster - merge their partial results through distributed shared memory.
+// What bounds it: with many heads HBM (K_hat, V_hat and the window are read once); with few the
+// latency of launch, first loads and merge, and on the host the launch itself, which is why the rotation of the
+// token and the merge are not kernels of their own: 32 heads over 256 + window rows took 1.9 + 7.4 + 3.1 us
+// in three kernels and 18.5 us per step on the host's side; now 9.5 us per step.  64 x 32 heads over 4096 + window
+// rows: 763 -> 716 us per step (6.57 TB/s), the set-up of a step under the tail of the one before.
+#include <cooperative_groups.h>
+
 #include "kvm_internal.h"
 #include "ln_rows.cuh"
 
@@ -14,138 +20,23 @@ __device__ __forceinline__ float rope_pair(float val, float oth, float cs, float
   return lower ? val * cs - oth * sn : oth * sn + val * cs;
 }
 
-// Rotates q and k of the new token, stores k, v, gate in the window ring and the rotated query
-// (rounded to bf16 exactly like the prefill staging) in decQ.
-__global__ void decode_ingest_kernel(const __nv_bfloat16* __restrict__ q, const __nv_bfloat16* __restrict__ k,
-                                     const __nv_bfloat16* __restrict__ v, const float* __restrict__ gate,
-                                     const double* __restrict__ inv_freq, __half* __restrict__ decQ,
-                                     __half* __restrict__ ringK, __half* __restrict__ ringV,
-                                     float* __restrict__ ringG, int nQ, int nKV, int d, int r, int64_t t,
-                                     int64_t ringCap, int64_t ringLen, int32_t* __restrict__ sat_counter) {
-  // blocks [0, nQ): query heads; blocks [nQ, nQ + nKV): kv units
-  const int x = threadIdx.x;
-  if (x >= d) return;
-  const int half = r >> 1;
-  float cs = 1.f, sn = 0.f;
-  int partner = x;
-  if (x < r) {
-    const int pidx = x < half ? x : x - half;
-    double s, c;
-    sincos((double)t * inv_freq[pidx], &s, &c);
-    cs = (float)c; sn = (float)s;
-    partner = x < half ? x + half : x - half;
-  }
-  if ((int)blockIdx.x < nQ) {
-    const __nv_bfloat16* row = q + (int64_t)blockIdx.x * d;
-    const float val = __bfloat162float(row[x]);
-    const float oth = __bfloat162float(row[partner]);
-    const float o = (x < r) ? rope_pair(val, oth, cs, sn, x < half) : val;
-    if (!(fabsf(o) <= 65504.f)) atomicAdd(sat_counter, 1);   // (clamped: counted for the debug counter)
-    decQ[(int64_t)blockIdx.x * d + x] = __float2half_rn(fminf(fmaxf(o, -65504.f), 65504.f));
-  } else {
-    const int u = blockIdx.x - nQ;
-    const __nv_bfloat16* row = k + (int64_t)u * d;
-    const float val = __bfloat162float(row[x]);
-    const float oth = __bfloat162float(row[partner]);
-    const float o = (x < r) ? rope_pair(val, oth, cs, sn, x < half) : val;
-    const int64_t rrow = (int64_t)u * ringCap + (t % ringLen);
-    const float vv = __bfloat162float(v[(int64_t)u * d + x]);
-    const int nsat = (!(fabsf(o) <= 65504.f) ? 1 : 0) + (!(fabsf(vv) <= 65504.f) ? 1 : 0);
-    if (nsat) atomicAdd(sat_counter, nsat);
-    ringK[rrow * d + x] = __float2half_rn(fminf(fmaxf(o, -65504.f), 65504.f));
-    ringV[rrow * d + x] = __float2half_rn(fminf(fmaxf(vv, -65504.f), 65504.f));
-    if (x == 0) ringG[rrow] = gate ? gate[u] : 1.0f;
-  }
-}
-
-// The same with LN_q / LN_k applied first (fused front end): one warp per head, d / 8 lanes hold the row as
-// eight channels each (ln_chunk8: the arithmetic of kvm_head_layernorm), the other lane groups compute
-// copies and store nothing.  Rotation as in decode_ingest_kernel, the partner channel comes from the lane
-// that holds it.
-template <int D>
-__global__ void __launch_bounds__(32) decode_ingest_ln_kernel(const __nv_bfloat16* __restrict__ q, const __nv_bfloat16* __restrict__ k,
-                                        const __nv_bfloat16* __restrict__ v, const float* __restrict__ gate,
-                                        const double* __restrict__ inv_freq, __half* __restrict__ decQ,
-                                        __half* __restrict__ ringK, __half* __restrict__ ringV, float* __restrict__ ringG,
-                                        int nQ, int nKV, int Hq, int Hkv, int r, int64_t t, int64_t ringCap, int64_t ringLen,
-                                        int32_t* __restrict__ sat_counter, const float* __restrict__ lnq_w,
-                                        const float* __restrict__ lnq_b, const float* __restrict__ lnk_w,
-                                        const float* __restrict__ lnk_b, float eps) {
-  constexpr int LPR = D / 8;
-  const int lane = threadIdx.x, sub = lane % LPR;
-  const bool store = lane < LPR;
-  const bool isq = (int)blockIdx.x < nQ;
-  const int idx = isq ? blockIdx.x : blockIdx.x - nQ;
-  const int h = isq ? idx % Hq : idx % Hkv;
-  const __nv_bfloat16* row = (isq ? q : k) + (int64_t)idx * D;
-  float x[8];
-  {
-    const uint4 raw = *reinterpret_cast<const uint4*>(row + sub * 8);
-    const __nv_bfloat162* pv = reinterpret_cast<const __nv_bfloat162*>(&raw);
-#pragma unroll
-    for (int i = 0; i < 4; ++i) {
-      const float2 f = __bfloat1622float2(pv[i]);
-      x[2 * i] = f.x; x[2 * i + 1] = f.y;
-    }
-  }
-  float w8[8], b8[8];
-  ln_load_affine<D>(isq ? lnq_w : lnk_w, isq ? lnq_b : lnk_b, h, sub, w8, b8);
-  ln_chunk8<D>(x, w8, b8, eps);
-  const int half = r >> 1;
-  float o[8];
-#pragma unroll
-  for (int i = 0; i < 8; ++i) o[i] = x[i];
-  if (r > 0) {   // (uniform; r / 2 is a multiple of 8, so a partner chunk is a whole lane's)
-    const int ch0 = sub * 8;
-    const bool inr = ch0 < r, lower = ch0 < half;
-    const int src = (lane & ~(LPR - 1)) + (inr ? (lower ? sub + half / 8 : sub - half / 8) : sub);
-#pragma unroll
-    for (int i = 0; i < 8; ++i) {
-      const float oth = __shfl_sync(0xffffffffu, x[i], src);
-      if (inr) {
-        const int pidx = (lower ? ch0 : ch0 - half) + i;
-        double sn, cs;
-        sincos((double)t * inv_freq[pidx], &sn, &cs);
-        o[i] = rope_pair(x[i], oth, (float)cs, (float)sn, lower);
-      }
-    }
-  }
-  if (!store) return;
-  int nsat = 0;
-  __half hv[8];
-#pragma unroll
-  for (int i = 0; i < 8; ++i) {
-    nsat += !(fabsf(o[i]) <= 65504.f) ? 1 : 0;
-    hv[i] = __float2half_rn(fminf(fmaxf(o[i], -65504.f), 65504.f));
-  }
-  if (isq) {
-    *reinterpret_cast<uint4*>(decQ + (int64_t)idx * D + sub * 8) = *reinterpret_cast<const uint4*>(hv);
-  } else {
-    const int64_t rrow = (int64_t)idx * ringCap + (t % ringLen);
-    *reinterpret_cast<uint4*>(ringK + rrow * D + sub * 8) = *reinterpret_cast<const uint4*>(hv);
-    __half vh[8];
-    const uint4 raw = *reinterpret_cast<const uint4*>(v + (int64_t)idx * D + sub * 8);
-    const __nv_bfloat162* pv = reinterpret_cast<const __nv_bfloat162*>(&raw);
-#pragma unroll
-    for (int i = 0; i < 4; ++i) {
-      const float2 f = __bfloat1622float2(pv[i]);
-      nsat += (!(fabsf(f.x) <= 65504.f) ? 1 : 0) + (!(fabsf(f.y) <= 65504.f) ? 1 : 0);
-      vh[2 * i] = __float2half_rn(fminf(fmaxf(f.x, -65504.f), 65504.f));
-      vh[2 * i + 1] = __float2half_rn(fminf(fmaxf(f.y, -65504.f), 65504.f));
-    }
-    *reinterpret_cast<uint4*>(ringV + rrow * D + sub * 8) = *reinterpret_cast<const uint4*>(vh);
-    if (sub == 0) ringG[rrow] = gate ? gate[idx] : 1.0f;
-  }
-  if (nsat) atomicAdd(sat_counter, nsat);
-}
-
 struct DecodeParams {
-  const __half *decQ, *Khat, *Vhat, *ringK, *ringV;
+  const __nv_bfloat16 *q, *k, *v;   // [B*Hq, D], [U, D]
+  const float* gate;                // [U] or NULL
+  const double* inv_freq;
+  const float *lnq_w, *lnq_b, *lnk_w, *lnk_b;
+  const __half *Khat, *Vhat;
+  __half *ringK, *ringV;
+  float* ringG;
   const float *tau_s, *tau_b;
   __nv_bfloat16* out;
-  float* part;     // [B*Hq, nsplit, D + 2]
-  int64_t Mcap, ringCap, ringLen, m, b, t;
-  int Hq, Hkv, G, nsplit;
+  int32_t* sat_counter;
+  int64_t Mcap, ringCap, t;
+  int m, n;              // state rows; all rows: m + window tokens, the new one last
+  int ringLen, slot_b;   // ring slot of the window's first token
+  int slot_t;            // ring slot of the new token
+  int Hq, Hkv, G, nsplit, r;
+  float qk_ln_eps;
 };
 
 __device__ __forceinline__ void unpack8(const uint4& w, float (&f)[8]) {
@@ -163,19 +54,144 @@ __device__ __forceinline__ uint4 ldg_stream(const void* p) {
   return r;
 }
 
-// grid (nsplit, B*Hq / GQ); block 256 = 8 warps.  LPR = D/8 lanes cover one row with 16-byte loads,
-// a warp covers RPW = 32/LPR rows per load instruction and UNR such instructions per step.  A CTA
-// serves GQ query heads that share one kv head (grouped queries): every key / value row is loaded
-// once and meets all GQ queries, so the bytes streamed per step do not grow with the group size.
+// The new token's share of a CTA's set-up: the query heads [bh0, bh0 + GQ) rotated into s_q, and, where `fresh`
+// (the CTA's rows end with the new token), its rotated key and its value into s_new; the first query head's CTA of a
+// kv group (`store`) also writes them to the window ring, and `count_q` says which CTA of a head counts the inputs that
+// had to be clamped to the fp16 range.  Plain rows: one thread per channel.
 template <int D, int GQ>
-__global__ void __launch_bounds__(256) decode_attn_kernel(DecodeParams p) {
+__device__ __forceinline__ void new_token(const DecodeParams& p, int bh0, int64_t u, bool fresh, bool store, bool count_q,
+                                          __half (*s_q)[D], __half (*s_new)[D]) {
+  const int x = threadIdx.x % D;
+  const int half = p.r >> 1;
+  float cs = 1.f, sn = 0.f;
+  int partner = x;
+  if (x < p.r) {
+    const int pidx = x < half ? x : x - half;
+    double s, c;
+    sincos((double)p.t * p.inv_freq[pidx], &s, &c);
+    cs = (float)c; sn = (float)s;
+    partner = x < half ? x + half : x - half;
+  }
+  // (the step before this one, or whatever wrote the inputs and the rows, may still be running up to here)
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  int nsat = 0;
+  for (int i = threadIdx.x / D; i < GQ + (fresh ? 1 : 0); i += 256 / D) {
+    const bool isq = i < GQ;
+    const __nv_bfloat16* row = isq ? p.q + (int64_t)(bh0 + i) * D : p.k + u * D;
+    const float val = __bfloat162float(row[x]), oth = __bfloat162float(row[partner]);
+    const float o = (x < p.r) ? rope_pair(val, oth, cs, sn, x < half) : val;
+    const __half h = __float2half_rn(fminf(fmaxf(o, -65504.f), 65504.f));
+    const int sat = !(fabsf(o) <= 65504.f) ? 1 : 0;
+    if (isq) {
+      s_q[i][x] = h;
+      if (count_q) nsat += sat;
+    } else {
+      const float vv = __bfloat162float(p.v[u * D + x]);
+      const __half hv = __float2half_rn(fminf(fmaxf(vv, -65504.f), 65504.f));
+      s_new[0][x] = h; s_new[1][x] = hv;
+      if (store) {
+        const int64_t at = (u * p.ringCap + p.slot_t) * D + x;
+        p.ringK[at] = h; p.ringV[at] = hv;
+        nsat += sat + (!(fabsf(vv) <= 65504.f) ? 1 : 0);
+      }
+    }
+  }
+  if (nsat) atomicAdd(p.sat_counter, nsat);
+}
+
+// The same with LN_q / LN_k applied first (fused front end): one warp per row, d / 8 lanes hold it as eight channels
+// each (ln_chunk8: the arithmetic of kvm_head_layernorm), the other lane groups compute copies and store nothing.
+// The partner channel of the rotation comes from the lane that holds it.
+template <int D, int GQ>
+__device__ __forceinline__ void new_token_ln(const DecodeParams& p, int bh0, int64_t u, bool fresh, bool store, bool count_q,
+                                             __half (*s_q)[D], __half (*s_new)[D]) {
+  constexpr int LPR = D / 8;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, sub = lane % LPR;
+  const int half = p.r >> 1, ch0 = sub * 8;
+  const bool inr = ch0 < p.r, lower = ch0 < half;   // (r / 2 is a multiple of 8: a partner chunk is a whole lane's)
+  float cs[8], sn[8];
+#pragma unroll
+  for (int i = 0; i < 8; ++i) { cs[i] = 1.f; sn[i] = 0.f; }
+  if (inr && warp < GQ + (fresh ? 1 : 0)) {
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+      double s, c;
+      sincos((double)p.t * p.inv_freq[(lower ? ch0 : ch0 - half) + i], &s, &c);
+      cs[i] = (float)c; sn[i] = (float)s;
+    }
+  }
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  int nsat = 0;
+  for (int row_i = warp; row_i < GQ + (fresh ? 1 : 0); row_i += 8) {   // (uniform over the warp)
+    const bool isq = row_i < GQ;
+    const int h = isq ? (bh0 + row_i) % p.Hq : (int)(u % p.Hkv);
+    float x[8];
+    {
+      const uint4 raw = *reinterpret_cast<const uint4*>((isq ? p.q + (int64_t)(bh0 + row_i) * D : p.k + u * D) + ch0);
+      const __nv_bfloat162* pv = reinterpret_cast<const __nv_bfloat162*>(&raw);
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        const float2 f = __bfloat1622float2(pv[i]);
+        x[2 * i] = f.x; x[2 * i + 1] = f.y;
+      }
+    }
+    float w8[8], b8[8];
+    ln_load_affine<D>(isq ? p.lnq_w : p.lnk_w, isq ? p.lnq_b : p.lnk_b, h, sub, w8, b8);
+    ln_chunk8<D>(x, w8, b8, p.qk_ln_eps);
+    const int src = (lane & ~(LPR - 1)) + (inr ? (lower ? sub + half / 8 : sub - half / 8) : sub);
+    alignas(16) __half hv[8];
+    int sat = 0;
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+      const float oth = __shfl_sync(0xffffffffu, x[i], src);
+      const float o = inr ? rope_pair(x[i], oth, cs[i], sn[i], lower) : x[i];
+      sat += !(fabsf(o) <= 65504.f) ? 1 : 0;
+      hv[i] = __float2half_rn(fminf(fmaxf(o, -65504.f), 65504.f));
+    }
+    if (lane >= LPR) continue;
+    if (isq) {
+      *reinterpret_cast<uint4*>(&s_q[row_i][ch0]) = *reinterpret_cast<const uint4*>(hv);
+      if (count_q) nsat += sat;
+    } else {
+      alignas(16) __half vh[8];
+      const uint4 raw = *reinterpret_cast<const uint4*>(p.v + u * D + ch0);
+      const __nv_bfloat162* pv = reinterpret_cast<const __nv_bfloat162*>(&raw);
+#pragma unroll
+      for (int i = 0; i < 4; ++i) {
+        const float2 f = __bfloat1622float2(pv[i]);
+        sat += (!(fabsf(f.x) <= 65504.f) ? 1 : 0) + (!(fabsf(f.y) <= 65504.f) ? 1 : 0);
+        vh[2 * i] = __float2half_rn(fminf(fmaxf(f.x, -65504.f), 65504.f));
+        vh[2 * i + 1] = __float2half_rn(fminf(fmaxf(f.y, -65504.f), 65504.f));
+      }
+      *reinterpret_cast<uint4*>(&s_new[0][ch0]) = *reinterpret_cast<const uint4*>(hv);
+      *reinterpret_cast<uint4*>(&s_new[1][ch0]) = *reinterpret_cast<const uint4*>(vh);
+      if (store) {
+        const int64_t at = (u * p.ringCap + p.slot_t) * D + ch0;
+        *reinterpret_cast<uint4*>(p.ringK + at) = *reinterpret_cast<const uint4*>(hv);
+        *reinterpret_cast<uint4*>(p.ringV + at) = *reinterpret_cast<const uint4*>(vh);
+        nsat += sat;
+      }
+    }
+  }
+  if (nsat) atomicAdd(p.sat_counter, nsat);
+}
+
+// grid (nsplit, B*Hq / GQ), the nsplit CTAs of a row a cluster; block 256 = 8 warps.  LPR = D/8 lanes cover one
+// row with 16-byte loads, a warp covers RPW = 32/LPR rows per load instruction and UNR such instructions per
+// step.  A CTA serves GQ query heads that share one kv head (grouped queries): every key / value row is loaded
+// once and meets all GQ queries, so the bytes streamed per step do not grow with the group size.
+template <int D, int GQ, bool LN>
+__global__ void __launch_bounds__(256) decode_step_kernel(DecodeParams p) {
   constexpr int LPR = D / 8;
   constexpr int RPW = 32 / LPR;
   constexpr int UNR = 4;
   constexpr int STEP = RPW * UNR;       // rows per warp per iteration
   __shared__ float s_m[8][GQ], s_l[8][GQ];
-  __shared__ float s_acc[8][GQ][D];
+  __shared__ __align__(16) float s_acc[8][GQ][D];
+  __shared__ float s_part[GQ][D + 2];   // this split's merged result: channels, maximum, sum
+  __shared__ __align__(16) __half s_q[GQ][D], s_new[2][D];
 
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   const int split = blockIdx.x;
   const int bh0 = blockIdx.y * GQ;                 // first query head of this CTA (GQ divides the group size G)
   const int bb = bh0 / p.Hq, hq0 = bh0 % p.Hq, hk = hq0 / p.G;
@@ -183,12 +199,17 @@ __global__ void __launch_bounds__(256) decode_attn_kernel(DecodeParams p) {
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int grp = lane / LPR, gl = lane % LPR;   // row group inside the warp, lane inside the row
 
-  const int64_t m = p.m;
-  const int64_t n = m + (p.t - p.b + 1);
-  int64_t per = (n + p.nsplit - 1) / p.nsplit;
+  const int m = p.m, n = p.n;
+  int per = (n + p.nsplit - 1) / p.nsplit;
   per = (per + 8 * STEP - 1) / (8 * STEP) * (8 * STEP);
-  const int64_t r0 = (int64_t)split * per;
-  const int64_t r1 = min(n, r0 + per);
+  const int r0 = split * per;
+  const int r1 = min(n, r0 + per);
+  const bool fresh = r0 < n && r1 == n;          // this CTA's rows end with the new token
+
+  if (LN) new_token_ln<D, GQ>(p, bh0, u, fresh, fresh && hq0 % p.G == 0, split == 0, s_q, s_new);
+  else new_token<D, GQ>(p, bh0, u, fresh, fresh && hq0 % p.G == 0, split == 0, s_q, s_new);
+  if (fresh && hq0 % p.G == 0 && tid == 0) p.ringG[u * p.ringCap + p.slot_t] = p.gate ? p.gate[u] : 1.0f;
+  __syncthreads();
 
   const float kLog2e = 1.4426950408889634f;
   float scale_s[GQ], scale_b[GQ];
@@ -197,8 +218,7 @@ __global__ void __launch_bounds__(256) decode_attn_kernel(DecodeParams p) {
   for (int g = 0; g < GQ; ++g) {
     scale_s[g] = p.tau_s[hq0 + g] * rsqrtf((float)D) * kLog2e;
     scale_b[g] = p.tau_b[hq0 + g] * rsqrtf((float)D) * kLog2e;
-    const uint4 qw = *reinterpret_cast<const uint4*>(p.decQ + (int64_t)(bh0 + g) * D + gl * 8);
-    unpack8(qw, qf[g]);
+    unpack8(*reinterpret_cast<const uint4*>(&s_q[g][gl * 8]), qf[g]);
   }
   float m_run[GQ], l_run[GQ];
   float acc[GQ][8];
@@ -209,32 +229,36 @@ __global__ void __launch_bounds__(256) decode_attn_kernel(DecodeParams p) {
     for (int c = 0; c < 8; ++c) acc[g][c] = 0.f;
   }
 
-  const __half* KhatU = p.Khat + u * p.Mcap * D;
-  const __half* VhatU = p.Vhat + u * p.Mcap * D;
-  const __half* ringKU = p.ringK + u * p.ringCap * D;
-  const __half* ringVU = p.ringV + u * p.ringCap * D;
+  const __half* KhatU = p.Khat + u * p.Mcap * D + gl * 8;
+  const __half* VhatU = p.Vhat + u * p.Mcap * D + gl * 8;
+  const __half* ringKU = p.ringK + u * p.ringCap * D + gl * 8;
+  const __half* ringVU = p.ringV + u * p.ringCap * D + gl * 8;
 
-  for (int64_t base = r0 + (int64_t)warp * STEP; base < r1; base += 8 * STEP) {
+  for (int base = r0 + warp * STEP; base < r1; base += 8 * STEP) {
     uint4 kw[UNR], vw[UNR];
     bool ok[UNR];
     bool st_[UNR];
 #pragma unroll
     for (int i = 0; i < UNR; ++i) {
-      const int64_t row = base + i * RPW + grp;
+      const int row = base + i * RPW + grp;
       ok[i] = row < r1;
       st_[i] = row < m;
-      if (ok[i]) {
+      if (ok[i] && row < n - 1) {
         const __half *kp, *vp;
         if (st_[i]) {
-          kp = KhatU + row * D;
-          vp = VhatU + row * D;
+          kp = KhatU + (int64_t)row * D;
+          vp = VhatU + (int64_t)row * D;
         } else {
-          const int64_t slot = (p.b + (row - m)) % p.ringLen;
-          kp = ringKU + slot * D;
-          vp = ringVU + slot * D;
+          int slot = p.slot_b + (row - m);   // (the window is no longer than the ring)
+          if (slot >= p.ringLen) slot -= p.ringLen;
+          kp = ringKU + (int64_t)slot * D;
+          vp = ringVU + (int64_t)slot * D;
         }
-        kw[i] = ldg_stream(kp + gl * 8);
-        vw[i] = ldg_stream(vp + gl * 8);
+        kw[i] = ldg_stream(kp);
+        vw[i] = ldg_stream(vp);
+      } else if (ok[i]) {   // the new token
+        kw[i] = *reinterpret_cast<const uint4*>(&s_new[0][gl * 8]);
+        vw[i] = *reinterpret_cast<const uint4*>(&s_new[1][gl * 8]);
       } else {
         kw[i] = make_uint4(0, 0, 0, 0);
         vw[i] = make_uint4(0, 0, 0, 0);
@@ -297,95 +321,95 @@ __global__ void __launch_bounds__(256) decode_attn_kernel(DecodeParams p) {
     }
   }
   __syncthreads();
-  if (tid < D) {
+  for (int e = tid; e < GQ * D; e += 256) {
+    const int g = e / D, x = e % D;
+    float mx = -INFINITY;
 #pragma unroll
-    for (int g = 0; g < GQ; ++g) {
-      float mx = -INFINITY;
+    for (int w = 0; w < 8; ++w) mx = fmaxf(mx, s_m[w][g]);
+    float l = 0.f, a = 0.f;
 #pragma unroll
-      for (int w = 0; w < 8; ++w) mx = fmaxf(mx, s_m[w][g]);
-      float l = 0.f, a = 0.f;
-#pragma unroll
-      for (int w = 0; w < 8; ++w) {
-        const float f = (s_m[w][g] == -INFINITY) ? 0.f : exp2f(s_m[w][g] - mx);
-        l += s_l[w][g] * f;
-        a += s_acc[w][g][tid] * f;
-      }
-      const int64_t bh = bh0 + g;
-      if (p.nsplit == 1) {
-        p.out[bh * D + tid] = __float2bfloat16_rn(a / l);
-      } else {
-        float* dst = p.part + (bh * p.nsplit + split) * (D + 2);
-        dst[tid] = a;
-        if (tid == 0) { dst[D] = mx; dst[D + 1] = l; }
-      }
+    for (int w = 0; w < 8; ++w) {
+      const float f = (s_m[w][g] == -INFINITY) ? 0.f : exp2f(s_m[w][g] - mx);
+      l += s_l[w][g] * f;
+      a += s_acc[w][g][x] * f;
+    }
+    if (p.nsplit == 1) {
+      p.out[(int64_t)(bh0 + g) * D + x] = __float2bfloat16_rn(a / l);
+    } else {
+      s_part[g][x] = a;
+      if (x == 0) { s_part[g][D] = mx; s_part[g][D + 1] = l; }
     }
   }
+  if (p.nsplit == 1) return;
+  // the splits of these heads: every CTA of the cluster merges its share of the channels
+  cooperative_groups::cluster_group cl = cooperative_groups::this_cluster();
+  cl.sync();
+  const int share = (GQ * D + p.nsplit - 1) / p.nsplit;
+  for (int e = split * share + tid; e < min(GQ * D, (split + 1) * share); e += 256) {
+    const int g = e / D, x = e % D;
+    const float* mine = &s_part[g][0];
+    float mx = -INFINITY;
+    for (int z = 0; z < p.nsplit; ++z) mx = fmaxf(mx, cl.map_shared_rank(mine, z)[D]);
+    float l = 0.f, a = 0.f;
+    for (int z = 0; z < p.nsplit; ++z) {
+      const float* pz = cl.map_shared_rank(mine, z);
+      const float ms = pz[D];
+      const float f = (ms == -INFINITY) ? 0.f : exp2f(ms - mx);
+      l += pz[D + 1] * f;
+      a += pz[x] * f;
+    }
+    p.out[(int64_t)(bh0 + g) * D + x] = __float2bfloat16_rn(a / l);
+  }
+  cl.sync();   // (no CTA leaves while another still reads its shared memory)
 }
 
-template <int D>
-__global__ void decode_combine_kernel(const float* __restrict__ part, __nv_bfloat16* __restrict__ out, int nsplit) {
-  const int bh = blockIdx.x, x = threadIdx.x;
-  if (x >= D) return;
-  const float* src = part + (int64_t)bh * nsplit * (D + 2);
-  float mx = -INFINITY;
-  for (int s = 0; s < nsplit; ++s) mx = fmaxf(mx, src[s * (D + 2) + D]);
-  float l = 0.f, a = 0.f;
-  for (int s = 0; s < nsplit; ++s) {
-    const float ms = src[s * (D + 2) + D];
-    const float f = (ms == -INFINITY) ? 0.f : exp2f(ms - mx);
-    l += src[s * (D + 2) + D + 1] * f;
-    a += src[s * (D + 2) + x] * f;
-  }
-  out[(int64_t)bh * D + x] = __float2bfloat16_rn(a / l);
+template <int D, int GQ, bool LN>
+static bool launch_decode_step(const DecodeParams& p, int ncta, bool early, cudaStream_t s) {
+  cudaLaunchConfig_t lc = {};
+  lc.gridDim = dim3(p.nsplit, ncta); lc.blockDim = dim3(256); lc.stream = s;
+  cudaLaunchAttribute at[2];
+  // the set-up of this step (launch, the rotation's angles) runs under the tail of the kernel before it on the stream
+  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[0].val.programmaticStreamSerializationAllowed = early ? 1 : 0;
+  at[1].id = cudaLaunchAttributeClusterDimension;
+  at[1].val.clusterDim.x = p.nsplit; at[1].val.clusterDim.y = 1; at[1].val.clusterDim.z = 1;
+  lc.attrs = at; lc.numAttrs = p.nsplit > 1 ? 2 : 1;
+  return cudaLaunchKernelEx(&lc, decode_step_kernel<D, GQ, LN>, p) == cudaSuccess;
 }
+
+// query heads of one kv group share a CTA: the largest of 8, 4, 2, 1 that divides the group size
+static int decode_heads_per_cta(const State* st) { return (st->G % 8 == 0) ? 8 : (st->G % 4 == 0) ? 4 : (st->G % 2 == 0) ? 2 : 1; }
+
+#define KVM_DEC_EACH(F)                                                                                                 \
+  F(128, 8, true) F(128, 4, true) F(128, 2, true) F(128, 1, true) F(64, 8, true) F(64, 4, true) F(64, 2, true) F(64, 1, true) \
+  F(128, 8, false) F(128, 4, false) F(128, 2, false) F(128, 1, false) F(64, 8, false) F(64, 4, false) F(64, 2, false) F(64, 1, false)
 
 int launch_decode(State* st, const DecodeArgs& a, cudaStream_t s) {
-  int launches = 0;
-  const int D = st->d;
-  const int nQ = st->B * st->Hq, nKV = st->U;
-  if (st->fusedLn) {
-#define KVM_DEC_LN(DD)                                                                                                        \
-    decode_ingest_ln_kernel<DD><<<nQ + nKV, 32, 0, s>>>(a.q, a.k, a.v, a.gate, st->inv_freq, st->decQ, st->ringK, st->ringV,   \
-                                                        st->ringG, nQ, nKV, st->Hq, st->Hkv, st->r, a.t,                      \
-                                                        (int64_t)st->w * st->Cmax, st->ringLen, st->status + 4, st->lnq_w,    \
-                                                        st->lnq_b, st->lnk_w, st->lnk_b, st->qk_ln_eps)
-    if (D == 128) { KVM_DEC_LN(128); } else { KVM_DEC_LN(64); }
-#undef KVM_DEC_LN
-  } else {
-    decode_ingest_kernel<<<nQ + nKV, D, 0, s>>>(a.q, a.k, a.v, a.gate, st->inv_freq, st->decQ, st->ringK, st->ringV,
-                                                st->ringG, nQ, nKV, D, st->r, a.t, (int64_t)st->w * st->Cmax,
-                                                st->ringLen, st->status + 4);
-  }
-  ++launches;
+  const int nQ = st->B * st->Hq, GQ = decode_heads_per_cta(st);
   DecodeParams p;
-  p.decQ = st->decQ; p.Khat = st->KhatBuf[st->nfolds & 1]; p.Vhat = st->VhatBuf[st->nfolds & 1]; p.ringK = st->ringK; p.ringV = st->ringV;
-  p.tau_s = st->tau_s; p.tau_b = st->tau_b; p.out = a.out; p.part = st->decPart;
-  p.Mcap = st->Mcap; p.ringCap = (int64_t)st->w * st->Cmax; p.ringLen = st->ringLen;
-  p.m = a.m; p.b = a.b; p.t = a.t;
-  p.Hq = st->Hq; p.Hkv = st->Hkv; p.G = st->G;
-  // query heads of one kv group share a CTA (the largest of 8, 4, 2, 1 that divides the group size)
-  const int GQ = (st->G % 8 == 0) ? 8 : (st->G % 4 == 0) ? 4 : (st->G % 2 == 0) ? 2 : 1;
-  const int nCta = nQ / GQ;
-  // splits: fill ~4 CTAs per SM, keep at least 256 rows per split
-  const int64_t n = a.m + (a.t - a.b + 1);
-  int64_t want = (4 * 148 + nCta - 1) / nCta;
-  int64_t maxs = (n + 255) / 256;
-  int nsplit = (int)(want < maxs ? want : maxs);
-  if (nsplit < 1) nsplit = 1;
-  if (nsplit > st->nsplitDec) nsplit = st->nsplitDec;
+  p.q = a.q; p.k = a.k; p.v = a.v; p.gate = a.gate; p.inv_freq = st->inv_freq;
+  p.lnq_w = st->lnq_w; p.lnq_b = st->lnq_b; p.lnk_w = st->lnk_w; p.lnk_b = st->lnk_b; p.qk_ln_eps = st->qk_ln_eps;
+  p.Khat = st->KhatBuf[st->nfolds & 1]; p.Vhat = st->VhatBuf[st->nfolds & 1];
+  p.ringK = st->ringK; p.ringV = st->ringV; p.ringG = st->ringG;
+  p.tau_s = st->tau_s; p.tau_b = st->tau_b; p.out = a.out; p.sat_counter = st->status + 4;
+  p.Mcap = st->Mcap; p.ringCap = (int64_t)st->w * st->Cmax; p.t = a.t;
+  p.m = (int)a.m; p.n = (int)(a.m + (a.t - a.b + 1));
+  p.ringLen = (int)st->ringLen; p.slot_b = (int)(a.b % st->ringLen); p.slot_t = (int)(a.t % st->ringLen);
+  p.Hq = st->Hq; p.Hkv = st->Hkv; p.G = st->G; p.r = st->r;
+  // Row splits: a power of two up to the portable cluster size (clusters of 16 took 13.5 us per step where 8 take 8.5),
+  // until there are two CTAs per SM, and no more than give every split one step of its eight warps (64 or 128 rows).
+  // Measured per step of 32 heads over 256 + window rows, one / two / three / four CTAs per SM: 9.7 / 9.5 / 9.7 /
+  // 10.2 us; of 8 groups of four heads: 11.3 / 10.6 / 10.7 / 10.7 us.
+  const int nCta = nQ / GQ, rows1 = 8 * 4 * (256 / st->d);
+  int nsplit = 1;
+  while (nsplit < 8 && nsplit * nCta < 2 * 148 && nsplit * rows1 < p.n) nsplit *= 2;
   p.nsplit = nsplit;
-  dim3 grid(nsplit, nCta);
-#define KVM_DEC(DD, GG) decode_attn_kernel<DD, GG><<<grid, 256, 0, s>>>(p)
-  if (D == 128) { if (GQ == 8) KVM_DEC(128, 8); else if (GQ == 4) KVM_DEC(128, 4); else if (GQ == 2) KVM_DEC(128, 2); else KVM_DEC(128, 1); }
-  else { if (GQ == 8) KVM_DEC(64, 8); else if (GQ == 4) KVM_DEC(64, 4); else if (GQ == 2) KVM_DEC(64, 2); else KVM_DEC(64, 1); }
-#undef KVM_DEC
-  ++launches;
-  if (nsplit > 1) {
-    if (D == 128) decode_combine_kernel<128><<<nQ, 128, 0, s>>>(st->decPart, a.out, nsplit);
-    else decode_combine_kernel<64><<<nQ, 64, 0, s>>>(st->decPart, a.out, nsplit);
-    ++launches;
-  }
-  return launches;
+  const bool early = st->prof_hook == nullptr;
+#define KVM_DEC_GO(DD, GG, LL) \
+  if (st->d == DD && GQ == GG && st->fusedLn == LL) launch_decode_step<DD, GG, LL>(p, nCta, early, s);
+  KVM_DEC_EACH(KVM_DEC_GO)
+#undef KVM_DEC_GO
+  return 1;
 }
 
 }  // namespace kvm

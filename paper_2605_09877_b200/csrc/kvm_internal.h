@@ -12,7 +12,7 @@ namespace kvm {
 constexpr int kMaxBlock = 256;      // largest block C (one thread per overflow token in the fold)
 constexpr int kTopK = 8;            // routing filter keeps at most K candidate rows per (token, row split)
 constexpr int kChunkCap = 16;       // 32-row chunks of approximate similarities the routing filter can record per (token, row split)
-constexpr int kMaxSplits = 32;      // routing filter / decode split count upper bound
+constexpr int kMaxSplits = 32;      // routing filter split count upper bound
 constexpr int kAttnSplitTiles = 37; // launches with at most this many (batch, head, query tile) CTAs - a quarter of the GPU - are split along the keys
 constexpr int kAttnMaxSplits = 8;
 constexpr int kRowAlign = 128;      // state capacity is rounded up to the attention key tile
@@ -114,10 +114,6 @@ struct State {
   // ---- split-KV attention scratch (device) ----
   float* attnPart;               // [kAttnSplitTiles][kAttnMaxSplits][d + 2][128]
   int32_t* attnCnt;              // [2 kAttnSplitTiles] tickets
-  // ---- decode scratch (device) ----
-  int nsplitDec;
-  float* decPart;                // [B*Hq, nsplitDec, d + 2]
-  __half* decQ;                  // [B*Hq, d] rotated query
   // ---- optional per-kernel timing hook (set by kvm_profile_enable): phase ids
   //      0 ingest, 1 attention, 2 memory keys, 3 routing filter, 4 decide, 5 apply, 6 decode ----
   void (*prof_hook)(void* ctx, int phase, int begin, cudaStream_t s);
