@@ -176,6 +176,26 @@ __device__ __forceinline__ void new_token_ln(const DecodeParams& p, int bh0, int
   if (nsat) atomicAdd(p.sat_counter, nsat);
 }
 
+// Sums of LEFT values over 2 O lanes: a lane with bit O set goes on with the upper half of the values that are left, the
+// other one with the lower half; a single value left is summed over the remaining lanes.
+template <int LEFT, int O, int N>
+__device__ __forceinline__ void lane_sums(float (&v)[N], int gl) {
+  if constexpr (O > 0) {
+    if constexpr (LEFT > 1) {
+      const bool up = gl & O;
+#pragma unroll
+      for (int k = 0; k < LEFT / 2; ++k) {
+        const float give = up ? v[k] : v[k + LEFT / 2], keep = up ? v[k + LEFT / 2] : v[k];
+        v[k] = keep + __shfl_xor_sync(0xffffffffu, give, O);
+      }
+      lane_sums<LEFT / 2, O / 2>(v, gl);
+    } else {
+      v[0] += __shfl_xor_sync(0xffffffffu, v[0], O);
+      lane_sums<1, O / 2>(v, gl);
+    }
+  }
+}
+
 // grid (nsplit, B*Hq / GQ), the nsplit CTAs of a row a cluster; block 256 = 8 warps.  LPR = D/8 lanes cover one
 // row with 16-byte loads, a warp covers RPW = 32/LPR rows per load instruction and UNR such instructions per
 // step.  A CTA serves GQ query heads that share one kv head (grouped queries): every key / value row is loaded
@@ -211,23 +231,26 @@ __global__ void __launch_bounds__(256) decode_step_kernel(DecodeParams p) {
   if (fresh && hq0 % p.G == 0 && tid == 0) p.ringG[u * p.ringCap + p.slot_t] = p.gate ? p.gate[u] : 1.0f;
   __syncthreads();
 
+  // Which of a step's GQ * UNR logits of a row group a lane ends up with (index g * UNR + i: head g, row i of the
+  // group): the reduction over the LPR lanes of a row halves the values together with the lanes, so every sum costs
+  // about one exchange instead of log2(LPR) and every exponential is taken once.
+  constexpr int NV = GQ * UNR;
+  constexpr int NVL = NV > LPR ? NV / LPR : 1;        // logits per lane
+  constexpr int LPV = NV > LPR ? 1 : LPR / NV;        // lanes that hold the same logit
+  const int v0 = gl / LPV * NVL;                      // this lane's first logit
+  const int my_g = v0 / UNR;
   const float kLog2e = 1.4426950408889634f;
-  float scale_s[GQ], scale_b[GQ];
+  const float scale_s = p.tau_s[hq0 + my_g] * rsqrtf((float)D) * kLog2e;
+  const float scale_b = p.tau_b[hq0 + my_g] * rsqrtf((float)D) * kLog2e;
   float qf[GQ][8];
 #pragma unroll
-  for (int g = 0; g < GQ; ++g) {
-    scale_s[g] = p.tau_s[hq0 + g] * rsqrtf((float)D) * kLog2e;
-    scale_b[g] = p.tau_b[hq0 + g] * rsqrtf((float)D) * kLog2e;
-    unpack8(*reinterpret_cast<const uint4*>(&s_q[g][gl * 8]), qf[g]);
-  }
-  float m_run[GQ], l_run[GQ];
+  for (int g = 0; g < GQ; ++g) unpack8(*reinterpret_cast<const uint4*>(&s_q[g][gl * 8]), qf[g]);
+  float m_run = -INFINITY, l_run = 0.f;   // of head my_g: maximum over the warp's rows, sum over this lane's
   float acc[GQ][8];
 #pragma unroll
-  for (int g = 0; g < GQ; ++g) {
-    m_run[g] = -INFINITY; l_run[g] = 0.f;
+  for (int g = 0; g < GQ; ++g)
 #pragma unroll
     for (int c = 0; c < 8; ++c) acc[g][c] = 0.f;
-  }
 
   const __half* KhatU = p.Khat + u * p.Mcap * D + gl * 8;
   const __half* VhatU = p.Vhat + u * p.Mcap * D + gl * 8;
@@ -236,16 +259,12 @@ __global__ void __launch_bounds__(256) decode_step_kernel(DecodeParams p) {
 
   for (int base = r0 + warp * STEP; base < r1; base += 8 * STEP) {
     uint4 kw[UNR], vw[UNR];
-    bool ok[UNR];
-    bool st_[UNR];
 #pragma unroll
     for (int i = 0; i < UNR; ++i) {
       const int row = base + i * RPW + grp;
-      ok[i] = row < r1;
-      st_[i] = row < m;
-      if (ok[i] && row < n - 1) {
+      if (row < r1 && row < n - 1) {
         const __half *kp, *vp;
-        if (st_[i]) {
+        if (row < m) {
           kp = KhatU + (int64_t)row * D;
           vp = VhatU + (int64_t)row * D;
         } else {
@@ -256,7 +275,7 @@ __global__ void __launch_bounds__(256) decode_step_kernel(DecodeParams p) {
         }
         kw[i] = ldg_stream(kp);
         vw[i] = ldg_stream(vp);
-      } else if (ok[i]) {   // the new token
+      } else if (row < r1) {   // the new token
         kw[i] = *reinterpret_cast<const uint4*>(&s_new[0][gl * 8]);
         vw[i] = *reinterpret_cast<const uint4*>(&s_new[1][gl * 8]);
       } else {
@@ -264,7 +283,7 @@ __global__ void __launch_bounds__(256) decode_step_kernel(DecodeParams p) {
         vw[i] = make_uint4(0, 0, 0, 0);
       }
     }
-    float lg[GQ][UNR];
+    float lg[NV];
 #pragma unroll
     for (int i = 0; i < UNR; ++i) {
       float kf[8];
@@ -274,50 +293,68 @@ __global__ void __launch_bounds__(256) decode_step_kernel(DecodeParams p) {
         float dot = 0.f;
 #pragma unroll
         for (int c = 0; c < 8; ++c) dot = fmaf(qf[g][c], kf[c], dot);
+        lg[g * UNR + i] = dot;
+      }
+    }
+    lane_sums<NV, LPR / 2>(lg, gl);
+    float tmax = -INFINITY;
 #pragma unroll
-        for (int o = LPR / 2; o > 0; o >>= 1) dot += __shfl_xor_sync(0xffffffffu, dot, o);
-        lg[g][i] = ok[i] ? dot * (st_[i] ? scale_s[g] : scale_b[g]) : -INFINITY;
+    for (int k = 0; k < NVL; ++k) {
+      const int row = base + (v0 + k) % UNR * RPW + grp;
+      lg[k] = row < r1 ? lg[k] * (row < m ? scale_s : scale_b) : -INFINITY;
+      tmax = fmaxf(tmax, lg[k]);
+    }
+    // maximum of the head over the rows of the step: the lanes of its other rows, the other row groups
+#pragma unroll
+    for (int o = LPV; o < LPV * UNR / NVL; o <<= 1) tmax = fmaxf(tmax, __shfl_xor_sync(0xffffffffu, tmax, o));
+#pragma unroll
+    for (int o = 16; o >= LPR; o >>= 1) tmax = fmaxf(tmax, __shfl_xor_sync(0xffffffffu, tmax, o));
+    // (a step has a valid row, so tmax is finite for every head)
+    if (__any_sync(0xffffffffu, tmax > m_run)) {
+      const float mnew = fmaxf(m_run, tmax);
+      const float corr = exp2f(m_run - mnew);
+      m_run = mnew;
+      l_run *= corr;
+#pragma unroll
+      for (int g = 0; g < GQ; ++g) {
+        const float cg = __shfl_sync(0xffffffffu, corr, g * UNR / NVL * LPV);
+#pragma unroll
+        for (int c = 0; c < 8; ++c) acc[g][c] *= cg;
       }
     }
 #pragma unroll
-    for (int g = 0; g < GQ; ++g) {
-      float tmax = lg[g][0];
+    for (int k = 0; k < NVL; ++k) {
+      lg[k] = exp2f(lg[k] - m_run);   // 0 for invalid rows
+      l_run += lg[k];
+    }
 #pragma unroll
-      for (int i = 1; i < UNR; ++i) tmax = fmaxf(tmax, lg[g][i]);
-      // maximum over the row groups of the warp
+    for (int i = 0; i < UNR; ++i) {
+      float vf[8];
+      unpack8(vw[i], vf);
 #pragma unroll
-      for (int o = 16; o >= LPR; o >>= 1) tmax = fmaxf(tmax, __shfl_xor_sync(0xffffffffu, tmax, o));
-      if (tmax == -INFINITY) continue;   // warp-uniform: no valid row in this step
-      const float mnew = fmaxf(m_run[g], tmax);
-      const float corr = exp2f(m_run[g] - mnew);
-      m_run[g] = mnew;
-      l_run[g] *= corr;
-#pragma unroll
-      for (int c = 0; c < 8; ++c) acc[g][c] *= corr;
-#pragma unroll
-      for (int i = 0; i < UNR; ++i) {
-        const float pr = exp2f(lg[g][i] - mnew);   // 0 for invalid rows
-        l_run[g] += pr;
-        float vf[8];
-        unpack8(vw[i], vf);
+      for (int g = 0; g < GQ; ++g) {
+        const int idx = g * UNR + i;   // held by lane idx / NVL * LPV of the row group
+        const float pr = __shfl_sync(0xffffffffu, lg[idx % NVL], grp * LPR + idx / NVL * LPV);
 #pragma unroll
         for (int c = 0; c < 8; ++c) acc[g][c] = fmaf(pr, vf[c], acc[g][c]);
       }
     }
   }
-  // merge the row groups of the warp (all share m_run; l_run is per group)
+  // merge the row groups of the warp (all share m_run; l_run is per lane)
+#pragma unroll
+  for (int o = LPV; o < LPV * UNR / NVL; o <<= 1) l_run += __shfl_xor_sync(0xffffffffu, l_run, o);
+#pragma unroll
+  for (int o = 16; o >= LPR; o >>= 1) l_run += __shfl_xor_sync(0xffffffffu, l_run, o);
+  if (grp == 0 && gl % (LPV * UNR / NVL) == 0) { s_m[warp][my_g] = m_run; s_l[warp][my_g] = l_run; }
 #pragma unroll
   for (int g = 0; g < GQ; ++g) {
 #pragma unroll
-    for (int o = 16; o >= LPR; o >>= 1) {
-      l_run[g] += __shfl_xor_sync(0xffffffffu, l_run[g], o);
+    for (int o = 16; o >= LPR; o >>= 1)
 #pragma unroll
       for (int c = 0; c < 8; ++c) acc[g][c] += __shfl_xor_sync(0xffffffffu, acc[g][c], o);
-    }
     if (grp == 0) {
 #pragma unroll
       for (int c = 0; c < 8; ++c) s_acc[warp][g][gl * 8 + c] = acc[g][c];
-      if (gl == 0) { s_m[warp][g] = m_run[g]; s_l[warp][g] = l_run[g]; }
     }
   }
   __syncthreads();
@@ -396,13 +433,19 @@ int launch_decode(State* st, const DecodeArgs& a, cudaStream_t s) {
   p.m = (int)a.m; p.n = (int)(a.m + (a.t - a.b + 1));
   p.ringLen = (int)st->ringLen; p.slot_b = (int)(a.b % st->ringLen); p.slot_t = (int)(a.t % st->ringLen);
   p.Hq = st->Hq; p.Hkv = st->Hkv; p.G = st->G; p.r = st->r;
-  // Row splits: a power of two up to the portable cluster size (clusters of 16 took 13.5 us per step where 8 take 8.5),
-  // until there are two CTAs per SM, and no more than give every split one step of its eight warps (64 or 128 rows).
-  // Measured per step of 32 heads over 256 + window rows, one / two / three / four CTAs per SM: 9.7 / 9.5 / 9.7 /
-  // 10.2 us; of 8 groups of four heads: 11.3 / 10.6 / 10.7 / 10.7 us.
-  const int nCta = nQ / GQ, rows1 = 8 * 4 * (256 / st->d);
+  // Row splits, up to the portable cluster size (clusters of 16 took 13.5 us per step where 8 take 8.5): waves of CTAs
+  // times the length of a CTA, its set-up and merge counted as 300 rows.  `slots` = CTAs that fit the GPU at once (3, 2,
+  // 2, 1 per SM by registers for 1, 2, 4, 8 heads).  This picks the fastest of 1, 2, 3, 4, 6, 8 splits, or one within 2 %
+  // of it, in all of 15 measured shapes (64 to 768 heads, 900 to 2400 rows; e.g. us per step of 256 heads over 2430
+  // rows: 59, 68, 55, 61, 64, 70; of 512 heads: 123, 109, 106, 108, 123, 131).
+  const int nCta = nQ / GQ, rows1 = 8 * 4 * (256 / st->d), slots = 148 * (GQ == 1 ? 3 : GQ == 8 ? 1 : 2);
   int nsplit = 1;
-  while (nsplit < 8 && nsplit * nCta < 2 * 148 && nsplit * rows1 < p.n) nsplit *= 2;
+  int64_t least = INT64_MAX;
+  for (int ns = 1; ns <= 8; ++ns) {
+    const int64_t rows = ((p.n + ns - 1) / ns + rows1 - 1) / rows1 * rows1;
+    const int64_t t = ((int64_t)nCta * ns + slots - 1) / slots * (rows + 300);
+    if (t < least) { least = t; nsplit = ns; }
+  }
   p.nsplit = nsplit;
   const bool early = st->prof_hook == nullptr;
 #define KVM_DEC_GO(DD, GG, LL) \
