@@ -369,8 +369,6 @@ KVM_API kvm_status_t kvm_state_create(const kvm_config_t* cfg, kvm_state_t** out
     A(s.foldPi[i], U * Cm); A(s.foldSorted[i], U * Cm); A(s.foldCreator[i], U * Cm); A(s.foldSegNew[i], U * Cm);
     A(s.foldNMerge[i], U);
   }
-  A(s.xScore, U * Cm); A(s.xBest, U * Cm); A(s.xArg, U * Cm); A(s.xCount, U);
-  if (rc == KVM_OK && cudaMemset(s.xCount, 0, U * sizeof(int32_t)) != cudaSuccess) rc = KVM_ERR_CUDA;
   A(s.candV, U * (size_t)s.nsplitRoute * Cm * kTopK); A(s.candI, U * (size_t)s.nsplitRoute * Cm * kTopK);
   A(s.chunkMeta, U * (size_t)s.nsplitRoute * Cm * kChunkCap); A(s.chunkMax, U * (size_t)s.nsplitRoute * Cm * kChunkCap);
   if (rc == KVM_OK) rc = dev_alloc(ks, &s.chunkVal, U * (size_t)s.nsplitRoute * Cm * kChunkCap * 32, false);

@@ -9,8 +9,8 @@
 //                           the rows within the rounding window of the best one, per token and row split
 //   3. fold_decide_kernel   exact fp64 similarities of the candidates, append selection, merge
 //                           routing against s_+ (new rows: filtered by the products of step 1, the few
-//                           contenders exactly), grouping of the merged tokens by target row; several CTAs
-//                           per unit share the refinement, the last one to finish takes the block-wide steps
+//                           contenders exactly), grouping of the merged tokens by target row; the CTAs of a unit
+//                           are a cluster that shares all of it
 //   4. fold_apply_kernel    one warp per touched row: creates appended rows, accumulates the
 //                           members in ascending token order (deterministic), refreshes the
 //                           readout cache (LN_s of the key sum, value-radius readout) in the readout
@@ -23,6 +23,7 @@
 // approximate similarity is within 2*eps of the best one, eps being a rigorous bound on the fp16
 // rounding error of the dot product, so the true arg max is always among the candidates.
 #include "kvm_internal.h"
+#include "tc_common.cuh"
 
 namespace kvm {
 
@@ -380,8 +381,6 @@ struct FoldDecideParams {
   const double* sumK;
   const double *kmu, *krstd;
   int32_t *pi, *sorted, *creator, *segnew, *nmerge;   // outputs, [U, Cmax] (nmerge [U])
-  double *xScore, *xBest;   // [U, Cmax] per-token results handed from the slice CTAs to the last one
-  int32_t *xArg, *xCount;   // [U, Cmax]; [U] ticket counter (zero between launches)
   int32_t* counters;   // debug: [0] tokens on the exhaustive path, [1] candidate pairs, [2] tokens decided
   int64_t Mcap, m;
   int C, Cmax, Hkv, S, n_append, nsplit;
@@ -389,12 +388,12 @@ struct FoldDecideParams {
   double ln_eps;
 };
 
-constexpr int kPairCap = 1536;
 constexpr int kPairPerTok = 24;
 
 constexpr int kDecideThreads = 512;
 constexpr int kDecideWarps = kDecideThreads / 32;
-static_assert(kDecideThreads == 2 * kMaxBlock, "the ranking loops give every token two threads");
+constexpr int kWarpPairs = 96;      // (token, row) pairs a warp holds at a time
+constexpr int kDecideMaxCtas = 8;   // CTAs per unit: the portable cluster size
 
 // The candidate rows (kTopK entries, -1 = none) of one token in one split: two 16-byte loads.
 __device__ __forceinline__ void load_cand_rows(const int32_t* candI, int64_t o, int (&i)[kTopK]) {
@@ -456,38 +455,52 @@ __device__ __forceinline__ void sort_n(K& key, int& val, K* sk, int* sv, int t) 
   }
 }
 
+// Decisions of a fold: the R CTAs of a unit are a cluster, CTA r takes the tokens [r C / R, (r + 1) C / R) and every warp
+// a run of those.  A warp takes its tokens from the filter's lists to the exact similarities (and later from the new
+// rows' products to the merge targets) without a barrier; what needs every token of the block - the order of the append
+// scores, the appended rows' positions, the members of a row - is exchanged through distributed shared memory in three
+// steps (asynchronous stores, counted on the receiver's barriers).
+// What bounds it: the latency of its chain of dependent loads and exchanges (a state with few units has no work to hide
+// them).  With the block-wide steps on one CTA per unit, reached through a ticket, and the lists read in three
+// rounds the kernel took 28 us for 8 units of 5000 rows, 30 for 32 of 2000, 18.5 for 32 full states of 512; now 16, 24, 9.
 // PER_SM = 2 for grids that fill the GPU twice over (64 registers, a few spills), 1 for the small grids
 // of chain-bound shapes, where a CTA has an SM to itself anyway and keeps everything in registers.
 template <int D, int PER_SM, bool RK>
-__global__ void __launch_bounds__(kDecideThreads, PER_SM) fold_decide_kernel(FoldDecideParams p) {
+__global__ void __launch_bounds__(kDecideThreads, PER_SM) fold_decide_kernel(const __grid_constant__ FoldDecideParams p) {
   constexpr int CH = D / 32;
-  __shared__ double s_score[kMaxBlock], s_best[kMaxBlock];
-  __shared__ int s_barg[kMaxBlock], s_pi[kMaxBlock], s_creator[kMaxBlock];
-  __shared__ int s_pstart[kMaxBlock], s_pcnt[kMaxBlock];
-  __shared__ unsigned char s_app[kMaxBlock], s_exh[kMaxBlock];
-  __shared__ int s_prow[kPairCap];
-  __shared__ unsigned short s_ptok[kPairCap];
-  __shared__ double s_pval[kPairCap];
-  __shared__ int s_np, s_nmerge, s_nexh, s_last;
-  __shared__ int s_wsum[kDecideWarps];
-  __shared__ int s_gmaxi[kMaxBlock], s_fill[kMaxBlock];
+  __shared__ unsigned long long s_key[kMaxBlock];    // append scores of all tokens (exchanged)
+  __shared__ unsigned s_tgt[kMaxBlock];              // row << 9 | token of all merged tokens (exchanged; all ones: appended)
+  __shared__ int s_app[kMaxBlock];                   // append flags of all tokens (exchanged)
+  __shared__ uint64_t s_bar[3];                      // the three exchanges: bytes received
+  __shared__ double s_score[kMaxBlock], s_best[kMaxBlock];   // (of this CTA's tokens, as everything below)
+  __shared__ int s_barg[kMaxBlock], s_creator[kMaxBlock];
   __shared__ float s_thr[kMaxBlock];
-  __shared__ __align__(16) __half s_hat[kGramOnTheFly][D];   // LN_s(kbar_a) of the rows a small fold appends
+  __shared__ signed char s_how[kMaxBlock];   // 0: its pairs are on the warp's list, 1: decided, 2: scan every row
+  __shared__ int s_np[kDecideWarps];
+  __shared__ int s_prow[kDecideWarps][kWarpPairs];
+  __shared__ unsigned char s_ptok[kDecideWarps][kWarpPairs];
+  __shared__ double s_pval[kDecideWarps][kWarpPairs];
+  __shared__ unsigned s_word[kMaxBlock / 32];
+  __shared__ int s_dead;
+  __shared__ int s_nexh, s_npair;
 
-  // grid (R, U): CTA r of a unit refines the candidates of tokens [jlo, jhi); the CTA of the unit
-  // that finishes last (a ticket, nobody waits) takes the decisions that need every token
+  const int R = gridDim.x, rank = blockIdx.x;
   const int u = blockIdx.y, hk = u % p.Hkv;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  const int C = p.C;
-  const int R = gridDim.x;
-  const int jlo = (int)blockIdx.x * ((C + R - 1) / R), jhi = min(C, jlo + (C + R - 1) / R);
+  const int C = p.C, n_a = p.n_append;
   const int64_t m = p.m;
-  const int n_a = p.n_append;
+  const int nsl = (C + R - 1) / R;
+  const int jlo = min(C, rank * nsl), jhi = min(C, jlo + nsl);
+  const int tpw = (nsl + kDecideWarps - 1) / kDecideWarps;
+  const int wj0 = min(jhi, jlo + warp * tpw), wj1 = min(jhi, wj0 + tpw);   // this warp's tokens (at most 16)
   const int64_t rowBase = (int64_t)u * p.Mcap;
   const int64_t tokBase = (int64_t)u * p.Cmax;
   KbarRows<D, RK> kbarU;
   kbarU.k64 = p.kbar64 + (int64_t)u * p.Cmax * D; kbarU.k16 = p.ok + (int64_t)u * p.unit_stride;
   kbarU.stat = p.kbarStat + tokBase; kbarU.r = p.r;
+  int* prow = s_prow[warp];
+  unsigned char* ptok = s_ptok[warp];
+  double* pval = s_pval[warp];
 
   double gam[CH], bet[CH];
 #pragma unroll
@@ -495,487 +508,392 @@ __global__ void __launch_bounds__(kDecideThreads, PER_SM) fold_decide_kernel(Fol
     gam[i] = (double)p.ln_w[hk * D + lane + 32 * i];
     bet[i] = (double)p.ln_b[hk * D + lane + 32 * i];
   }
-  if (tid == 0) { s_np = 0; s_nmerge = 0; s_nexh = 0; }
-  if (tid < kMaxBlock) {
-    s_app[tid] = 0; s_exh[tid] = 0; s_pcnt[tid] = 0; s_pstart[tid] = 0; s_pi[tid] = -1;
-    s_best[tid] = -INFINITY; s_barg[tid] = -1; s_score[tid] = -INFINITY; s_creator[tid] = -1;
-    s_gmaxi[tid] = (int)0x80000000; s_fill[tid] = 0; s_thr[tid] = 0.f;
+  if (tid == 0) {
+    s_nexh = 0; s_npair = 0; s_dead = 0;
+    const uint32_t bytes[3] = {8, 4, 4};   // per token
+    for (int i = 0; i < 3; ++i) tc::mbar_init(&s_bar[i], 1);
+    tc::fence_barrier_init();
+    for (int i = 0; i < 3; ++i) tc::mbar_expect_tx(&s_bar[i], bytes[i] * (uint32_t)C);
   }
-  // everything above reads parameters and writes shared memory only; the routing filter's lists are
-  // read, and global memory is written, from here on
+  if (tid < kDecideWarps) s_np[tid] = 0;
+  if (tid < kMaxBlock) s_creator[tid] = 0;
+  if (tid < kMaxBlock && (tid >= C || n_a == 0)) { s_tgt[tid] = 0xffffffffu; s_app[tid] = 0; }   // (what the exchanges leave out)
+  __syncthreads();
+  // the exchanges: one value per token and CTA of the unit, its bytes counted on the receiver's barrier (a cluster
+  // barrier per exchange cost about 2000 cycles, this less than half).  A CTA's barriers exist, and a CTA is there, from
+  // here on; it leaves when the others have, at the end.  A unit's only CTA stores to itself: st.async is for clusters
+  // (in a launch without one it raised an illegal instruction).
+  const bool many = R > 1;
+  if (many) asm volatile("barrier.cluster.arrive.release;" ::: "memory");
+  auto give32 = [&](int* arr, int bar, int j, int r, int v) {
+    if (!many) { arr[j] = v; return; }
+    asm volatile("st.async.weak.shared::cluster.mbarrier::complete_tx::bytes.b32 [%0], %1, [%2];"
+                 ::"r"(tc::cluster_addr(arr + j, r)), "r"(v), "r"(tc::cluster_addr(&s_bar[bar], r)) : "memory");
+  };
+  auto give64 = [&](unsigned long long* arr, int bar, int j, int r, unsigned long long v) {
+    if (!many) { arr[j] = v; return; }
+    asm volatile("st.async.weak.shared::cluster.mbarrier::complete_tx::bytes.b64 [%0], %1, [%2];"
+                 ::"r"(tc::cluster_addr(arr + j, r)), "l"(v), "r"(tc::cluster_addr(&s_bar[bar], r)) : "memory");
+  };
+  auto received = [&](int bar) {   // every thread calls; the wait is bounded
+    if (!many) __syncthreads();
+    else if (!tc::mbar_wait_cluster(&s_bar[bar], 0)) s_dead = 1;
+  };
+  // everything above reads parameters and writes shared memory only
   asm volatile("griddepcontrol.wait;" ::: "memory");
-  if (tid < p.Cmax && tid < kMaxBlock) p.segnew[tokBase + tid] = -1;
-  __syncthreads();
 
-  // ---- A1/A2: candidate pairs from the filter lists.  The work items are (token of the slice, split),
-  //      consecutive threads taking consecutive tokens of one split, in three rounds: the maximum over
-  //      the splits per token; the number of pairs per token; the pairs themselves, into the token's
-  //      segment of the pair list (order inside a segment does not matter to what follows).
-  //      A split keeps its candidates when its own maximum is within the window of the global one;
-  //      sink rows (< S) only matter for the append score and are kept whenever rows are appended. ----
-  const int nslice = jhi - jlo;
-  const int nitems = nslice > 0 ? nslice * p.nsplit : 0;
-  const int64_t ostep = (int64_t)p.Cmax * kTopK;
-  const int64_t obase = (int64_t)u * p.nsplit * p.Cmax * kTopK;
-  for (int it = tid; it < nitems; it += kDecideThreads) {
-    const int sp = it / nslice, j = jlo + it % nslice;
-    const int vi = __float_as_int(p.candV[obase + sp * ostep + (int64_t)j * kTopK]);
-    atomicMax(&s_gmaxi[j], vi >= 0 ? vi : vi ^ 0x7fffffff);   // order-preserving integer image of the float
-    if (sp == 0) s_thr[j] = p.thr_coeff * p.kbarNorm[tokBase + j] + 1e-5f;
-  }
-  __syncthreads();
-  for (int it = tid; it < nitems; it += kDecideThreads) {
-    const int sp = it / nslice, j = jlo + it % nslice;
-    const int gi = s_gmaxi[j];
-    const float gmax = __int_as_float(gi >= 0 ? gi : gi ^ 0x7fffffff);
-    if (!(gmax > -INFINITY)) { s_exh[j] = 1; continue; }
-    const int64_t o = obase + sp * ostep + (int64_t)j * kTopK;
-    const float2 hd = *reinterpret_cast<const float2*>(p.candV + o);
-    int i[kTopK];
-    load_cand_rows(p.candI, o, i);
-    const bool keep = hd.x >= gmax - s_thr[j];
-    if (hd.y > (float)kTopK && (keep || (n_a > 0 && sp == 0))) s_exh[j] = 1;   // list overflowed
-    int c = 0;
+  // ---- A: candidate pairs of the warp's tokens from the filter's lists, TL lanes (splits) per token.  A split keeps
+  //      its candidates when its own maximum is within the window of the global one; sink rows (< S) only matter
+  //      for the append score and are kept whenever rows are appended. ----
+  const int TL = p.nsplit <= 1 ? 1 : 1 << (32 - __clz(p.nsplit - 1));   // (nsplit <= 32)
+  const int TB = 32 / TL;
+  const int sp = lane & (TL - 1);
+  float2 hd_n;
+  int4 i0_n, i1_n;
+  float norm_n;
+  auto fetch = [&](int j) {   // this lane's share of token j's lists (the next batch's while one is worked on)
+    hd_n = make_float2(-INFINITY, 0.f);
+    i0_n = i1_n = make_int4(-1, -1, -1, -1);
+    norm_n = 0.f;
+    if (j < wj1) {
+      norm_n = p.kbarNorm[tokBase + j];
+      if (sp < p.nsplit) {
+        const int64_t o = (((int64_t)u * p.nsplit + sp) * p.Cmax + j) * kTopK;
+        static_assert(kTopK == 8, "list loads are written for 8 entries");
+        hd_n = *reinterpret_cast<const float2*>(p.candV + o);
+        i0_n = *reinterpret_cast<const int4*>(p.candI + o);
+        i1_n = *reinterpret_cast<const int4*>(p.candI + o + 4);
+      }
+    }
+  };
+  fetch(wj0 + lane / TL);
+  for (int jb = wj0; jb < wj1; jb += TB) {
+    const int j = jb + lane / TL;
+    const bool tok = j < wj1;
+    const float smax = hd_n.x, cnt = hd_n.y;
+    const int i[kTopK] = {i0_n.x, i0_n.y, i0_n.z, i0_n.w, i1_n.x, i1_n.y, i1_n.z, i1_n.w};
+    const float thr = tok ? p.thr_coeff * norm_n + 1e-5f : 0.f;
+    fetch(j + TB);
+    float gmax = smax;
+    for (int o = TL >> 1; o > 0; o >>= 1) gmax = fmaxf(gmax, __shfl_xor_sync(0xffffffffu, gmax, o));
+    const bool keep = smax >= gmax - thr && smax > -INFINITY;
+    unsigned use = 0;
 #pragma unroll
     for (int k = 0; k < kTopK; ++k)
-      if (i[k] >= 0 && (i[k] < p.S ? n_a > 0 : keep)) ++c;
-    if (c > 0) atomicAdd(&s_pcnt[j], c);
-  }
-  __syncthreads();
-  {   // segment starts: exclusive prefix sum over the slice's tokens, one token per thread
-    const int j = jlo + tid;
-    const bool mine = tid < nslice;
-    int c = 0;
-    bool exh = false, single = false;
-    if (mine) {
-      c = s_pcnt[j];
-      exh = s_exh[j] != 0 || c > kPairPerTok;
-      if (exh) c = 0;
-      // A fold that appends nothing needs no scores, and the true arg max is always among the
-      // candidates: a token with a single candidate is decided without the exact similarity
-      // (it takes no room in the pair list).
-      if (n_a == 0 && c == 1) { single = true; c = 0; }
+      if (i[k] >= 0 && (i[k] < p.S ? n_a > 0 : keep)) use |= 1u << k;
+    const int c = __popc(use);
+    // a list overflowed, or there is no maximum: every row exactly
+    bool exh = !(gmax > -INFINITY) || (cnt > (float)kTopK && (keep || (n_a > 0 && sp == 0)));
+    // A fold that appends nothing needs no scores, and the true arg max is always among the candidates: a token
+    // with a single candidate is decided without the exact similarity.
+    bool single = false;
+    const unsigned group = (TL == 32 ? 0xffffffffu : (1u << TL) - 1u) << (lane & ~(TL - 1));
+    if (n_a == 0) {
+      const unsigned one = __ballot_sync(0xffffffffu, c >= 1) & group, two = __ballot_sync(0xffffffffu, c >= 2) & group;
+      single = two == 0u && __popc(one) == 1;
     }
-    int incl = c;
-#pragma unroll
-    for (int o2 = 1; o2 < 32; o2 <<= 1) {
-      const int v = __shfl_up_sync(0xffffffffu, incl, o2);
-      if (lane >= o2) incl += v;
+    exh = (__ballot_sync(0xffffffffu, exh) & group) != 0u;
+    if (tok && sp == 0) {
+      s_thr[j] = thr;
+      s_how[j] = exh ? 2 : single ? 1 : 0;
     }
-    if (lane == 31) s_wsum[warp] = incl;
-    __syncthreads();
-    int start = incl - c;
-    for (int w = 0; w < warp; ++w) start += s_wsum[w];
-    if (mine) {
-      // a list that would pass the end of the pair buffer is dropped (so are the lists behind it):
-      // those tokens are scanned exactly instead
-      if (start + c > kPairCap) { exh = true; c = 0; }
-      s_pstart[j] = start;
-      s_pcnt[j] = c;
-      s_fill[j] = (single && !exh) ? -1 : 0;
-      s_exh[j] = exh ? 1 : 0;
-    }
-    // pairs of the lists that were kept form a prefix of the buffer: its end, one atomic per warp
-    // (256 atomics on one shared-memory word serialise)
-    const unsigned wend = __reduce_max_sync(0xffffffffu, (unsigned)((mine && c > 0) ? start + c : 0));
-    if (lane == 0 && wend > 0) atomicMax(&s_np, (int)wend);
-    const int ne = __syncthreads_count(mine && exh);   // tokens of the slice that take the exhaustive path
-    if (tid == 0) s_nexh += ne;
-  }
-  __syncthreads();
-  for (int it = tid; it < nitems; it += kDecideThreads) {
-    const int sp = it / nslice, j = jlo + it % nslice;
-    if (s_exh[j]) continue;
-    const int gi = s_gmaxi[j];
-    const float gmax = __int_as_float(gi >= 0 ? gi : gi ^ 0x7fffffff);
-    const int64_t o = obase + sp * ostep + (int64_t)j * kTopK;
-    const bool keep = p.candV[o] >= gmax - s_thr[j];
-    int i[kTopK];
-    load_cand_rows(p.candI, o, i);
-    int c = 0;
+    __syncwarp();
+    if (tok && !exh && c > 0) {
+      int w = single ? 0 : atomicAdd(&s_np[warp], c);   // (the order of a warp's pairs does not matter)
+      if (!single && w + c > kWarpPairs) {   // no room: the token is scanned, what is left of the list filled with copies of a row
+        s_how[j] = 2;
+        for (; w < kWarpPairs; ++w) { prow[w] = p.S; ptok[w] = (unsigned char)j; }
+      }
 #pragma unroll
-    for (int k = 0; k < kTopK; ++k)
-      if (i[k] >= 0 && (i[k] < p.S ? n_a > 0 : keep)) ++c;
-    if (c == 0) continue;
-    if (s_fill[j] < 0) {   // the token's only candidate: its row is the merge target
-#pragma unroll
-      for (int k = 0; k < kTopK; ++k)
-        if (i[k] >= 0 && (i[k] < p.S ? n_a > 0 : keep)) s_barg[j] = i[k];
-      continue;
-    }
-    int w = s_pstart[j] + atomicAdd(&s_fill[j], c);
-#pragma unroll
-    for (int k = 0; k < kTopK; ++k) {
-      if (i[k] >= 0 && (i[k] < p.S ? n_a > 0 : keep)) {
-        s_prow[w] = i[k];
-        s_ptok[w] = (unsigned short)j;
-        ++w;
+      for (int k = 0; k < kTopK; ++k) {
+        if (use & (1u << k)) {
+          if (single) s_barg[j] = i[k];
+          else if (w < kWarpPairs) { prow[w] = i[k]; ptok[w] = (unsigned char)j; ++w; }
+        }
       }
     }
   }
-  __syncthreads();
-  // ---- A3: exact fp64 similarity of every candidate pair, one warp per pair, eight in flight
-  //      (the loads of a pair hang on one another: pair list -> rows -> statistics) ----
-  const int np = min(s_np, kPairCap);
-  for (int q0 = warp; q0 < np; q0 += 8 * kDecideWarps) {
-    double part[8];
-#pragma unroll
-    for (int k = 0; k < 8; ++k) {
-      const int q = min(q0 + k * kDecideWarps, np - 1);   // clamped duplicates are computed and dropped
-      const int j = s_ptok[q], i = s_prow[q];
+  __syncwarp();
+  int np = min(s_np[warp], kWarpPairs);
+  // exact fp64 values of the warp's pairs, one pair at a time over its lanes, eight in flight: similarities with
+  // state rows, kbar_j . LN_s(s^K_i), or (fresh) with rows this fold appends, kbar_j . LN_s(kbar_c), c the creator
+  auto pair_share = [&](int q, int n, bool fresh) -> double {   // this lane's share of pair q (past the end: a copy, dropped)
+    q = min(q, n - 1);
+    const int j = ptok[q], i = prow[q];
+    double acc = 0.0;
+    if (!fresh) {
       const double* sk = p.sumK + (rowBase + i) * D;
       const double mu = p.kmu[rowBase + i], rs = p.krstd[rowBase + i];
-      double acc = 0.0;
 #pragma unroll
       for (int c = 0; c < CH; ++c)
         acc += kbarU.at(j, lane + 32 * c, gam[c], bet[c]) * (gam[c] * ((sk[lane + 32 * c] - mu) * rs) + bet[c]);
-      part[k] = acc;
-    }
-    const double z0 = warp_reduce4(part[0], part[1], part[2], part[3], lane);
-    const double z1 = warp_reduce4(part[4], part[5], part[6], part[7], lane);
-    if ((lane & 7) == 0) {   // lanes 0, 8, 16, 24 hold pairs 0..3 of z0 and 4..7 of z1
-      const int qa = q0 + (lane >> 3) * kDecideWarps, qb = qa + 4 * kDecideWarps;
-      if (qa < np) s_pval[qa] = z0;
-      if (qb < np) s_pval[qb] = z1;
-    }
-  }
-  __syncthreads();
-  // ---- A4: per-token reduction (ties: lowest row) ----
-  if (jlo + tid < jhi && !s_exh[jlo + tid] && s_fill[jlo + tid] >= 0) {
-    const int j = jlo + tid;
-    double score = -INFINITY, best = -INFINITY;
-    int barg = -1;
-    const int st0 = s_pstart[j];
-    for (int q = st0; q < st0 + s_pcnt[j]; ++q) {
-      const double v = s_pval[q];
-      const int i = s_prow[q];
-      if (v > score) score = v;
-      if (i >= p.S && (v > best || (v == best && i < barg))) { best = v; barg = i; }
-    }
-    s_score[j] = score;
-    s_best[j] = best;
-    s_barg[j] = barg;
-  }
-  // ---- A5: exhaustive path for flagged tokens: one warp per token, rows in sequence ----
-  for (int j = jlo + warp; j < jhi; j += kDecideWarps) {
-    if (!s_exh[j]) continue;
-    double kb[CH];
+    } else {
+      const int jc = s_creator[i];
+      const double2 hs = p.kbarHatStat[tokBase + jc];
 #pragma unroll
-    for (int i = 0; i < CH; ++i) kb[i] = kbarU.at(j, lane + 32 * i, gam[i], bet[i]);
-    double score = -INFINITY, best = -INFINITY;
-    int barg = -1;
-    for (int64_t i = 0; i < m; ++i) {
-      const double acc = warp_sim<CH>(kb, p.sumK + (rowBase + i) * D, p.kmu[rowBase + i], p.krstd[rowBase + i], gam, bet, lane);
-      if (acc > score) score = acc;
-      if (i >= p.S && acc > best) { best = acc; barg = (int)i; }
-    }
-    if (lane == 0) { s_score[j] = score; s_best[j] = best; s_barg[j] = barg; }
-  }
-  __syncthreads();
-  if (R > 1) {
-    // hand the slice's results over; the last CTA of the unit to get here carries on with all of them
-    if (jlo + tid < jhi) {
-      const int j = jlo + tid;
-      p.xScore[tokBase + j] = s_score[j];
-      p.xBest[tokBase + j] = s_best[j];
-      p.xArg[tokBase + j] = s_barg[j];
-    }
-    __threadfence();
-    __syncthreads();
-    if (tid == 0) {
-      atomicAdd(&p.counters[0], s_nexh);
-      atomicAdd(&p.counters[1], min(s_np, kPairCap));
-      s_last = atomicAdd(&p.xCount[u], 1) == R - 1 ? 1 : 0;
-    }
-    __syncthreads();
-    if (!s_last) return;
-    __threadfence();
-    if (tid == 0) { p.xCount[u] = 0; s_nexh = 0; s_np = 0; }
-    if (tid < C) {   // read past the L1, which may hold stale lines of these arrays
-      s_score[tid] = __ldcg(p.xScore + tokBase + tid);
-      s_best[tid] = __ldcg(p.xBest + tokBase + tid);
-      s_barg[tid] = __ldcg(p.xArg + tokBase + tid);
-    }
-    __syncthreads();
-  }
-  // ---- B: append selection: the n_a smallest scores, ties to the smaller token index ----
-  if (n_a > 0) {
-    // rank of every token in the order (score, token): the n_a lowest are appended.  Counted, not sorted: two
-    // threads per token, each over half of the other tokens (a 256-entry bitonic sort is 36 dependent stages,
-    // six of them through shared memory and barriers; this is 128 independent compare-and-adds per thread).
-    {
-      unsigned long long* skey = reinterpret_cast<unsigned long long*>(s_pval);   // (the pair list is idle here)
-      if (tid < kMaxBlock) {
-        unsigned long long kbits = ~0ull;
-        if (tid < C) {   // order-preserving integer image of the double
-          const long long bits = __double_as_longlong(s_score[tid]);
-          kbits = (unsigned long long)bits ^ (bits < 0 ? ~0ull : 0x8000000000000000ull);
-        }
-        skey[tid] = kbits;
-        s_fill[tid] = 0;   // (idle here: the rank)
+      for (int c = 0; c < CH; ++c) {
+        const double hat = gam[c] * ((kbarU.at(jc, lane + 32 * c, gam[c], bet[c]) - hs.x) * hs.y) + bet[c];
+        acc += kbarU.at(j, lane + 32 * c, gam[c], bet[c]) * hat;
       }
-      __syncthreads();
-      const int j = tid & (kMaxBlock - 1), h = tid / kMaxBlock;   // kDecideThreads == 2 kMaxBlock
-      if (j < C) {
-        const unsigned long long kj = skey[j];
-        const int half_n = (C + 1) / 2, i0 = h * half_n, i1 = min(C, i0 + half_n);
-        int cnt = 0;
+    }
+    return acc;
+  };
+  auto exact_pairs = [&](int n, bool fresh) {
+    int q0 = 0;
+    for (; n - q0 > 4; q0 += 8) {
+      double part[8];
+#pragma unroll
+      for (int k = 0; k < 8; ++k) part[k] = pair_share(q0 + k, n, fresh);
+      const double z0 = warp_reduce4(part[0], part[1], part[2], part[3], lane);
+      const double z1 = warp_reduce4(part[4], part[5], part[6], part[7], lane);
+      if ((lane & 7) == 0) {   // lanes 0, 8, 16, 24 hold pairs 0..3 of z0 and 4..7 of z1
+        const int qa = q0 + (lane >> 3), qb = qa + 4;
+        if (qa < n) pval[qa] = z0;
+        if (qb < n) pval[qb] = z1;
+      }
+    }
+    if (q0 < n) {
+      const double p0 = pair_share(q0, n, fresh), p1 = pair_share(q0 + 1, n, fresh), p2 = pair_share(q0 + 2, n, fresh),
+                   p3 = pair_share(q0 + 3, n, fresh);
+      const double z0 = warp_reduce4(p0, p1, p2, p3, lane);
+      if ((lane & 7) == 0 && q0 + (lane >> 3) < n) pval[q0 + (lane >> 3)] = z0;
+    }
+    __syncwarp();
+  };
+  exact_pairs(np, false);
+  int npair = np;
+  // per-token reduction (ties: lowest row), one lane per token
+  int nexh = 0;
+  {
+    const int j = wj0 + lane;
+    const int how = j < wj1 ? s_how[j] : 1;
+    if (how == 0) {   // (a token has a pair at least: the filter's maximum is on its list)
+      double score = -INFINITY, best = -INFINITY;
+      int barg = -1;
+      for (int q = 0; q < np; ++q) {   // (of all the warp's tokens)
+        if (ptok[q] != j) continue;
+        const double v = pval[q];
+        const int i = prow[q];
+        if (v > score) score = v;
+        if (i >= p.S && (v > best || (v == best && i < barg))) { best = v; barg = i; }
+      }
+      s_score[j] = score; s_best[j] = best; s_barg[j] = barg;
+    }
+    // exhaustive path: rows in sequence
+    unsigned todo = __ballot_sync(0xffffffffu, how == 2);
+    nexh = __popc(todo);
+    while (todo) {
+      const int jx = wj0 + __ffs(todo) - 1;
+      todo &= todo - 1;
+      double kb[CH];
+#pragma unroll
+      for (int i = 0; i < CH; ++i) kb[i] = kbarU.at(jx, lane + 32 * i, gam[i], bet[i]);
+      double score = -INFINITY, best = -INFINITY;
+      int barg = -1;
+      for (int64_t i = 0; i < m; ++i) {
+        const double acc = warp_sim<CH>(kb, p.sumK + (rowBase + i) * D, p.kmu[rowBase + i], p.krstd[rowBase + i], gam, bet, lane);
+        if (acc > score) score = acc;
+        if (i >= p.S && acc > best) { best = acc; barg = (int)i; }
+      }
+      if (lane == 0) { s_score[jx] = score; s_best[jx] = best; s_barg[jx] = barg; }
+    }
+    __syncwarp();
+  }
+  if (many) asm volatile("barrier.cluster.wait.acquire;" ::: "memory");   // (all CTAs of the unit are set up)
+
+  if (n_a > 0) {
+    // ---- B: append selection: the n_a smallest scores, ties to the smaller token index.  Every CTA gets all keys
+    //      and counts the ranks of its own tokens, q threads per token. ----
+    for (int e = lane; e < (wj1 - wj0) * R; e += 32) {
+      const int j = wj0 + e / R;
+      const long long bits = __double_as_longlong(s_score[j]);   // order-preserving integer image of the double
+      give64(s_key, 0, j, e % R, (unsigned long long)bits ^ (bits < 0 ? ~0ull : 0x8000000000000000ull));
+    }
+    received(0);
+    {
+      int q = 1;
+      while (2 * q * nsl <= kDecideThreads && q < 32) q *= 2;
+      const int j = jlo + tid / q, part = tid & (q - 1);
+      const bool mine = j < jhi;
+      const unsigned long long kj = mine ? s_key[j] : 0ull;
+      int cnt = 0;
+      if (mine) {
 #pragma unroll 4
-        for (int i = i0; i < i1; ++i) {
-          const unsigned long long ki = skey[i];
+        for (int i = part; i < C; i += q) {
+          const unsigned long long ki = s_key[i];
           cnt += (ki < kj || (ki == kj && i < j)) ? 1 : 0;
         }
-        atomicAdd(&s_fill[j], cnt);
       }
-      __syncthreads();
-      if (tid < C) s_app[tid] = s_fill[tid] < n_a ? 1 : 0;
+      for (int o = q >> 1; o > 0; o >>= 1) cnt += __shfl_xor_sync(0xffffffffu, cnt, o);
+      if (mine)
+        for (int r = part; r < R; r += q) give32(s_app, 1, j, r, cnt < n_a ? 1 : 0);
     }
-    __syncthreads();
+    received(1);
     // rows are laid down in ascending token order: position of an appended token = appended tokens before it
+    bool ap = false;
+    unsigned bal = 0;
     if (tid < kMaxBlock) {
-      const bool ap = tid < C && s_app[tid];
-      const unsigned bal = __ballot_sync(0xffffffffu, ap);
-      if (lane == 0) s_fill[warp] = __popc(bal);   // (s_fill is idle here)
-      __syncwarp();
-      s_pcnt[tid] = __popc(bal & ((1u << lane) - 1u));   // appended tokens before this one inside its warp
+      ap = tid < C && s_app[tid];
+      bal = __ballot_sync(0xffffffffu, ap);
+      if (lane == 0) s_word[warp] = bal;
     }
     __syncthreads();
-    if (tid < C && s_app[tid]) {
-      int before = s_pcnt[tid];
-      for (int wq = 0; wq < warp; ++wq) before += s_fill[wq];
+    if (ap) {
+      int before = __popc(bal & ((1u << lane) - 1u));
+      for (int w = 0; w < warp; ++w) before += __popc(s_word[w]);
       s_creator[before] = tid;
     }
     __syncthreads();
-  }
-  // ---- D: merge target against s_+ = old rows (best exact similarity known from A) and the rows
-  //      appended by this fold.  The tensor-core products gramT[a][j] ~ kbarHat_a . kbar_j are within
-  //      eps_j = thr_j / 2 of the exact values, so a new row can only win when its approximate value
-  //      plus eps_j reaches both the exact best old value and (best approximate new value - eps_j).
-  //      Those few pairs are recomputed in fp64; everything else is decided by the bound. ----
-  if (tid == 0) { atomicAdd(&p.counters[1], min(s_np, kPairCap)); s_np = 0; }
-  __syncthreads();
-  // A fold that appends only a few rows (n_a <= kGramOnTheFly, i.e. nearly every fold of a growing state)
-  // computes the approximate products itself, fp16 x fp16 -> fp32 on the scalar cores, against the new rows'
-  // keys LN_s(kbar_a) rounded to fp16 in shared memory: n_a x C products instead of the C x C that the
-  // batched tensor-core product of the block's token pairs holds.  The error bound is the same (fp16
-  // rounding of both operands; fp32 accumulation errs less than the tensor core's).
-  const bool otf = n_a <= p.otf_max;
-  if (n_a > 0 && otf) {
-    for (int a = warp; a < n_a; a += kDecideWarps) {
-      const int jc = s_creator[a];
-      const double2 hs = p.kbarHatStat[tokBase + jc];
+    // ---- D: merge target against s_+ = old rows (best exact similarity known from A) and the rows appended by this
+    //      fold.  The tensor-core products gramT[a][j] ~ kbarHat_a . kbar_j are within eps_j = thr_j / 2 of the exact
+    //      values, so a new row can only win when its approximate value plus eps_j reaches both the exact best old
+    //      value and (best approximate new value - eps_j).  Those few pairs are recomputed in fp64. ----
+    const float* gram = p.gramT + (int64_t)u * p.Cmax * p.Cmax;
+    np = 0;
+    bool over = false;
+    {   // LT lanes per token, each a share of the new rows
+      int LT = 32;
+      while (LT * tpw > 32) LT >>= 1;
+      const int j = wj0 + lane / LT, part = lane & (LT - 1);
+      const bool merged = j < wj1 && !s_app[j];
+      float pv[4], gm = -INFINITY;   // (the first products stay in registers)
 #pragma unroll
-      for (int c = 0; c < CH; ++c)
-        s_hat[a][lane + 32 * c] =
-            __float2half_rn((float)(gam[c] * ((kbarU.at(jc, lane + 32 * c, gam[c], bet[c]) - hs.x) * hs.y) + bet[c]));
-    }
-    __syncthreads();
-  }
-  if (n_a > 0 && tid < C) {
-    const int j = tid;
-    s_pcnt[j] = 0;
-    s_exh[j] = 0;
-    if (!s_app[j]) {
-      const double eps = 0.5 * (double)(p.thr_coeff * p.kbarNorm[tokBase + j] + 1e-5f);
-      const double best_old = s_best[j];
-      // one pass over the products with the new rows, ascending a: contenders are kept while they reach the
-      // running bar (which only rises: a superset) and pruned against the final bar afterwards
-      float gm = -INFINITY;
-      int cntc = 0, ca[4] = {0, 0, 0, 0};
-      float cp[4] = {0.f, 0.f, 0.f, 0.f};
-      auto consider = [&](int a, float pv) {
-        gm = fmaxf(gm, pv);
-        if ((double)pv >= fmax(best_old, (double)gm - eps) - eps) {
+      for (int t = 0; t < 4; ++t) {
+        const int a = part + t * LT;
+        pv[t] = merged && a < n_a ? gram[(int64_t)s_creator[a] * p.Cmax + j] : -INFINITY;
+      }
+      for (int a = part + 4 * LT; merged && a < n_a; a += LT) gm = fmaxf(gm, gram[(int64_t)s_creator[a] * p.Cmax + j]);
 #pragma unroll
-          for (int k = 0; k < 4; ++k)
-            if (k == cntc) { ca[k] = a; cp[k] = pv; }
-          ++cntc;
+      for (int t = 0; t < 4; ++t) gm = fmaxf(gm, pv[t]);
+      for (int o = LT >> 1; o > 0; o >>= 1) gm = fmaxf(gm, __shfl_xor_sync(0xffffffffu, gm, o));
+      double bar = INFINITY;
+      if (merged) {
+        const double eps = 0.5 * (double)s_thr[j];
+        bar = fmax(s_best[j], (double)gm - eps) - eps;
+      }
+      for (int t = 0; t * LT < n_a; ++t) {
+        const int a = part + t * LT;
+        const float v = t == 0 ? pv[0] : t == 1 ? pv[1] : t == 2 ? pv[2] : t == 3 ? pv[3]
+                        : merged && a < n_a ? gram[(int64_t)s_creator[a] * p.Cmax + j] : -INFINITY;
+        const bool in = merged && a < n_a && (double)v >= bar;
+        const unsigned hit = __ballot_sync(0xffffffffu, in);
+        if (np + __popc(hit) > kWarpPairs) { over = true; break; }
+        if (in) {
+          const int w = np + __popc(hit & ((1u << lane) - 1u));
+          prow[w] = a; ptok[w] = (unsigned char)j;
         }
-      };
-      if (otf) {
-        const __half* kj = p.kbarH + ((int64_t)u * p.CbarRows + j) * D;
-        for (int a0 = 0; a0 < n_a; a0 += 4) {
-          float acc[4] = {0.f, 0.f, 0.f, 0.f};
-#pragma unroll 2
-          for (int ch = 0; ch < D / 8; ++ch) {
-            const uint4 kw = *reinterpret_cast<const uint4*>(kj + 8 * ch);
-            const __half2* kh = reinterpret_cast<const __half2*>(&kw);
-            float2 kf[4];
+        np += __popc(hit);
+      }
+      if (over) np = 0;
+    }
+    __syncwarp();
+    exact_pairs(np, true);
+    npair += np;
+    {
+      const int j = wj0 + lane;
+      const bool merged = j < wj1 && !s_app[j];
+      if (merged && np > 0) {
+        double best = s_best[j];
+        int arg = s_barg[j];
+        for (int q = 0; q < np; ++q) {   // (few, of all the warp's tokens; ties: the lowest row)
+          const double v = pval[q];
+          const int row = (int)m + prow[q];
+          if (ptok[q] == j && (v > best || (v == best && row < arg))) { best = v; arg = row; }
+        }
+        s_barg[j] = arg;
+      }
+      unsigned todo = __ballot_sync(0xffffffffu, merged && over);   // more contenders than the list holds: every new row exactly
+      nexh += __popc(todo);
+      while (todo) {
+        const int jx = wj0 + __ffs(todo) - 1;
+        todo &= todo - 1;
+        double kb[CH];
 #pragma unroll
-            for (int q = 0; q < 4; ++q) kf[q] = __half22float2(kh[q]);
+        for (int c = 0; c < CH; ++c) kb[c] = kbarU.at(jx, lane + 32 * c, gam[c], bet[c]);
+        double best = s_best[jx];
+        int arg = s_barg[jx];
+        for (int a = 0; a < n_a; ++a) {
+          const int jc = s_creator[a];
+          const double2 hs = p.kbarHatStat[tokBase + jc];
+          double acc = 0.0;
 #pragma unroll
-            for (int t = 0; t < 4; ++t) {
-              const int a = min(a0 + t, n_a - 1);   // (a clamped duplicate is computed and dropped)
-              const uint4 hw = *reinterpret_cast<const uint4*>(&s_hat[a][8 * ch]);
-              const __half2* hh = reinterpret_cast<const __half2*>(&hw);
-#pragma unroll
-              for (int q = 0; q < 4; ++q) {
-                const float2 hf = __half22float2(hh[q]);
-                acc[t] = fmaf(kf[q].x, hf.x, acc[t]);
-                acc[t] = fmaf(kf[q].y, hf.y, acc[t]);
-              }
-            }
+          for (int c = 0; c < CH; ++c) {
+            const double hat = gam[c] * ((kbarU.at(jc, lane + 32 * c, gam[c], bet[c]) - hs.x) * hs.y) + bet[c];
+            acc += kb[c] * hat;
           }
-#pragma unroll
-          for (int t = 0; t < 4; ++t)
-            if (a0 + t < n_a) consider(a0 + t, acc[t]);
+          acc = warp_sum_d(acc);
+          if (acc > best) { best = acc; arg = (int)m + a; }
         }
-      } else {
-        // (all loads of a batch in flight before the first product is looked at)
-        const float* gcol = p.gramT + (int64_t)u * p.Cmax * p.Cmax + j;
-        for (int a0 = 0; a0 < n_a; a0 += 16) {
-          float pv[16];
-#pragma unroll
-          for (int t = 0; t < 16; ++t) pv[t] = a0 + t < n_a ? gcol[(int64_t)s_creator[a0 + t] * p.Cmax] : 0.f;
-#pragma unroll
-          for (int t = 0; t < 16; ++t)
-            if (a0 + t < n_a) consider(a0 + t, pv[t]);
-        }
+        if (lane == 0) s_barg[jx] = arg;
       }
-      bool exh = cntc > 4;   // more than four contenders: every new row exactly
-      if (!exh) {            // prune against the final bar (order kept: ascending new-row index)
-        const double bar = fmax(best_old, (double)gm - eps) - eps;
-        int kept = 0;
-#pragma unroll
-        for (int k = 0; k < 4; ++k) {
-          if (k < cntc && (double)cp[k] >= bar) {
-#pragma unroll
-            for (int k2 = 0; k2 < 4; ++k2)
-              if (k2 == kept) ca[k2] = ca[k];
-            ++kept;
-          }
-        }
-        cntc = kept;
-      }
-      int start = 0;
-      if (!exh && cntc > 0) {
-        start = atomicAdd(&s_np, cntc);
-        if (start + cntc > kPairCap) exh = true;
-      }
-      if (!exh && cntc > 0) {
-#pragma unroll
-        for (int k = 0; k < 4; ++k) {
-          if (k < cntc) {
-            s_prow[start + k] = ca[k];          // index of the new row, ascending within a token
-            s_ptok[start + k] = (unsigned short)j;
-          }
-        }
-        s_pstart[j] = start;
-        s_pcnt[j] = cntc;
-      }
-      s_exh[j] = exh ? 1 : 0;
-      if (exh) atomicAdd(&s_nexh, 1);
+      __syncwarp();
     }
   }
+  // ---- E: every CTA of the unit gets all merge targets ----
+  for (int e = lane; e < (wj1 - wj0) * R; e += 32) {
+    const int j = wj0 + e / R;
+    // (rows < 2^23, tokens < 2^9)
+    give32(reinterpret_cast<int*>(s_tgt), 2, j, e % R, s_app[j] ? -1 : (int)(((unsigned)s_barg[j] << 9) | (unsigned)j));
+  }
+  if (lane == 0 && nexh) atomicAdd(&s_nexh, nexh);
+  if (lane == 0 && npair) atomicAdd(&s_npair, npair);
+  received(2);
   __syncthreads();
-  if (n_a > 0) {
-    const int np2 = min(s_np, kPairCap);
-    for (int q0 = warp; q0 < np2; q0 += 8 * kDecideWarps) {
-      double part[8];
-#pragma unroll
-      for (int k = 0; k < 8; ++k) {
-        const int q = min(q0 + k * kDecideWarps, np2 - 1);
-        const int jt = s_ptok[q];
-        const int jc = s_creator[s_prow[q]];
-        const double2 hs = p.kbarHatStat[tokBase + jc];
-        double acc = 0.0;
-#pragma unroll
-        for (int c = 0; c < CH; ++c) {
-          const double hat = gam[c] * ((kbarU.at(jc, lane + 32 * c, gam[c], bet[c]) - hs.x) * hs.y) + bet[c];
-          acc += kbarU.at(jt, lane + 32 * c, gam[c], bet[c]) * hat;
-        }
-        part[k] = acc;
-      }
-      const double z0 = warp_reduce4(part[0], part[1], part[2], part[3], lane);
-      const double z1 = warp_reduce4(part[4], part[5], part[6], part[7], lane);
-      if ((lane & 7) == 0) {
-        const int qa = q0 + (lane >> 3) * kDecideWarps, qb = qa + 4 * kDecideWarps;
-        if (qa < np2) s_pval[qa] = z0;
-        if (qb < np2) s_pval[qb] = z1;
-      }
-    }
-    // tokens whose candidate list did not fit: every new row exactly, one warp per token
-    for (int j = warp; j < C; j += kDecideWarps) {
-      if (!s_exh[j]) continue;
-      double kb[CH];
-#pragma unroll
-      for (int c = 0; c < CH; ++c) kb[c] = kbarU.at(j, lane + 32 * c, gam[c], bet[c]);
-      double best = s_best[j];
-      int arg = s_barg[j];
-      for (int a = 0; a < n_a; ++a) {
-        const int jc = s_creator[a];
-        const double2 hs = p.kbarHatStat[tokBase + jc];
-        double acc = 0.0;
-#pragma unroll
-        for (int c = 0; c < CH; ++c) {
-          const double hat = gam[c] * ((kbarU.at(jc, lane + 32 * c, gam[c], bet[c]) - hs.x) * hs.y) + bet[c];
-          acc += kb[c] * hat;
-        }
-        acc = warp_sum_d(acc);
-        if (acc > best) { best = acc; arg = (int)m + a; }
-      }
-      if (lane == 0) { s_best[j] = best; s_barg[j] = arg; }
-    }
-  }
-  __syncthreads();
-  const bool merged = tid < C && !s_app[tid];
-  if (merged) {
-    double best = s_best[tid];
-    int arg = s_barg[tid];
-    if (n_a > 0 && !s_exh[tid]) {
-      const int st0 = s_pstart[tid];
-      for (int q = st0; q < st0 + s_pcnt[tid]; ++q) {   // ascending new-row index: the first maximum wins
-        const double v = s_pval[q];
-        if (v > best) { best = v; arg = (int)m + s_prow[q]; }
-      }
-    }
-    s_pi[tid] = arg;
-  }
-  {   // number of merged tokens: a block-wide count (an atomic per token on one word would serialise)
-    const int nm = __syncthreads_count(merged);
-    if (tid == 0) s_nmerge = nm;
-  }
-  // ---- E: order merged tokens by (row, token); publish ----
-  {   // (ranks counted as in the append selection; keys of merged tokens are distinct, the others go last)
-    unsigned* ekey = reinterpret_cast<unsigned*>(s_prow);   // (the pair list is idle here)
-    unsigned* ukey = ekey + 256;                             // unsorted keys
-    if (tid < kMaxBlock) {
-      const int pj = tid < C ? s_pi[tid] : -1;
-      ukey[tid] = pj >= 0 ? (((unsigned)pj << 9) | (unsigned)tid) : 0xffffffffu;   // rows < 2^23, tokens < 2^9
-      ekey[tid] = 0xffffffffu;
-      s_fill[tid] = 0;
-      if (tid < C) {
-        p.pi[tokBase + tid] = pj;
-        p.creator[tokBase + tid] = s_creator[tid];
-      }
-    }
-    __syncthreads();
-    const int j = tid & (kMaxBlock - 1), h = tid / kMaxBlock;
-    const unsigned kj = ukey[j];
-    if (j < C && kj != 0xffffffffu) {
-      const int half_n = (C + 1) / 2, i0 = h * half_n, i1 = min(C, i0 + half_n);
-      int cnt = 0;
-#pragma unroll 4
-      for (int i = i0; i < i1; ++i) cnt += ukey[i] < kj ? 1 : 0;
-      atomicAdd(&s_fill[j], cnt);
-    }
-    __syncthreads();
-    if (tid < C && ukey[tid] != 0xffffffffu) ekey[s_fill[tid]] = ukey[tid];   // ranks 0 .. nmerge-1
-    __syncthreads();
-    const unsigned kq = tid < kMaxBlock ? ekey[tid] : 0xffffffffu;
-    if (kq != 0xffffffffu) {
-      const int rowq = (int)(kq >> 9);
-      p.sorted[tokBase + tid] = (int)(kq & 511u);
-      const bool head = tid == 0 || (int)(ekey[tid - 1] >> 9) != rowq;
-      if (head && rowq >= m) p.segnew[tokBase + (rowq - (int)m)] = tid;
-    }
+  if (many) asm volatile("barrier.cluster.arrive.release;" ::: "memory");
+  if (s_dead) {   // (a wait ran out: nothing is applied)
+    if (tid == 0) atomicExch(p.counters - 1, (int)KVM_ERR_TIMEOUT);
+    if (many) asm volatile("barrier.cluster.wait.acquire;" ::: "memory");
+    return;
   }
   if (tid == 0) {
-    p.nmerge[u] = s_nmerge;
-    atomicAdd(&p.counters[0], s_nexh);
-    atomicAdd(&p.counters[1], min(s_np, kPairCap));
-    atomicAdd(&p.counters[2], C);
+    if (s_nexh) atomicAdd(&p.counters[0], s_nexh);
+    if (s_npair) atomicAdd(&p.counters[1], s_npair);
+    atomicAdd(&p.counters[2], jhi - jlo);
   }
+
+  // ---- F: publish, q threads per token of this CTA: a merged token's rank in the order (row, token), whether it heads
+  //      its row's segment; an appended token's row, and where that row's segment begins ----
+  {
+    int q = 1;
+    while (2 * q * nsl <= kDecideThreads && q < 32) q *= 2;
+    const int j = jlo + tid / q, part = tid & (q - 1);
+    const bool mine = j < jhi;
+    int pos = 0;
+    bool app = false;
+    unsigned key = 0u;   // (an appended token: the lowest key of its row)
+    if (mine) {
+      app = s_app[j] != 0;
+      key = s_tgt[j];
+      if (app) {
+        pos = __popc(s_word[j >> 5] & ((1u << (j & 31)) - 1u));
+        for (int w = 0; w < (j >> 5); ++w) pos += __popc(s_word[w]);
+        key = (unsigned)(m + pos) << 9;
+      }
+    }
+    int less = 0;   // merged tokens before `key` in the order (row, token)
+    bool members = false;
+    if (mine) {
+#pragma unroll 4
+      for (int i = part; i < C; i += q) less += s_tgt[i] < key ? 1 : 0;
+      if (app)
+        for (int i = part; i < C; i += q) members |= (s_tgt[i] >> 9) == (key >> 9);
+    }
+    int cnt = less | (members ? 1 << 16 : 0);
+    for (int o = q >> 1; o > 0; o >>= 1) cnt += __shfl_xor_sync(0xffffffffu, cnt, o);
+    less = cnt & 0xffff; members = cnt >> 16 != 0;
+    if (mine && part == 0) {
+      if (app) {
+        p.pi[tokBase + j] = -1;
+        p.creator[tokBase + pos] = j;
+        p.segnew[tokBase + pos] = members ? less : -1;
+      } else {
+        p.pi[tokBase + j] = (int)(key >> 9);
+        p.sorted[tokBase + less] = j;
+      }
+    }
+    if (tid == 0 && rank == 0) p.nmerge[u] = C - n_a;
+  }
+  if (many) asm volatile("barrier.cluster.wait.acquire;" ::: "memory");   // (nobody leaves before everybody has received)
 }
 
 // ------------------------------------------------------------------------------------------
@@ -1005,8 +923,8 @@ __device__ __forceinline__ void mma_m16n8k16(float (&c)[4], uint32_t a0, uint32_
                : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1));
 }
 
-template <int D, bool RK>
-__global__ void __launch_bounds__(kPrunedThreads, 4) fold_decide_pruned_kernel(FoldDecideParams p) {
+template <int D, int PER_SM, bool RK>
+__global__ void __launch_bounds__(kPrunedThreads, PER_SM) fold_decide_pruned_kernel(FoldDecideParams p) {
   constexpr int CH = D / 32;
   constexpr int HS = D + 32;   // row stride of the new rows' keys in halves: consecutive rows start 16 banks apart
   __shared__ double s_lo[kMaxBlock], s_hi[kMaxBlock];   // bounds of the score; then exact score / exact best of scored tokens
@@ -2090,6 +2008,27 @@ int launch_prev_copy(State* st, cudaStream_t s) {
   return 1;
 }
 
+template <int PER_SM>
+static void launch_pruned(const State* st, const cudaLaunchConfig_t& lc, const FoldDecideParams& p) {
+  if (st->d == 128) {
+    if (st->recomputeK) cudaLaunchKernelEx(&lc, fold_decide_pruned_kernel<128, PER_SM, true>, p);
+    else cudaLaunchKernelEx(&lc, fold_decide_pruned_kernel<128, PER_SM, false>, p);
+  } else {
+    if (st->recomputeK) cudaLaunchKernelEx(&lc, fold_decide_pruned_kernel<64, PER_SM, true>, p);
+    else cudaLaunchKernelEx(&lc, fold_decide_pruned_kernel<64, PER_SM, false>, p);
+  }
+}
+template <int PER_SM>
+static void launch_decide(const State* st, const cudaLaunchConfig_t& lc, const FoldDecideParams& p) {
+  if (st->d == 128) {
+    if (st->recomputeK) cudaLaunchKernelEx(&lc, fold_decide_kernel<128, PER_SM, true>, p);
+    else cudaLaunchKernelEx(&lc, fold_decide_kernel<128, PER_SM, false>, p);
+  } else {
+    if (st->recomputeK) cudaLaunchKernelEx(&lc, fold_decide_kernel<64, PER_SM, true>, p);
+    else cudaLaunchKernelEx(&lc, fold_decide_kernel<64, PER_SM, false>, p);
+  }
+}
+
 int launch_fold(State* st, const FoldArgs& a, cudaStream_t s) {
   int launches = 0;
   const int C = st->C, D = st->d;
@@ -2134,51 +2073,41 @@ int launch_fold(State* st, const FoldArgs& a, cudaStream_t s) {
     p.pi = st->foldPi[dst]; p.sorted = st->foldSorted[dst]; p.creator = st->foldCreator[dst];
     p.segnew = st->foldSegNew[dst]; p.nmerge = st->foldNMerge[dst];
     p.counters = st->status + 1;
-    p.xScore = st->xScore; p.xBest = st->xBest; p.xArg = st->xArg; p.xCount = st->xCount;
     p.Mcap = st->Mcap; p.m = a.m;
     p.C = C; p.Cmax = st->Cmax; p.Hkv = st->Hkv; p.S = st->S; p.n_append = a.n_append; p.nsplit = nsplit;
     p.thr_coeff = route_thr_coeff(st);
     p.ln_eps = (double)st->ln_eps;
     KernelTimer kt(st, 4, s);
-    // CTAs per unit (measured on U = 1, 8, 32, 256): about 64 CTAs in all, at least two per unit while
-    // 2U CTAs fit the GPU in one wave, at most eight, at least 16 tokens each - beyond that the
-    // hand-over costs more than the shorter slices save.  A fold that appends nothing has few pairs
-    // to refine (most tokens have one candidate and need no exact similarity): one CTA per unit.
-    int R = 64 / st->U;
-    if (R < 2 && 2 * st->U <= 2 * 148) R = 2;
-    if (R > 8) R = 8;
-    if (R > C / 16) R = C / 16;
-    if (R < 1 || a.n_append == 0) R = 1;
-    dim3 dgrid(R, st->U);
+    // CTAs per unit: about 64 in all - with 128, what shorter slices save is lost to the attention kernel beside them,
+    // which needs whole SMs (measured, 32 units: 9.0 against 8.5 ms for 32768 tokens; 8 units: no difference) -, two per
+    // unit while those fit the GPU, at least 16 tokens each
+    int ctas = 64 / st->U;
+    if (ctas < 2 && 2 * st->U <= 148) ctas = 2;
+    if (ctas > C / 16) ctas = C / 16;
+    int R = 1;
+    while (2 * R <= ctas && R < kDecideMaxCtas) R *= 2;
     // programmatic dependent launch: the CTAs may start (and set up their shared memory) while the
     // routing filter is still running; they wait for it before the first read of its output
+    // (measured off / on: 24 units with 96 query heads 2.15 / 1.84 ms for 5000 tokens, one unit 351 / 308 us for 1024,
+    // 32 units 8.77 / 8.56 ms for 32768)
     cudaLaunchConfig_t lc = {};
-    lc.gridDim = dgrid; lc.blockDim = dim3(kDecideThreads); lc.dynamicSmemBytes = 0; lc.stream = s;
-    cudaLaunchAttribute at[1];
+    lc.gridDim = dim3(R, st->U); lc.blockDim = dim3(kDecideThreads); lc.dynamicSmemBytes = 0; lc.stream = s;
+    cudaLaunchAttribute at[2];
     at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    at[0].val.programmaticStreamSerializationAllowed = 1;
-    // Measured: the early start pays when the filter, these CTAs and the attention CTAs of a block
-    // all find room on the GPU at once (or when every kernel fills it anyway); in between, CTAs
-    // that sit waiting keep the attention kernel, which needs whole SMs, off them.
-    const int sms_wanted = nsplit * st->U + (R * st->U + 1) / 2 + st->B * st->Hq * ((C + 127) / 128);
-    const bool pdl = st->prof_hook == nullptr && !(st->flags & KVM_FLAG_SIMT_ROUTING) &&
-                     (sms_wanted <= 148 || st->U >= 148);
-    lc.attrs = at; lc.numAttrs = pdl ? 1 : 0;
-    const bool roomy = R * st->U <= 148;
-#define KVM_DECIDE(DD, PP, RR) cudaLaunchKernelEx(&lc, fold_decide_kernel<DD, PP, RR>, p)
-    const bool rk = st->recomputeK;
+    at[0].val.programmaticStreamSerializationAllowed = st->prof_hook == nullptr && !(st->flags & KVM_FLAG_SIMT_ROUTING) ? 1 : 0;
+    at[1].id = cudaLaunchAttributeClusterDimension;
+    at[1].val.clusterDim.x = R; at[1].val.clusterDim.y = 1; at[1].val.clusterDim.z = 1;
+    lc.attrs = at; lc.numAttrs = R > 1 ? 2 : 1;
     if (st->U > 148 && a.n_append > 0) {   // (R == 1 here) more units than SMs: bounds first, few exact pairs
       lc.blockDim = dim3(kPrunedThreads);
-      if (D == 128) { if (rk) cudaLaunchKernelEx(&lc, fold_decide_pruned_kernel<128, true>, p); else cudaLaunchKernelEx(&lc, fold_decide_pruned_kernel<128, false>, p); }
-      else { if (rk) cudaLaunchKernelEx(&lc, fold_decide_pruned_kernel<64, true>, p); else cudaLaunchKernelEx(&lc, fold_decide_pruned_kernel<64, false>, p); }
-    } else if (D == 128) {
-      if (roomy) { if (rk) KVM_DECIDE(128, 1, true); else KVM_DECIDE(128, 1, false); }
-      else { if (rk) KVM_DECIDE(128, 2, true); else KVM_DECIDE(128, 2, false); }
+      // 128 registers (every load of the exact passes in flight) while one wave holds all units: measured, 256 units: 93 ->
+      // 71 us; 512 units, in two waves: 112 -> 123 us
+      if (st->U <= 2 * 148) launch_pruned<2>(st, lc, p);
+      else launch_pruned<4>(st, lc, p);
     } else {
-      if (roomy) { if (rk) KVM_DECIDE(64, 1, true); else KVM_DECIDE(64, 1, false); }
-      else { if (rk) KVM_DECIDE(64, 2, true); else KVM_DECIDE(64, 2, false); }
+      if (R * st->U <= 148) launch_decide<1>(st, lc, p);
+      else launch_decide<2>(st, lc, p);
     }
-#undef KVM_DECIDE
     ++launches;
   }
   FoldApplyParams q;

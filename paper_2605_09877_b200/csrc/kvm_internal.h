@@ -16,7 +16,7 @@ constexpr int kMaxSplits = 32;      // routing filter split count upper bound
 constexpr int kAttnSplitTiles = 37; // launches with at most this many (batch, head, query tile) CTAs - a quarter of the GPU - are split along the keys
 constexpr int kAttnMaxSplits = 8;
 constexpr int kRowAlign = 128;      // state capacity is rounded up to the attention key tile
-constexpr int kGramOnTheFly = 32;   // in a state with enough units to fill the GPU (State::serial), folds that append at most this
+constexpr int kGramOnTheFly = 32;   // in a state with enough units to fill the GPU (gram_from), folds that append at most this
                                     // many rows compute the products of the other tokens with the new rows inside the decision
                                     // kernel; all other folds read them from the batched tensor-core product of all token pairs of
                                     // the block (gramT), computed off the folds' critical path - most of it never read
@@ -101,8 +101,6 @@ struct State {
   float* gramT;                  // [kbSlots][U, Cmax, Cmax]  approximate kbarHat_a . kbar_j at [a][j] (new-row filter)
   // decisions of the fold being computed ([(nfolds+1) & 1]) and of the one before ([nfolds & 1])
   int32_t *foldPi[2], *foldSorted[2], *foldCreator[2], *foldSegNew[2], *foldNMerge[2];
-  double *xScore, *xBest;        // [U, Cmax] hand-over between the CTAs of the decide kernel
-  int32_t *xArg, *xCount;        // [U, Cmax]; [U]
   int nsplitRoute;               // splits the routing filter may use
   float* candV;                  // [U, nsplitRoute, Cmax, kTopK]  routing filter output: (split maximum, candidate count, ...)
   int32_t* candI;                // [U, nsplitRoute, Cmax, kTopK]  candidate rows
@@ -133,7 +131,7 @@ struct State {
 
 inline int64_t budget_of(const kvm_growth_t& g, int64_t e);
 // folds that append more rows than this (and not the whole block) take the batched product of the block's token pairs
-inline int gram_from(const State* st) { return st->serial ? kGramOnTheFly : 0; }
+inline int gram_from(const State* st) { return st->serial && st->U > 148 ? kGramOnTheFly : 0; }
 
 // ---------------- launchers (each returns the number of kernels it launched) ----------------
 

@@ -211,3 +211,56 @@ def test_shape_sweep_with_more_units_than_sms(case):
     stats = _sampled(wl, units, params=params, gate=gate, decode_from=(T - dec) if dec else None,
                      flags=kvm.FLAG_SERIAL_FOLDS if serial else 0)
     print(case, stats)
+
+
+_DECIDE = [
+    # (B, Hq, Hkv, d, C, blocks, extra, growth kwargs, r, S, w, kind, flags_serial, gate)
+    (1, 1, 1, 64, 16, 12, 5, dict(growth="sqrt", sqrt_coeff=3), 0, 0, 2, "normal", False, False),          # one CTA
+    (1, 1, 1, 128, 256, 9, 1, dict(growth="sqrt", sqrt_coeff=16), 32, 1, 2, "mixture", False, True),       # eight CTAs
+    (1, 3, 3, 64, 136, 10, 40, dict(growth="fixed", fixed_slots=200), 16, 4, 3, "needles", False, True),   # slices of 17
+    (3, 6, 3, 128, 200, 7, 0, dict(growth="power", sqrt_coeff=6, pow_num=2, pow_den=3), 0, 0, 1, "scaled_keys", False, False),
+    (2, 20, 10, 64, 72, 11, 3, dict(growth="saturating", fixed_slots=300, sat_half=400), 0, 1, 2, "mixture", True, True),
+    (4, 10, 10, 128, 256, 5, 9, dict(growth="sqrt", sqrt_coeff=20), 32, 2, 2, "normal", True, False),      # keys recomputed
+    (5, 15, 15, 64, 104, 6, 0, dict(growth="fixed", fixed_slots=104), 0, 1, 2, "normal", False, False),    # one CTA per unit
+    (4, 37, 37, 64, 48, 6, 7, dict(growth="sqrt", sqrt_coeff=5), 16, 1, 2, "mixture", False, True),        # 148 units
+    (10, 15, 15, 64, 48, 8, 0, dict(growth="fixed", fixed_slots=64), 0, 2, 2, "normal", False, True),      # decisions alone
+]
+
+
+@pytest.mark.parametrize("case", range(len(_DECIDE)))
+def test_decisions_over_cluster_sizes_and_slices(case):
+    """One to eight CTAs per unit, slices of the block that are no multiple of a warp, every budget rule, full states
+    that append nothing, one and two readout copies, up to 150 units."""
+    from paper_2605_09877_b200 import kvm
+    B, Hq, Hkv, d, C, nb, extra, gk, r, S, w, kind, serial, gate = _DECIDE[case]
+    wl = synth.Workload("step", B, Hq, Hkv, d, C * nb + extra, C, r=r, S=S, w=w, seed=300 + case, kind=kind, **gk)
+    params = synth.make_layer_params(wl, trivial=(case % 2 == 0))
+    units = [(0, 0), (B // 2, Hkv // 2), (B - 1, Hkv - 1)]
+    print(case, _sampled(wl, units, params=params, gate=gate, flags=kvm.FLAG_SERIAL_FOLDS if serial else 0))
+
+
+def test_decisions_scan_every_row_for_tokens_with_too_many_candidates():
+    """Keys repeated over whole blocks: most rows of the state tie, the filter's lists overflow, and the tokens are
+    scored against every row (and, where rows are appended, against every new row)."""
+    wl = synth.Workload("t", 1, 4, 4, 64, 64 * 8 + 3, 64, "sqrt", sqrt_coeff=8, r=0, S=2, seed=320)
+    tensors = synth.make_inputs(wl)
+    tensors["k"][:, 0] = tensors["k"][:, 0, :1]                        # one key
+    for j in range(wl.T):
+        tensors["k"][:, 1, j] = tensors["k"][:, 1, j % 3]             # three keys in turn
+    tensors["k"][:, 2, 64:] = tensors["k"][:, 2, 64:65]
+    params = synth.make_layer_params(wl)
+    y_gpu, st = pu.run_gpu(wl, tensors, params)
+    y_ref, o = pu.run_oracle(wl, tensors, params)
+    print(pu.compare(wl, y_gpu, st, y_ref, o))
+    assert st.debug_counters()["exhaustive_tokens"] > 0
+    st.free()
+
+
+@pytest.mark.parametrize("B,Hq,Hkv,d,pos,steps", [
+    (1, 1, 1, 64, 40, 30), (1, 2, 1, 128, 900, 20), (3, 32, 4, 64, 1300, 10), (7, 21, 21, 128, 300, 9), (9, 64, 64, 64, 700, 6),
+    (40, 32, 8, 128, 300, 4)])
+def test_decode_row_splits_from_one_to_eight(B, Hq, Hkv, d, pos, steps):
+    """Clusters of one, two, four and eight CTAs per head, one to eight query heads per CTA, splits without rows."""
+    wl = synth.Workload("dec", B, Hq, Hkv, d, pos + steps, 64, "sqrt", sqrt_coeff=20, r=32, seed=330 + pos)
+    params = synth.make_layer_params(wl, trivial=False)
+    print(_sampled(wl, [(0, 0), (B - 1, Hkv - 1)], params=params, decode_from=pos))
