@@ -89,6 +89,28 @@ __device__ __forceinline__ void kbar_run4(const KbarRows<D, RK>& kr, int j, int 
   }
 }
 
+// The same with LN_s weight and bias of the unit in fp64 (shared memory): the conversions of the two, eight cycles of the
+// conversion unit each, were two thirds of what a recomputed channel asked of it (apply kernel, 256 full units of 256
+// rows: 74.9 -> 65.4 us; 256 units of 2000 rows: 68 -> 65; 512 units: 144 -> 138).
+template <int D, bool RK>
+__device__ __forceinline__ void kbar_run4(const KbarRows<D, RK>& kr, int j, int x, const double* w64, const double* b64, double (&out)[4]) {
+  if (!RK) {
+    const double* kb = kr.k64 + (int64_t)j * D + x;
+    const double2 k01 = *reinterpret_cast<const double2*>(kb), k23 = *reinterpret_cast<const double2*>(kb + 2);
+    out[0] = k01.x; out[1] = k01.y; out[2] = k23.x; out[3] = k23.y;
+  } else {
+    alignas(8) __half hv[4];
+    *reinterpret_cast<uint2*>(hv) = *reinterpret_cast<const uint2*>(kr.k16 + (int64_t)j * D + x);
+    const double2 w01 = *reinterpret_cast<const double2*>(w64 + x), w23 = *reinterpret_cast<const double2*>(w64 + x + 2);
+    const double2 b01 = *reinterpret_cast<const double2*>(b64 + x), b23 = *reinterpret_cast<const double2*>(b64 + x + 2);
+    const double wv[4] = {w01.x, w01.y, w23.x, w23.y}, bv[4] = {b01.x, b01.y, b23.x, b23.y};
+    const double2 st = kr.stat[j];
+#pragma unroll
+    for (int e = 0; e < 4; ++e)
+      out[e] = ln_affine(x + e < kr.r ? 0.0 : (double)__half2float(hv[e]), st.x, st.y, wv[e], bv[e]);
+  }
+}
+
 // ------------------------------------------------------------------------------------------
 // 1. memory keys (one warp per overflow token)
 
@@ -1660,6 +1682,7 @@ __global__ void __launch_bounds__(256, 2) fold_apply_rows4_kernel(FoldApplyParam
   constexpr double inv_d = 1.0 / D;   // D is a power of two: multiplying is dividing, exactly
   __shared__ int s_pi[kMaxBlock], s_sorted[kMaxBlock], s_creator[kMaxBlock], s_segnew[kMaxBlock];
   __shared__ int s_nmerge;
+  __shared__ __align__(16) double s_w[D], s_b[D];   // LN_s weight and bias of the unit
   // the routing filter of the next fold may start its set-up now; it waits for this grid to finish
   // before it reads the readout keys written here
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
@@ -1674,14 +1697,16 @@ __global__ void __launch_bounds__(256, 2) fold_apply_rows4_kernel(FoldApplyParam
       s_creator[i] = p.creator[tokBase + i];
       s_segnew[i] = p.segnew[tokBase + i];
     }
-    __syncthreads();
   }
+  if (threadIdx.x < D) {
+    s_w[threadIdx.x] = (double)p.ln_w[hk * D + threadIdx.x];
+    s_b[threadIdx.x] = (double)p.ln_b[hk * D + threadIdx.x];
+  }
+  __syncthreads();
   const int64_t rowBase = (int64_t)u * p.Mcap;
   KbarRows<D, RK> kbarU;
   kbarU.k64 = p.kbar64 + tokBase * D; kbarU.k16 = p.ok + (int64_t)u * p.unit_stride;
   kbarU.stat = p.kbarStat + tokBase; kbarU.r = p.r;
-  const float* lnwH = p.ln_w + hk * D;
-  const float* lnbH = p.ln_b + hk * D;
   const __half* ovU = p.ov + (int64_t)u * p.unit_stride;
   const float* ogU = p.og + (int64_t)u * p.gate_stride;
   const int nmerge = p.all_append ? 0 : s_nmerge;
@@ -1729,7 +1754,7 @@ __global__ void __launch_bounds__(256, 2) fold_apply_rows4_kernel(FoldApplyParam
         for (int i = 0; i < NI; ++i) {
           const int x = 32 * i + 4 * sub;
           double k4[4];
-          kbar_run4<D, RK>(kbarU, jc, x, lnwH, lnbH, k4);
+          kbar_run4<D, RK>(kbarU, jc, x, s_w, s_b, k4);
           kx[4 * i] = k4[0]; kx[4 * i + 1] = k4[1]; kx[4 * i + 2] = k4[2]; kx[4 * i + 3] = k4[3];
           alignas(8) __half hv[4];
           *reinterpret_cast<uint2*>(hv) = *reinterpret_cast<const uint2*>(vr + x);
@@ -1771,7 +1796,7 @@ __global__ void __launch_bounds__(256, 2) fold_apply_rows4_kernel(FoldApplyParam
         for (int i = 0; i < NI; ++i) {
           const int x = 32 * i + 4 * sub;
           double k4[4];
-          kbar_run4<D, RK>(kbarU, j, x, lnwH, lnbH, k4);
+          kbar_run4<D, RK>(kbarU, j, x, s_w, s_b, k4);
           kx[4 * i] += (double)g * k4[0]; kx[4 * i + 1] += (double)g * k4[1];
           kx[4 * i + 2] += (double)g * k4[2]; kx[4 * i + 3] += (double)g * k4[3];
           alignas(8) __half hv[4];
@@ -1807,12 +1832,13 @@ __global__ void __launch_bounds__(256, 2) fold_apply_rows4_kernel(FoldApplyParam
 #pragma unroll
     for (int i = 0; i < NI; ++i) {
       const int x = 32 * i + 4 * sub;
-      const float4 w4 = *reinterpret_cast<const float4*>(p.ln_w + hk * D + x), b4 = *reinterpret_cast<const float4*>(p.ln_b + hk * D + x);
-      const float wv[4] = {w4.x, w4.y, w4.z, w4.w}, bv[4] = {b4.x, b4.y, b4.z, b4.w};
+      const double2 w01 = *reinterpret_cast<const double2*>(s_w + x), w23 = *reinterpret_cast<const double2*>(s_w + x + 2);
+      const double2 b01 = *reinterpret_cast<const double2*>(s_b + x), b23 = *reinterpret_cast<const double2*>(s_b + x + 2);
+      const double wv[4] = {w01.x, w01.y, w23.x, w23.y}, bv[4] = {b01.x, b01.y, b23.x, b23.y};
       alignas(8) __half kh[4], vh[4];
 #pragma unroll
       for (int e = 0; e < 4; ++e) {
-        const double hat = (double)wv[e] * ((kx[4 * i + e] - mu) * rs) + (double)bv[e];
+        const double hat = wv[e] * ((kx[4 * i + e] - mu) * rs) + bv[e];
         kh[e] = __float2half_rn((float)hat);
         vh[e] = __float2half_rn((float)((double)vx[4 * i + e] * vscale));
       }
