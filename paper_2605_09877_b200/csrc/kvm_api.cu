@@ -141,11 +141,14 @@ void free_all(kvm_state* ks) {
 }
 
 struct DeviceGuard {
-  int prev = -1;
+  int prev = -1;   // the device to go back to, if another one was current
   bool ok = true;
   explicit DeviceGuard(int dev) {
-    if (cudaGetDevice(&prev) != cudaSuccess) { ok = false; cudaGetLastError(); return; }
-    if (prev != dev && cudaSetDevice(dev) != cudaSuccess) { ok = false; cudaGetLastError(); }
+    int cur = -1;
+    if (cudaGetDevice(&cur) != cudaSuccess) { ok = false; cudaGetLastError(); return; }
+    if (cur == dev) return;
+    prev = cur;
+    if (cudaSetDevice(dev) != cudaSuccess) { ok = false; cudaGetLastError(); }
   }
   ~DeviceGuard() { if (prev >= 0) cudaSetDevice(prev); }
 };

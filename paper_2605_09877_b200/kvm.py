@@ -177,9 +177,12 @@ def _fp(a):
 
 
 def _stream_ptr(stream):
-    if stream is None:
-        stream = torch.cuda.current_stream()
-    return C.c_void_p(stream.cuda_stream)
+    if stream is not None:
+        return stream.cuda_stream
+    if not torch.cuda.is_initialized():
+        return torch.cuda.current_stream().cuda_stream
+    # the current stream of the current device, without the Stream object around it
+    return torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice())
 
 
 def attend_rows_noalloc(q, keys, values, scale: float, out=None, stream=None):
@@ -281,9 +284,10 @@ class KVMState:
         assert q.is_contiguous() and k.is_contiguous() and v.is_contiguous()
         if out is None:
             out = torch.empty(q.shape, dtype=torch.bfloat16, device=q.device)
-        gp = C.c_void_p(gate.data_ptr()) if gate is not None else None
-        rc = lib.kvm_decode_step(C.c_void_p(q.data_ptr()), C.c_void_p(k.data_ptr()), C.c_void_p(v.data_ptr()),
-                                 self._h, gp, C.c_void_p(out.data_ptr()), _stream_ptr(stream))
+        # (plain integers: ctypes converts them by the argument types, and a step is short enough for the
+        # objects around a pointer to show)
+        rc = lib.kvm_decode_step(q.data_ptr(), k.data_ptr(), v.data_ptr(), self._h,
+                                 gate.data_ptr() if gate is not None else None, out.data_ptr(), _stream_ptr(stream))
         if rc != KVM_OK:
             raise KVMError(rc, "kvm_decode_step")
         return out
