@@ -179,6 +179,11 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant__
       tc::tma_load_3d(dst + kb * Cfg::BOX_BYTES, map, full, kb * 64, row, u);
     return true;
   };
+  // (launched behind the kernel before it on the stream: what that one wrote - staged tokens, readout rows - is read, and
+  // anything is written, from here on.  The kernel behind this one may then take the SMs that this grid's last CTAs
+  // leave idle: see the routing filter.)
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   if (tid == 0) {
     // the first loads start before the tensor memory is allocated and the roles split: they need
     // nothing but their own barriers (no stage is waited for yet)
@@ -578,10 +583,19 @@ int launch_attn_tc(State* st, const AttnArgs& a, cudaStream_t s) {
   dim3 grid(n_whole + (tiles - n_whole) * nsp_rest);
   const CUtensorMap* tm = reinterpret_cast<const CUtensorMap*>(st->tmaps);
   const int ks = (st->nfolds & 1) ? 6 : 1, vs = (st->nfolds & 1) ? 7 : 2;   // readout copy of the current version
+  // where every kernel has the GPU to itself this one's CTAs start as the kernel before leaves the SMs
+  cudaLaunchConfig_t lc = {};
+  lc.gridDim = grid; lc.blockDim = dim3(384); lc.stream = s;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[0].val.programmaticStreamSerializationAllowed = 1;
+  lc.attrs = at; lc.numAttrs = st->serial && st->prof_hook == nullptr ? 1 : 0;
   if (st->d == 128) {
-    attn_tc_kernel<128><<<grid, 384, AttnTcCfg<128>::SMEM_BYTES, s>>>(tm[0], tm[ks], tm[vs], tm[3], tm[4], p);
+    lc.dynamicSmemBytes = AttnTcCfg<128>::SMEM_BYTES;
+    cudaLaunchKernelEx(&lc, attn_tc_kernel<128>, tm[0], tm[ks], tm[vs], tm[3], tm[4], p);
   } else {
-    attn_tc_kernel<64><<<grid, 384, AttnTcCfg<64>::SMEM_BYTES, s>>>(tm[0], tm[ks], tm[vs], tm[3], tm[4], p);
+    lc.dynamicSmemBytes = AttnTcCfg<64>::SMEM_BYTES;
+    cudaLaunchKernelEx(&lc, attn_tc_kernel<64>, tm[0], tm[ks], tm[vs], tm[3], tm[4], p);
   }
   return 1;
 }

@@ -43,6 +43,7 @@ struct RouteTcParams {
   float thr_coeff;         // candidate window = thr_coeff * ||kbar_j|| + 1e-5
   int64_t m;
   int C, Cmax, nsplit, S;
+  int ahead;               // the readout keys are complete when this grid may start (see the launch): wait at the end only
 };
 
 template <int D>
@@ -127,7 +128,7 @@ route_filter_tc_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_co
           tc::tma_load_3d(sA + mt * Cfg::TILE_BYTES + kb * Cfg::BOX_BYTES, gram ? &mapH : &mapA, &bars[RB_AFULL], kb * 64, mt * 128, a_unit);
       // the readout keys are written by the apply kernel of the fold before this one: wait for it here
       // (the set-up above and the load of the block's own keys run beside its tail)
-      asm volatile("griddepcontrol.wait;" ::: "memory");
+      if (!p.ahead) asm volatile("griddepcontrol.wait;" ::: "memory");
       for (int j = 0; j < nsteps; ++j) {
         const int s = j % Cfg::NS;
         const int jt = j;
@@ -347,6 +348,8 @@ route_filter_tc_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_co
       }
     }
   }
+  // (this grid does not end before the kernel that it ran beside)
+  if (p.ahead) asm volatile("griddepcontrol.wait;" ::: "memory");
   tc::tc_fence_before();
   __syncthreads();
   if (warp == 1) {
@@ -361,6 +364,10 @@ int launch_route_filter_tc(State* st, int64_t m, int nsplit, int slot, bool earl
   p.C = st->C; p.Cmax = st->Cmax; p.nsplit = nsplit; p.S = st->S;
   p.kbarNorm = st->kbarNorm + (int64_t)slot * st->U * st->Cmax; p.thr_coeff = route_thr_coeff(st);
   p.a_unit0 = slot * st->U; p.gramT = st->gramT; p.gram_mode = 0; p.U = st->U;
+  // A state with one readout copy runs this kernel behind the block's attention, which lets it start once it has itself
+  // waited for the fold that wrote the readout keys: nothing here depends on the attention, so it fills the SMs that the
+  // attention's last wave leaves idle.
+  p.ahead = early_start && st->serial && st->prof_hook == nullptr && !(st->flags & KVM_FLAG_SIMT_ATTENTION) ? 1 : 0;
   const CUtensorMap* tm = reinterpret_cast<const CUtensorMap*>(st->tmaps);
   dim3 grid(nsplit, st->U);
   const int ks = (st->nfolds & 1) ? 6 : 1;   // the fold reads the readout copy of the current version
@@ -384,7 +391,7 @@ int launch_gram_tc(State* st, int slot0, int nblk, cudaStream_t s) {
   p.candV = st->candV; p.candI = st->candI; p.chunkMax = st->chunkMax; p.chunkMeta = st->chunkMeta; p.chunkVal = st->chunkVal; p.status = st->status; p.m = 0;
   p.C = st->C; p.Cmax = st->Cmax; p.nsplit = 1; p.S = st->S;
   p.kbarNorm = st->kbarNorm; p.thr_coeff = 0.f;
-  p.a_unit0 = slot0 * st->U; p.gramT = st->gramT; p.gram_mode = 1; p.U = st->U;
+  p.a_unit0 = slot0 * st->U; p.gramT = st->gramT; p.gram_mode = 1; p.U = st->U; p.ahead = 0;
   const CUtensorMap* tm = reinterpret_cast<const CUtensorMap*>(st->tmaps);
   dim3 grid(1, st->U, nblk);
   if (st->d == 128) route_filter_tc_kernel<128><<<grid, 352, RouteTcCfg<128>::SMEM_BYTES, s>>>(tm[5], tm[1], tm[8], p);
