@@ -862,7 +862,7 @@ __global__ void __launch_bounds__(kDecideThreads, PER_SM) fold_decide_kernel(con
   received(2);
   __syncthreads();
   if (many) asm volatile("barrier.cluster.arrive.release;" ::: "memory");
-  if (s_dead) {   // (a wait ran out: nothing is applied)
+  if (s_dead) {   // (a wait ran out: nothing is published)
     if (tid == 0) atomicExch(p.counters - 1, (int)KVM_ERR_TIMEOUT);
     if (many) asm volatile("barrier.cluster.wait.acquire;" ::: "memory");
     return;
