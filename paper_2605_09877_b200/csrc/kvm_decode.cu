@@ -47,9 +47,11 @@ __device__ __forceinline__ void unpack8(const uint4& w, float (&f)[8]) {
   f[0] = a.x; f[1] = a.y; f[2] = b.x; f[3] = b.y; f[4] = c.x; f[5] = c.y; f[6] = e.x; f[7] = e.y;
 }
 
+// A row that is read once.  Not the non-coherent path (.nc): a step is resident while the kernel before it still writes
+// window slots or readout rows, and only ordinary loads are ordered by griddepcontrol.wait.
 __device__ __forceinline__ uint4 ldg_stream(const void* p) {
   uint4 r;
-  asm volatile("ld.global.nc.L1::no_allocate.v4.u32 {%0,%1,%2,%3}, [%4];"
+  asm volatile("ld.global.L1::no_allocate.v4.u32 {%0,%1,%2,%3}, [%4];"
                : "=r"(r.x), "=r"(r.y), "=r"(r.z), "=r"(r.w) : "l"(p));
   return r;
 }

@@ -440,9 +440,10 @@ __device__ __forceinline__ double warp_reduce4(double v0, double v1, double v2, 
   return z;
 }
 
-// kb . LN_s(row) with the row's statistics given; channels are strided over the lanes of a warp.
+// kb . LN_s(row) with the row's statistics given; channels are strided over the lanes of a warp.  (The row is no
+// __restrict__ pointer: a decision CTA is resident while the apply kernel before it still writes rows.)
 template <int CH>
-__device__ __forceinline__ double warp_sim(const double (&kb)[CH], const double* __restrict__ row, double mu, double rs,
+__device__ __forceinline__ double warp_sim(const double (&kb)[CH], const double* row, double mu, double rs,
                                            const double (&g)[CH], const double (&b)[CH], int lane) {
   double acc = 0.0;
 #pragma unroll

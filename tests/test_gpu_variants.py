@@ -264,3 +264,29 @@ def test_decode_row_splits_from_one_to_eight(B, Hq, Hkv, d, pos, steps):
     wl = synth.Workload("dec", B, Hq, Hkv, d, pos + steps, 64, "sqrt", sqrt_coeff=20, r=32, seed=330 + pos)
     params = synth.make_layer_params(wl, trivial=False)
     print(_sampled(wl, [(0, 0), (B - 1, Hkv - 1)], params=params, decode_from=pos))
+
+
+@pytest.mark.parametrize("B,Hq,Hkv,d,serial", [(1, 2, 1, 64, False), (1, 4, 4, 128, False), (2, 8, 2, 128, True)])
+def test_decode_steps_launched_back_to_back_equal_steps_one_at_a_time(B, Hq, Hkv, d, serial):
+    """A step is on the GPU while the one before it stores its token, and while a fold rewrites readout rows: every slot
+    of the window ring is reused several times, and the outputs are those of steps that are waited for one by one."""
+    from paper_2605_09877_b200 import kvm
+    wl = synth.Workload("pdl", B, Hq, Hkv, d, 40 + 16 * 13, 16, "sqrt", sqrt_coeff=5, r=16, seed=360 + Hq)
+    params = synth.make_layer_params(wl, trivial=False)
+    t = {n: x.cuda() for n, x in synth.make_inputs(wl).items() if n in "qkv"}
+    outs = []
+    for wait in (False, True):
+        st, g = pu.gpu_layer(wl, params, flags=kvm.FLAG_SERIAL_FOLDS if serial else 0)
+        st.prefill(t["q"][:, :, :40], t["k"][:, :, :40], t["v"][:, :, :40], wl.C, g, wl.r)
+        steps = [[t[n][:, :, i].contiguous() for n in "qkv"] for i in range(40, wl.T)]
+        y = [torch.empty_like(s[0]) for s in steps]
+        torch.cuda.synchronize()
+        for s, o in zip(steps, y):
+            st.decode_step(*s, out=o)
+            if wait:
+                torch.cuda.synchronize()
+        torch.cuda.synchronize()
+        assert st.check() == 0
+        outs.append(torch.stack(y))
+        st.free()
+    assert torch.equal(outs[0], outs[1])
