@@ -285,6 +285,12 @@ kvm_status_t kvm_profile_read(kvm_state_t* state, double* ms, int64_t* groups);
  * `out` has room for four values.  32-bit device counters. */
 kvm_status_t kvm_debug_counters(kvm_state_t* state, int64_t* out, void* cuda_stream);
 
+/* How a decode step over n_rows rows (state and window) is cut, for tests: out[0] query heads per CTA, out[1] CTAs per
+ * cluster (row splits merged through shared memory), out[2] clusters per group of heads (merged through global memory).
+ * Host arithmetic only. */
+kvm_status_t kvm_debug_decode_plan(int32_t batch, int32_t n_q_heads, int32_t n_kv_heads, int32_t head_dim, int64_t n_rows,
+                                   int32_t* out);
+
 /* Number of kernels the library has launched for this state so far (host counter). */
 int64_t kvm_launch_count(const kvm_state_t* state);
 

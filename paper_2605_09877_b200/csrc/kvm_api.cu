@@ -378,6 +378,7 @@ KVM_API kvm_status_t kvm_state_create(const kvm_config_t* cfg, kvm_state_t** out
   // (tiles x splits: up to kAttnSplitTiles x kAttnMaxSplits, or 2 kAttnSplitTiles tiles of two splits)
   A(s.attnPart, (size_t)kAttnSplitTiles * kAttnMaxSplits * (d + 2) * 128); A(s.attnCnt, (size_t)2 * kAttnSplitTiles);
   if (rc == KVM_OK && cudaMemset(s.attnCnt, 0, 2 * kAttnSplitTiles * sizeof(int32_t)) != cudaSuccess) rc = KVM_ERR_CUDA;
+  A(s.decPart, (size_t)kDecodePartCtas * (d + 2)); A(s.decTicket, (size_t)kDecodePartCtas);
   A(s.status, (size_t)16);   // [0] status word, [1..3] fold debug counters
   if (s.Tassign > 0) { A(s.slotTok, U * (size_t)s.Tassign); A(s.appTok, U * (size_t)s.Tassign); }
 #undef A
@@ -485,6 +486,15 @@ KVM_API kvm_status_t kvm_state_check(kvm_state_t* ks, void* cuda_stream) {
   if (w == 0) return KVM_OK;
   if (cudaMemsetAsync(ks->s.status, 0, sizeof(w), stream) != cudaSuccess) return KVM_ERR_CUDA;   // reported once
   return w == KVM_ERR_TIMEOUT ? KVM_ERR_TIMEOUT : KVM_ERR_CUDA;
+}
+
+KVM_API kvm_status_t kvm_debug_decode_plan(int32_t batch, int32_t n_q_heads, int32_t n_kv_heads, int32_t head_dim,
+                                           int64_t n_rows, int32_t* out) {
+  if (batch < 1 || n_q_heads < 1 || n_kv_heads < 1 || n_q_heads % n_kv_heads || n_rows < 1 || !out) return KVM_ERR_INVALID_ARG;
+  if (head_dim != 64 && head_dim != 128) return KVM_ERR_UNSUPPORTED;
+  const DecodePlan p = plan_decode(batch * n_q_heads, n_q_heads / n_kv_heads, head_dim, n_rows);
+  out[0] = p.heads; out[1] = p.splits; out[2] = p.clusters;
+  return KVM_OK;
 }
 
 KVM_API kvm_status_t kvm_debug_expire_wait(kvm_state_t* ks, int32_t spins, void* cuda_stream) {

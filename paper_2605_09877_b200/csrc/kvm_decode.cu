@@ -2,13 +2,16 @@
 // m readout rows of the state plus the window tokens [b, t].  ONE kernel per step: every CTA rotates
 // the query heads it serves (and, where its rows end with the new token, that token's key), streams
 // its share of the rows with 16-byte loads into an online softmax, and the row splits of a head - a
-// thread-block cluster - merge their partial results through distributed shared memory.
+// thread-block cluster - merge their partial results through distributed shared memory; few heads over many rows take several
+// clusters per head (plan_decode), of which the last to arrive merges.
 // What bounds it: with many heads HBM (K_hat, V_hat and the window are read once); with few the
 // latency of launch, first loads and merge, and on the host the launch itself, which is why the rotation of the
 // token and the merge are not kernels of their own: 32 heads over 256 + window rows took 1.9 + 7.4 + 3.1 us
 // in three kernels and 18.5 us per step on the host's side; now 9.5 us per step.  64 x 32 heads over 4096 + window
 // rows: 763 -> 716 us per step (6.57 TB/s), the set-up of a step under the tail of the one before.
 #include <cooperative_groups.h>
+
+#include <utility>
 
 #include "kvm_internal.h"
 #include "ln_rows.cuh"
@@ -36,6 +39,9 @@ struct DecodeParams {
   int ringLen, slot_b;   // ring slot of the window's first token
   int slot_t;            // ring slot of the new token
   int Hq, Hkv, G, nsplit, r;
+  int nclus;             // clusters of nsplit CTAs per group of heads
+  float* part;           // (nclus > 1) merged results of the clusters, [CTA group][rank][cluster][share + 2]
+  int32_t* ticket;       // (nclus > 1) [CTA group][rank], zero between launches
   float qk_ln_eps;
 };
 
@@ -198,11 +204,12 @@ __device__ __forceinline__ void lane_sums(float (&v)[N], int gl) {
   }
 }
 
-// grid (nsplit, B*Hq / GQ), the nsplit CTAs of a row a cluster; block 256 = 8 warps.  LPR = D/8 lanes cover one
+// grid (nsplit * nclus, B*Hq / GQ), nsplit CTAs of a row a cluster; block 256 = 8 warps.  LPR = D/8 lanes cover one
 // row with 16-byte loads, a warp covers RPW = 32/LPR rows per load instruction and UNR such instructions per
 // step.  A CTA serves GQ query heads that share one kv head (grouped queries): every key / value row is loaded
-// once and meets all GQ queries, so the bytes streamed per step do not grow with the group size.
-template <int D, int GQ, bool LN>
+// once and meets all GQ queries, so the bytes streamed per step do not grow with the group size.  MULTI: nclus > 1 (a build of
+// its own: the steps of one cluster, 5 us each for few rows, took 1 to 3 % longer with the merge of several in the kernel).
+template <int D, int GQ, bool LN, bool MULTI>
 __global__ void __launch_bounds__(256) decode_step_kernel(DecodeParams p) {
   constexpr int LPR = D / 8;
   constexpr int RPW = 32 / LPR;
@@ -212,6 +219,7 @@ __global__ void __launch_bounds__(256) decode_step_kernel(DecodeParams p) {
   __shared__ __align__(16) float s_acc[8][GQ][D];
   __shared__ float s_part[GQ][D + 2];   // this split's merged result: channels, maximum, sum
   __shared__ __align__(16) __half s_q[GQ][D], s_new[2][D];
+  __shared__ int s_last;
 
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   const int split = blockIdx.x;
@@ -221,8 +229,8 @@ __global__ void __launch_bounds__(256) decode_step_kernel(DecodeParams p) {
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int grp = lane / LPR, gl = lane % LPR;   // row group inside the warp, lane inside the row
 
-  const int m = p.m, n = p.n;
-  int per = (n + p.nsplit - 1) / p.nsplit;
+  const int m = p.m, n = p.n, ns_all = MULTI ? p.nsplit * p.nclus : p.nsplit;
+  int per = (n + ns_all - 1) / ns_all;
   per = (per + 8 * STEP - 1) / (8 * STEP) * (8 * STEP);
   const int r0 = split * per;
   const int r1 = min(n, r0 + per);
@@ -372,19 +380,21 @@ __global__ void __launch_bounds__(256) decode_step_kernel(DecodeParams p) {
       l += s_l[w][g] * f;
       a += s_acc[w][g][x] * f;
     }
-    if (p.nsplit == 1) {
+    if (!MULTI && ns_all == 1) {
       p.out[(int64_t)(bh0 + g) * D + x] = __float2bfloat16_rn(a / l);
     } else {
       s_part[g][x] = a;
       if (x == 0) { s_part[g][D] = mx; s_part[g][D + 1] = l; }
     }
   }
-  if (p.nsplit == 1) return;
+  if (!MULTI && ns_all == 1) return;
   // the splits of these heads: every CTA of the cluster merges its share of the channels
   cooperative_groups::cluster_group cl = cooperative_groups::this_cluster();
   cl.sync();
-  const int share = (GQ * D + p.nsplit - 1) / p.nsplit;
-  for (int e = split * share + tid; e < min(GQ * D, (split + 1) * share); e += 256) {
+  const int rank = MULTI ? (int)cl.block_rank() : split, share = (GQ * D + p.nsplit - 1) / p.nsplit, e0 = rank * share;
+  // several clusters: nsplit == 8, a share lies in one head
+  float* part = p.part + ((int64_t)blockIdx.y * p.nsplit + rank) * p.nclus * (share + 2);
+  for (int e = e0 + tid; e < min(GQ * D, e0 + share); e += 256) {
     const int g = e / D, x = e % D;
     const float* mine = &s_part[g][0];
     float mx = -INFINITY;
@@ -397,15 +407,80 @@ __global__ void __launch_bounds__(256) decode_step_kernel(DecodeParams p) {
       l += pz[D + 1] * f;
       a += pz[x] * f;
     }
-    p.out[(int64_t)(bh0 + g) * D + x] = __float2bfloat16_rn(a / l);
+    if (!MULTI) {
+      p.out[(int64_t)(bh0 + g) * D + x] = __float2bfloat16_rn(a / l);
+    } else {
+      float* mine_out = part + split / p.nsplit * (share + 2);
+      mine_out[e - e0] = a;
+      if (e == e0) { mine_out[share] = mx; mine_out[share + 1] = l; }
+    }
   }
-  cl.sync();   // (no CTA leaves while another still reads its shared memory)
+  // (no CTA leaves while another still reads its shared memory)
+  if constexpr (!MULTI) {
+    cl.sync();
+  } else {
+    auto gone = cl.barrier_arrive();
+    // the clusters of these heads: of the CTAs with the same share the one that arrives last merges it (nobody waits)
+    __threadfence();
+    __syncthreads();
+    int32_t* ticket = p.ticket + (int64_t)blockIdx.y * p.nsplit + rank;
+    if (tid == 0) s_last = atomicAdd(ticket, 1) == p.nclus - 1 ? 1 : 0;
+    __syncthreads();
+    if (s_last) {
+      __threadfence();
+      if (tid == 0) *ticket = 0;
+      const float* all = part;
+      // (s_acc is idle by now) weight of every cluster; then the partial sums of the thread groups
+      float *s_w = &s_acc[0][0][0], *s_sum = s_w + 128;
+      static_assert(8 * 64 >= 128 + 256, "scratch of the merge");
+      if (warp == 0) {   // (at most 64 clusters: plan_decode)
+        float ms[2], ls[2];
+#pragma unroll
+        for (int k = 0; k < 2; ++k) {
+          const int z = lane + 32 * k;
+          ms[k] = z < p.nclus ? __ldcg(all + z * (share + 2) + share) : -INFINITY;
+          ls[k] = z < p.nclus ? __ldcg(all + z * (share + 2) + share + 1) : 0.f;
+        }
+        float mx = fmaxf(ms[0], ms[1]), l = 0.f;
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+#pragma unroll
+        for (int k = 0; k < 2; ++k) {
+          const float f = (ms[k] == -INFINITY) ? 0.f : exp2f(ms[k] - mx);
+          s_w[lane + 32 * k] = f;
+          l += ls[k] * f;
+        }
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) l += __shfl_xor_sync(0xffffffffu, l, o);
+        if (lane == 0) s_w[64] = l;
+      }
+      __syncthreads();
+      // a group of `share` threads takes every (256 / share)-th cluster, four loads in flight
+      const int ng = 256 / share, grp_z = tid / share, ch = tid % share;
+      float a = 0.f;
+      for (int z0 = grp_z; z0 < p.nclus; z0 += 4 * ng) {
+        float v[4];
+#pragma unroll
+        for (int k = 0; k < 4; ++k) v[k] = z0 + k * ng < p.nclus ? __ldcg(all + (z0 + k * ng) * (share + 2) + ch) : 0.f;
+#pragma unroll
+        for (int k = 0; k < 4; ++k) a += v[k] * (z0 + k * ng < p.nclus ? s_w[z0 + k * ng] : 0.f);
+      }
+      s_sum[tid] = a;
+      __syncthreads();
+      if (tid < share) {
+        a = 0.f;
+        for (int k = 0; k < ng; ++k) a += s_sum[k * share + tid];
+        p.out[(int64_t)bh0 * D + e0 + tid] = __float2bfloat16_rn(a / s_w[64]);
+      }
+    }
+    cl.barrier_wait(std::move(gone));
+  }
 }
 
-template <int D, int GQ, bool LN>
+template <int D, int GQ, bool LN, bool MULTI>
 static bool launch_decode_step(const DecodeParams& p, int ncta, bool early, cudaStream_t s) {
   cudaLaunchConfig_t lc = {};
-  lc.gridDim = dim3(p.nsplit, ncta); lc.blockDim = dim3(256); lc.stream = s;
+  lc.gridDim = dim3(p.nsplit * p.nclus, ncta); lc.blockDim = dim3(256); lc.stream = s;
   cudaLaunchAttribute at[2];
   // the set-up of this step (launch, the rotation's angles) runs under the tail of the kernel before it on the stream
   at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
@@ -413,18 +488,59 @@ static bool launch_decode_step(const DecodeParams& p, int ncta, bool early, cuda
   at[1].id = cudaLaunchAttributeClusterDimension;
   at[1].val.clusterDim.x = p.nsplit; at[1].val.clusterDim.y = 1; at[1].val.clusterDim.z = 1;
   lc.attrs = at; lc.numAttrs = p.nsplit > 1 ? 2 : 1;
-  return cudaLaunchKernelEx(&lc, decode_step_kernel<D, GQ, LN>, p) == cudaSuccess;
+  return cudaLaunchKernelEx(&lc, decode_step_kernel<D, GQ, LN, MULTI>, p) == cudaSuccess;
 }
 
-// query heads of one kv group share a CTA: the largest of 8, 4, 2, 1 that divides the group size
-static int decode_heads_per_cta(const State* st) { return (st->G % 8 == 0) ? 8 : (st->G % 4 == 0) ? 4 : (st->G % 2 == 0) ? 2 : 1; }
+// How a step over n rows is cut.  Query heads per CTA (they share a kv head): the largest of 8, 4, 2, 1 that divides the group
+// size, but four of eight while all splits of four fit at once, two CTAs per SM: the rows are fetched twice, mostly from L2, by
+// twice the warps (us per step of 8 and 4: 64 heads on 8, 900 rows 10.0, 8.7; 16600 rows 69, 41 in two clusters; 96 on 12, 2400
+// rows 15.6, 14.2; 50000 rows 197, 179; 128 on 16 - 16 clusters of eight CTAs do not fit at one per SM - 900 rows 19, 10).
+DecodePlan plan_decode(int nQ, int G, int d, int64_t n) {
+  int heads = (G % 8 == 0) ? 8 : (G % 4 == 0) ? 4 : (G % 2 == 0) ? 2 : 1;
+  if (heads == 8 && nQ / 4 <= 33) heads = 4;
+  DecodePlan pl;
+  pl.heads = heads;
+  pl.splits = pl.clusters = 1;
+  // Row splits, up to the portable cluster size (clusters of 16 took 13.5 us per step where 8 take 8.5): waves of clusters
+  // times the length of a CTA, its set-up and merge counted as 300 rows.  kFit: clusters of 1 to 8 CTAs that the GPU holds at
+  // once at 1, 2, 3 CTAs per SM (cudaOccupancyMaxActiveClusters; a cluster lies in one group of SMs, and one too many is another
+  // wave: 136 heads on 17, 900 rows, clusters of 8: 18.6 us, of 6: 12).  By registers 3, 2, 2, 1 CTAs of 1, 2, 4, 8 heads fit an SM.
+  // This picks the fastest of 1, 2, 3, 4, 6, 8 splits, or one within 2 % of it, in all of 15 measured shapes (64 to 768 heads,
+  // 900 to 2400 rows; e.g. us per step of 256 heads over 2430 rows: 59, 68, 55, 61, 64, 70; of 512 heads: 123, 109, 106, 108,
+  // 123, 131).  (The fewest of equal counts.)
+  static const int kFit[3][kDecodeCluster] = {{148, 74, 45, 33, 26, 22, 15, 15}, {296, 148, 93, 71, 56, 45, 37, 33}, {444, 222, 142, 104, 82, 71, 56, 48}};
+  const int* fit = kFit[heads == 1 ? 2 : heads == 8 ? 0 : 1];
+  const int64_t ncta = nQ / heads, rows1 = 8 * 4 * (256 / d);
+  auto rows_of = [&](int64_t ns) { return ((n + ns - 1) / ns + rows1 - 1) / rows1 * rows1; };
+  int64_t t = INT64_MAX;
+  for (int ns = 1; ns <= kDecodeCluster; ++ns) {
+    const int64_t tn = (ncta + fit[ns - 1] - 1) / fit[ns - 1] * (rows_of(ns) + 300);
+    if (tn < t) { t = tn; pl.splits = ns; }
+  }
+  // Few heads over many rows: several clusters of eight per group of heads, while all of them fit at once (another wave costs
+  // what the shorter CTAs save), merged through global memory by the CTAs that arrive last.  That takes 1.5 us and 5 to 9 ns per CTA longer, where a CTA takes 80 (1, 2 heads)
+  // or 45 rows of 128 channels per us.  Measured, us per step, one cluster and as chosen: 1 head of 128 channels over 2300
+  // rows 7.5, 6.7; 6400 rows 13.3, 7.9; 131072 rows 281, 19; 8 heads on one, 50000 rows 171, 21; 8 on 8,
+  // 16600 rows 41, 19; 32 on 8, 50000 rows 158, 61; 16 on 16, 50000 rows 127, 67.  Left in one cluster: 32 on 8, 1300 rows 8.8
+  // (10.2 with three); 2 x 8 heads of 64 channels, 4400 rows 9.4 (10.2).  A twentieth has to be gained: 32 on 8 over 1870
+  // rows 10.6, 11.9 with four.
+  t -= t / 20;
+  for (int64_t nc = 2; ncta * nc <= fit[kDecodeCluster - 1]; ++nc) {
+    const int64_t merge = ((heads <= 2 ? 120 : 70) + 2 * kDecodeCluster * ncta * nc / 5) * 128 / d;
+    const int64_t tn = rows_of(kDecodeCluster * nc) + 300 + merge;
+    if (tn < t) { t = tn; pl.splits = kDecodeCluster; pl.clusters = (int)nc; }
+  }
+  return pl;
+}
 
-#define KVM_DEC_EACH(F)                                                                                                 \
-  F(128, 8, true) F(128, 4, true) F(128, 2, true) F(128, 1, true) F(64, 8, true) F(64, 4, true) F(64, 2, true) F(64, 1, true) \
-  F(128, 8, false) F(128, 4, false) F(128, 2, false) F(128, 1, false) F(64, 8, false) F(64, 4, false) F(64, 2, false) F(64, 1, false)
+#define KVM_DEC_EACH(F, L) \
+  F(128, 8, L, false) F(128, 4, L, false) F(128, 2, L, false) F(128, 1, L, false) F(64, 8, L, false) F(64, 4, L, false) F(64, 2, L, false) F(64, 1, L, false) \
+  F(128, 4, L, true) F(128, 2, L, true) F(128, 1, L, true) F(64, 4, L, true) F(64, 2, L, true) F(64, 1, L, true)
 
 int launch_decode(State* st, const DecodeArgs& a, cudaStream_t s) {
-  const int nQ = st->B * st->Hq, GQ = decode_heads_per_cta(st);
+  const int nQ = st->B * st->Hq;
+  const DecodePlan pl = plan_decode(nQ, st->G, st->d, a.m + (a.t - a.b + 1));
+  const int GQ = pl.heads;
   DecodeParams p;
   p.q = a.q; p.k = a.k; p.v = a.v; p.gate = a.gate; p.inv_freq = st->inv_freq;
   p.lnq_w = st->lnq_w; p.lnq_b = st->lnq_b; p.lnk_w = st->lnk_w; p.lnk_b = st->lnk_b; p.qk_ln_eps = st->qk_ln_eps;
@@ -435,24 +551,12 @@ int launch_decode(State* st, const DecodeArgs& a, cudaStream_t s) {
   p.m = (int)a.m; p.n = (int)(a.m + (a.t - a.b + 1));
   p.ringLen = (int)st->ringLen; p.slot_b = (int)(a.b % st->ringLen); p.slot_t = (int)(a.t % st->ringLen);
   p.Hq = st->Hq; p.Hkv = st->Hkv; p.G = st->G; p.r = st->r;
-  // Row splits, up to the portable cluster size (clusters of 16 took 13.5 us per step where 8 take 8.5): waves of CTAs
-  // times the length of a CTA, its set-up and merge counted as 300 rows.  `slots` = CTAs that fit the GPU at once (3, 2,
-  // 2, 1 per SM by registers for 1, 2, 4, 8 heads).  This picks the fastest of 1, 2, 3, 4, 6, 8 splits, or one within 2 %
-  // of it, in all of 15 measured shapes (64 to 768 heads, 900 to 2400 rows; e.g. us per step of 256 heads over 2430
-  // rows: 59, 68, 55, 61, 64, 70; of 512 heads: 123, 109, 106, 108, 123, 131).
-  const int nCta = nQ / GQ, rows1 = 8 * 4 * (256 / st->d), slots = 148 * (GQ == 1 ? 3 : GQ == 8 ? 1 : 2);
-  int nsplit = 1;
-  int64_t least = INT64_MAX;
-  for (int ns = 1; ns <= 8; ++ns) {
-    const int64_t rows = ((p.n + ns - 1) / ns + rows1 - 1) / rows1 * rows1;
-    const int64_t t = ((int64_t)nCta * ns + slots - 1) / slots * (rows + 300);
-    if (t < least) { least = t; nsplit = ns; }
-  }
-  p.nsplit = nsplit;
+  p.nsplit = pl.splits; p.nclus = pl.clusters; p.part = st->decPart; p.ticket = st->decTicket;
   const bool early = st->prof_hook == nullptr;
-#define KVM_DEC_GO(DD, GG, LL) \
-  if (st->d == DD && GQ == GG && st->fusedLn == LL) launch_decode_step<DD, GG, LL>(p, nCta, early, s);
-  KVM_DEC_EACH(KVM_DEC_GO)
+#define KVM_DEC_GO(DD, GG, LL, MM) \
+  if (st->d == DD && GQ == GG && st->fusedLn == LL && (pl.clusters > 1) == MM) launch_decode_step<DD, GG, LL, MM>(p, nQ / GQ, early, s);
+  KVM_DEC_EACH(KVM_DEC_GO, true)
+  KVM_DEC_EACH(KVM_DEC_GO, false)
 #undef KVM_DEC_GO
   return 1;
 }

@@ -15,6 +15,8 @@ constexpr int kChunkCap = 16;       // 32-row chunks of approximate similarities
 constexpr int kMaxSplits = 32;      // routing filter split count upper bound
 constexpr int kAttnSplitTiles = 37; // launches with at most this many (batch, head, query tile) CTAs - a quarter of the GPU - are split along the keys
 constexpr int kAttnMaxSplits = 8;
+constexpr int kDecodeCluster = 8;   // most CTAs of a decode step that share a cluster (the portable size)
+constexpr int kDecodePartCtas = 48 * kDecodeCluster;   // most CTAs of a decode step that merge through global memory (plan_decode)
 constexpr int kRowAlign = 128;      // state capacity is rounded up to the attention key tile
 constexpr int kGramOnTheFly = 32;   // in a state with enough units to fill the GPU (gram_from), folds that append at most this
                                     // many rows compute the products of the other tokens with the new rows inside the decision
@@ -112,6 +114,9 @@ struct State {
   // ---- split-KV attention scratch (device) ----
   float* attnPart;               // [kAttnSplitTiles][kAttnMaxSplits][d + 2][128]
   int32_t* attnCnt;              // [2 kAttnSplitTiles] tickets
+  // ---- decode scratch (device): clusters of the same heads merge through it ----
+  float* decPart;                // [kDecodePartCtas][d + 2]
+  int32_t* decTicket;            // [kDecodePartCtas], zero between launches
   // ---- optional per-kernel timing hook (set by kvm_profile_enable): phase ids
   //      0 ingest, 1 attention, 2 memory keys, 3 routing filter, 4 decide, 5 apply, 6 decode ----
   void (*prof_hook)(void* ctx, int phase, int begin, cudaStream_t s);
@@ -200,6 +205,8 @@ struct DecodeArgs {
   int64_t m;
 };
 int launch_decode(State* st, const DecodeArgs& a, cudaStream_t s);
+struct DecodePlan { int heads, splits, clusters; };   // query heads per CTA, CTAs per cluster, clusters per group of heads
+DecodePlan plan_decode(int n_q, int group, int d, int64_t n_rows);
 
 // Self test of the bounded waits: one thread waits `spins` iterations on a barrier nobody arrives at and
 // records KVM_ERR_TIMEOUT in the status word.

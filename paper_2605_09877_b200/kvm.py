@@ -26,7 +26,8 @@ EXPORTS = ["kvm_plan_capacity", "kvm_state_create", "kvm_prefill", "kvm_decode_s
            "kvm_decode_step_host", "kvm_state_free", "kvm_state_info", "kvm_state_check", "kvm_state_export",
            "kvm_debug_assignments", "kvm_launch_count", "kvm_status_string", "kvm_state_reset",
            "kvm_profile_enable", "kvm_profile_read", "kvm_debug_counters", "kvm_attend_rows_noalloc", "kvm_merge_gate", "kvm_head_layernorm",
-           "kvm_state_snapshot_info", "kvm_state_export_window", "kvm_state_import", "kvm_debug_expire_wait"]
+           "kvm_state_snapshot_info", "kvm_state_export_window", "kvm_state_import", "kvm_debug_expire_wait",
+           "kvm_debug_decode_plan"]
 
 
 class KVMError(RuntimeError):
@@ -106,6 +107,8 @@ def _load():
     L.kvm_attend_rows_noalloc.argtypes = [vp, vp, vp, C.c_int32, C.c_int64, C.c_int32, C.c_float, vp, vp]
     L.kvm_merge_gate.restype = C.c_int
     L.kvm_merge_gate.argtypes = [vp, vp, C.c_int32, C.c_int64, C.c_int32, C.c_int32, vp, vp, vp]
+    L.kvm_debug_decode_plan.restype = C.c_int
+    L.kvm_debug_decode_plan.argtypes = [C.c_int32, C.c_int32, C.c_int32, C.c_int32, C.c_int64, C.POINTER(C.c_int32)]
     L.kvm_debug_expire_wait.restype = C.c_int
     L.kvm_debug_expire_wait.argtypes = [vp, C.c_int32, vp]
     L.kvm_head_layernorm.restype = C.c_int
@@ -163,6 +166,15 @@ def head_layernorm(x: "torch.Tensor", weight=None, bias=None, eps: float = 1e-5,
     if rc != 0:
         raise KVMError(rc, "kvm_head_layernorm")
     return x
+
+
+def decode_plan(batch: int, n_q_heads: int, n_kv_heads: int, head_dim: int, n_rows: int):
+    """(query heads per CTA, CTAs per cluster, clusters per group of heads) of a decode step over n_rows rows."""
+    out = (C.c_int32 * 3)()
+    rc = lib.kvm_debug_decode_plan(batch, n_q_heads, n_kv_heads, head_dim, n_rows, out)
+    if rc != KVM_OK:
+        raise KVMError(rc, "kvm_debug_decode_plan")
+    return tuple(out)
 
 
 def kvm_plan_capacity(block: int, n_bswa_chunks: int, g: Growth, seq_len: int) -> int:

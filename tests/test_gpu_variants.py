@@ -256,12 +256,27 @@ def test_decisions_scan_every_row_for_tokens_with_too_many_candidates():
     st.free()
 
 
-@pytest.mark.parametrize("B,Hq,Hkv,d,pos,steps", [
-    (1, 1, 1, 64, 40, 30), (1, 2, 1, 128, 900, 20), (3, 32, 4, 64, 1300, 10), (7, 21, 21, 128, 300, 9), (9, 64, 64, 64, 700, 6),
-    (40, 32, 8, 128, 300, 4)])
-def test_decode_row_splits_from_one_to_eight(B, Hq, Hkv, d, pos, steps):
-    """Clusters of one, two, four and eight CTAs per head, one to eight query heads per CTA, splits without rows."""
+def _decode_rows(wl, t):
+    """State rows and window tokens that the decode step at position t attends over."""
+    from paper_2605_09877_b200 import kvm
+    g = kvm.growth(wl.growth, wl.fixed_slots, wl.sqrt_coeff, wl.pow_num, wl.pow_den, wl.sat_half)
+    return kvm.kvm_plan_capacity(wl.C, wl.w, g, t // wl.C * wl.C) + t + 1 - max(0, (t // wl.C + 1 - wl.w) * wl.C)
+
+
+@pytest.mark.parametrize("B,Hq,Hkv,d,pos,steps,plans", [
+    (1, 1, 1, 64, 40, 30, {(1, 1, 1)}), (1, 2, 1, 128, 900, 20, {(2, 6, 1)}), (3, 32, 4, 64, 1300, 10, {(4, 7, 1)}),
+    (7, 21, 21, 128, 300, 9, {(1, 2, 1)}), (9, 64, 64, 64, 700, 6, {(1, 1, 1)}), (40, 32, 8, 128, 300, 4, {(4, 1, 1)}),
+    (1, 1, 1, 128, 60, 20, {(1, 1, 1), (1, 2, 1)}), (1, 2, 2, 128, 110, 10, {(1, 2, 1)}), (1, 3, 3, 64, 400, 5, {(1, 4, 1)}),
+    (1, 1, 1, 64, 1000, 5, {(1, 6, 1)}), (1, 2, 2, 128, 260, 5, {(1, 5, 1)}),
+    (1, 2, 2, 128, 452, 5, {(1, 8, 1)}), (6, 32, 16, 128, 70, 8, {(2, 2, 1)}), (10, 32, 8, 64, 500, 5, {(4, 2, 1)}),
+    (5, 32, 4, 64, 20, 5, {(8, 1, 1)}), (5, 32, 4, 128, 130, 8, {(8, 3, 1)}), (12, 32, 4, 128, 300, 5, {(8, 2, 1)}),
+    (5, 32, 4, 128, 392, 5, {(8, 4, 1)}), (1, 2, 2, 128, 392, 5, {(1, 7, 1)})])
+def test_decode_row_splits_from_one_to_eight(B, Hq, Hkv, d, pos, steps, plans):
+    """One to eight CTAs in the cluster of a group of heads, one to eight query heads per CTA; every case asserts how its
+    steps are cut (query heads per CTA, CTAs per cluster, clusters)."""
+    from paper_2605_09877_b200 import kvm
     wl = synth.Workload("dec", B, Hq, Hkv, d, pos + steps, 64, "sqrt", sqrt_coeff=20, r=32, seed=330 + pos)
+    assert {kvm.decode_plan(B, Hq, Hkv, d, _decode_rows(wl, t)) for t in range(pos, pos + steps)} == plans
     params = synth.make_layer_params(wl, trivial=False)
     print(_sampled(wl, [(0, 0), (B - 1, Hkv - 1)], params=params, decode_from=pos))
 
@@ -290,3 +305,29 @@ def test_decode_steps_launched_back_to_back_equal_steps_one_at_a_time(B, Hq, Hkv
         outs.append(torch.stack(y))
         st.free()
     assert torch.equal(outs[0], outs[1])
+
+
+@pytest.mark.parametrize("B,Hq,Hkv,d,slots,clusters", [
+    (1, 1, 1, 128, 3000, 7), (1, 8, 1, 128, 2500, 6), (1, 4, 2, 128, 4000, 9), (1, 2, 2, 64, 9000, 10), (1, 32, 8, 128, 4200, 3),
+    (2, 8, 8, 64, 9000, 3), (1, 16, 1, 64, 6000, 7), (1, 64, 8, 128, 4200, 2)])
+def test_decode_clusters_of_the_same_heads_merge_through_global_memory(B, Hq, Hkv, d, slots, clusters):
+    """Few heads over many rows: one to four query heads per CTA, an odd number of clusters, the last ones with few rows or
+    none; steps across a block boundary, with a fold between them, against the oracle and from run to run."""
+    from paper_2605_09877_b200 import kvm
+    C = 256
+    start = (slots // C + 4) * C - 5
+    wl = synth.Workload("far", B, Hq, Hkv, d, start + 9, C, "fixed", fixed_slots=slots, r=32, seed=370 + slots)
+    got = {kvm.decode_plan(B, Hq, Hkv, d, slots + n)[1:] for n in (2 * C - 5, 2 * C, C + 1, C + 4)}
+    assert all(s == 8 and c > 1 for s, c in got) and any(c == clusters for _, c in got), got
+    params = synth.make_layer_params(wl, trivial=False)
+    tensors = synth.make_inputs(wl)
+    ys = []
+    for _ in range(2):
+        y, st = pu.run_gpu(wl, tensors, params, decode_from=start)
+        ys.append(y)
+        if len(ys) == 1:
+            units = [(0, 0), (B - 1, Hkv - 1)]
+            y_ref, o = pu.run_oracle(wl, tensors, params, units=units)
+            print(pu.compare(wl, y, st, y_ref, o, units=units))
+        st.free()
+    assert torch.equal(ys[0], ys[1])
