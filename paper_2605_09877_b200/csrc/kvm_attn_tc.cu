@@ -39,6 +39,8 @@ struct AttnTcParams {
   int32_t* status;
   float* part;       // split-KV partial results, [tile][split][D + 2][128] (see the epilogue)
   int32_t* part_cnt; // [tile] tickets, zero between launches
+  uint32_t* fold_seen; // (TELL) where this launch says that the fold before it is complete, by its number
+  uint32_t fold_no;
   int nq, Hq, Hkv, G;
   int qtiles;        // query tiles per (batch, head)
   int n_whole;       // the first n_whole (batch, head, query tile) tiles have one CTA each,
@@ -105,7 +107,9 @@ struct AttnTcCfg {
 enum { BAR_QFULL = 0, BAR_KFULL = 1, BAR_KFREE = 4, BAR_VFULL = 7, BAR_VFREE = 9, BAR_SFULL = 11, BAR_PFULL = 14,
        BAR_PVDONE = 17, BAR_XM = 20, BAR_COUNT = 22 };
 
-template <int D>
+// TELL: the routing filter of the block may run beside this grid (see launch_route_filter_tc).  (A build of its own: the shapes that
+// do not need it, bound by their chain of launches, took up to 5 % longer with the store in the kernel, executed or not.)
+template <int D, bool TELL>
 __global__ void __launch_bounds__(384, 1)
 attn_tc_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant__ CUtensorMap mapKs,
                const __grid_constant__ CUtensorMap mapVs, const __grid_constant__ CUtensorMap mapKw,
@@ -282,7 +286,10 @@ attn_tc_kernel(const __grid_constant__ CUtensorMap mapQ, const __grid_constant__
       if (dead) { atomicExch(p.status, (int)KVM_ERR_TIMEOUT); *abort_flag = 1; }
     }
   } else if (warp == 3) {
-    // spare warp: keeps the softmax warps aligned to the TMEM lane quarters
+    // spare warp: keeps the softmax warps aligned to the TMEM lane quarters; says that the fold before this grid is complete
+    // (this thread has waited for it)
+    if (TELL && blockIdx.x == 0 && lane == 0)
+      asm volatile("st.release.gpu.global.u32 [%0], %1;" ::"l"(p.fold_seen), "r"(p.fold_no) : "memory");
   } else {
     // ------------------------------ softmax / epilogue ------------------------------
     // Two warpgroups split every key tile by columns: half 0 owns keys 0..63 of the tile, half 1
@@ -556,6 +563,9 @@ int launch_attn_tc(State* st, const AttnArgs& a, cudaStream_t s) {
   p.out = a.out; p.tau_s = st->tau_s; p.tau_b = st->tau_b; p.status = st->status;
   p.nq = a.nq; p.Hq = st->Hq; p.Hkv = st->Hkv; p.G = st->G;
   p.part = st->attnPart; p.part_cnt = st->attnCnt;
+  const bool tell = st->serial && st->prof_hook == nullptr;
+  if (tell && ++st->foldNo == 0) ++st->foldNo;   // (0 says nothing)
+  p.fold_seen = st->foldSeen; p.fold_no = st->foldNo;
   p.out_vec = (reinterpret_cast<uintptr_t>(a.out) % 16 == 0 && a.so[0] % 8 == 0 && a.so[1] % 8 == 0 && a.so[2] % 8 == 0) ? 1 : 0;
   // key splits when there are few query tiles: up to a quarter of the GPU (the folds of the block
   // before run beside this kernel and are usually the longer chain; measured: a wider attention
@@ -589,14 +599,12 @@ int launch_attn_tc(State* st, const AttnArgs& a, cudaStream_t s) {
   cudaLaunchAttribute at[1];
   at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   at[0].val.programmaticStreamSerializationAllowed = 1;
-  lc.attrs = at; lc.numAttrs = st->serial && st->prof_hook == nullptr ? 1 : 0;
-  if (st->d == 128) {
-    lc.dynamicSmemBytes = AttnTcCfg<128>::SMEM_BYTES;
-    cudaLaunchKernelEx(&lc, attn_tc_kernel<128>, tm[0], tm[ks], tm[vs], tm[3], tm[4], p);
-  } else {
-    lc.dynamicSmemBytes = AttnTcCfg<64>::SMEM_BYTES;
-    cudaLaunchKernelEx(&lc, attn_tc_kernel<64>, tm[0], tm[ks], tm[vs], tm[3], tm[4], p);
-  }
+  lc.attrs = at; lc.numAttrs = tell ? 1 : 0;
+#define KVM_ATTN(DD, TT) cudaLaunchKernelEx(&lc, attn_tc_kernel<DD, TT>, tm[0], tm[ks], tm[vs], tm[3], tm[4], p)
+  lc.dynamicSmemBytes = st->d == 128 ? AttnTcCfg<128>::SMEM_BYTES : AttnTcCfg<64>::SMEM_BYTES;
+  if (st->d == 128) { if (tell) KVM_ATTN(128, true); else KVM_ATTN(128, false); }
+  else { if (tell) KVM_ATTN(64, true); else KVM_ATTN(64, false); }
+#undef KVM_ATTN
   return 1;
 }
 
@@ -620,8 +628,10 @@ bool setup_attn_tc(State* st) {
   ok = ok && encode_tmap_rows(&tm[3], st->stK, st->d, st->stRows, st->U, 128);
   ok = ok && encode_tmap_rows(&tm[4], st->stV, st->d, st->stRows, st->U, 128);
   if (!ok) return false;
-  if (cudaFuncSetAttribute(attn_tc_kernel<128>, cudaFuncAttributeMaxDynamicSharedMemorySize, AttnTcCfg<128>::SMEM_BYTES) != cudaSuccess) return false;
-  if (cudaFuncSetAttribute(attn_tc_kernel<64>, cudaFuncAttributeMaxDynamicSharedMemorySize, AttnTcCfg<64>::SMEM_BYTES) != cudaSuccess) return false;
+  for (auto k : {attn_tc_kernel<128, false>, attn_tc_kernel<128, true>})
+    if (cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, AttnTcCfg<128>::SMEM_BYTES) != cudaSuccess) return false;
+  for (auto k : {attn_tc_kernel<64, false>, attn_tc_kernel<64, true>})
+    if (cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, AttnTcCfg<64>::SMEM_BYTES) != cudaSuccess) return false;
   return true;
 }
 

@@ -114,6 +114,8 @@ struct State {
   // ---- split-KV attention scratch (device) ----
   float* attnPart;               // [kAttnSplitTiles][kAttnMaxSplits][d + 2][128]
   int32_t* attnCnt;              // [2 kAttnSplitTiles] tickets
+  uint32_t* foldSeen;            // (serial states) number of the attention launch that has met the end of the fold before it
+  uint32_t foldNo;               // number of the last attention launch (host)
   // ---- decode scratch (device): clusters of the same heads merge through it ----
   float* decPart;                // [kDecodePartCtas][d + 2]
   int32_t* decTicket;            // [kDecodePartCtas], zero between launches

@@ -43,7 +43,8 @@ struct RouteTcParams {
   float thr_coeff;         // candidate window = thr_coeff * ||kbar_j|| + 1e-5
   int64_t m;
   int C, Cmax, nsplit, S;
-  int ahead;               // the readout keys are complete when this grid may start (see the launch): wait at the end only
+  uint32_t* fold_seen;     // (AHEAD) holds fold_no once the attention kernel that this grid may run beside has met the end of the
+  uint32_t fold_no;        // fold that wrote the readout keys
 };
 
 template <int D>
@@ -66,7 +67,8 @@ struct RouteTcCfg {
 
 enum { RB_AFULL = 0, RB_BFULL = 1, RB_BFREE = 4, RB_SFULL = 7, RB_ACCFREE = 9, RB_COUNT = 11 };
 
-template <int D>
+// AHEAD: runs beside the attention kernel before it on the stream (see the launch).
+template <int D, bool AHEAD>
 __global__ void __launch_bounds__(352, 1)
 route_filter_tc_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CUtensorMap mapB,
                        const __grid_constant__ CUtensorMap mapH, const RouteTcParams p) {
@@ -107,6 +109,12 @@ route_filter_tc_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_co
     *abort_flag = 0;
     tc::fence_barrier_init();
   }
+  volatile int* seen = abort_flag + 1;
+  if (AHEAD && tid == 96) {   // (by a thread with nothing else to do: the load takes as long as the tensor memory's allocation)
+    uint32_t no;
+    asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(no) : "l"(p.fold_seen) : "memory");
+    *seen = no == p.fold_no;
+  }
   if (warp == 1) {
     tc::tmem_alloc(tmem_slot, Cfg::TMEM_COLS);
     tc::tmem_relinquish();
@@ -128,7 +136,8 @@ route_filter_tc_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_co
           tc::tma_load_3d(sA + mt * Cfg::TILE_BYTES + kb * Cfg::BOX_BYTES, gram ? &mapH : &mapA, &bars[RB_AFULL], kb * 64, mt * 128, a_unit);
       // the readout keys are written by the apply kernel of the fold before this one: wait for it here
       // (the set-up above and the load of the block's own keys run beside its tail)
-      if (!p.ahead) asm volatile("griddepcontrol.wait;" ::: "memory");
+      if (AHEAD && *seen) asm volatile("fence.proxy.async.global;" ::: "memory");   // (rows stored by threads, read by TMA)
+      else asm volatile("griddepcontrol.wait;" ::: "memory");
       for (int j = 0; j < nsteps; ++j) {
         const int s = j % Cfg::NS;
         const int jt = j;
@@ -140,6 +149,10 @@ route_filter_tc_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_co
         for (int kb = 0; kb < Cfg::NKB; ++kb)
           tc::tma_load_3d(sB + s * Cfg::TILE_BYTES + kb * Cfg::BOX_BYTES, gram ? &mapA : &mapB, &bars[RB_BFULL + s], kb * 64,
                           (int)(i0 + (int64_t)jt * 128), gram ? a_unit : u);
+      }
+      if (AHEAD) {   // (this grid does not end before the kernel that it ran beside)
+        asm volatile("griddepcontrol.wait;" ::: "memory");
+        if (blockIdx.x == 0 && blockIdx.y == 0) *p.fold_seen = 0;   // (CTAs that have not looked yet wait for the attention)
       }
     }
   } else if (warp == 1 || warp == 10) {
@@ -348,8 +361,6 @@ route_filter_tc_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_co
       }
     }
   }
-  // (this grid does not end before the kernel that it ran beside)
-  if (p.ahead) asm volatile("griddepcontrol.wait;" ::: "memory");
   tc::tc_fence_before();
   __syncthreads();
   if (warp == 1) {
@@ -366,8 +377,10 @@ int launch_route_filter_tc(State* st, int64_t m, int nsplit, int slot, bool earl
   p.a_unit0 = slot * st->U; p.gramT = st->gramT; p.gram_mode = 0; p.U = st->U;
   // A state with one readout copy runs this kernel behind the block's attention, which lets it start once it has itself
   // waited for the fold that wrote the readout keys: nothing here depends on the attention, so it fills the SMs that the
-  // attention's last wave leaves idle.
-  p.ahead = early_start && st->serial && st->prof_hook == nullptr && !(st->flags & KVM_FLAG_SIMT_ATTENTION) ? 1 : 0;
+  // attention's last wave leaves idle.  (A launch that may start says nothing about memory: the attention stores the number
+  // of its launch with release behind its wait, and a CTA here reads it with acquire before it reads the keys.)
+  const bool ahead = early_start && st->serial && st->prof_hook == nullptr && !(st->flags & KVM_FLAG_SIMT_ATTENTION);
+  p.fold_seen = st->foldSeen; p.fold_no = st->foldNo;
   const CUtensorMap* tm = reinterpret_cast<const CUtensorMap*>(st->tmaps);
   dim3 grid(nsplit, st->U);
   const int ks = (st->nfolds & 1) ? 6 : 1;   // the fold reads the readout copy of the current version
@@ -380,8 +393,11 @@ int launch_route_filter_tc(State* st, int64_t m, int nsplit, int slot, bool earl
   at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   at[0].val.programmaticStreamSerializationAllowed = 1;
   lc.attrs = at; lc.numAttrs = (early_start && st->prof_hook == nullptr) ? 1 : 0;
-  if (st->d == 128) { lc.dynamicSmemBytes = RouteTcCfg<128>::SMEM_BYTES; cudaLaunchKernelEx(&lc, route_filter_tc_kernel<128>, tm[5], tm[ks], tm[8], p); }
-  else { lc.dynamicSmemBytes = RouteTcCfg<64>::SMEM_BYTES; cudaLaunchKernelEx(&lc, route_filter_tc_kernel<64>, tm[5], tm[ks], tm[8], p); }
+#define KVM_ROUTE(DD, AA) cudaLaunchKernelEx(&lc, route_filter_tc_kernel<DD, AA>, tm[5], tm[ks], tm[8], p)
+  lc.dynamicSmemBytes = st->d == 128 ? RouteTcCfg<128>::SMEM_BYTES : RouteTcCfg<64>::SMEM_BYTES;
+  if (st->d == 128) { if (ahead) KVM_ROUTE(128, true); else KVM_ROUTE(128, false); }
+  else { if (ahead) KVM_ROUTE(64, true); else KVM_ROUTE(64, false); }
+#undef KVM_ROUTE
   return 1;
 }
 
@@ -391,11 +407,11 @@ int launch_gram_tc(State* st, int slot0, int nblk, cudaStream_t s) {
   p.candV = st->candV; p.candI = st->candI; p.chunkMax = st->chunkMax; p.chunkMeta = st->chunkMeta; p.chunkVal = st->chunkVal; p.status = st->status; p.m = 0;
   p.C = st->C; p.Cmax = st->Cmax; p.nsplit = 1; p.S = st->S;
   p.kbarNorm = st->kbarNorm; p.thr_coeff = 0.f;
-  p.a_unit0 = slot0 * st->U; p.gramT = st->gramT; p.gram_mode = 1; p.U = st->U; p.ahead = 0;
+  p.a_unit0 = slot0 * st->U; p.gramT = st->gramT; p.gram_mode = 1; p.U = st->U; p.fold_seen = nullptr; p.fold_no = 0;
   const CUtensorMap* tm = reinterpret_cast<const CUtensorMap*>(st->tmaps);
   dim3 grid(1, st->U, nblk);
-  if (st->d == 128) route_filter_tc_kernel<128><<<grid, 352, RouteTcCfg<128>::SMEM_BYTES, s>>>(tm[5], tm[1], tm[8], p);
-  else route_filter_tc_kernel<64><<<grid, 352, RouteTcCfg<64>::SMEM_BYTES, s>>>(tm[5], tm[1], tm[8], p);
+  if (st->d == 128) route_filter_tc_kernel<128, false><<<grid, 352, RouteTcCfg<128>::SMEM_BYTES, s>>>(tm[5], tm[1], tm[8], p);
+  else route_filter_tc_kernel<64, false><<<grid, 352, RouteTcCfg<64>::SMEM_BYTES, s>>>(tm[5], tm[1], tm[8], p);
   return 1;
 }
 
@@ -403,8 +419,10 @@ bool setup_route_tc(State* st) {
   CUtensorMap* tm = reinterpret_cast<CUtensorMap*>(st->tmaps);
   if (!encode_tmap_rows(&tm[5], st->kbarH, st->d, st->CbarRows, (int64_t)st->kbSlots * st->U, 128)) return false;
   if (!encode_tmap_rows(&tm[8], st->kbarHatH, st->d, st->CbarRows, (int64_t)st->kbSlots * st->U, 128)) return false;
-  if (cudaFuncSetAttribute(route_filter_tc_kernel<128>, cudaFuncAttributeMaxDynamicSharedMemorySize, RouteTcCfg<128>::SMEM_BYTES) != cudaSuccess) return false;
-  if (cudaFuncSetAttribute(route_filter_tc_kernel<64>, cudaFuncAttributeMaxDynamicSharedMemorySize, RouteTcCfg<64>::SMEM_BYTES) != cudaSuccess) return false;
+  for (auto k : {route_filter_tc_kernel<128, false>, route_filter_tc_kernel<128, true>})
+    if (cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, RouteTcCfg<128>::SMEM_BYTES) != cudaSuccess) return false;
+  for (auto k : {route_filter_tc_kernel<64, false>, route_filter_tc_kernel<64, true>})
+    if (cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, RouteTcCfg<64>::SMEM_BYTES) != cudaSuccess) return false;
   return true;
 }
 

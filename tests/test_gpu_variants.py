@@ -331,3 +331,28 @@ def test_decode_clusters_of_the_same_heads_merge_through_global_memory(B, Hq, Hk
             print(pu.compare(wl, y, st, y_ref, o, units=units))
         st.free()
     assert torch.equal(ys[0], ys[1])
+
+
+@pytest.mark.parametrize("B,Hq,Hkv,d,C,T,slots", [(1, 3, 3, 128, 64, 1500, 700), (8, 32, 32, 64, 64, 1111, 200), (4, 128, 64, 128, 128, 1400, 300)])
+def test_kernels_that_start_under_the_ones_before_equal_kernels_one_at_a_time(B, Hq, Hkv, d, C, T, slots):
+    """One readout copy: attention under the end of the fold, the routing filter under the attention.  With the timing hook on
+    nothing starts early; outputs, sums, rows and the slots of all tokens are the same, in calls of whole and of odd pieces."""
+    from paper_2605_09877_b200 import kvm
+    wl = synth.Workload("early", B, Hq, Hkv, d, T, C, "fixed", fixed_slots=slots, r=32, seed=400 + B, kind="mixture")
+    params = synth.make_layer_params(wl, trivial=False)
+    t = {n: x.cuda() for n, x in synth.make_inputs(wl).items() if n in "qkv"}
+    outs = []
+    for hook in (True, False, False):
+        st, g = pu.gpu_layer(wl, params, flags=kvm.FLAG_SERIAL_FOLDS)
+        st.profile_enable(hook)
+        y = torch.zeros_like(t["q"])
+        for a, z in ((0, 5 * C), (5 * C, 7 * C + 13), (7 * C + 13, T)):
+            st.prefill(t["q"][:, :, a:z], t["k"][:, :, a:z], t["v"][:, :, a:z], C, g, wl.r, out=y[:, :, a:z])
+        torch.cuda.synchronize()
+        assert st.check() == 0
+        e = st.export()
+        outs.append([y.cpu().view(torch.int16).numpy(), e["sum_k"], e["sum_v"], e["k_read"].view(torch.int16).numpy(), e["v_read"].view(torch.int16).numpy()] + list(st.assignments()))
+        st.free()
+    for o in outs[1:]:
+        for a, b in zip(outs[0], o):
+            assert np.array_equal(a, b)
