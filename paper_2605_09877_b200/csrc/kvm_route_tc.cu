@@ -38,8 +38,8 @@ struct RouteTcParams {
   int32_t* status;
   const float* kbarNorm;   // [U, Cmax] upper bound of ||kbar_j||
   int a_unit0;             // first unit of this block's slot in the memory-key tensor map
-  float* gramT;            // [slots][U, Cmax, Cmax]: output of the new-row filter launch (gram_mode), see below
-  int gram_mode, U;        // gram_mode: grid (1, U, blocks), block z uses slot a_unit0 / U + z
+  float* gramT;            // [slots][U, Cmax, Cmax]: output of the new-row filter launch (ROUTE_GRAM), see below
+  int U;                   // (ROUTE_GRAM: grid (1, U, blocks), block z uses slot a_unit0 / U + z)
   float thr_coeff;         // candidate window = thr_coeff * ||kbar_j|| + 1e-5
   int64_t m;
   int C, Cmax, nsplit, S;
@@ -67,12 +67,14 @@ struct RouteTcCfg {
 
 enum { RB_AFULL = 0, RB_BFULL = 1, RB_BFREE = 4, RB_SFULL = 7, RB_ACCFREE = 9, RB_COUNT = 11 };
 
-// AHEAD: runs beside the attention kernel before it on the stream (see the launch).
-template <int D, bool AHEAD>
+// MODE: the filter; the filter that may run beside the attention kernel before it on the stream (see the launch); the new-row products.
+enum { ROUTE_FILTER = 0, ROUTE_AHEAD = 1, ROUTE_GRAM = 2 };
+template <int D, int MODE>
 __global__ void __launch_bounds__(352, 1)
 route_filter_tc_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CUtensorMap mapB,
                        const __grid_constant__ CUtensorMap mapH, const RouteTcParams p) {
   using Cfg = RouteTcCfg<D>;
+  constexpr bool AHEAD = MODE == ROUTE_AHEAD;
   extern __shared__ uint8_t smem_raw[];
   uint8_t* base = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   uint8_t* sA = base + Cfg::OFF_A;
@@ -87,7 +89,7 @@ route_filter_tc_kernel(const __grid_constant__ CUtensorMap mapA, const __grid_co
   // New-row filter mode (a launch of its own, ahead of the folds: it needs the block's keys only):
   // the would-be row keys LN_s(kbar_a) are the M operand, the memory keys kbar_j the N operand, one
   // pass, and the products themselves are stored, gramT[a][j]; which rows a exist is known later.
-  const bool gram = p.gram_mode != 0;
+  constexpr bool gram = MODE == ROUTE_GRAM;
   const int a_unit = p.a_unit0 + (gram ? (int)blockIdx.z * p.U : 0) + u;
   int64_t per = (p.m + p.nsplit - 1) / p.nsplit;
   per = (per + 127) / 128 * 128;
@@ -374,7 +376,7 @@ int launch_route_filter_tc(State* st, int64_t m, int nsplit, int slot, bool earl
   p.candV = st->candV; p.candI = st->candI; p.chunkMax = st->chunkMax; p.chunkMeta = st->chunkMeta; p.chunkVal = st->chunkVal; p.status = st->status; p.m = m;
   p.C = st->C; p.Cmax = st->Cmax; p.nsplit = nsplit; p.S = st->S;
   p.kbarNorm = st->kbarNorm + (int64_t)slot * st->U * st->Cmax; p.thr_coeff = route_thr_coeff(st);
-  p.a_unit0 = slot * st->U; p.gramT = st->gramT; p.gram_mode = 0; p.U = st->U;
+  p.a_unit0 = slot * st->U; p.gramT = st->gramT; p.U = st->U;
   // A state with one readout copy runs this kernel behind the block's attention, which lets it start once it has itself
   // waited for the fold that wrote the readout keys: nothing here depends on the attention, so it fills the SMs that the
   // attention's last wave leaves idle.  (A launch that may start says nothing about memory: the attention stores the number
@@ -395,8 +397,8 @@ int launch_route_filter_tc(State* st, int64_t m, int nsplit, int slot, bool earl
   lc.attrs = at; lc.numAttrs = (early_start && st->prof_hook == nullptr) ? 1 : 0;
 #define KVM_ROUTE(DD, AA) cudaLaunchKernelEx(&lc, route_filter_tc_kernel<DD, AA>, tm[5], tm[ks], tm[8], p)
   lc.dynamicSmemBytes = st->d == 128 ? RouteTcCfg<128>::SMEM_BYTES : RouteTcCfg<64>::SMEM_BYTES;
-  if (st->d == 128) { if (ahead) KVM_ROUTE(128, true); else KVM_ROUTE(128, false); }
-  else { if (ahead) KVM_ROUTE(64, true); else KVM_ROUTE(64, false); }
+  if (st->d == 128) { if (ahead) KVM_ROUTE(128, ROUTE_AHEAD); else KVM_ROUTE(128, ROUTE_FILTER); }
+  else { if (ahead) KVM_ROUTE(64, ROUTE_AHEAD); else KVM_ROUTE(64, ROUTE_FILTER); }
 #undef KVM_ROUTE
   return 1;
 }
@@ -407,11 +409,11 @@ int launch_gram_tc(State* st, int slot0, int nblk, cudaStream_t s) {
   p.candV = st->candV; p.candI = st->candI; p.chunkMax = st->chunkMax; p.chunkMeta = st->chunkMeta; p.chunkVal = st->chunkVal; p.status = st->status; p.m = 0;
   p.C = st->C; p.Cmax = st->Cmax; p.nsplit = 1; p.S = st->S;
   p.kbarNorm = st->kbarNorm; p.thr_coeff = 0.f;
-  p.a_unit0 = slot0 * st->U; p.gramT = st->gramT; p.gram_mode = 1; p.U = st->U; p.fold_seen = nullptr; p.fold_no = 0;
+  p.a_unit0 = slot0 * st->U; p.gramT = st->gramT; p.U = st->U; p.fold_seen = nullptr; p.fold_no = 0;
   const CUtensorMap* tm = reinterpret_cast<const CUtensorMap*>(st->tmaps);
   dim3 grid(1, st->U, nblk);
-  if (st->d == 128) route_filter_tc_kernel<128, false><<<grid, 352, RouteTcCfg<128>::SMEM_BYTES, s>>>(tm[5], tm[1], tm[8], p);
-  else route_filter_tc_kernel<64, false><<<grid, 352, RouteTcCfg<64>::SMEM_BYTES, s>>>(tm[5], tm[1], tm[8], p);
+  if (st->d == 128) route_filter_tc_kernel<128, ROUTE_GRAM><<<grid, 352, RouteTcCfg<128>::SMEM_BYTES, s>>>(tm[5], tm[1], tm[8], p);
+  else route_filter_tc_kernel<64, ROUTE_GRAM><<<grid, 352, RouteTcCfg<64>::SMEM_BYTES, s>>>(tm[5], tm[1], tm[8], p);
   return 1;
 }
 
@@ -419,9 +421,9 @@ bool setup_route_tc(State* st) {
   CUtensorMap* tm = reinterpret_cast<CUtensorMap*>(st->tmaps);
   if (!encode_tmap_rows(&tm[5], st->kbarH, st->d, st->CbarRows, (int64_t)st->kbSlots * st->U, 128)) return false;
   if (!encode_tmap_rows(&tm[8], st->kbarHatH, st->d, st->CbarRows, (int64_t)st->kbSlots * st->U, 128)) return false;
-  for (auto k : {route_filter_tc_kernel<128, false>, route_filter_tc_kernel<128, true>})
+  for (auto k : {route_filter_tc_kernel<128, ROUTE_FILTER>, route_filter_tc_kernel<128, ROUTE_AHEAD>, route_filter_tc_kernel<128, ROUTE_GRAM>})
     if (cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, RouteTcCfg<128>::SMEM_BYTES) != cudaSuccess) return false;
-  for (auto k : {route_filter_tc_kernel<64, false>, route_filter_tc_kernel<64, true>})
+  for (auto k : {route_filter_tc_kernel<64, ROUTE_FILTER>, route_filter_tc_kernel<64, ROUTE_AHEAD>, route_filter_tc_kernel<64, ROUTE_GRAM>})
     if (cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, RouteTcCfg<64>::SMEM_BYTES) != cudaSuccess) return false;
   return true;
 }
