@@ -478,6 +478,168 @@ __device__ __forceinline__ void sort_n(K& key, int& val, K* sk, int* sv, int t) 
   }
 }
 
+struct DecideShared {
+  unsigned long long key[kMaxBlock];   // append scores of all tokens (exchanged)
+  unsigned tgt[kMaxBlock];             // row << 9 | token of all merged tokens (exchanged; all ones: appended)
+  int app[kMaxBlock];                  // append flags of all tokens (exchanged)
+  uint64_t bar[4];                     // the three exchanges and the results of row scans: bytes received
+  double score[kMaxBlock], best[kMaxBlock];   // (of this CTA's tokens, as everything below)
+  int barg[kMaxBlock], creator[kMaxBlock];
+  float thr[kMaxBlock];
+  signed char how[kMaxBlock];          // 0: its pairs are on the warp's list, 1: decided, 2: scan every row
+  int np[kDecideWarps];
+  int prow[kDecideWarps][kWarpPairs];
+  unsigned char ptok[kDecideWarps][kWarpPairs];
+  double pval[kDecideWarps][kWarpPairs];
+  unsigned word[kMaxBlock / 32];
+  int dead;
+  int nexh, npair;
+};
+
+// The exchanges: one value per token and CTA of the unit, its bytes counted on the receiver's barrier (a cluster barrier per
+// exchange cost about 2000 cycles, this less than half).  A unit's only CTA stores to itself: st.async is for clusters (in a
+// launch without one it raised an illegal instruction).
+__device__ __forceinline__ void decide_give32(int* arr, uint64_t* bar, int j, int r, int v, bool many) {
+  if (!many) { arr[j] = v; return; }
+  asm volatile("st.async.weak.shared::cluster.mbarrier::complete_tx::bytes.b32 [%0], %1, [%2];"
+               ::"r"(tc::cluster_addr(arr + j, r)), "r"(v), "r"(tc::cluster_addr(bar, r)) : "memory");
+}
+__device__ __forceinline__ void decide_give64(unsigned long long* arr, uint64_t* bar, int j, int r, unsigned long long v, bool many) {
+  if (!many) { arr[j] = v; return; }
+  asm volatile("st.async.weak.shared::cluster.mbarrier::complete_tx::bytes.b64 [%0], %1, [%2];"
+               ::"r"(tc::cluster_addr(arr + j, r)), "l"(v), "r"(tc::cluster_addr(bar, r)) : "memory");
+}
+__device__ __forceinline__ void decide_received(DecideShared& sm, int bar, bool many, uint32_t limit) {   // every thread calls; the wait is bounded
+  if (!many) __syncthreads();
+  else if (!tc::mbar_wait_cluster(&sm.bar[bar], 0, limit)) sm.dead = 1;
+}
+// order-preserving integer image of a score (never NaN: all ones is no image)
+__device__ __forceinline__ unsigned long long decide_key(double score) {
+  const long long bits = __double_as_longlong(score);
+  return (unsigned long long)bits ^ (bits < 0 ? ~0ull : 0x8000000000000000ull);
+}
+constexpr unsigned long long kScanKey = ~0ull;
+constexpr unsigned kScanTgt = 0xfffffffeu;   // (there is no token 510)
+
+// The tokens without a usable list, marked in an exchange in place of a score or target, so that every CTA of the unit knows all
+// of them and no other wait has to last as long as a scan of the state.  They are dealt over the CTAs in groups of up to four; all
+// warps of a CTA share the rows, a row is read once for the group, lanes 8 t .. 8 t + 7 keep the result of its token t.  What
+// is missing then goes out: the score (or, nothing being appended, the target) to every CTA, the best row to the token's own.
+// With each token scanned by the warp that had listed it, a run of equal tokens was one warp's work and the others waited (16
+// equal keys at the start of every block, 16384 tokens: 1 unit 50.6 -> 7.8 ms, 100 units 749 -> 83 ms with one token at a time).  The
+// wait is bounded by more than the scans can take.  Every thread calls; the pair lists are idle.
+template <int D, bool RK, bool APP>
+__device__ __forceinline__ void decide_scan_marked(const FoldDecideParams& p, DecideShared& sm, bool marked, const double (&gam)[D / 32],
+                                                   const double (&bet)[D / 32]) {
+  constexpr int CH = D / 32;
+  const int R = gridDim.x, rank = blockIdx.x, u = blockIdx.y;
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int nsl = (p.C + R - 1) / R;
+  const bool many = R > 1;
+  const int64_t rowBase = (int64_t)u * p.Mcap, tokBase = (int64_t)u * p.Cmax;
+  KbarRows<D, RK> kbarU;
+  kbarU.k64 = p.kbar64 + tokBase * D; kbarU.k16 = p.ok + (int64_t)u * p.unit_stride;
+  kbarU.stat = p.kbarStat + tokBase; kbarU.r = p.r;
+  if (tid < kMaxBlock) {
+    const unsigned bal = __ballot_sync(0xffffffffu, marked);
+    if (lane == 0) sm.word[warp] = bal;
+  }
+  __syncthreads();
+  int n = 0, own = 0;
+  for (int w = 0; w < kMaxBlock / 32; ++w) {
+    n += __popc(sm.word[w]);
+    for (unsigned b = sm.word[w]; b != 0; b &= b - 1) own += (32 * w + __ffs(b) - 1) / nsl == rank ? 1 : 0;
+  }
+  if (many && tid == 0) tc::mbar_expect_tx(&sm.bar[3], APP ? 8 * n + 12 * own : 4 * n);
+  const int gsz = min(4, (n + R - 1) / R);
+  int w = 0;
+  unsigned bits = sm.word[0];
+  for (int k = 0; k * gsz < n; ++k) {
+    int jt[4];   // the tokens of the group (past its end: the last one again)
+#pragma unroll
+    for (int t = 0; t < 4; ++t) {
+      if (t > 0) jt[t] = jt[t - 1];
+      if (t >= gsz || k * gsz + t >= n) continue;
+      while (bits == 0) bits = sm.word[++w];
+      jt[t] = 32 * w + __ffs(bits) - 1;
+      bits &= bits - 1;
+    }
+    if (k % R != rank) continue;
+    double kb[4][CH];
+#pragma unroll
+    for (int t = 0; t < 4; ++t)
+#pragma unroll
+      for (int c = 0; c < CH; ++c) kb[t][c] = kbarU.at(jt[t], lane + 32 * c, gam[c], bet[c]);
+    double score = -INFINITY, best = -INFINITY;   // of token lane >> 3 over this warp's rows
+    int arg = -1;
+    for (int64_t i0 = warp; i0 < p.m; i0 += 2 * kDecideWarps) {
+      double x[2][CH], mu[2], rs[2];
+#pragma unroll
+      for (int q = 0; q < 2; ++q) {   // (past the end: a copy of the last row, dropped)
+        const int64_t row = rowBase + min(i0 + q * kDecideWarps, p.m - 1);
+        mu[q] = p.kmu[row]; rs[q] = p.krstd[row];
+#pragma unroll
+        for (int c = 0; c < CH; ++c) x[q][c] = p.sumK[row * D + lane + 32 * c];
+      }
+#pragma unroll
+      for (int q = 0; q < 2; ++q) {
+        double acc[4] = {0.0, 0.0, 0.0, 0.0};
+#pragma unroll
+        for (int c = 0; c < CH; ++c) {
+          const double hat = gam[c] * ((x[q][c] - mu[q]) * rs[q]) + bet[c];
+#pragma unroll
+          for (int t = 0; t < 4; ++t) acc[t] += kb[t][c] * hat;
+        }
+        const double v = warp_reduce4(acc[0], acc[1], acc[2], acc[3], lane);
+        const int64_t i = i0 + q * kDecideWarps;
+        if (i < p.m) {   // (ascending rows: the lowest of equals)
+          if (v > score) score = v;
+          if (i >= p.S && v > best) { best = v; arg = (int)i; }
+        }
+      }
+    }
+    if ((lane & 7) == 0) { sm.pval[warp][lane >> 3] = score; sm.pval[warp][4 + (lane >> 3)] = best; sm.prow[warp][lane >> 3] = arg; }
+    __syncthreads();
+    const int t = tid / R, r = tid % R;
+    if (t < gsz && k * gsz + t < n) {   // one thread per token of the group and CTA of the unit
+      const int j = t == 0 ? jt[0] : t == 1 ? jt[1] : t == 2 ? jt[2] : jt[3];
+      score = best = -INFINITY;
+      arg = -1;
+      for (int z = 0; z < kDecideWarps; ++z) {
+        score = fmax(score, sm.pval[z][t]);
+        const double be = sm.pval[z][4 + t];
+        const int ar = sm.prow[z][t];
+        if (be > best || (be == best && ar < arg)) { best = be; arg = ar; }
+      }
+      if (APP) {
+        decide_give64(sm.key, &sm.bar[3], j, r, decide_key(score), many);
+        if (r == j / nsl) {
+          decide_give64(reinterpret_cast<unsigned long long*>(sm.best), &sm.bar[3], j, r, (unsigned long long)__double_as_longlong(best), many);
+          decide_give32(sm.barg, &sm.bar[3], j, r, arg, many);
+        }
+      } else {
+        decide_give32(reinterpret_cast<int*>(sm.tgt), &sm.bar[3], j, r, (int)(((unsigned)arg << 9) | (unsigned)j), many);
+      }
+    }
+    __syncthreads();
+  }
+  decide_received(sm, 3, many, (uint32_t)min((int64_t)0xffffffff, (int64_t)tc::kSpinLimit + (n + R - 1) / R * p.m));
+  __syncthreads();
+}
+
+// The same out of line, for the build whose registers are few (inlined it spilled in the common path).
+template <int D, bool RK, bool APP>
+__device__ __noinline__ void decide_scan_marked_call(const FoldDecideParams& p, DecideShared& sm, bool marked) {
+  const int lane = threadIdx.x & 31, hk = (int)blockIdx.y % p.Hkv;
+  double gam[D / 32], bet[D / 32];
+#pragma unroll
+  for (int c = 0; c < D / 32; ++c) {
+    gam[c] = (double)p.ln_w[hk * D + lane + 32 * c];
+    bet[c] = (double)p.ln_b[hk * D + lane + 32 * c];
+  }
+  decide_scan_marked<D, RK, APP>(p, sm, marked, gam, bet);
+}
+
 // Decisions of a fold: the R CTAs of a unit are a cluster, CTA r takes the tokens [r C / R, (r + 1) C / R) and every warp
 // a run of those.  A warp takes its tokens from the filter's lists to the exact similarities (and later from the new
 // rows' products to the merge targets) without a barrier; what needs every token of the block - the order of the append
@@ -486,31 +648,22 @@ __device__ __forceinline__ void sort_n(K& key, int& val, K* sk, int* sv, int t) 
 // What bounds it: the latency of its chain of dependent loads and exchanges (a state with few units has no work to hide
 // them).  With the block-wide steps on one CTA per unit, reached through a ticket, and the lists read in three
 // rounds the kernel took 28 us for 8 units of 5000 rows, 30 for 32 of 2000, 18.5 for 32 full states of 512; now 16, 24, 9.
-// PER_SM = 2 for grids that fill the GPU twice over (64 registers, a few spills), 1 for the small grids
-// of chain-bound shapes, where a CTA has an SM to itself anyway and keeps everything in registers.
-template <int D, int PER_SM, bool RK>
+// APP: the fold appends rows (n_append > 0): scores, append selection, new rows; without it only the targets are left.
+// PER_SM = 2 (64 registers) for states of more units than SMs, whose folds come here when they append nothing; 1 for the small
+// grids of chain-bound shapes, where a CTA has an SM to itself anyway and keeps everything in registers.
+template <int D, int PER_SM, bool RK, bool APP>
 __global__ void __launch_bounds__(kDecideThreads, PER_SM) fold_decide_kernel(const __grid_constant__ FoldDecideParams p) {
   constexpr int CH = D / 32;
-  __shared__ unsigned long long s_key[kMaxBlock];    // append scores of all tokens (exchanged)
-  __shared__ unsigned s_tgt[kMaxBlock];              // row << 9 | token of all merged tokens (exchanged; all ones: appended)
-  __shared__ int s_app[kMaxBlock];                   // append flags of all tokens (exchanged)
-  __shared__ uint64_t s_bar[3];                      // the three exchanges: bytes received
-  __shared__ double s_score[kMaxBlock], s_best[kMaxBlock];   // (of this CTA's tokens, as everything below)
-  __shared__ int s_barg[kMaxBlock], s_creator[kMaxBlock];
-  __shared__ float s_thr[kMaxBlock];
-  __shared__ signed char s_how[kMaxBlock];   // 0: its pairs are on the warp's list, 1: decided, 2: scan every row
-  __shared__ int s_np[kDecideWarps];
-  __shared__ int s_prow[kDecideWarps][kWarpPairs];
-  __shared__ unsigned char s_ptok[kDecideWarps][kWarpPairs];
-  __shared__ double s_pval[kDecideWarps][kWarpPairs];
-  __shared__ unsigned s_word[kMaxBlock / 32];
-  __shared__ int s_dead;
-  __shared__ int s_nexh, s_npair;
+  __shared__ DecideShared sm;
+  auto &s_key = sm.key; auto &s_tgt = sm.tgt; auto &s_app = sm.app; auto &s_bar = sm.bar; auto &s_score = sm.score; auto &s_best = sm.best;
+  auto &s_barg = sm.barg; auto &s_creator = sm.creator; auto &s_thr = sm.thr; auto &s_how = sm.how; auto &s_np = sm.np; auto &s_prow = sm.prow;
+  auto &s_ptok = sm.ptok; auto &s_pval = sm.pval; auto &s_word = sm.word;
+  int &s_dead = sm.dead, &s_nexh = sm.nexh, &s_npair = sm.npair;
 
   const int R = gridDim.x, rank = blockIdx.x;
   const int u = blockIdx.y, hk = u % p.Hkv;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  const int C = p.C, n_a = p.n_append;
+  const int C = p.C, n_a = APP ? p.n_append : 0;
   const int64_t m = p.m;
   const int nsl = (C + R - 1) / R;
   const int jlo = min(C, rank * nsl), jhi = min(C, jlo + nsl);
@@ -534,34 +687,18 @@ __global__ void __launch_bounds__(kDecideThreads, PER_SM) fold_decide_kernel(con
   if (tid == 0) {
     s_nexh = 0; s_npair = 0; s_dead = 0;
     const uint32_t bytes[3] = {8, 4, 4};   // per token
-    for (int i = 0; i < 3; ++i) tc::mbar_init(&s_bar[i], 1);
+    for (int i = 0; i < 4; ++i) tc::mbar_init(&s_bar[i], 1);
     tc::fence_barrier_init();
     for (int i = 0; i < 3; ++i) tc::mbar_expect_tx(&s_bar[i], bytes[i] * (uint32_t)C);
   }
   if (tid < kDecideWarps) s_np[tid] = 0;
   if (tid < kMaxBlock) s_creator[tid] = 0;
-  if (tid < kMaxBlock && (tid >= C || n_a == 0)) { s_tgt[tid] = 0xffffffffu; s_app[tid] = 0; }   // (what the exchanges leave out)
+  if (tid < kMaxBlock && (tid >= C || !APP)) { s_tgt[tid] = 0xffffffffu; s_app[tid] = 0; }   // (what the exchanges leave out)
   __syncthreads();
-  // the exchanges: one value per token and CTA of the unit, its bytes counted on the receiver's barrier (a cluster
-  // barrier per exchange cost about 2000 cycles, this less than half).  A CTA's barriers exist, and a CTA is there, from
-  // here on; it leaves when the others have, at the end.  A unit's only CTA stores to itself: st.async is for clusters
-  // (in a launch without one it raised an illegal instruction).
+  // A CTA's barriers exist, and a CTA is there, from here on; it leaves when the others have, at the end.
   const bool many = R > 1;
   if (many) asm volatile("barrier.cluster.arrive.release;" ::: "memory");
-  auto give32 = [&](int* arr, int bar, int j, int r, int v) {
-    if (!many) { arr[j] = v; return; }
-    asm volatile("st.async.weak.shared::cluster.mbarrier::complete_tx::bytes.b32 [%0], %1, [%2];"
-                 ::"r"(tc::cluster_addr(arr + j, r)), "r"(v), "r"(tc::cluster_addr(&s_bar[bar], r)) : "memory");
-  };
-  auto give64 = [&](unsigned long long* arr, int bar, int j, int r, unsigned long long v) {
-    if (!many) { arr[j] = v; return; }
-    asm volatile("st.async.weak.shared::cluster.mbarrier::complete_tx::bytes.b64 [%0], %1, [%2];"
-                 ::"r"(tc::cluster_addr(arr + j, r)), "l"(v), "r"(tc::cluster_addr(&s_bar[bar], r)) : "memory");
-  };
-  auto received = [&](int bar) {   // every thread calls; the wait is bounded
-    if (!many) __syncthreads();
-    else if (!tc::mbar_wait_cluster(&s_bar[bar], 0)) s_dead = 1;
-  };
+  auto received = [&](int bar) { decide_received(sm, bar, many, tc::kSpinLimit); };
   // everything above reads parameters and writes shared memory only
   asm volatile("griddepcontrol.wait;" ::: "memory");
 
@@ -603,15 +740,15 @@ __global__ void __launch_bounds__(kDecideThreads, PER_SM) fold_decide_kernel(con
     unsigned use = 0;
 #pragma unroll
     for (int k = 0; k < kTopK; ++k)
-      if (i[k] >= 0 && (i[k] < p.S ? n_a > 0 : keep)) use |= 1u << k;
+      if (i[k] >= 0 && (i[k] < p.S ? APP : keep)) use |= 1u << k;
     const int c = __popc(use);
     // a list overflowed, or there is no maximum: every row exactly
-    bool exh = !(gmax > -INFINITY) || (cnt > (float)kTopK && (keep || (n_a > 0 && sp == 0)));
+    bool exh = !(gmax > -INFINITY) || (cnt > (float)kTopK && (keep || (APP && sp == 0)));
     // A fold that appends nothing needs no scores, and the true arg max is always among the candidates: a token
     // with a single candidate is decided without the exact similarity.
     bool single = false;
     const unsigned group = (TL == 32 ? 0xffffffffu : (1u << TL) - 1u) << (lane & ~(TL - 1));
-    if (n_a == 0) {
+    if (!APP) {
       const unsigned one = __ballot_sync(0xffffffffu, c >= 1) & group, two = __ballot_sync(0xffffffffu, c >= 2) & group;
       single = two == 0u && __popc(one) == 1;
     }
@@ -702,37 +839,21 @@ __global__ void __launch_bounds__(kDecideThreads, PER_SM) fold_decide_kernel(con
       }
       s_score[j] = score; s_best[j] = best; s_barg[j] = barg;
     }
-    // exhaustive path: rows in sequence
-    unsigned todo = __ballot_sync(0xffffffffu, how == 2);
-    nexh = __popc(todo);
-    while (todo) {
-      const int jx = wj0 + __ffs(todo) - 1;
-      todo &= todo - 1;
-      double kb[CH];
-#pragma unroll
-      for (int i = 0; i < CH; ++i) kb[i] = kbarU.at(jx, lane + 32 * i, gam[i], bet[i]);
-      double score = -INFINITY, best = -INFINITY;
-      int barg = -1;
-      for (int64_t i = 0; i < m; ++i) {
-        const double acc = warp_sim<CH>(kb, p.sumK + (rowBase + i) * D, p.kmu[rowBase + i], p.krstd[rowBase + i], gam, bet, lane);
-        if (acc > score) score = acc;
-        if (i >= p.S && acc > best) { best = acc; barg = (int)i; }
-      }
-      if (lane == 0) { s_score[jx] = score; s_best[jx] = best; s_barg[jx] = barg; }
-    }
+    nexh = __popc(__ballot_sync(0xffffffffu, how == 2));
     __syncwarp();
   }
   if (many) asm volatile("barrier.cluster.wait.acquire;" ::: "memory");   // (all CTAs of the unit are set up)
 
-  if (n_a > 0) {
+  if constexpr (APP) {
     // ---- B: append selection: the n_a smallest scores, ties to the smaller token index.  Every CTA gets all keys
     //      and counts the ranks of its own tokens, q threads per token. ----
     for (int e = lane; e < (wj1 - wj0) * R; e += 32) {
       const int j = wj0 + e / R;
-      const long long bits = __double_as_longlong(s_score[j]);   // order-preserving integer image of the double
-      give64(s_key, 0, j, e % R, (unsigned long long)bits ^ (bits < 0 ? ~0ull : 0x8000000000000000ull));
+      decide_give64(s_key, &s_bar[0], j, e % R, s_how[j] == 2 ? kScanKey : decide_key(s_score[j]), many);
     }
     received(0);
+    const bool marked = tid < C && s_key[tid] == kScanKey;
+    if (__syncthreads_or(marked) && !s_dead) decide_scan_marked<D, RK, APP>(p, sm, marked, gam, bet);
     {
       int q = 1;
       while (2 * q * nsl <= kDecideThreads && q < 32) q *= 2;
@@ -749,7 +870,7 @@ __global__ void __launch_bounds__(kDecideThreads, PER_SM) fold_decide_kernel(con
       }
       for (int o = q >> 1; o > 0; o >>= 1) cnt += __shfl_xor_sync(0xffffffffu, cnt, o);
       if (mine)
-        for (int r = part; r < R; r += q) give32(s_app, 1, j, r, cnt < n_a ? 1 : 0);
+        for (int r = part; r < R; r += q) decide_give32(s_app, &s_bar[1], j, r, cnt < n_a ? 1 : 0, many);
     }
     received(1);
     // rows are laid down in ascending token order: position of an appended token = appended tokens before it
@@ -856,12 +977,21 @@ __global__ void __launch_bounds__(kDecideThreads, PER_SM) fold_decide_kernel(con
   for (int e = lane; e < (wj1 - wj0) * R; e += 32) {
     const int j = wj0 + e / R;
     // (rows < 2^23, tokens < 2^9)
-    give32(reinterpret_cast<int*>(s_tgt), 2, j, e % R, s_app[j] ? -1 : (int)(((unsigned)s_barg[j] << 9) | (unsigned)j));
+    decide_give32(reinterpret_cast<int*>(s_tgt), &s_bar[2], j, e % R,
+                  s_app[j] ? -1 : !APP && s_how[j] == 2 ? (int)kScanTgt : (int)(((unsigned)s_barg[j] << 9) | (unsigned)j), many);
   }
   if (lane == 0 && nexh) atomicAdd(&s_nexh, nexh);
   if (lane == 0 && npair) atomicAdd(&s_npair, npair);
   received(2);
-  __syncthreads();
+  if constexpr (APP) {
+    __syncthreads();
+  } else {
+    const bool marked = tid < C && s_tgt[tid] == kScanTgt;
+    if (__syncthreads_or(marked) && !s_dead) {
+      if constexpr (PER_SM == 1) decide_scan_marked<D, RK, APP>(p, sm, marked, gam, bet);
+      else decide_scan_marked_call<D, RK, APP>(p, sm, marked);
+    }
+  }
   if (many) asm volatile("barrier.cluster.arrive.release;" ::: "memory");
   if (s_dead) {   // (a wait ran out: nothing is published)
     if (tid == 0) atomicExch(p.counters - 1, (int)KVM_ERR_TIMEOUT);
@@ -2045,14 +2175,14 @@ static void launch_pruned(const State* st, const cudaLaunchConfig_t& lc, const F
     else cudaLaunchKernelEx(&lc, fold_decide_pruned_kernel<64, PER_SM, false>, p);
   }
 }
-template <int PER_SM>
+template <int PER_SM, bool APP>
 static void launch_decide(const State* st, const cudaLaunchConfig_t& lc, const FoldDecideParams& p) {
   if (st->d == 128) {
-    if (st->recomputeK) cudaLaunchKernelEx(&lc, fold_decide_kernel<128, PER_SM, true>, p);
-    else cudaLaunchKernelEx(&lc, fold_decide_kernel<128, PER_SM, false>, p);
+    if (st->recomputeK) cudaLaunchKernelEx(&lc, fold_decide_kernel<128, PER_SM, true, APP>, p);
+    else cudaLaunchKernelEx(&lc, fold_decide_kernel<128, PER_SM, false, APP>, p);
   } else {
-    if (st->recomputeK) cudaLaunchKernelEx(&lc, fold_decide_kernel<64, PER_SM, true>, p);
-    else cudaLaunchKernelEx(&lc, fold_decide_kernel<64, PER_SM, false>, p);
+    if (st->recomputeK) cudaLaunchKernelEx(&lc, fold_decide_kernel<64, PER_SM, true, APP>, p);
+    else cudaLaunchKernelEx(&lc, fold_decide_kernel<64, PER_SM, false, APP>, p);
   }
 }
 
@@ -2132,8 +2262,10 @@ int launch_fold(State* st, const FoldArgs& a, cudaStream_t s) {
       if (st->U <= 2 * 148) launch_pruned<2>(st, lc, p);
       else launch_pruned<4>(st, lc, p);
     } else {
-      if (R * st->U <= 148) launch_decide<1>(st, lc, p);
-      else launch_decide<2>(st, lc, p);
+      // (folds that append rows to more units than SMs went the other way)
+      if (a.n_append > 0) launch_decide<1, true>(st, lc, p);
+      else if (R * st->U <= 148) launch_decide<1, false>(st, lc, p);
+      else launch_decide<2, false>(st, lc, p);
     }
     ++launches;
   }

@@ -356,3 +356,63 @@ def test_kernels_that_start_under_the_ones_before_equal_kernels_one_at_a_time(B,
     for o in outs[1:]:
         for a, b in zip(outs[0], o):
             assert np.array_equal(a, b)
+
+
+def _equal_keys(wl, where):
+    """Inputs in which the tokens `where(position in block)` of every block have one and the same key per head."""
+    tensors = synth.make_inputs(wl)
+    pos = [t for t in range(wl.T) if where(t % wl.C)]
+    tensors["k"][:, :, pos] = tensors["k"][:, :, :1].clone()
+    return tensors
+
+
+@pytest.mark.parametrize("B,Hkv,d,C,T,kind", [
+    (1, 1, 64, 256, 256 * 9 + 3, dict(growth="sqrt", sqrt_coeff=16)),      # eight CTAs per unit
+    (1, 9, 128, 256, 256 * 7, dict(growth="sqrt", sqrt_coeff=20)),         # four
+    (1, 1, 128, 128, 128 * 12, dict(growth="fixed", fixed_slots=300)),     # eight, nothing appended
+    (2, 20, 64, 64, 64 * 9 + 1, dict(growth="fixed", fixed_slots=150)),    # two, nothing appended
+    (2, 20, 64, 256, 256 * 6, dict(growth="sqrt", sqrt_coeff=16)),         # two
+    (4, 25, 64, 256, 256 * 6, dict(growth="sqrt", sqrt_coeff=16)),         # one CTA per unit
+    (10, 16, 64, 128, 128 * 8, dict(growth="fixed", fixed_slots=128)),     # more units than SMs, nothing appended
+])
+def test_runs_of_equal_keys_in_one_slice_of_the_block(B, Hkv, d, C, T, kind):
+    """The tokens whose candidate lists overflow are neighbours, all in the slice of one CTA (and of one or two of its warps); the
+    other CTAs of the unit have none.  Scores, targets and slots against the oracle."""
+    wl = synth.Workload("runs", B, Hkv, Hkv, d, T, C, r=0, S=1, seed=410 + Hkv, **kind)
+    params = synth.make_layer_params(wl)
+    for lo, hi in ((0, 16), (C - 21, C)):
+        tensors = _equal_keys(wl, lambda p: lo <= p < hi)
+        y_gpu, st = pu.run_gpu(wl, tensors, params)
+        units = [(0, 0), (B - 1, Hkv - 1)]
+        y_ref, o = pu.run_oracle(wl, tensors, params, units=units)
+        print(pu.compare(wl, y_gpu, st, y_ref, o, units=units))
+        assert st.debug_counters()["exhaustive_tokens"] > 0
+        st.free()
+
+
+@pytest.mark.parametrize("units", [1, 40, 100])
+def test_runs_of_equal_keys_cost_what_scattered_ones_cost(units):
+    """Sixteen tokens of every block scan the state: neighbours (one or two warps' own tokens) or one every sixteen tokens
+    (one per warp).  The same number of scans, dealt over all warps of the unit: about the same time (ten times more for
+    the neighbours when every warp scanned for its own tokens)."""
+    from paper_2605_09877_b200 import kvm
+    wl = synth.Workload("deal", 1, units, units, 64, 256 * 14, 256, "fixed", fixed_slots=1500, r=0, seed=430)
+    ms = []
+    for where in (lambda p: p < 16, lambda p: p % 16 == 0):
+        t = {n: x.cuda() for n, x in _equal_keys(wl, where).items() if n in "qkv"}
+        st, g = pu.gpu_layer(wl, {})
+        best = float("inf")
+        for _ in range(3):
+            a, b = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+            st.reset()
+            a.record()
+            st.prefill(t["q"], t["k"], t["v"], wl.C, g, 0)
+            b.record()
+            torch.cuda.synchronize()
+            best = min(best, a.elapsed_time(b))
+        ms.append(best)
+        assert st.check() == 0 and st.debug_counters()["exhaustive_tokens"] > 100 * units
+        st.free()
+    print(units, ms)
+    assert ms[0] < 2 * ms[1], ms
+
