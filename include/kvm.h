@@ -285,6 +285,12 @@ kvm_status_t kvm_profile_read(kvm_state_t* state, double* ms, int64_t* groups);
  * `out` has room for four values.  32-bit device counters. */
 kvm_status_t kvm_debug_counters(kvm_state_t* state, int64_t* out, void* cuda_stream);
 
+/* Failure test: in the next fold that decides on state rows, the last of the thread blocks that share unit `unit` (batch row *
+ * n_kv_heads + kv head) loses the targets that it should send to the others (no effect where one block serves a unit).  Their wait
+ * (shortened) runs out, kvm_state_check reports KVM_ERR_TIMEOUT, the unit keeps the rows that it had (those the fold should have
+ * appended are undefined), the other units fold as ever. */
+kvm_status_t kvm_debug_drop_exchange(kvm_state_t* state, int32_t unit);
+
 /* How a decode step over n_rows rows (state and window) is cut, for tests: out[0] query heads per CTA, out[1] CTAs per
  * cluster (row splits merged through shared memory), out[2] clusters per group of heads (merged through global memory).
  * Host arithmetic only. */

@@ -296,6 +296,7 @@ KVM_API kvm_status_t kvm_state_create(const kvm_config_t* cfg, kvm_state_t** out
   s.rope_base = cfg->rope_base; s.ln_eps = cfg->ln_eps; s.norm_eps = cfg->norm_eps;
   s.flags = cfg->flags; s.device = cfg->device;
   s.stRows = (int64_t)s.w * s.Cmax + s.Tcall;
+  s.dropUnit = -1;
 
   const int d = s.d;
   std::vector<float> lw((size_t)s.Hkv * d, 1.f), lb((size_t)s.Hkv * d, 0.f), ts(s.Hq, 1.f), tb(s.Hq, 1.f);
@@ -487,6 +488,12 @@ KVM_API kvm_status_t kvm_state_check(kvm_state_t* ks, void* cuda_stream) {
   if (w == 0) return KVM_OK;
   if (cudaMemsetAsync(ks->s.status, 0, sizeof(w), stream) != cudaSuccess) return KVM_ERR_CUDA;   // reported once
   return w == KVM_ERR_TIMEOUT ? KVM_ERR_TIMEOUT : KVM_ERR_CUDA;
+}
+
+KVM_API kvm_status_t kvm_debug_drop_exchange(kvm_state_t* ks, int32_t unit) {
+  if (!ks || unit < 0 || unit >= ks->s.U) return KVM_ERR_INVALID_ARG;
+  ks->s.dropUnit = unit;
+  return KVM_OK;
 }
 
 KVM_API kvm_status_t kvm_debug_decode_plan(int32_t batch, int32_t n_q_heads, int32_t n_kv_heads, int32_t head_dim,

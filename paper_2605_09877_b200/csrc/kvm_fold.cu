@@ -406,6 +406,7 @@ struct FoldDecideParams {
   int32_t* counters;   // debug: [0] tokens on the exhaustive path, [1] candidate pairs, [2] tokens decided
   int64_t Mcap, m;
   int C, Cmax, Hkv, S, n_append, nsplit;
+  int drop_unit;       // kvm_debug_drop_exchange: the unit whose last CTA loses its targets (-1: none)
   float thr_coeff;
   double ln_eps;
 };
@@ -698,7 +699,8 @@ __global__ void __launch_bounds__(kDecideThreads, PER_SM) fold_decide_kernel(con
   // A CTA's barriers exist, and a CTA is there, from here on; it leaves when the others have, at the end.
   const bool many = R > 1;
   if (many) asm volatile("barrier.cluster.arrive.release;" ::: "memory");
-  auto received = [&](int bar) { decide_received(sm, bar, many, tc::kSpinLimit); };
+  const uint32_t spins = u == p.drop_unit ? 1u << 16 : tc::kSpinLimit;
+  auto received = [&](int bar) { decide_received(sm, bar, many, spins); };
   // everything above reads parameters and writes shared memory only
   asm volatile("griddepcontrol.wait;" ::: "memory");
 
@@ -974,7 +976,8 @@ __global__ void __launch_bounds__(kDecideThreads, PER_SM) fold_decide_kernel(con
     }
   }
   // ---- E: every CTA of the unit gets all merge targets ----
-  for (int e = lane; e < (wj1 - wj0) * R; e += 32) {
+  const bool drop = u == p.drop_unit && rank == R - 1;   // (failure test: what this CTA should send is lost)
+  for (int e = lane; e < (drop ? 0 : (wj1 - wj0) * R); e += 32) {
     const int j = wj0 + e / R;
     // (rows < 2^23, tokens < 2^9)
     decide_give32(reinterpret_cast<int*>(s_tgt), &s_bar[2], j, e % R,
@@ -992,10 +995,12 @@ __global__ void __launch_bounds__(kDecideThreads, PER_SM) fold_decide_kernel(con
       else decide_scan_marked_call<D, RK, APP>(p, sm, marked);
     }
   }
+  if (tid == 0 && rank == 0) p.nmerge[u] = C - n_a;
   if (many) asm volatile("barrier.cluster.arrive.release;" ::: "memory");
-  if (s_dead) {   // (a wait ran out: nothing is published)
+  if (s_dead) {   // a wait ran out: whatever the unit's other CTAs publish, the apply kernel leaves the unit as it is
     if (tid == 0) atomicExch(p.counters - 1, (int)KVM_ERR_TIMEOUT);
     if (many) asm volatile("barrier.cluster.wait.acquire;" ::: "memory");
+    if (tid == 0) p.nmerge[u] = -1;   // (behind the first CTA's store)
     return;
   }
   if (tid == 0) {
@@ -1044,7 +1049,6 @@ __global__ void __launch_bounds__(kDecideThreads, PER_SM) fold_decide_kernel(con
         p.sorted[tokBase + less] = j;
       }
     }
-    if (tid == 0 && rank == 0) p.nmerge[u] = C - n_a;
   }
   if (many) asm volatile("barrier.cluster.wait.acquire;" ::: "memory");   // (nobody leaves before everybody has received)
 }
@@ -1686,6 +1690,7 @@ __global__ void __launch_bounds__(256, 4) fold_apply_kernel(FoldApplyParams p) {
   const __half* ovU = p.ov + (int64_t)u * p.unit_stride;
   const float* ogU = p.og + (int64_t)u * p.gate_stride;
   const int nmerge = p.all_append ? 0 : p.nmerge[u];
+  if (nmerge < 0) return;   // (the unit's decisions were not completed)
   const int m = (int)p.m;
 
   // task 0: the q-th appended row; task 1: the segment of an old row whose head sits at sorted[q]
@@ -1841,6 +1846,7 @@ __global__ void __launch_bounds__(256, 2) fold_apply_rows4_kernel(FoldApplyParam
   const __half* ovU = p.ov + (int64_t)u * p.unit_stride;
   const float* ogU = p.og + (int64_t)u * p.gate_stride;
   const int nmerge = p.all_append ? 0 : s_nmerge;
+  if (nmerge < 0) return;   // (the unit's decisions were not completed)
   const int m = (int)p.m;
 
   // A warp takes groups of four row slots in turn (with few CTAs per unit the stores of one group drain
@@ -2234,6 +2240,7 @@ int launch_fold(State* st, const FoldArgs& a, cudaStream_t s) {
     p.C = C; p.Cmax = st->Cmax; p.Hkv = st->Hkv; p.S = st->S; p.n_append = a.n_append; p.nsplit = nsplit;
     p.thr_coeff = route_thr_coeff(st);
     p.ln_eps = (double)st->ln_eps;
+    p.drop_unit = st->dropUnit; st->dropUnit = -1;
     KernelTimer kt(st, 4, s);
     // CTAs per unit: about 64 in all - with 128, what shorter slices save is lost to the attention kernel beside them,
     // which needs whole SMs (measured, 32 units: 9.0 against 8.5 ms for 32768 tokens; 8 units: no difference) -, two per

@@ -119,6 +119,7 @@ struct State {
   // ---- decode scratch (device): clusters of the same heads merge through it ----
   float* decPart;                // [kDecodePartCtas][d + 2]
   int32_t* decTicket;            // [kDecodePartCtas], zero between launches
+  int dropUnit;                  // (host) unit that loses an exchange of the next fold's decisions, -1 (kvm_debug_drop_exchange)
   // ---- optional per-kernel timing hook (set by kvm_profile_enable): phase ids
   //      0 ingest, 1 attention, 2 memory keys, 3 routing filter, 4 decide, 5 apply, 6 decode ----
   void (*prof_hook)(void* ctx, int phase, int begin, cudaStream_t s);

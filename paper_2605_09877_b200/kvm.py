@@ -27,7 +27,7 @@ EXPORTS = ["kvm_plan_capacity", "kvm_state_create", "kvm_prefill", "kvm_decode_s
            "kvm_debug_assignments", "kvm_launch_count", "kvm_status_string", "kvm_state_reset",
            "kvm_profile_enable", "kvm_profile_read", "kvm_debug_counters", "kvm_attend_rows_noalloc", "kvm_merge_gate", "kvm_head_layernorm",
            "kvm_state_snapshot_info", "kvm_state_export_window", "kvm_state_import", "kvm_debug_expire_wait",
-           "kvm_debug_decode_plan"]
+           "kvm_debug_decode_plan", "kvm_debug_drop_exchange"]
 
 
 class KVMError(RuntimeError):
@@ -107,6 +107,8 @@ def _load():
     L.kvm_attend_rows_noalloc.argtypes = [vp, vp, vp, C.c_int32, C.c_int64, C.c_int32, C.c_float, vp, vp]
     L.kvm_merge_gate.restype = C.c_int
     L.kvm_merge_gate.argtypes = [vp, vp, C.c_int32, C.c_int64, C.c_int32, C.c_int32, vp, vp, vp]
+    L.kvm_debug_drop_exchange.restype = C.c_int
+    L.kvm_debug_drop_exchange.argtypes = [vp, C.c_int32]
     L.kvm_debug_decode_plan.restype = C.c_int
     L.kvm_debug_decode_plan.argtypes = [C.c_int32, C.c_int32, C.c_int32, C.c_int32, C.c_int64, C.POINTER(C.c_int32)]
     L.kvm_debug_expire_wait.restype = C.c_int
@@ -366,6 +368,11 @@ class KVMState:
         rc = lib.kvm_debug_expire_wait(self._h, spins, _stream_ptr(stream))
         if rc != KVM_OK:
             raise KVMError(rc, "kvm_debug_expire_wait")
+
+    def debug_drop_exchange(self, unit: int):
+        rc = lib.kvm_debug_drop_exchange(self._h, unit)
+        if rc != KVM_OK:
+            raise KVMError(rc, "kvm_debug_drop_exchange")
 
     def launch_count(self):
         return lib.kvm_launch_count(self._h)

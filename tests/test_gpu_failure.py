@@ -76,3 +76,43 @@ def test_gate_status_word_stays_clear_on_the_success_path():
     gate = kvm.merge_gate(x, w, status=status)      # 16 heads, d_model % 64 == 0: the tensor-core path
     torch.cuda.synchronize()
     assert int(status.item()) == 0 and torch.isfinite(gate).all()
+
+
+@pytest.mark.parametrize("Hkv,d,growth", [(3, 64, dict(growth="sqrt", sqrt_coeff=20)), (3, 128, dict(growth="fixed", fixed_slots=200)),
+                                          (40, 64, dict(growth="sqrt", sqrt_coeff=20))])
+def test_a_fold_whose_decisions_are_incomplete_leaves_its_unit_as_it_was(Hkv, d, growth):
+    """One of the thread blocks of a unit loses what it should send: the others' bounded wait runs out, the call is reported
+    once, none of the unit's rows is touched by decisions that are not all there, and the other units fold as in a run
+    without the loss (one and four rows per warp in the apply kernel).  The state works on."""
+    from paper_2605_09877_b200 import kvm
+    wl = synth.Workload("lost", 1, Hkv, Hkv, d, 256 * 6, 256, seed=54, **growth)
+    params = synth.make_layer_params(wl)
+    q, k, v = (synth.make_inputs(wl)[n].cuda() for n in "qkv")
+    cut, end, unit = 256 * 4, 256 * 5, Hkv - 2
+
+    def run(st, g, a, z):
+        st.prefill(q[:, :, a:z], k[:, :, a:z], v[:, :, a:z], wl.C, g, wl.r)
+        torch.cuda.synchronize()
+        return st.export()
+
+    st, g = pu.gpu_layer(wl, params)
+    run(st, g, 0, cut)
+    whole = run(st, g, cut, end)
+    assert st.check() == 0
+    st.free()
+    st, g = pu.gpu_layer(wl, params)
+    before = run(st, g, 0, cut)
+    m = st.info()["n_slots"]
+    with pytest.raises(kvm.KVMError):
+        st.debug_drop_exchange(Hkv)
+    st.debug_drop_exchange(unit)
+    after = run(st, g, cut, end)
+    assert st.check() == 7 and st.check() == 0          # KVM_ERR_TIMEOUT, reported once
+    others = [u for u in range(Hkv) if u != unit]
+    for n in ("sum_k", "sum_v", "radius", "weight", "count", "k_read", "v_read"):
+        a, w, b = (np.asarray(x[n]) for x in (after, whole, before))
+        assert np.array_equal(a[others], w[others]), n
+        assert np.array_equal(a[unit, :m], b[unit, :m]), n
+    run(st, g, end, wl.T)
+    assert st.check() == 0
+    st.free()
