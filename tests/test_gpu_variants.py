@@ -416,3 +416,17 @@ def test_runs_of_equal_keys_cost_what_scattered_ones_cost(units):
     print(units, ms)
     assert ms[0] < 2 * ms[1], ms
 
+
+@pytest.mark.parametrize("Hkv,d,C", [(80, 64, 256), (148, 64, 256), (100, 128, 128), (160, 64, 256), (40, 64, 256), (9, 128, 256), (1, 64, 256)])
+def test_crowded_runs_are_compared_pair_by_pair(Hkv, d, C):
+    """Every key of a block occurs eight times, the same keys in every block: each token has eight candidate rows, the most that
+    a list holds, and up to sixteen neighbouring tokens share a warp's list.  None is scanned against every row."""
+    wl = synth.Workload("crowd", 1, Hkv, Hkv, d, C * 6 + 5, C, "fixed", fixed_slots=C, r=0, S=1, seed=440 + Hkv)
+    tensors = synth.make_inputs(wl)
+    tensors["k"] = tensors["k"][:, :, torch.arange(wl.T) % C // 8 * 8].clone()
+    y_gpu, st = pu.run_gpu(wl, tensors, synth.make_layer_params(wl))
+    units = [(0, 0), (0, Hkv - 1)]
+    y_ref, o = pu.run_oracle(wl, tensors, synth.make_layer_params(wl), units=units)
+    print(pu.compare(wl, y_gpu, st, y_ref, o, units=units), st.debug_counters())
+    assert st.debug_counters()["exhaustive_tokens"] == 0
+    st.free()
