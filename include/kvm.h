@@ -287,8 +287,8 @@ kvm_status_t kvm_debug_counters(kvm_state_t* state, int64_t* out, void* cuda_str
 
 /* Failure test: in the next fold that decides on state rows, the last of the thread blocks that share unit `unit` (batch row *
  * n_kv_heads + kv head) loses the targets that it should send to the others (no effect where one block serves a unit).  Their wait
- * (shortened) runs out, kvm_state_check reports KVM_ERR_TIMEOUT, the unit keeps the rows that it had (those the fold should have
- * appended are undefined), the other units fold as ever. */
+ * (shortened) runs out, kvm_state_check reports KVM_ERR_TIMEOUT, the unit keeps the rows that it had (what the fold should
+ * have appended are rows of single tokens of the block, nothing is merged), the other units fold as ever. */
 kvm_status_t kvm_debug_drop_exchange(kvm_state_t* state, int32_t unit);
 
 /* How a decode step over n_rows rows (state and window) is cut, for tests: out[0] query heads per CTA, out[1] CTAs per

@@ -1000,10 +1000,11 @@ __global__ void __launch_bounds__(kDecideThreads, PER_SM) fold_decide_kernel(con
   }
   if (tid == 0 && rank == 0) p.nmerge[u] = C - n_a;
   if (many) asm volatile("barrier.cluster.arrive.release;" ::: "memory");
-  if (s_dead) {   // a wait ran out: whatever the unit's other CTAs publish, the apply kernel leaves the unit as it is
+  if (s_dead) {   // a wait ran out: no row of the unit has members (nmerge, behind the first CTA's store), new rows are some tokens of the block
     if (tid == 0) atomicExch(p.counters - 1, (int)KVM_ERR_TIMEOUT);
     if (many) asm volatile("barrier.cluster.wait.acquire;" ::: "memory");
-    if (tid == 0) p.nmerge[u] = -1;   // (behind the first CTA's store)
+    for (int i = tid; i < C; i += kDecideThreads) { p.creator[tokBase + i] = i; p.segnew[tokBase + i] = -1; }
+    if (tid == 0) p.nmerge[u] = -1;
     return;
   }
   if (tid == 0) {
@@ -1693,7 +1694,6 @@ __global__ void __launch_bounds__(256, 4) fold_apply_kernel(FoldApplyParams p) {
   const __half* ovU = p.ov + (int64_t)u * p.unit_stride;
   const float* ogU = p.og + (int64_t)u * p.gate_stride;
   const int nmerge = p.all_append ? 0 : p.nmerge[u];
-  if (nmerge < 0) return;   // (the unit's decisions were not completed)
   const int m = (int)p.m;
 
   // task 0: the q-th appended row; task 1: the segment of an old row whose head sits at sorted[q]
@@ -1849,7 +1849,6 @@ __global__ void __launch_bounds__(256, 2) fold_apply_rows4_kernel(FoldApplyParam
   const __half* ovU = p.ov + (int64_t)u * p.unit_stride;
   const float* ogU = p.og + (int64_t)u * p.gate_stride;
   const int nmerge = p.all_append ? 0 : s_nmerge;
-  if (nmerge < 0) return;   // (the unit's decisions were not completed)
   const int m = (int)p.m;
 
   // A warp takes groups of four row slots in turn (with few CTAs per unit the stores of one group drain
