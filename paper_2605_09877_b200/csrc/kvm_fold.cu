@@ -664,7 +664,7 @@ __global__ void __launch_bounds__(kDecideThreads, PER_SM) fold_decide_kernel(con
   auto &s_ptok = sm.ptok; auto &s_pval = sm.pval; auto &s_word = sm.word;
   int &s_dead = sm.dead, &s_nexh = sm.nexh, &s_npair = sm.npair;
 
-  const int R = gridDim.x, rank = blockIdx.x;
+  const int R = PER_SM == 2 ? 1 : (int)gridDim.x, rank = PER_SM == 2 ? 0 : (int)blockIdx.x;
   const int u = blockIdx.y, hk = u % p.Hkv;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int C = p.C, n_a = APP ? p.n_append : 0;
@@ -702,8 +702,7 @@ __global__ void __launch_bounds__(kDecideThreads, PER_SM) fold_decide_kernel(con
   // A CTA's barriers exist, and a CTA is there, from here on; it leaves when the others have, at the end.
   const bool many = R > 1;
   if (many) asm volatile("barrier.cluster.arrive.release;" ::: "memory");
-  const uint32_t spins = u == p.drop_unit ? 1u << 16 : tc::kSpinLimit;
-  auto received = [&](int bar) { decide_received(sm, bar, many, spins); };
+  auto received = [&](int bar) { decide_received(sm, bar, many, u == p.drop_unit ? 1u << 16 : tc::kSpinLimit); };
   // everything above reads parameters and writes shared memory only
   asm volatile("griddepcontrol.wait;" ::: "memory");
 
@@ -2245,22 +2244,28 @@ int launch_fold(State* st, const FoldArgs& a, cudaStream_t s) {
     p.drop_unit = st->dropUnit; st->dropUnit = -1;
     KernelTimer kt(st, 4, s);
     // CTAs per unit: about 64 in all - with 128, what shorter slices save is lost to the attention kernel beside them,
-    // which needs whole SMs (measured, 32 units: 9.0 against 8.5 ms for 32768 tokens; 8 units: no difference) -, two per
-    // unit while those fit the GPU, at least 16 tokens each
+    // which needs whole SMs (measured, 32 units: 9.0 against 8.5 ms for 32768 tokens; 8 units: no difference) -, at least 16
+    // tokens each.  Between 33 and 64 units two, where rows are appended (40 units, 8192 tokens, one and two: 2745, 2292 us; 56:
+    // 3218, 3033; 72: 5150, 5320); a fold that appends nothing has little to decide, from 32 units on for one (fixed 512
+    // rows, 4096 tokens, 32 units: 947, 976; 48 with fixed 256 rows, 8192 tokens: 1621, 1787; 64: 1350, 1396).
     int ctas = 64 / st->U;
-    if (ctas < 2 && 2 * st->U <= 148) ctas = 2;
+    if (a.n_append > 0 && ctas < 2 && st->U <= 64) ctas = 2;
+    if (a.n_append == 0 && st->U >= 32) ctas = 1;
     if (ctas > C / 16) ctas = C / 16;
     int R = 1;
     while (2 * R <= ctas && R < kDecideMaxCtas) R *= 2;
-    // programmatic dependent launch: the CTAs may start (and set up their shared memory) while the
-    // routing filter is still running; they wait for it before the first read of its output
-    // (measured off / on: 24 units with 96 query heads 2.15 / 1.84 ms for 5000 tokens, one unit 351 / 308 us for 1024,
-    // 32 units 8.77 / 8.56 ms for 32768)
+    // programmatic dependent launch: the CTAs may start (and set up their shared memory) while the routing filter is still
+    // running; they wait for it before the first read of its output.  Not from about 64 units to the number from which every
+    // kernel fills the GPU anyway: CTAs that sit waiting there keep the attention kernel, which needs whole SMs, off them.
+    // Measured off / on, 8192 tokens (fixed 512 rows: 4096): 16 units 1394 / 1348 us (square-root state), 839 / 795 (fixed 512); 32:
+    // 2049 / 2027, 979 / 947; 56: 3080 / 3033, 1200 / 1156; 64, 16384 tokens: 7130 (one CTA) / 6976 (two); 72, grouped queries: 5148 / 5295, 1972 / 2030; 96: 4635 / 4692, 1795 /
+    // 1895; 148: 6365 / 6561, 2295 / 2583; 160: 6741 / 7107, 2946 / 3017, fixed 256 4685 / 4607; 192: 7907 / 7741, 3315 / 3258.
+    const bool early = st->U < 64 + (a.n_append > 0 ? 1 : 0) || st->U > (a.n_append > 0 ? 175 : 148);
     cudaLaunchConfig_t lc = {};
     lc.gridDim = dim3(R, st->U); lc.blockDim = dim3(kDecideThreads); lc.dynamicSmemBytes = 0; lc.stream = s;
     cudaLaunchAttribute at[2];
     at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    at[0].val.programmaticStreamSerializationAllowed = st->prof_hook == nullptr && !(st->flags & KVM_FLAG_SIMT_ROUTING) ? 1 : 0;
+    at[0].val.programmaticStreamSerializationAllowed = early && st->prof_hook == nullptr && !(st->flags & KVM_FLAG_SIMT_ROUTING) ? 1 : 0;
     at[1].id = cudaLaunchAttributeClusterDimension;
     at[1].val.clusterDim.x = R; at[1].val.clusterDim.y = 1; at[1].val.clusterDim.z = 1;
     lc.attrs = at; lc.numAttrs = R > 1 ? 2 : 1;

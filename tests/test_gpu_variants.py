@@ -370,7 +370,8 @@ def _equal_keys(wl, where):
     (1, 1, 64, 256, 256 * 9 + 3, dict(growth="sqrt", sqrt_coeff=16)),      # eight CTAs per unit
     (1, 9, 128, 256, 256 * 7, dict(growth="sqrt", sqrt_coeff=20)),         # four
     (1, 1, 128, 128, 128 * 12, dict(growth="fixed", fixed_slots=300)),     # eight, nothing appended
-    (2, 20, 64, 64, 64 * 9 + 1, dict(growth="fixed", fixed_slots=150)),    # two, nothing appended
+    (1, 20, 64, 64, 64 * 9 + 1, dict(growth="fixed", fixed_slots=150)),    # two, nothing appended
+    (2, 20, 64, 64, 64 * 9 + 1, dict(growth="fixed", fixed_slots=150)),    # one, nothing appended
     (2, 20, 64, 256, 256 * 6, dict(growth="sqrt", sqrt_coeff=16)),         # two
     (4, 25, 64, 256, 256 * 6, dict(growth="sqrt", sqrt_coeff=16)),         # one CTA per unit
     (10, 16, 64, 128, 128 * 8, dict(growth="fixed", fixed_slots=128)),     # more units than SMs, nothing appended
