@@ -7,8 +7,8 @@
 // What bounds it: with many heads HBM (K_hat, V_hat and the window are read once); with few the
 // latency of launch, first loads and merge, and on the host the launch itself, which is why the rotation of the
 // token and the merge are not kernels of their own: 32 heads over 256 + window rows took 1.9 + 7.4 + 3.1 us
-// in three kernels and 18.5 us per step on the host's side; now 9.5 us per step.  64 x 32 heads over 4096 + window
-// rows: 763 -> 716 us per step (6.57 TB/s), the set-up of a step under the tail of the one before.
+// in three kernels and 18.5 us per step on the host's side; now 7.0 us per step.  64 x 32 heads over 4096 + window
+// rows: 763 -> 695 us per step with its share of the block's fold, the set-up of a step under the tail of the one before.
 #include <cooperative_groups.h>
 
 #include <utility>

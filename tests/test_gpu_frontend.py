@@ -86,7 +86,7 @@ def test_fused_qk_layernorm_equals_standalone_kernel_then_plain_calls(d, r, C):
 
 @pytest.mark.parametrize("G", [2, 8])
 def test_decode_grouped_queries_share_a_cta(G):
-    """G query heads per kv head: the decode kernel serves the whole group from one pass over the rows."""
+    """G query heads per kv head: the decode kernel serves a whole group, or four heads of it, from one pass over the rows."""
     wl = synth.Workload("gq", 2, 2 * G, 2, 64 if G == 8 else 128, 300 + 70, 64, "sqrt", sqrt_coeff=7, r=16, seed=63 + G)
     params = synth.make_layer_params(wl, trivial=False)
     tensors = synth.make_inputs(wl)

@@ -2,7 +2,7 @@
 still selects it, against the fp64 oracle on sampled (batch, head) units (units are independent end to
 end, so the oracle run on a unit alone is that unit's exact reference):
 
-  * the fold-decision kernel built for grids of more than 148 CTAs (two CTAs per SM, 64 registers);
+  * the fold-decision kernels of states with more units than SMs;
   * the decode kernel's direct-output branch (one row split per head) at head_dim 128, with and without
     grouped queries;
   * config 5's structure at a batch wide enough to select the kernels that the full batch selects;
@@ -34,26 +34,31 @@ def _sampled(wl, units, params=None, gate=False, decode_from=None, flags=0):
 
 
 def test_fold_decide_two_ctas_per_sm_variant_head_dim_128():
-    """160 units x block 256 at head_dim 128: one decision CTA per unit, 160 > 148 CTAs, so the 64-register
-    build runs (the one every many-unit shape uses); gates and affine LayerNorm included."""
+    """160 units x block 256 at head_dim 128, more units than SMs: folds that append rows take the bounds-first decision
+    kernel (its 128-register build, two CTAs per SM); gates and affine LayerNorm included."""
     wl = synth.Workload("t", 1, 160, 160, 128, 4 * 256 + 70, 256, "sqrt", sqrt_coeff=14, r=32, seed=31, kind="mixture")
     params = synth.make_layer_params(wl, trivial=False)
     print(_sampled(wl, [(0, 0), (0, 37), (0, 101), (0, 148), (0, 159)], params=params, gate=True))
 
 
 def test_decode_direct_output_branch_head_dim_128():
-    """640 query heads need no row split (nsplit == 1): the decode kernel writes its output directly.
-    40 steps from position 1004 cross the block boundary at 1024, so one of them folds."""
-    wl = synth.Workload("t", 20, 32, 32, 128, 1004 + 40, 256, "sqrt", r=0, seed=32)
-    print(_sampled(wl, [(0, 0), (7, 13), (19, 31)], decode_from=1004))
+    """416 query heads need no row split: the decode kernel writes its output directly.  40 steps from position 1004
+    cross the block boundary at 1024, so one of them folds."""
+    from paper_2605_09877_b200 import kvm
+    wl = synth.Workload("t", 13, 32, 32, 128, 1004 + 40, 256, "sqrt", r=0, seed=32)
+    assert {kvm.decode_plan(13, 32, 32, 128, _decode_rows(wl, t)) for t in range(1004, wl.T)} == {(1, 1, 1)}
+    print(_sampled(wl, [(0, 0), (7, 13), (12, 31)], decode_from=1004))
 
 
 def test_decode_grouped_queries_direct_and_split():
     """Four query heads per kv head: 640 query heads (direct output) and 8 query heads (row splits)."""
+    from paper_2605_09877_b200 import kvm
     wl = synth.Workload("t", 5, 128, 32, 128, 500 + 30, 128, "sqrt", r=32, seed=33)
+    assert {kvm.decode_plan(5, 128, 32, 128, _decode_rows(wl, t)) for t in range(500, wl.T)} == {(4, 1, 1)}
     params = synth.make_layer_params(wl, trivial=False)
     print(_sampled(wl, [(0, 0), (2, 17), (4, 31)], params=params, decode_from=500))
     wl = synth.Workload("t", 1, 8, 2, 128, 700 + 30, 128, "sqrt", r=32, seed=34)
+    assert all(kvm.decode_plan(1, 8, 2, 128, _decode_rows(wl, t))[1] > 1 for t in range(700, wl.T))
     print(_sampled(wl, [(0, 0), (0, 1)], decode_from=700))
 
 
