@@ -88,7 +88,7 @@ def prefill_flops(wl, T):
 
 
 # DRAM traffic (dram__bytes_read.sum + dram__bytes_write.sum) of the kernels that carry a roofline, from the ncu
-# captures summarised under profiles/ncu_full_cfg5_small_case_prefill_and_decode_kernels.md.  The captures run a
+# captures summarised under profiles/ncu_full_cfg5_small_case_prefill_kernels.md.  The captures run a
 # small case of the same kernels (256 units instead of 2048; 640 decode heads instead of 2048); both kernels read
 # every key / value row of a (batch, head) unit once per launch, so the traffic of a launch grows in proportion to
 # units x rows: the figure reported for a full-size launch is the algorithmic bytes of that launch times the
