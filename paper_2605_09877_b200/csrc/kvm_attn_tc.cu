@@ -26,6 +26,8 @@
 // results are merged by the CTA that finishes last; with many, the tiles that would make up a last,
 // less than half full wave of CTAs are each split in two, so that the wave is half as long.
 // Every mbarrier wait is bounded; on expiry the CTA records KVM_ERR_TIMEOUT and tears down.
+#include <algorithm>
+
 #include "kvm_internal.h"
 #include "tc_common.cuh"
 
@@ -567,19 +569,15 @@ int launch_attn_tc(State* st, const AttnArgs& a, cudaStream_t s) {
   if (tell && ++st->foldNo == 0) ++st->foldNo;   // (0 says nothing)
   p.fold_seen = st->foldSeen; p.fold_no = st->foldNo;
   p.out_vec = (reinterpret_cast<uintptr_t>(a.out) % 16 == 0 && a.so[0] % 8 == 0 && a.so[1] % 8 == 0 && a.so[2] % 8 == 0) ? 1 : 0;
-  // key splits when there are few query tiles: up to a quarter of the GPU (the folds of the block
-  // before run beside this kernel and are usually the longer chain; measured: a wider attention
-  // kernel only takes SMs away from them), at least two key tiles per split
+  // key splits when there are few query tiles: up to a quarter of the GPU (the folds of the block before run beside this kernel and
+  // are usually the longer chain), at least two key tiles per split; up to three quarters where a split still has nine or so, for
+  // there the attention is the longer chain (ms, a quarter and as chosen: 16 heads on 4, 65536 tokens 12.1, 8.64; 8 heads 10.4, 9.0; 16
+  // heads, 4096 rows, 32768 tokens 7.31, 5.37.  Three quarters where splits have two or three tiles: 24 heads on 8, 512 rows, 3.04, 3.24)
   const int qtiles = (a.nq + 127) / 128;
   const int ctas = qtiles * st->B * st->Hq;
-  int nsp = 1;
-  if (ctas <= kAttnSplitTiles) {
-    nsp = kAttnSplitTiles / ctas;
-    const int ntot_min = (int)((a.m + 127) / 128) + 1;
-    if (nsp > ntot_min / 2) nsp = ntot_min / 2;
-    if (nsp > kAttnMaxSplits) nsp = kAttnMaxSplits;
-    if (nsp < 1) nsp = 1;
-  }
+  const int ntot_min = (int)((a.m + 127) / 128) + 1;
+  int nsp = std::max(std::min(kAttnSplitTiles / ctas, ntot_min / 2), std::min(3 * kAttnSplitTiles / ctas, (ntot_min + 8) / 9));
+  nsp = std::max(1, std::min(nsp, kAttnMaxSplits));
   // Many tiles: when the last wave of one-CTA-per-SM would be less than half full, its tiles are split
   // in two (the partial-result buffer holds 2 * kAttnSplitTiles tiles of two splits).
   const int tiles = qtiles * st->B * st->Hq;

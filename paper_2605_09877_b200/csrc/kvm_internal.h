@@ -13,7 +13,7 @@ constexpr int kMaxBlock = 256;      // largest block C (one thread per overflow 
 constexpr int kTopK = 8;            // routing filter keeps at most K candidate rows per (token, row split)
 constexpr int kChunkCap = 16;       // 32-row chunks of approximate similarities the routing filter can record per (token, row split)
 constexpr int kMaxSplits = 32;      // routing filter split count upper bound
-constexpr int kAttnSplitTiles = 37; // launches with at most this many (batch, head, query tile) CTAs - a quarter of the GPU - are split along the keys
+constexpr int kAttnSplitTiles = 37; // a quarter of the GPU: launches of few (batch, head, query tile) CTAs are split along the keys (launch_attn_tc)
 constexpr int kAttnMaxSplits = 8;
 constexpr int kDecodeCluster = 8;   // most CTAs of a decode step that share a cluster (the portable size)
 constexpr int kDecodePartCtas = 48 * kDecodeCluster;   // most CTAs of a decode step that merge through global memory (plan_decode)

@@ -436,3 +436,10 @@ def test_crowded_runs_are_compared_pair_by_pair(Hkv, d, C):
     print(pu.compare(wl, y_gpu, st, y_ref, o, units=units), st.debug_counters())
     assert st.debug_counters()["exhaustive_tokens"] == 0
     st.free()
+
+
+@pytest.mark.parametrize("Hq,Hkv,d,blocks", [(8, 8, 128, 21), (16, 4, 128, 22), (24, 8, 64, 23), (3, 3, 128, 25)])
+def test_attention_of_few_heads_over_many_rows_splits_the_keys(Hq, Hkv, d, blocks):
+    """Key splits of launches of 6 to 48 tiles over 10 to 40 key tiles: two to eight splits, ragged last ones."""
+    wl = synth.Workload("t", 1, Hq, Hkv, d, 256 * blocks + 70, 256, "unbounded", r=32, seed=62)
+    print(_sampled(wl, [(0, 0), (0, Hkv - 1)]))
