@@ -1666,18 +1666,30 @@ struct FoldApplyParams {
 };
 
 // One touched row per warp: the shorter chain per row; used when a launch has too few rows to fill the
-// GPU, where the latency of a row is what counts.
+// GPU, where the latency of a row is what counts.  Slot q is the q-th appended row or, behind those, the row whose members
+// start at sorted[q - n_append]: a warp has one row.  What bounds it: the decisions, the row with its members, the reductions - three
+// latencies after another; so up to kApplyBatch members (cp.async into shared memory: no registers) are under way together with the
+// row's own sums, and added in their order when they are there.  (A member fetched after the one before was added, and a warp's
+// appended row before its merged one: 2 x 16 heads, 512 rows, 8192 tokens 1.947 ms, now 1.893; 32 heads on 8, 3 x 5003 tokens
+// 1.260, 1.215.  Four consecutive channels per lane - half-used sectors and bank conflicts - 1.978.)
+constexpr int kApplyBatch = 4;
+__device__ __forceinline__ void cp_async16(void* dst, const void* src) {
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(tc::smem_u32(dst)), "l"(src) : "memory");
+}
 template <int D>
 __global__ void __launch_bounds__(256, 4) fold_apply_kernel(FoldApplyParams p) {
-  constexpr int CH = D / 32;
+  constexpr int CH = D / 32;   // channels per lane: 2 lane + 64 i and the one behind
   __shared__ int s_pi[kMaxBlock], s_sorted[kMaxBlock], s_creator[kMaxBlock], s_segnew[kMaxBlock];
+  __shared__ __align__(16) double s_kb[8][kApplyBatch][D];
+  __shared__ __align__(16) __half s_v[8][kApplyBatch][D];
   // the routing filter of the next fold may start its set-up now; it waits for this grid to finish
   // before it reads the readout keys written here
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   const int u = blockIdx.y, hk = u % p.Hkv;
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, x0 = 2 * lane;
   const int q = blockIdx.x * 8 + warp;
   const int64_t tokBase = (int64_t)u * p.Cmax;
+  const int nmerge = p.all_append ? 0 : p.nmerge[u];
   if (!p.all_append) {   // the decisions of this unit, read once per CTA instead of chased per warp
     for (int i = threadIdx.x; i < p.C; i += 256) {
       s_pi[i] = p.pi[tokBase + i];
@@ -1692,106 +1704,131 @@ __global__ void __launch_bounds__(256, 4) fold_apply_kernel(FoldApplyParams p) {
   const double* kbarU = p.kbar64 + tokBase * D;
   const __half* ovU = p.ov + (int64_t)u * p.unit_stride;
   const float* ogU = p.og + (int64_t)u * p.gate_stride;
-  const int nmerge = p.all_append ? 0 : p.nmerge[u];
   const int m = (int)p.m;
 
-  // task 0: the q-th appended row; task 1: the segment of an old row whose head sits at sorted[q]
-  for (int task = 0; task < 2; ++task) {
-    int rowi, seg, jc = -1;
-    if (task == 0) {
-      if (q >= p.n_append) continue;
-      rowi = m + q;
-      jc = p.all_append ? q : s_creator[q];
-      seg = p.all_append ? -1 : s_segnew[q];
-    } else {
-      if (q >= nmerge) continue;
-      const int j0 = s_sorted[q];
-      rowi = s_pi[j0];
-      if (rowi >= m) continue;                                 // new rows are task 0
-      if (q > 0 && s_pi[s_sorted[q - 1]] == rowi) continue;    // not a head
-      seg = q;
+  const bool fresh = q < p.n_append;
+  int rowi, seg, jc = -1;
+  if (fresh) {
+    rowi = m + q;
+    jc = p.all_append ? q : s_creator[q];
+    seg = p.all_append ? -1 : s_segnew[q];
+  } else {
+    seg = q - p.n_append;
+    if (seg >= nmerge) return;
+    rowi = s_pi[s_sorted[seg]];
+    if (rowi >= m || (seg > 0 && s_pi[s_sorted[seg - 1]] == rowi)) return;   // an appended row's member, or not a head
+  }
+  int nmem = 0;   // members of the row: a run of `sorted`
+  for (int b = seg; seg >= 0; b += 32) {
+    const unsigned same = __ballot_sync(0xffffffffu, b + lane < nmerge && s_pi[s_sorted[min(b + lane, p.C - 1)]] == rowi);
+    nmem += same == 0xffffffffu ? 32 : __ffs(~same) - 1;
+    if (same != 0xffffffffu) break;
+  }
+  const int64_t row = rowBase + rowi;
+  double kx[CH];
+  float vx[CH];
+  double wacc = 1.0, rad = 0.0;
+  int nacc = 1;
+  const double2* k2 = reinterpret_cast<const double2*>(fresh ? kbarU + (int64_t)jc * D + x0 : p.sumK + row * D + x0);
+#pragma unroll
+  for (int i = 0; i < CH / 2; ++i) {
+    const double2 k = k2[32 * i];
+    kx[2 * i] = k.x; kx[2 * i + 1] = k.y;
+  }
+  if (fresh) {
+    const __half2* vr = reinterpret_cast<const __half2*>(ovU + (int64_t)jc * D + x0);
+#pragma unroll
+    for (int i = 0; i < CH / 2; ++i) {
+      const float2 v = __half22float2(vr[32 * i]);
+      vx[2 * i] = v.x; vx[2 * i + 1] = v.y;
     }
-    const int64_t row = rowBase + rowi;
-    double kx[CH];
-    float vx[CH];
-    double wacc, rad;
-    int nacc;
-    if (task == 0) {
-      const double* kb = kbarU + (int64_t)jc * D;
-      const __half* vr = ovU + (int64_t)jc * D;
-      double v2 = 0.0;
+  } else {
+    const float2* vr = reinterpret_cast<const float2*>(p.sumV + row * D + x0);
 #pragma unroll
-      for (int i = 0; i < CH; ++i) {
-        const int x = lane + 32 * i;
-        kx[i] = kb[x];
-        vx[i] = __half2float(vr[x]);
-        v2 += (double)vx[i] * (double)vx[i];
-      }
-      rad = (double)(float)sqrt(warp_sum_d(v2));   // the radius is kept in fp32
-      wacc = 1.0;
-      nacc = 1;
-      if (lane == 0 && p.slotTok && p.b + jc < p.Tassign) {
-        p.slotTok[(int64_t)u * p.Tassign + p.b + jc] = rowi;
-        p.appTok[(int64_t)u * p.Tassign + p.b + jc] = 1;
-      }
-    } else {
-#pragma unroll
-      for (int i = 0; i < CH; ++i) {
-        const int x = lane + 32 * i;
-        kx[i] = p.sumK[row * D + x];
-        vx[i] = p.sumV[row * D + x];
-      }
-      wacc = p.wsum[row];
-      nacc = p.cnt[row];
-      rad = (double)p.rho[row];
+    for (int i = 0; i < CH / 2; ++i) {
+      const float2 v = vr[32 * i];
+      vx[2 * i] = v.x; vx[2 * i + 1] = v.y;
     }
-    if (seg >= 0) {
-      for (int qq = seg; qq < nmerge; ++qq) {
-        const int j = s_sorted[qq];
-        if (s_pi[j] != rowi) break;
-        const float g = ogU[j];
-        const double* kb = kbarU + (int64_t)j * D;
-        const __half* vr = ovU + (int64_t)j * D;
-#pragma unroll
-        for (int i = 0; i < CH; ++i) {
-          const int x = lane + 32 * i;
-          kx[i] += (double)g * kb[x];
-          vx[i] = fmaf(g, __half2float(vr[x]), vx[i]);
-        }
-        wacc += (double)g;
-        nacc += 1;
-        if (lane == 0 && p.slotTok && p.b + j < p.Tassign) {
-          p.slotTok[(int64_t)u * p.Tassign + p.b + j] = rowi;
-          p.appTok[(int64_t)u * p.Tassign + p.b + j] = 0;
-        }
+    wacc = p.wsum[row];
+    nacc = p.cnt[row];
+    rad = (double)p.rho[row];
+  }
+  float g = 0.f;   // lane t: gate of the batch's member t
+  auto fetch = [&](int k0) {
+    const int n = min(kApplyBatch, nmem - k0);
+    int j = 0;
+    if (lane < n) {
+      j = s_sorted[seg + k0 + lane];
+      g = ogU[j];
+      if (p.slotTok && p.b + j < p.Tassign) {
+        p.slotTok[(int64_t)u * p.Tassign + p.b + j] = rowi;
+        p.appTok[(int64_t)u * p.Tassign + p.b + j] = 0;
       }
     }
-    double mu, rs;
-    row_stats<CH>(kx, D, p.ln_eps, mu, rs);
+    for (int t = 0; t < n; ++t) {
+      const int jt = __shfl_sync(0xffffffffu, j, t);
+      for (int e = lane; e < D / 2; e += 32) cp_async16(&s_kb[warp][t][2 * e], kbarU + (int64_t)jt * D + 2 * e);
+      if (lane < D / 8) cp_async16(&s_v[warp][t][8 * lane], ovU + (int64_t)jt * D + 8 * lane);
+    }
+  };
+  fetch(0);
+  if (fresh) {   // the radius is the norm of the creator's value, kept in fp32
     double v2 = 0.0;
 #pragma unroll
     for (int i = 0; i < CH; ++i) v2 += (double)vx[i] * (double)vx[i];
-    const double vnorm = sqrt(warp_sum_d(v2));
-    const double den = vnorm > p.norm_eps ? vnorm : p.norm_eps;
-    // one fp64 divide per row instead of one per channel (the readout values are rounded to fp16)
-    const double vscale = p.radius_on ? rad / den : 1.0 / wacc;
+    rad = (double)(float)sqrt(warp_sum_d(v2));
+    if (lane == 0 && p.slotTok && p.b + jc < p.Tassign) {
+      p.slotTok[(int64_t)u * p.Tassign + p.b + jc] = rowi;
+      p.appTok[(int64_t)u * p.Tassign + p.b + jc] = 1;
+    }
+  }
+  for (int k0 = 0; k0 < nmem; k0 += kApplyBatch) {
+    asm volatile("cp.async.wait_all;" ::: "memory");
+    __syncwarp();
+    for (int t = 0; t < min(kApplyBatch, nmem - k0); ++t) {   // ascending tokens
+      const float gt = __shfl_sync(0xffffffffu, g, t);
 #pragma unroll
-    for (int i = 0; i < CH; ++i) {
-      const int x = lane + 32 * i;
-      const double hat = (double)p.ln_w[hk * D + x] * ((kx[i] - mu) * rs) + (double)p.ln_b[hk * D + x];
-      p.sumK[row * D + x] = kx[i];
-      p.sumV[row * D + x] = vx[i];
-      p.Khat[row * D + x] = __float2half_rn((float)hat);
-      const double vo = (double)vx[i] * vscale;
-      p.Vhat[row * D + x] = __float2half_rn((float)vo);
+      for (int i = 0; i < CH; ++i) {
+        const int x = x0 + 64 * (i >> 1) + (i & 1);
+        kx[i] += (double)gt * s_kb[warp][t][x];
+        vx[i] = fmaf(gt, __half2float(s_v[warp][t][x]), vx[i]);
+      }
+      wacc += (double)gt;
     }
-    if (lane == 0) {
-      p.rho[row] = (float)rad;
-      p.wsum[row] = wacc;
-      p.cnt[row] = nacc;
-      p.kmu[row] = mu;
-      p.krstd[row] = rs;
-    }
+    __syncwarp();
+    if (k0 + kApplyBatch < nmem) fetch(k0 + kApplyBatch);
+  }
+  nacc += nmem;
+  double mu, rs;
+  row_stats<CH>(kx, D, p.ln_eps, mu, rs);
+  double v2 = 0.0;
+#pragma unroll
+  for (int i = 0; i < CH; ++i) v2 += (double)vx[i] * (double)vx[i];
+  const double vnorm = sqrt(warp_sum_d(v2));
+  const double den = vnorm > p.norm_eps ? vnorm : p.norm_eps;
+  // one fp64 divide per row instead of one per channel (the readout values are rounded to fp16)
+  const double vscale = p.radius_on ? rad / den : 1.0 / wacc;
+  __half2 kh[CH / 2], vh[CH / 2];
+#pragma unroll
+  for (int i = 0; i < CH / 2; ++i) {
+    const float2 w = *reinterpret_cast<const float2*>(p.ln_w + hk * D + x0 + 64 * i), c = *reinterpret_cast<const float2*>(p.ln_b + hk * D + x0 + 64 * i);
+    const double h0 = (double)w.x * ((kx[2 * i] - mu) * rs) + (double)c.x, h1 = (double)w.y * ((kx[2 * i + 1] - mu) * rs) + (double)c.y;
+    kh[i] = __halves2half2(__float2half_rn((float)h0), __float2half_rn((float)h1));
+    vh[i] = __halves2half2(__float2half_rn((float)((double)vx[2 * i] * vscale)), __float2half_rn((float)((double)vx[2 * i + 1] * vscale)));
+    reinterpret_cast<double2*>(p.sumK + row * D + x0)[32 * i] = make_double2(kx[2 * i], kx[2 * i + 1]);
+    reinterpret_cast<float2*>(p.sumV + row * D + x0)[32 * i] = make_float2(vx[2 * i], vx[2 * i + 1]);
+  }
+#pragma unroll
+  for (int i = 0; i < CH / 2; ++i) {
+    reinterpret_cast<__half2*>(p.Khat + row * D + x0)[32 * i] = kh[i];
+    reinterpret_cast<__half2*>(p.Vhat + row * D + x0)[32 * i] = vh[i];
+  }
+  if (lane == 0) {
+    p.rho[row] = (float)rad;
+    p.wsum[row] = wacc;
+    p.cnt[row] = nacc;
+    p.kmu[row] = mu;
+    p.krstd[row] = rs;
   }
 }
 
@@ -1852,28 +1889,24 @@ __global__ void __launch_bounds__(256, 2) fold_apply_rows4_kernel(FoldApplyParam
 
   // A warp takes groups of four row slots in turn (with few CTAs per unit the stores of one group drain
   // while the next group's rows are fetched, and the decisions are read once for more work).
-  // task 0: the q-th appended row; task 1: the segment of an old row whose head sits at sorted[q]
-  for (int qg = blockIdx.x * 8 + warp; qg * kApplyRowsPerWarp < p.C; qg += gridDim.x * 8)
-  for (int task = 0; task < 2; ++task) {
+  // Slot q: the q-th appended row (fresh) or, behind those, the segment of an old row whose head sits at sorted[q - n_append].
+  for (int qg = blockIdx.x * 8 + warp; qg * kApplyRowsPerWarp < p.C; qg += gridDim.x * 8) {
     const int q = qg * kApplyRowsPerWarp + (lane >> 3);
+    const bool fresh = q < p.n_append;
     bool act = q < p.C;
     int rowi = 0, seg = -1, jc = -1;
     if (act) {
-      if (task == 0) {
-        if (q >= p.n_append) act = false;
-        else {
-          rowi = m + q;
-          jc = p.all_append ? q : s_creator[q];
-          seg = p.all_append ? -1 : s_segnew[q];
-        }
+      if (fresh) {
+        rowi = m + q;
+        jc = p.all_append ? q : s_creator[q];
+        seg = p.all_append ? -1 : s_segnew[q];
       } else {
-        if (q >= nmerge) act = false;
+        seg = q - p.n_append;
+        if (seg >= nmerge) act = false;
         else {
-          const int j0 = s_sorted[q];
-          rowi = s_pi[j0];
-          if (rowi >= m) act = false;                                          // new rows are task 0
-          else if (q > 0 && s_pi[s_sorted[q - 1]] == rowi) act = false;        // not a head
-          seg = q;
+          rowi = s_pi[s_sorted[seg]];
+          if (rowi >= m) act = false;                                                // a new row's member
+          else if (seg > 0 && s_pi[s_sorted[seg - 1]] == rowi) act = false;          // not a head
         }
       }
     }
@@ -1886,7 +1919,7 @@ __global__ void __launch_bounds__(256, 2) fold_apply_rows4_kernel(FoldApplyParam
 #pragma unroll
     for (int c = 0; c < NC; ++c) { kx[c] = 0.0; vx[c] = 0.f; }
     if (act) {
-      if (task == 0) {
+      if (fresh) {
         const __half* vr = ovU + (int64_t)jc * D;
 #pragma unroll
         for (int i = 0; i < NI; ++i) {
@@ -1923,7 +1956,7 @@ __global__ void __launch_bounds__(256, 2) fold_apply_rows4_kernel(FoldApplyParam
     }
     // radius of a new row = the norm of its creator's value, kept in fp32 (all lanes: group reduction)
     v2 = group8_sum_d(v2);
-    if (task == 0) rad = (double)(float)sqrt(v2);
+    if (fresh) rad = (double)(float)sqrt(v2);
     if (act && seg >= 0) {
       for (int qq = seg; qq < nmerge; ++qq) {
         const int j = s_sorted[qq];
@@ -2073,8 +2106,8 @@ __global__ void __launch_bounds__(256) refresh_rows_kernel(RefreshParams p) {
     float vx[CH];
 #pragma unroll
     for (int i = 0; i < CH; ++i) {
-      kx[i] = p.sumK[row * D + lane + 32 * i];
-      vx[i] = p.sumV[row * D + lane + 32 * i];
+      kx[i] = p.sumK[row * D + 2 * lane + 64 * (i >> 1) + (i & 1)];
+      vx[i] = p.sumV[row * D + 2 * lane + 64 * (i >> 1) + (i & 1)];
     }
     const double wacc = p.wsum[row], rad = (double)p.rho[row];
     double mu, rs;
@@ -2087,7 +2120,7 @@ __global__ void __launch_bounds__(256) refresh_rows_kernel(RefreshParams p) {
     const double vscale = p.radius_on ? rad / den : 1.0 / wacc;
 #pragma unroll
     for (int i = 0; i < CH; ++i) {
-      const int x = lane + 32 * i;
+      const int x = 2 * lane + 64 * (i >> 1) + (i & 1);
       const double hat = (double)p.ln_w[hk * D + x] * ((kx[i] - mu) * rs) + (double)p.ln_b[hk * D + x];
       const __half kh = __float2half_rn((float)hat);
       const __half vh = __float2half_rn((float)((double)vx[i] * vscale));
@@ -2098,10 +2131,18 @@ __global__ void __launch_bounds__(256) refresh_rows_kernel(RefreshParams p) {
   }
 }
 
-// which apply kernel the folds of this state run (fixed per state and block): four rows per warp when
-// the launch is bound by throughput (measured: better from 8192 rows on: U = 32, C = 256; worse at
-// 4096 and 2048 rows, where the longer chain per row shows)
-static bool apply_uses_rows4(const State* st) { return (int64_t)st->C * st->U >= 8192; }
+// Which apply kernel the folds of this state run (fixed per state and block).  Four rows per warp where the keys are recomputed and
+// otherwise only for blocks of more than 128 tokens of a middling number of units.  Measured (ms, 24 blocks; one row per warp, four):
+// 128 channels, blocks of 256, square-root state: 64 units 2.19, 2.30; 72 2.50, 2.42; 96 3.49, 3.33; 128 3.86, 4.02; 148 4.59, 4.56;
+// 160 4.74, 4.87; 192 5.22, 5.58; 512 rows: 64 units 1.50, 1.55; 96 2.14, 2.20; 128 2.49, 2.61; 160 3.19, 3.60.  64 channels, 256
+// rows: 48 units 1.21, 1.25; 64 1.25, 1.18; 148 2.04, 1.86; 224 2.98, 2.80 (with four CTAs per unit).  Blocks of 64 and 128, 64 to 224
+// units: one row per warp is up to 12 % faster, nowhere more than 1 % slower.
+static bool apply_uses_rows4(const State* st) {
+  if (st->recomputeK) return true;
+  if (st->C <= 128) return false;
+  if (st->d == 64) return (int64_t)st->C * st->U > 12288;
+  return (int64_t)st->C * st->U > 16384 && st->U < 128;
+}
 
 int launch_refresh_rows(State* st, int64_t m, cudaStream_t s) {
   if (m <= 0) return 0;
@@ -2300,8 +2341,9 @@ int launch_fold(State* st, const FoldArgs& a, cudaStream_t s) {
   KernelTimer kt(st, 5, s);
   if (apply_uses_rows4(st)) {
     // CTAs per unit: one when the units alone fill the GPU's CTA slots (measured at 256 and 2048 units: 1 beats
-    // 2, 4 and 8), else enough to fill them, at most one per 32 row slots
-    const int R = std::max(1, std::min(2 * 148 / st->U, (C + kApplyRowsPerCta - 1) / kApplyRowsPerCta));
+    // 2, 4 and 8), four where they nearly do (64 channels, 256 rows, one and four: 160 units 2.28, 2.12 ms; 192 2.59, 2.46; 224
+    // 2.85, 2.80), else enough to fill them; at most one per 32 row slots
+    const int R = std::max(1, std::min(st->U > 148 && !st->recomputeK ? 4 : 2 * 148 / st->U, (C + kApplyRowsPerCta - 1) / kApplyRowsPerCta));
     dim3 grid(R, st->U);
     if (D == 128) { if (st->recomputeK) fold_apply_rows4_kernel<128, true><<<grid, 256, 0, s>>>(q); else fold_apply_rows4_kernel<128, false><<<grid, 256, 0, s>>>(q); }
     else { if (st->recomputeK) fold_apply_rows4_kernel<64, true><<<grid, 256, 0, s>>>(q); else fold_apply_rows4_kernel<64, false><<<grid, 256, 0, s>>>(q); }

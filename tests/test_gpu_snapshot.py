@@ -31,7 +31,7 @@ SERIAL = 1 << 5   # KVM_FLAG_SERIAL_FOLDS
     (synth.Workload("snapA", 2, 4, 2, 128, 256 * 6 + 90, 256, "sqrt", sqrt_coeff=10, r=32, seed=41), 256 * 3 + 77, False, True, 0),
     (synth.Workload("snapB", 1, 3, 3, 64, 64 * 20 + 5, 64, "fixed", fixed_slots=200, r=0, seed=42, kind="mixture"), 64 * 9, True, False, 0),
     (synth.Workload("snapC", 1, 2, 2, 64, 300, 32, "sqrt", sqrt_coeff=6, r=16, seed=43, w=3), 17, True, False, 0),   # cut before any fold
-    (synth.Workload("snapD", 1, 40, 40, 128, 256 * 5 + 33, 256, "sqrt", r=0, seed=44), 256 * 4 + 1, True, False, 0),  # four-rows-per-warp apply
+    (synth.Workload("snapD", 1, 40, 40, 128, 256 * 5 + 33, 256, "sqrt", r=0, seed=44), 256 * 4 + 1, True, False, 0),
     # one readout copy, folds on the caller's stream
     (synth.Workload("snapF", 1, 4, 2, 128, 128 * 9 + 60, 128, "sqrt", sqrt_coeff=5, r=32, seed=46), 128 * 4 + 9, False, True, SERIAL),
     # the same with 64 units x block 128: no fp64 memory keys are kept, the import rebuilds the per-row statistics

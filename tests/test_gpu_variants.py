@@ -438,6 +438,25 @@ def test_crowded_runs_are_compared_pair_by_pair(Hkv, d, C):
     st.free()
 
 
+@pytest.mark.parametrize("B,Hkv,d,C,slots,rows4", [
+    (1, 3, 128, 256, 64, False),    # one row per warp: four members a row on average, many rows with more than a batch of four
+    (1, 2, 64, 200, 24, False),
+    (2, 9, 128, 64, 1, False),      # every token of a block joins one of the 64 rows of the first fold
+    (3, 24, 128, 256, 300, True),   # four rows per warp with stored memory keys
+    (2, 25, 64, 256, 256, True),
+    (5, 32, 64, 192, 64, True),     # (four CTAs per unit)
+])
+def test_rows_with_many_members_in_both_apply_kernels(B, Hkv, d, C, slots, rows4):
+    """The kernel that a state's folds run to write the touched rows, at rows with none, one and many members, appended rows
+    among them; the state means and readout rows against the oracle, and again after a snapshot's import."""
+    assert rows4 == (C > 128 and C * B * Hkv > (12288 if d == 64 else 16384) and (d == 64 or B * Hkv < 128))
+    wl = synth.Workload("t", B, Hkv, Hkv, d, C * 5 + 11, C, "fixed", fixed_slots=slots, r=32, seed=61, kind="mixture")
+    params = synth.make_layer_params(wl, trivial=False)
+    units = sorted({(0, 0), (B - 1, Hkv - 1)})
+    stats = _sampled(wl, units, params=params, gate=True)
+    print(stats)
+
+
 @pytest.mark.parametrize("Hq,Hkv,d,blocks", [(8, 8, 128, 21), (16, 4, 128, 22), (24, 8, 64, 23), (3, 3, 128, 25)])
 def test_attention_of_few_heads_over_many_rows_splits_the_keys(Hq, Hkv, d, blocks):
     """Key splits of launches of 6 to 48 tiles over 10 to 40 key tiles: two to eight splits, ragged last ones."""
