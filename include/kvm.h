@@ -291,7 +291,8 @@ kvm_status_t kvm_debug_counters(kvm_state_t* state, int64_t* out, void* cuda_str
  * have appended are rows of single tokens of the block, nothing is merged), the other units fold as ever. */
 kvm_status_t kvm_debug_drop_exchange(kvm_state_t* state, int32_t unit);
 
-/* How a decode step over n_rows rows (state and window) is cut, for tests: out[0] query heads per CTA, out[1] CTAs per
+/* How a decode step over n_rows rows (state and window) is cut where it runs the kernel that loops over them (few heads over few
+ * rows are cut otherwise, unless the timing hook is on), for tests: out[0] query heads per CTA, out[1] CTAs per
  * cluster (row splits merged through shared memory), out[2] clusters per group of heads (merged through global memory).
  * Host arithmetic only. */
 kvm_status_t kvm_debug_decode_plan(int32_t batch, int32_t n_q_heads, int32_t n_kv_heads, int32_t head_dim, int64_t n_rows,

@@ -380,6 +380,7 @@ KVM_API kvm_status_t kvm_state_create(const kvm_config_t* cfg, kvm_state_t** out
   A(s.attnPart, (size_t)kAttnSplitTiles * kAttnMaxSplits * (d + 2) * 128); A(s.attnCnt, (size_t)2 * kAttnSplitTiles);
   if (rc == KVM_OK && cudaMemset(s.attnCnt, 0, 2 * kAttnSplitTiles * sizeof(int32_t)) != cudaSuccess) rc = KVM_ERR_CUDA;
   A(s.foldSeen, (size_t)1);
+  A(s.decSeen, (size_t)1); s.decNo = s.decBase = 1;   // (0 says nothing)
   A(s.decPart, (size_t)kDecodePartCtas * (d + 2)); A(s.decTicket, (size_t)kDecodePartCtas);
   A(s.status, (size_t)16);   // [0] status word, [1..3] fold debug counters
   if (s.Tassign > 0) { A(s.slotTok, U * (size_t)s.Tassign); A(s.appTok, U * (size_t)s.Tassign); }
@@ -441,7 +442,7 @@ KVM_API kvm_status_t kvm_debug_counters(kvm_state_t* ks, int64_t* out, void* cud
 KVM_API kvm_status_t kvm_state_reset(kvm_state_t* ks) {
   if (!ks) return KVM_ERR_INVALID_ARG;
   State& s = ks->s;
-  s.bound = false; s.pos = 0; s.m = 0; s.nfolds = 0; s.prevValid = false;
+  s.bound = false; s.pos = 0; s.m = 0; s.decBase = s.decNo; s.nfolds = 0; s.prevValid = false;
   if (s.slotTok) s.assignDirty = true;   // debug recording only: the next prefill forgets the old assignments, on its stream
   return KVM_OK;
 }
@@ -687,6 +688,7 @@ KVM_API kvm_status_t kvm_prefill(const void* q, const void* k, const void* v, kv
   }
   if (ovf && fold_pending >= 0) ev_ok = ev_ok && cudaStreamWaitEvent(stream, s.evFold[fold_pending], 0) == cudaSuccess;
   s.pos = pos1;
+  s.decBase = s.decNo;
   if (!ev_ok) { cudaGetLastError(); return KVM_ERR_CUDA; }
   return launch_ok() ? KVM_OK : KVM_ERR_CUDA;
 }
@@ -729,6 +731,7 @@ KVM_API kvm_status_t kvm_decode_step(const void* q, const void* k, const void* v
     s.launches += launch_fold(&s, fa, stream);
     s.m += n_a;
     s.nfolds += 1;
+    s.decBase = s.decNo;
   }
   s.pos = t + 1;
   return launch_ok() ? KVM_OK : KVM_ERR_CUDA;
@@ -928,7 +931,7 @@ KVM_API kvm_status_t kvm_state_import(kvm_state_t* ks, const kvm_snapshot_info_t
 
   kvm_state_reset(ks);
   bind_state(s, C, info->growth, r);
-  s.pos = info->position; s.m = info->n_slots; s.nfolds = info->n_folds;
+  s.pos = info->position; s.m = info->n_slots; s.nfolds = info->n_folds; s.decBase = s.decNo;
   const size_t m = (size_t)s.m, M = (size_t)s.Mcap, d = (size_t)s.d, U = (size_t)s.U;
   bool ok = true;
   if (m > 0) {

@@ -11,10 +11,13 @@
 // rows: 763 -> 695 us per step with its share of the block's fold, the set-up of a step under the tail of the one before.
 #include <cooperative_groups.h>
 
+#include <algorithm>
+
 #include <utility>
 
 #include "kvm_internal.h"
 #include "ln_rows.cuh"
+#include "tc_common.cuh"
 
 namespace kvm {
 
@@ -42,6 +45,10 @@ struct DecodeParams {
   int nclus;             // clusters of nsplit CTAs per group of heads
   float* part;           // (nclus > 1) merged results of the clusters, [CTA group][rank][cluster][share + 2]
   int32_t* ticket;       // (nclus > 1) [CTA group][rank], zero between launches
+  uint32_t *seen;        // (short steps) the step that has last met the end of the one before it, by its number
+  uint32_t no, base;     // number of this step, and of the first one since a kernel other than a step wrote rows or window slots
+  int rpw;               // (short steps) rows per warp
+  int32_t* status;
   float qk_ln_eps;
 };
 
@@ -66,9 +73,9 @@ __device__ __forceinline__ uint4 ldg_stream(const void* p) {
 // (the CTA's rows end with the new token), its rotated key and its value into s_new; the first query head's CTA of a
 // kv group (`store`) also writes them to the window ring, and `count_q` says which CTA of a head counts the inputs that
 // had to be clamped to the fp16 range.  Plain rows: one thread per channel.
-template <int D, int GQ>
+template <int D, int GQ, typename F>
 __device__ __forceinline__ void new_token(const DecodeParams& p, int bh0, int64_t u, bool fresh, bool store, bool count_q,
-                                          __half (*s_q)[D], __half (*s_new)[D]) {
+                                          __half (*s_q)[D], __half (*s_new)[D], F&& behind_wait) {
   const int x = threadIdx.x % D;
   const int half = p.r >> 1;
   float cs = 1.f, sn = 0.f;
@@ -82,6 +89,7 @@ __device__ __forceinline__ void new_token(const DecodeParams& p, int bh0, int64_
   }
   // (the step before this one, or whatever wrote the inputs and the rows, may still be running up to here)
   asm volatile("griddepcontrol.wait;" ::: "memory");
+  behind_wait();
   int nsat = 0;
   for (int i = threadIdx.x / D; i < GQ + (fresh ? 1 : 0); i += 256 / D) {
     const bool isq = i < GQ;
@@ -110,9 +118,9 @@ __device__ __forceinline__ void new_token(const DecodeParams& p, int bh0, int64_
 // The same with LN_q / LN_k applied first (fused front end): one warp per row, d / 8 lanes hold it as eight channels
 // each (ln_chunk8: the arithmetic of kvm_head_layernorm), the other lane groups compute copies and store nothing.
 // The partner channel of the rotation comes from the lane that holds it.
-template <int D, int GQ>
+template <int D, int GQ, typename F>
 __device__ __forceinline__ void new_token_ln(const DecodeParams& p, int bh0, int64_t u, bool fresh, bool store, bool count_q,
-                                             __half (*s_q)[D], __half (*s_new)[D]) {
+                                             __half (*s_q)[D], __half (*s_new)[D], F&& behind_wait) {
   constexpr int LPR = D / 8;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, sub = lane % LPR;
   const int half = p.r >> 1, ch0 = sub * 8;
@@ -129,6 +137,7 @@ __device__ __forceinline__ void new_token_ln(const DecodeParams& p, int bh0, int
     }
   }
   asm volatile("griddepcontrol.wait;" ::: "memory");
+  behind_wait();
   int nsat = 0;
   for (int row_i = warp; row_i < GQ + (fresh ? 1 : 0); row_i += 8) {   // (uniform over the warp)
     const bool isq = row_i < GQ;
@@ -236,8 +245,8 @@ __global__ void __launch_bounds__(256) decode_step_kernel(DecodeParams p) {
   const int r1 = min(n, r0 + per);
   const bool fresh = r0 < n && r1 == n;          // this CTA's rows end with the new token
 
-  if (LN) new_token_ln<D, GQ>(p, bh0, u, fresh, fresh && hq0 % p.G == 0, split == 0, s_q, s_new);
-  else new_token<D, GQ>(p, bh0, u, fresh, fresh && hq0 % p.G == 0, split == 0, s_q, s_new);
+  if (LN) new_token_ln<D, GQ>(p, bh0, u, fresh, fresh && hq0 % p.G == 0, split == 0, s_q, s_new, [] {});
+  else new_token<D, GQ>(p, bh0, u, fresh, fresh && hq0 % p.G == 0, split == 0, s_q, s_new, [] {});
   if (fresh && hq0 % p.G == 0 && tid == 0) p.ringG[u * p.ringCap + p.slot_t] = p.gate ? p.gate[u] : 1.0f;
   __syncthreads();
 
@@ -477,6 +486,240 @@ __global__ void __launch_bounds__(256) decode_step_kernel(DecodeParams p) {
   }
 }
 
+// A step over few rows (a warp has at most 8 * RPW of them): bound by latencies, so what does not depend on the kernel before it is
+// done under that one's tail.  The rows are fetched before griddepcontrol.wait as far as they are known to be complete: a step
+// that has waited for everything before it stores its number with release, a later one that reads it with acquire may read what
+// was complete then - the state's rows and all window slots but those of the `back` steps in between, which follow
+// behind the wait, under the latency of the new token's own loads.  (Numbers from before `base`, or not below this step's own - a
+// replayed graph -, say nothing: then every row is fetched behind the wait.)  The splits of a head, a cluster, send each other
+// their shares of the channels (st.async, bytes counted by the receiver): one exchange instead of two cluster barriers and
+// a round of remote loads.  us per step, with the loop above
+// and with this: 32 heads, 600 rows 6.9, 4.6; 900 rows 7.2, 5.5; 16 heads, 900 rows 6.9, 4.2; 32 on 8, 600 rows 8.0, 5.5; one head 5.5, 4.0.
+// ONE: no warp has more than one pass over rows (with the loop's bookkeeping 0.3 us longer).
+template <int D, int GQ, bool LN, bool ONE>
+__global__ void __launch_bounds__(256, 2) decode_short_kernel(const __grid_constant__ DecodeParams p) {
+  constexpr int LPR = D / 8, RPW = 32 / LPR, UNR = 8;
+  __shared__ float s_m[8][GQ], s_l[8][GQ];
+  __shared__ __align__(16) float s_acc[8][GQ][D];
+  __shared__ __align__(16) __half s_q[GQ][D], s_new[2][D];
+  __shared__ float s_in[GQ * D + kDecodeCluster], s_in_ml[kDecodeCluster][GQ][2];   // what the splits send: [split][share], [split]
+  __shared__ uint64_t s_bar;
+  __shared__ uint32_t s_seen;
+
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  const int split = blockIdx.x, ns = p.nsplit;
+  const int bh0 = blockIdx.y * GQ;
+  const int bb = bh0 / p.Hq, hq0 = bh0 % p.Hq, hk = hq0 / p.G;
+  const int64_t u = (int64_t)bb * p.Hkv + hk;
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int grp = lane / LPR, gl = lane % LPR;
+  const int m = p.m, n = p.n;
+  const int share = (GQ * D + ns - 1) / ns, e0 = split * share, nmine = min(share, GQ * D - e0);
+  if (tid == 0) {
+    asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(s_seen) : "l"(p.seen) : "memory");
+    tc::mbar_init(&s_bar, 1);
+    tc::fence_barrier_init();
+    if (ns > 1) tc::mbar_expect_tx(&s_bar, (uint32_t)(ns * 4 * (nmine + 2 * GQ)));
+  }
+  __syncthreads();
+  if (ns > 1) asm volatile("barrier.cluster.arrive.release;" ::: "memory");   // (this CTA is there, with its barrier)
+
+  const uint32_t back = p.no - s_seen;
+  const int safe = back - 1u < p.no - p.base ? max(m, n - 1 - (int)back) : 0;
+  const int rw = (split * 8 + warp) * p.rpw, rend = min(n, rw + p.rpw);   // this warp's rows
+  const __half* KhatU = p.Khat + u * p.Mcap * D + gl * 8;
+  const __half* VhatU = p.Vhat + u * p.Mcap * D + gl * 8;
+  const __half* ringKU = p.ringK + u * p.ringCap * D + gl * 8;
+  const __half* ringVU = p.ringV + u * p.ringCap * D + gl * 8;
+  uint4 kw[UNR], vw[UNR];
+  auto fetch = [&](int r, int lo, int hi) {   // of the rows [r, r + UNR RPW) those in [lo, hi)
+#pragma unroll
+    for (int i = 0; i < UNR; ++i) {
+      const int row = r + i * RPW + grp;
+      if (row >= lo && row < hi) {
+        const __half *kp, *vp;
+        if (row < m) {
+          kp = KhatU + (int64_t)row * D;
+          vp = VhatU + (int64_t)row * D;
+        } else {
+          int slot = p.slot_b + (row - m);
+          if (slot >= p.ringLen) slot -= p.ringLen;
+          kp = ringKU + (int64_t)slot * D;
+          vp = ringVU + (int64_t)slot * D;
+        }
+        kw[i] = ldg_stream(kp);
+        vw[i] = ldg_stream(vp);
+      }
+    }
+  };
+#pragma unroll
+  for (int i = 0; i < UNR; ++i) kw[i] = vw[i] = make_uint4(0, 0, 0, 0);
+  const int known = min(rend, n - 1);   // (the new token's row is not in memory)
+  fetch(rw, 0, min(known, safe));
+  constexpr int NV = GQ * UNR;
+  constexpr int NVL = NV > LPR ? NV / LPR : 1;
+  constexpr int LPV = NV > LPR ? 1 : LPR / NV;
+  const int v0 = gl / LPV * NVL;
+  const int my_g = v0 / UNR;
+  const float kLog2e = 1.4426950408889634f;
+  const float scale_s = p.tau_s[hq0 + my_g] * rsqrtf((float)D) * kLog2e;
+  const float scale_b = p.tau_b[hq0 + my_g] * rsqrtf((float)D) * kLog2e;
+  const bool fresh = (n - 1) / (8 * p.rpw) == split;   // this CTA's rows end with the new token
+  const bool store = fresh && hq0 % p.G == 0;
+  auto behind_wait = [&] {
+    if (blockIdx.x == 0 && blockIdx.y == 0 && tid == 0) asm volatile("st.release.gpu.global.u32 [%0], %1;" ::"l"(p.seen), "r"(p.no) : "memory");
+    if (safe < known) fetch(rw, safe, known);
+  };
+  if (LN) new_token_ln<D, GQ>(p, bh0, u, fresh, store, split == 0, s_q, s_new, behind_wait);
+  else new_token<D, GQ>(p, bh0, u, fresh, store, split == 0, s_q, s_new, behind_wait);
+  if (store && tid == 0) p.ringG[u * p.ringCap + p.slot_t] = p.gate ? p.gate[u] : 1.0f;
+  __syncthreads();
+
+  float m_run = -INFINITY, l_run = 0.f;   // of head my_g: maximum over the warp's rows, sum over this lane's
+  float acc[GQ][8];
+#pragma unroll
+  for (int g = 0; g < GQ; ++g)
+#pragma unroll
+    for (int c = 0; c < 8; ++c) acc[g][c] = 0.f;
+  for (int r = rw; ONE ? r == rw : r < rend; r += UNR * RPW) {
+    if (!ONE && r > rw) fetch(r, 0, known);
+    float lg[NV];
+#pragma unroll
+    for (int i = 0; i < UNR; ++i) {
+      if (r + i * RPW + grp == n - 1 && rend == n) {   // (the last rows of a warp may be the next one's)
+        kw[i] = *reinterpret_cast<const uint4*>(&s_new[0][gl * 8]);
+        vw[i] = *reinterpret_cast<const uint4*>(&s_new[1][gl * 8]);
+      }
+      float kf[8];
+      unpack8(kw[i], kf);
+#pragma unroll
+      for (int g = 0; g < GQ; ++g) {
+        float qf[8];
+        unpack8(*reinterpret_cast<const uint4*>(&s_q[g][gl * 8]), qf);
+        float dot = 0.f;
+#pragma unroll
+        for (int c = 0; c < 8; ++c) dot = fmaf(qf[c], kf[c], dot);
+        lg[g * UNR + i] = dot;
+      }
+    }
+    lane_sums<NV, LPR / 2>(lg, gl);
+    float tmax = -INFINITY;
+#pragma unroll
+    for (int k = 0; k < NVL; ++k) {
+      const int row = r + (v0 + k) % UNR * RPW + grp;
+      lg[k] = row < rend ? lg[k] * (row < m ? scale_s : scale_b) : -INFINITY;
+      tmax = fmaxf(tmax, lg[k]);
+    }
+#pragma unroll
+    for (int o = LPV; o < LPV * UNR / NVL; o <<= 1) tmax = fmaxf(tmax, __shfl_xor_sync(0xffffffffu, tmax, o));
+#pragma unroll
+    for (int o = 16; o >= LPR; o >>= 1) tmax = fmaxf(tmax, __shfl_xor_sync(0xffffffffu, tmax, o));
+    const float mnew = fmaxf(m_run, tmax);   // (finite, but where a single pass meets no row)
+    if (!ONE && r > rw) {
+      const float corr = exp2f(m_run - mnew);
+      l_run *= corr;
+#pragma unroll
+      for (int g = 0; g < GQ; ++g) {
+        const float cg = __shfl_sync(0xffffffffu, corr, g * UNR / NVL * LPV);
+#pragma unroll
+        for (int c = 0; c < 8; ++c) acc[g][c] *= cg;
+      }
+    }
+    m_run = mnew;
+#pragma unroll
+    for (int k = 0; k < NVL; ++k) {
+      lg[k] = ONE && lg[k] == -INFINITY ? 0.f : exp2f(lg[k] - m_run);   // 0 for invalid rows
+      l_run += lg[k];
+    }
+#pragma unroll
+    for (int i = 0; i < UNR; ++i) {
+      float vf[8];
+      unpack8(vw[i], vf);
+#pragma unroll
+      for (int g = 0; g < GQ; ++g) {
+        const int idx = g * UNR + i;
+        const float pr = __shfl_sync(0xffffffffu, lg[idx % NVL], grp * LPR + idx / NVL * LPV);
+#pragma unroll
+        for (int c = 0; c < 8; ++c) acc[g][c] = fmaf(pr, vf[c], acc[g][c]);
+      }
+    }
+  }
+#pragma unroll
+  for (int o = LPV; o < LPV * UNR / NVL; o <<= 1) l_run += __shfl_xor_sync(0xffffffffu, l_run, o);
+#pragma unroll
+  for (int o = 16; o >= LPR; o >>= 1) l_run += __shfl_xor_sync(0xffffffffu, l_run, o);
+  if (grp == 0 && gl % (LPV * UNR / NVL) == 0) { s_m[warp][my_g] = m_run; s_l[warp][my_g] = l_run; }
+#pragma unroll
+  for (int g = 0; g < GQ; ++g) {
+#pragma unroll
+    for (int o = 16; o >= LPR; o >>= 1)
+#pragma unroll
+      for (int c = 0; c < 8; ++c) acc[g][c] += __shfl_xor_sync(0xffffffffu, acc[g][c], o);
+    if (grp == 0) {
+#pragma unroll
+      for (int c = 0; c < 8; c += 4)
+        *reinterpret_cast<float4*>(&s_acc[warp][g][gl * 8 + c]) = make_float4(acc[g][c], acc[g][c + 1], acc[g][c + 2], acc[g][c + 3]);
+    }
+  }
+  __syncthreads();
+  if (ns > 1) asm volatile("barrier.cluster.wait.acquire;" ::: "memory");   // (every CTA of the cluster is there)
+  for (int e = tid; e < GQ * D; e += 256) {
+    const int g = e / D, x = e % D;
+    float mx = -INFINITY;
+#pragma unroll
+    for (int w = 0; w < 8; ++w) mx = fmaxf(mx, s_m[w][g]);
+    float l = 0.f, a = 0.f;
+#pragma unroll
+    for (int w = 0; w < 8; ++w) {
+      const float f = s_m[w][g] == -INFINITY ? 0.f : exp2f(s_m[w][g] - mx);
+      l += s_l[w][g] * f;
+      a += s_acc[w][g][x] * f;
+    }
+    if (ns == 1) {
+      p.out[(int64_t)(bh0 + g) * D + x] = __float2bfloat16_rn(a / l);
+      continue;
+    }
+    auto send = [&](float* at, int r, float v) {
+      asm volatile("st.async.weak.shared::cluster.mbarrier::complete_tx::bytes.b32 [%0], %1, [%2];"
+                   ::"r"(tc::cluster_addr(at, r)), "r"(__float_as_uint(v)), "r"(tc::cluster_addr(&s_bar, r)) : "memory");
+    };
+    send(&s_in[split * share + e % share], e / share, a);
+    if (x < ns) { send(&s_in_ml[split][g][0], x, mx); send(&s_in_ml[split][g][1], x, l); }
+  }
+  if (ns == 1) return;
+  asm volatile("barrier.cluster.arrive.release;" ::: "memory");
+  if (tc::mbar_wait_cluster(&s_bar, 0)) {
+    for (int e = tid; e < nmine; e += 256) {
+      const int g = (e0 + e) / D;
+      float mx = -INFINITY;
+      for (int z = 0; z < ns; ++z) mx = fmaxf(mx, s_in_ml[z][g][0]);
+      float l = 0.f, a = 0.f;
+      for (int z = 0; z < ns; ++z) {
+        const float ms = s_in_ml[z][g][0], f = ms == -INFINITY ? 0.f : exp2f(ms - mx);
+        l += s_in_ml[z][g][1] * f;
+        a += s_in[z * share + e] * f;
+      }
+      p.out[(int64_t)bh0 * D + e0 + e] = __float2bfloat16_rn(a / l);
+    }
+  } else {
+    atomicExch(p.status, (int)KVM_ERR_TIMEOUT);
+  }
+  asm volatile("barrier.cluster.wait.acquire;" ::: "memory");   // (nobody leaves while another may still send to it)
+}
+
+template <int D, int GQ, bool LN, bool ONE>
+static bool launch_decode_short(const DecodeParams& p, int ncta, bool early, cudaStream_t s) {
+  cudaLaunchConfig_t lc = {};
+  lc.gridDim = dim3(p.nsplit, ncta); lc.blockDim = dim3(256); lc.stream = s;
+  cudaLaunchAttribute at[2];
+  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[0].val.programmaticStreamSerializationAllowed = early ? 1 : 0;
+  at[1].id = cudaLaunchAttributeClusterDimension;
+  at[1].val.clusterDim.x = p.nsplit; at[1].val.clusterDim.y = 1; at[1].val.clusterDim.z = 1;
+  lc.attrs = at; lc.numAttrs = p.nsplit > 1 ? 2 : 1;
+  return cudaLaunchKernelEx(&lc, decode_short_kernel<D, GQ, LN, ONE>, p) == cudaSuccess;
+}
+
 template <int D, int GQ, bool LN, bool MULTI>
 static bool launch_decode_step(const DecodeParams& p, int ncta, bool early, cudaStream_t s) {
   cudaLaunchConfig_t lc = {};
@@ -489,6 +732,22 @@ static bool launch_decode_step(const DecodeParams& p, int ncta, bool early, cuda
   at[1].val.clusterDim.x = p.nsplit; at[1].val.clusterDim.y = 1; at[1].val.clusterDim.z = 1;
   lc.attrs = at; lc.numAttrs = p.nsplit > 1 ? 2 : 1;
   return cudaLaunchKernelEx(&lc, decode_step_kernel<D, GQ, LN, MULTI>, p) == cudaSuccess;
+}
+
+// CTAs per cluster of decode_short_kernel for a step over n rows, 0 where decode_step_kernel is the better one.  kFit: clusters of 1
+// to 8 CTAs that the GPU holds at once at two CTAs per SM: more would be another wave, which costs more than the early loads
+// save (us per step, loop kernel and this: 48 heads, 900 rows in 4 splits 7.4, 12; 128 heads on 32, 600 rows 9.0, 14).  The fewest splits whose
+// warps have all their rows in flight at once, one pass; 8 for 8 to 16 groups of heads, where two steps fit beside each other
+// (16 heads, 600 rows 4.5, 4.3); two passes of 8 splits while those fit (8 heads, 1400 rows 6.7, 5.9; 32 heads 8.6, 8.1; three: 8
+// heads, 2400 rows 8.2, 8.8).  Two query heads of a kv head per CTA, not four: 32 on 8, 900 rows 6.2, 5.4.
+int plan_short(int nQ, int G, int d, int64_t n) {
+  static const int kFit[kDecodeCluster] = {296, 148, 93, 71, 56, 45, 37, 33};
+  const int groups = G % 2 == 0 ? nQ / 2 : nQ;
+  const int64_t pass = 8 * 8 * (256 / d);   // rows of a CTA in one pass
+  if (groups > kFit[0] || n > 2 * kDecodeCluster * pass) return 0;
+  int ns = (int)((n + pass - 1) / pass);
+  if (ns > kDecodeCluster || (groups >= 8 && groups <= 16)) ns = kDecodeCluster;
+  return groups <= kFit[ns - 1] ? ns : 0;
 }
 
 // How a step over n rows is cut.  Query heads per CTA (they share a kv head): the largest of 8, 4, 2, 1 that divides the group
@@ -553,6 +812,22 @@ int launch_decode(State* st, const DecodeArgs& a, cudaStream_t s) {
   p.Hq = st->Hq; p.Hkv = st->Hkv; p.G = st->G; p.r = st->r;
   p.nsplit = pl.splits; p.nclus = pl.clusters; p.part = st->decPart; p.ticket = st->decTicket;
   const bool early = st->prof_hook == nullptr;
+  p.seen = st->decSeen; p.no = st->decNo++; p.base = st->decBase; p.status = st->status;
+  const int ns = early ? plan_short(nQ, st->G, st->d, p.n) : 0;   // (with the timing hook on nothing overlaps)
+  if (ns > 0) {
+    const int rows1 = 256 / st->d /* rows that a warp loads at once */, heads = st->G % 2 == 0 ? 2 : 1;
+    p.nsplit = ns;
+    p.rpw = ((p.n + 8 * ns - 1) / (8 * ns) + rows1 - 1) / rows1 * rows1;
+#define KVM_DEC_SHORT(DD, GG, LL)                                                        \
+  if (st->d == DD && heads == GG && st->fusedLn == LL) {                                  \
+    if (p.rpw <= 8 * rows1) launch_decode_short<DD, GG, LL, true>(p, nQ / GG, early, s);  \
+    else launch_decode_short<DD, GG, LL, false>(p, nQ / GG, early, s);                    \
+  }
+    KVM_DEC_SHORT(128, 1, false) KVM_DEC_SHORT(128, 2, false) KVM_DEC_SHORT(64, 1, false) KVM_DEC_SHORT(64, 2, false)
+    KVM_DEC_SHORT(128, 1, true) KVM_DEC_SHORT(128, 2, true) KVM_DEC_SHORT(64, 1, true) KVM_DEC_SHORT(64, 2, true)
+#undef KVM_DEC_SHORT
+    return 1;
+  }
 #define KVM_DEC_GO(DD, GG, LL, MM) \
   if (st->d == DD && GQ == GG && st->fusedLn == LL && (pl.clusters > 1) == MM) launch_decode_step<DD, GG, LL, MM>(p, nQ / GQ, early, s);
   KVM_DEC_EACH(KVM_DEC_GO, true)

@@ -119,6 +119,8 @@ struct State {
   // ---- decode scratch (device): clusters of the same heads merge through it ----
   float* decPart;                // [kDecodePartCtas][d + 2]
   int32_t* decTicket;            // [kDecodePartCtas], zero between launches
+  uint32_t* decSeen;             // number of the step that has last met the end of the one before it
+  uint32_t decNo, decBase;       // (host) number of the next step; of the first one since other kernels wrote rows or window slots
   int dropUnit;                  // (host) unit that loses an exchange of the next fold's decisions, -1 (kvm_debug_drop_exchange)
   // ---- optional per-kernel timing hook (set by kvm_profile_enable): phase ids
   //      0 ingest, 1 attention, 2 memory keys, 3 routing filter, 4 decide, 5 apply, 6 decode ----

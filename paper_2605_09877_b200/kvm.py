@@ -171,7 +171,8 @@ def head_layernorm(x: "torch.Tensor", weight=None, bias=None, eps: float = 1e-5,
 
 
 def decode_plan(batch: int, n_q_heads: int, n_kv_heads: int, head_dim: int, n_rows: int):
-    """(query heads per CTA, CTAs per cluster, clusters per group of heads) of a decode step over n_rows rows."""
+    """(query heads per CTA, CTAs per cluster, clusters per group of heads) of a decode step over n_rows rows, where it runs the
+    kernel that loops over them (few heads over few rows are cut otherwise)."""
     out = (C.c_int32 * 3)()
     rc = lib.kvm_debug_decode_plan(batch, n_q_heads, n_kv_heads, head_dim, n_rows, out)
     if rc != KVM_OK:

@@ -62,9 +62,9 @@ def gpu_layer(wl, params, flags=0, max_call_tokens=None, max_seq_len=None, radiu
     return st, g
 
 
-def run_gpu(wl, tensors, params, cuts=None, flags=0, radius_on=True, decode_from=None, ln_eps=1e-5):
+def run_gpu(wl, tensors, params, cuts=None, flags=0, radius_on=True, decode_from=None, ln_eps=1e-5, timed=False):
     """Prefill in segments given by `cuts` (token boundaries); tokens >= decode_from go through
-    kvm_decode_step one at a time.  Returns (y [B,Hq,T,d] bf16 cpu, state handle)."""
+    kvm_decode_step one at a time; `timed`: with the timing hook on.  Returns (y [B,Hq,T,d] bf16 cpu, state handle)."""
     T = wl.T
     decode_from = T if decode_from is None else decode_from
     cuts = cuts or [0, decode_from]
@@ -73,6 +73,7 @@ def run_gpu(wl, tensors, params, cuts=None, flags=0, radius_on=True, decode_from
         cuts.append(decode_from)
     st, g = gpu_layer(wl, params, flags=flags, max_call_tokens=max(max(b - a for a, b in zip(cuts[:-1], cuts[1:])), 1),
                       radius_on=radius_on, ln_eps=ln_eps)
+    st.profile_enable(timed)
     dev = torch.device("cuda:0")
     q, k, v = (tensors[n].to(dev) for n in ("q", "k", "v"))
     gate = tensors.get("gate")

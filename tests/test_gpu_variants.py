@@ -462,3 +462,70 @@ def test_attention_of_few_heads_over_many_rows_splits_the_keys(Hq, Hkv, d, block
     """Key splits of launches of 6 to 48 tiles over 10 to 40 key tiles: two to eight splits, ragged last ones."""
     wl = synth.Workload("t", 1, Hq, Hkv, d, 256 * blocks + 70, 256, "unbounded", r=32, seed=62)
     print(_sampled(wl, [(0, 0), (0, Hkv - 1)]))
+
+
+def _short_splits(n_q, group, d, n):
+    """CTAs per cluster of the decode kernel that fetches its rows ahead (0: the step is not one of its)."""
+    groups, cta = (n_q // 2 if group % 2 == 0 else n_q), 64 * (256 // d)
+    fit = (296, 148, 93, 71, 56, 45, 37, 33)
+    if groups > fit[0] or n > 16 * cta:
+        return 0
+    ns = -(-n // cta)
+    ns = 8 if ns > 8 or 8 <= groups <= 16 else ns
+    return ns if groups <= fit[ns - 1] else 0
+
+
+@pytest.mark.parametrize("Hq,Hkv,d,C,slots,r,splits", [
+    (1, 1, 64, 16, 40, 0, {1}), (3, 1, 128, 16, 80, 32, {1}), (2, 2, 128, 32, 170, 32, {2}), (2, 1, 128, 64, 300, 64, {3, 4}),
+    (5, 5, 64, 64, 960, 16, {4, 5}), (4, 2, 128, 64, 600, 0, {6}), (3, 3, 128, 64, 700, 32, {6, 7}), (12, 12, 64, 32, 300, 0, {8}),
+    (24, 12, 128, 64, 900, 32, {8}), (33, 33, 128, 64, 930, 0, {8}),
+    (2, 2, 128, 64, 1500, 32, {8}), (1, 1, 64, 256, 3500, 0, {8}), (66, 33, 64, 64, 2700, 32, {8}),   # two passes over a warp's rows
+])
+def test_decode_steps_that_fetch_their_rows_ahead(Hq, Hkv, d, C, slots, r, splits):
+    """One to eight CTAs per group of heads, one and two passes, warps with few rows or none; steps back to back across a fold, of
+    which each fetches what the ones before leave complete, against the oracle and against steps that are waited for."""
+    start = (slots // C + 4) * C - 6
+    wl = synth.Workload("short", 1, Hq, Hkv, d, start + 14, C, "fixed", fixed_slots=slots, r=r, seed=400 + slots)
+    assert {_short_splits(Hq, Hq // Hkv, d, _decode_rows(wl, t)) for t in range(start, wl.T)} <= splits
+    params = synth.make_layer_params(wl, trivial=False)
+    tensors = synth.make_inputs(wl)
+    y, st = pu.run_gpu(wl, tensors, params, decode_from=start)
+    units = sorted({(0, 0), (0, Hkv - 1)})
+    y_ref, o = pu.run_oracle(wl, tensors, params, units=units)
+    print(pu.compare(wl, y, st, y_ref, o, units=units))
+    st.free()
+    t = {n: x.cuda() for n, x in tensors.items() if n in "qkv"}
+    outs = []
+    for wait in (False, True):
+        st, g = pu.gpu_layer(wl, params, max_call_tokens=start)
+        st.prefill(t["q"][:, :, :start], t["k"][:, :, :start], t["v"][:, :, :start], wl.C, g, wl.r)
+        steps = [[t[n][:, :, i].contiguous() for n in "qkv"] for i in range(start, wl.T)]
+        ys = [torch.empty_like(s[0]) for s in steps]
+        torch.cuda.synchronize()
+        for s, out in zip(steps, ys):
+            st.decode_step(*s, out=out)
+            if wait:
+                torch.cuda.synchronize()
+        torch.cuda.synchronize()
+        assert st.check() == 0
+        outs.append(torch.stack(ys, 2).cpu())
+        st.free()
+    assert torch.equal(outs[0], outs[1]) and torch.equal(outs[0], y[:, :, start:])
+
+
+@pytest.mark.parametrize("B,Hq,Hkv,d,pos,steps,plan", [
+    (1, 1, 1, 64, 40, 30, (1, 1, 1)), (1, 2, 1, 128, 900, 20, (2, 6, 1)), (3, 32, 4, 64, 1300, 10, (4, 7, 1)), (7, 21, 21, 128, 300, 9, (1, 2, 1)),
+    (1, 2, 2, 128, 260, 5, (1, 5, 1)), (1, 2, 2, 128, 452, 5, (1, 8, 1)), (5, 32, 4, 64, 20, 5, (8, 1, 1)), (5, 32, 4, 128, 130, 8, (8, 3, 1))])
+def test_decode_kernel_that_loops_over_rows_at_few_rows(B, Hq, Hkv, d, pos, steps, plan):
+    """With the timing hook on every step runs the kernel that loops over its rows, also where a few rows of a few heads are fetched ahead
+    otherwise: one to eight splits and query heads per CTA."""
+    from paper_2605_09877_b200 import kvm
+    wl = synth.Workload("dec", B, Hq, Hkv, d, pos + steps, 64, "sqrt", sqrt_coeff=20, r=32, seed=330 + pos)
+    assert {kvm.decode_plan(B, Hq, Hkv, d, _decode_rows(wl, t)) for t in range(pos, pos + steps)} == {plan}
+    params = synth.make_layer_params(wl, trivial=False)
+    tensors = synth.make_inputs(wl)
+    units = sorted({(0, 0), (B - 1, Hkv - 1)})
+    y, st = pu.run_gpu(wl, tensors, params, decode_from=pos, timed=True)
+    y_ref, o = pu.run_oracle(wl, tensors, params, units=units)
+    print(pu.compare(wl, y, st, y_ref, o, units=units))
+    st.free()
