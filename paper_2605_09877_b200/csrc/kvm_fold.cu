@@ -904,33 +904,46 @@ __global__ void __launch_bounds__(kDecideThreads, PER_SM) fold_decide_kernel(con
       while (LT * tpw > 32) LT >>= 1;
       const int j = wj0 + lane / LT, part = lane & (LT - 1);
       const bool merged = j < wj1 && !s_app[j];
-      float pv[4], gm = -INFINITY;   // (the first products stay in registers)
+      // eight products under way at a time, the first eight stay in registers (one after the
+      // other before: 32 heads on 8, 3 x 5003 tokens 1.220 ms, now 1.172; 96 heads, 8192 tokens 4.49, 4.28; 148 6.23, 5.96)
+      constexpr int NB = 8;
+      auto fetch8 = [&](int t0, float (&v)[NB]) {
 #pragma unroll
-      for (int t = 0; t < 4; ++t) {
-        const int a = part + t * LT;
-        pv[t] = merged && a < n_a ? gram[(int64_t)s_creator[a] * p.Cmax + j] : -INFINITY;
+        for (int t = 0; t < NB; ++t) {
+          const int a = part + (t0 + t) * LT;
+          v[t] = merged && a < n_a ? gram[(int64_t)s_creator[a] * p.Cmax + j] : -INFINITY;
+        }
+      };
+      float pv[NB], gm = -INFINITY;
+      fetch8(0, pv);
+      for (int t0 = NB; t0 * LT < n_a; t0 += NB) {
+        float v[NB];
+        fetch8(t0, v);
+#pragma unroll
+        for (int t = 0; t < NB; ++t) gm = fmaxf(gm, v[t]);
       }
-      for (int a = part + 4 * LT; merged && a < n_a; a += LT) gm = fmaxf(gm, gram[(int64_t)s_creator[a] * p.Cmax + j]);
 #pragma unroll
-      for (int t = 0; t < 4; ++t) gm = fmaxf(gm, pv[t]);
+      for (int t = 0; t < NB; ++t) gm = fmaxf(gm, pv[t]);
       for (int o = LT >> 1; o > 0; o >>= 1) gm = fmaxf(gm, __shfl_xor_sync(0xffffffffu, gm, o));
       double bar = INFINITY;
       if (merged) {
         const double eps = 0.5 * (double)s_thr[j];
         bar = fmax(s_best[j], (double)gm - eps) - eps;
       }
-      for (int t = 0; t * LT < n_a; ++t) {
-        const int a = part + t * LT;
-        const float v = t == 0 ? pv[0] : t == 1 ? pv[1] : t == 2 ? pv[2] : t == 3 ? pv[3]
-                        : merged && a < n_a ? gram[(int64_t)s_creator[a] * p.Cmax + j] : -INFINITY;
-        const bool in = merged && a < n_a && (double)v >= bar;
-        const unsigned hit = __ballot_sync(0xffffffffu, in);
-        if (np + __popc(hit) > kWarpPairs) { over = true; break; }
-        if (in) {
-          const int w = np + __popc(hit & ((1u << lane) - 1u));
-          prow[w] = a; ptok[w] = (unsigned char)j;
+      for (int t0 = 0; t0 * LT < n_a && !over; t0 += NB) {
+        if (t0 > 0) fetch8(t0, pv);
+#pragma unroll
+        for (int t = 0; t < NB; ++t) {
+          const bool in = merged && part + (t0 + t) * LT < n_a && (double)pv[t] >= bar;
+          const unsigned hit = __ballot_sync(0xffffffffu, in);
+          if (hit == 0) continue;
+          if (np + __popc(hit) > kWarpPairs) { over = true; break; }
+          if (in) {
+            const int w = np + __popc(hit & ((1u << lane) - 1u));
+            prow[w] = part + (t0 + t) * LT; ptok[w] = (unsigned char)j;
+          }
+          np += __popc(hit);
         }
-        np += __popc(hit);
       }
       if (over) np = 0;
     }
