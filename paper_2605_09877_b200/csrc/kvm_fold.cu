@@ -482,7 +482,7 @@ __device__ __forceinline__ void sort_n(K& key, int& val, K* sk, int* sv, int t) 
   }
 }
 
-struct DecideShared {
+struct __align__(16) DecideShared {
   unsigned long long key[kMaxBlock];   // append scores of all tokens (exchanged)
   unsigned tgt[kMaxBlock];             // row << 9 | token of all merged tokens (exchanged; all ones: appended)
   int app[kMaxBlock];                  // append flags of all tokens (exchanged)
@@ -867,9 +867,9 @@ __global__ void __launch_bounds__(kDecideThreads, PER_SM) fold_decide_kernel(con
       int cnt = 0;
       if (mine) {
 #pragma unroll 4
-        for (int i = part; i < C; i += q) {
-          const unsigned long long ki = s_key[i];
-          cnt += (ki < kj || (ki == kj && i < j)) ? 1 : 0;
+        for (int i = 2 * part; i < C; i += 2 * q) {   // (two keys per load; equal scores: the lower token first)
+          const ulonglong2 k2 = *reinterpret_cast<const ulonglong2*>(&s_key[i]);
+          cnt += (k2.x < kj + (i < j ? 1ull : 0ull) ? 1 : 0) + (k2.y < kj + (i + 1 < j ? 1ull : 0ull) ? 1 : 0);
         }
       }
       for (int o = q >> 1; o > 0; o >>= 1) cnt += __shfl_xor_sync(0xffffffffu, cnt, o);
@@ -1048,9 +1048,18 @@ __global__ void __launch_bounds__(kDecideThreads, PER_SM) fold_decide_kernel(con
     bool members = false;
     if (mine) {
 #pragma unroll 4
-      for (int i = part; i < C; i += q) less += s_tgt[i] < key ? 1 : 0;
-      if (app)
-        for (int i = part; i < C; i += q) members |= (s_tgt[i] >> 9) == (key >> 9);
+      for (int i = 4 * part; i < C; i += 4 * q) {   // (four keys per load)
+        const uint4 k4 = *reinterpret_cast<const uint4*>(&s_tgt[i]);
+        less += (k4.x < key ? 1 : 0) + (k4.y < key ? 1 : 0) + (k4.z < key ? 1 : 0) + (k4.w < key ? 1 : 0);
+      }
+      if (app) {
+#pragma unroll 4
+        for (int i = 4 * part; i < C; i += 4 * q) {
+          const uint4 k4 = *reinterpret_cast<const uint4*>(&s_tgt[i]);
+          const unsigned row = key >> 9;
+          members |= (k4.x >> 9) == row || (k4.y >> 9) == row || (k4.z >> 9) == row || (k4.w >> 9) == row;
+        }
+      }
     }
     int cnt = less | (members ? 1 << 16 : 0);
     for (int o = q >> 1; o > 0; o >>= 1) cnt += __shfl_xor_sync(0xffffffffu, cnt, o);
