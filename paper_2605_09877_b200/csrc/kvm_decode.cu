@@ -736,12 +736,13 @@ static bool launch_decode_step(const DecodeParams& p, int ncta, bool early, cuda
 
 // CTAs per cluster of decode_short_kernel for a step over n rows, 0 where decode_step_kernel is the better one.  kFit: clusters of 1
 // to 8 CTAs that the GPU holds at once at two CTAs per SM: more would be another wave, which costs more than the early loads
-// save (us per step, loop kernel and this: 48 heads, 900 rows in 4 splits 7.4, 12; 128 heads on 32, 600 rows 9.0, 14).  The fewest splits whose
+// save (us per step, loop kernel and this: 48 heads, 900 rows in 8 splits 7.4, 12; 128 heads on 32, 600 rows 9.0, 14; 93 heads in 3
+// splits, which fill the GPU to the last cluster, 7.1, 7.9: 88 there).  The fewest splits whose
 // warps have all their rows in flight at once, one pass; 8 for 8 to 16 groups of heads, where two steps fit beside each other
 // (16 heads, 600 rows 4.5, 4.3); two passes of 8 splits while those fit (8 heads, 1400 rows 6.7, 5.9; 32 heads 8.6, 8.1; three: 8
 // heads, 2400 rows 8.2, 8.8).  Two query heads of a kv head per CTA, not four: 32 on 8, 900 rows 6.2, 5.4.
 int plan_short(int nQ, int G, int d, int64_t n) {
-  static const int kFit[kDecodeCluster] = {296, 148, 93, 71, 56, 45, 37, 33};
+  static const int kFit[kDecodeCluster] = {296, 148, 88, 71, 56, 45, 37, 33};
   const int groups = G % 2 == 0 ? nQ / 2 : nQ;
   const int64_t pass = 8 * 8 * (256 / d);   // rows of a CTA in one pass
   if (groups > kFit[0] || n > 2 * kDecodeCluster * pass) return 0;

@@ -2154,16 +2154,17 @@ __global__ void __launch_bounds__(256) refresh_rows_kernel(RefreshParams p) {
 }
 
 // Which apply kernel the folds of this state run (fixed per state and block).  Four rows per warp where the keys are recomputed and
-// otherwise only for blocks of more than 128 tokens of a middling number of units.  Measured (ms, 24 blocks; one row per warp, four):
-// 128 channels, blocks of 256, square-root state: 64 units 2.19, 2.30; 72 2.50, 2.42; 96 3.49, 3.33; 128 3.86, 4.02; 148 4.59, 4.56;
-// 160 4.74, 4.87; 192 5.22, 5.58; 512 rows: 64 units 1.50, 1.55; 96 2.14, 2.20; 128 2.49, 2.61; 160 3.19, 3.60.  64 channels, 256
-// rows: 48 units 1.21, 1.25; 64 1.25, 1.18; 148 2.04, 1.86; 224 2.98, 2.80 (with four CTAs per unit).  Blocks of 64 and 128, 64 to 224
-// units: one row per warp is up to 12 % faster, nowhere more than 1 % slower.
+// otherwise for blocks of 256 of a middling number of units, and for 64 channels, whose rows are half as much to fetch, from fewer
+// rows on.  Measured (ms, 24 blocks; one row per warp, four): 128 channels, blocks of 256, square-root state: 64 units 2.19, 2.30; 72
+// 2.50, 2.42; 96 3.49, 3.33; 128 3.86, 4.02; 148 4.59, 4.56; 160 4.74, 4.87; 192 5.22, 5.58; 512 rows: 64 units 1.50, 1.55; 96
+// 2.14, 2.20; 128 2.49, 2.61; 160 3.19, 3.60; blocks of 64 and 128, 64 to 224 units: one is up to 12 % faster, nowhere more than 1 %
+// slower.  64 channels, 256 rows, blocks of 256: 48 units 1.21, 1.25; 64 1.25, 1.18; 148 2.04, 1.86; 224 2.98, 2.80; of 128: 48 units
+// 0.653, 0.630; 64 0.733, 0.705; 128 1.08, 0.98; 192 1.44, 1.34; of 64: 64 units 0.608, 0.629; 96 0.773, 0.712; 224 1.10, 1.06.
 static bool apply_uses_rows4(const State* st) {
+  const int64_t rows = (int64_t)st->C * st->U;
   if (st->recomputeK) return true;
-  if (st->C <= 128) return false;
-  if (st->d == 64) return (int64_t)st->C * st->U > 12288;
-  return (int64_t)st->C * st->U > 16384 && st->U < 128;
+  if (st->d == 64) return st->C > 128 ? rows > 12288 : rows >= 6144;
+  return st->C > 128 && rows > 16384 && st->U < 128;
 }
 
 int launch_refresh_rows(State* st, int64_t m, cudaStream_t s) {

@@ -445,11 +445,14 @@ def test_crowded_runs_are_compared_pair_by_pair(Hkv, d, C):
     (3, 24, 128, 256, 300, True),   # four rows per warp with stored memory keys
     (2, 25, 64, 256, 256, True),
     (5, 32, 64, 192, 64, True),     # (four CTAs per unit)
+    (2, 24, 64, 128, 90, True),
+    (1, 47, 64, 128, 300, False),
 ])
 def test_rows_with_many_members_in_both_apply_kernels(B, Hkv, d, C, slots, rows4):
     """The kernel that a state's folds run to write the touched rows, at rows with none, one and many members, appended rows
     among them; the state means and readout rows against the oracle, and again after a snapshot's import."""
-    assert rows4 == (C > 128 and C * B * Hkv > (12288 if d == 64 else 16384) and (d == 64 or B * Hkv < 128))
+    rows = C * B * Hkv
+    assert rows4 == ((rows > 12288 if C > 128 else rows >= 6144) if d == 64 else C > 128 and rows > 16384 and B * Hkv < 128)
     wl = synth.Workload("t", B, Hkv, Hkv, d, C * 5 + 11, C, "fixed", fixed_slots=slots, r=32, seed=61, kind="mixture")
     params = synth.make_layer_params(wl, trivial=False)
     units = sorted({(0, 0), (B - 1, Hkv - 1)})
@@ -467,7 +470,7 @@ def test_attention_of_few_heads_over_many_rows_splits_the_keys(Hq, Hkv, d, block
 def _short_splits(n_q, group, d, n):
     """CTAs per cluster of the decode kernel that fetches its rows ahead (0: the step is not one of its)."""
     groups, cta = (n_q // 2 if group % 2 == 0 else n_q), 64 * (256 // d)
-    fit = (296, 148, 93, 71, 56, 45, 37, 33)
+    fit = (296, 148, 88, 71, 56, 45, 37, 33)
     if groups > fit[0] or n > 16 * cta:
         return 0
     ns = -(-n // cta)
