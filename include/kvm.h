@@ -291,12 +291,22 @@ kvm_status_t kvm_debug_counters(kvm_state_t* state, int64_t* out, void* cuda_str
  * have appended are rows of single tokens of the block, nothing is merged), the other units fold as ever. */
 kvm_status_t kvm_debug_drop_exchange(kvm_state_t* state, int32_t unit);
 
-/* How a decode step over n_rows rows (state and window) is cut where it runs the kernel that loops over them (few heads over few
- * rows are cut otherwise, unless the timing hook is on), for tests: out[0] query heads per CTA, out[1] CTAs per
- * cluster (row splits merged through shared memory), out[2] clusters per group of heads (merged through global memory).
- * Host arithmetic only. */
+/* How the library cuts its launches, for tests (host arithmetic only; no state is needed):
+ * - kvm_debug_decode_ahead: a decode step over n_rows rows (state and window).  out[0] CTAs per group of query heads where the step
+ *   runs the kernel that fetches its rows ahead (few heads over few rows), 0 where it runs the one that loops over them
+ *   (kvm_debug_decode_plan); out[1] query heads per CTA, out[2] rows per warp.
+ * - kvm_debug_decode_plan: the same step in the looping kernel.  out[0] query heads per CTA, out[1] CTAs per cluster (row splits
+ *   merged through shared memory), out[2] clusters per group of heads (merged through global memory).
+ * - kvm_debug_apply_plan: the kernel that writes the rows a fold touches, for n_units = batch * n_kv_heads; serial: with
+ *   KVM_FLAG_SERIAL_FOLDS.  out[0] rows per warp (1 or 4), out[1] CTAs per unit.
+ * - kvm_debug_attention_plan: the attention of n_queries tokens of a block over n_slots state rows.  out[0] (batch, head, query tile)
+ *   CTAs that run whole, out[1] key splits of each of the others. */
+kvm_status_t kvm_debug_decode_ahead(int32_t batch, int32_t n_q_heads, int32_t n_kv_heads, int32_t head_dim, int64_t n_rows,
+                                    int32_t* out);
 kvm_status_t kvm_debug_decode_plan(int32_t batch, int32_t n_q_heads, int32_t n_kv_heads, int32_t head_dim, int64_t n_rows,
                                    int32_t* out);
+kvm_status_t kvm_debug_apply_plan(int64_t n_units, int32_t head_dim, int32_t block, int32_t serial, int32_t* out);
+kvm_status_t kvm_debug_attention_plan(int32_t batch, int32_t n_q_heads, int32_t n_queries, int64_t n_slots, int32_t* out);
 
 /* Number of kernels the library has launched for this state so far (host counter). */
 int64_t kvm_launch_count(const kvm_state_t* state);

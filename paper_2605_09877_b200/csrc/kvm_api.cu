@@ -179,12 +179,16 @@ kvm_status_t validate_prefill(const State& s, int32_t block, const kvm_growth_t&
   return KVM_OK;
 }
 
+// No fp64 memory keys are kept: states with one readout copy, where a block has enough tokens for the four-rows-per-warp apply
+// kernel, which recomputes them.
+bool recomputes_keys(bool serial, int block, int64_t units) { return serial && block * units >= 8192; }
+
 // Binds block / growth / rope_dims (host bookkeeping only; called once the call can no longer fail).
 void bind_state(State& s, int32_t block, const kvm_growth_t& growth, int32_t r) {
   s.C = block; s.r = r; s.growth = growth; s.ringLen = (int64_t)s.w * block;
   const int k = r / 2;
   s.inv_freq = s.inv_freq_all + (int64_t)k * (k - 1) / 2;
-  s.recomputeK = s.serial && (int64_t)block * s.U >= 8192;   // (the threshold of the four-rows-per-warp apply kernel)
+  s.recomputeK = recomputes_keys(s.serial, block, s.U);
   s.bound = true;
 }
 
@@ -503,6 +507,30 @@ KVM_API kvm_status_t kvm_debug_decode_plan(int32_t batch, int32_t n_q_heads, int
   if (head_dim != 64 && head_dim != 128) return KVM_ERR_UNSUPPORTED;
   const DecodePlan p = plan_decode(batch * n_q_heads, n_q_heads / n_kv_heads, head_dim, n_rows);
   out[0] = p.heads; out[1] = p.splits; out[2] = p.clusters;
+  return KVM_OK;
+}
+
+KVM_API kvm_status_t kvm_debug_decode_ahead(int32_t batch, int32_t n_q_heads, int32_t n_kv_heads, int32_t head_dim,
+                                            int64_t n_rows, int32_t* out) {
+  if (batch < 1 || n_q_heads < 1 || n_kv_heads < 1 || n_q_heads % n_kv_heads || n_rows < 1 || !out) return KVM_ERR_INVALID_ARG;
+  if (head_dim != 64 && head_dim != 128) return KVM_ERR_UNSUPPORTED;
+  const DecodeShortPlan p = plan_decode_short(batch * n_q_heads, n_q_heads / n_kv_heads, head_dim, n_rows);
+  out[0] = p.splits; out[1] = p.heads; out[2] = p.rows_per_warp;
+  return KVM_OK;
+}
+
+KVM_API kvm_status_t kvm_debug_apply_plan(int64_t n_units, int32_t head_dim, int32_t block, int32_t serial, int32_t* out) {
+  if (n_units < 1 || block < 8 || block > kMaxBlock || block % 8 || !out) return KVM_ERR_INVALID_ARG;
+  if (head_dim != 64 && head_dim != 128) return KVM_ERR_UNSUPPORTED;
+  const ApplyPlan p = plan_apply(n_units, head_dim, block, recomputes_keys(serial != 0 || n_units >= kSerialUnits, block, n_units));
+  out[0] = p.rows_per_warp; out[1] = p.ctas;
+  return KVM_OK;
+}
+
+KVM_API kvm_status_t kvm_debug_attention_plan(int32_t batch, int32_t n_q_heads, int32_t n_queries, int64_t n_slots, int32_t* out) {
+  if (batch < 1 || n_q_heads < 1 || n_queries < 1 || n_slots < 0 || !out) return KVM_ERR_INVALID_ARG;
+  const AttnPlan p = plan_attn((int64_t)batch * n_q_heads * ((n_queries + 127) / 128), n_slots);
+  out[0] = p.n_whole; out[1] = p.nsp_rest;
   return KVM_OK;
 }
 

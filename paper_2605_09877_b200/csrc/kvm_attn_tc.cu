@@ -558,6 +558,22 @@ bool encode_tmap_rows(CUtensorMap* map, const void* base, int d, int64_t rows, i
             CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
+// Key splits of a launch of `tiles` CTAs over m state rows.  Few query tiles: up to a quarter of the GPU (the folds of the block before
+// run beside this kernel and are usually the longer chain), at least two key tiles per split; up to three quarters where a split
+// still has nine or so, for there the attention is the longer chain (ms, a quarter and as chosen: 16 heads on 4, 65536 tokens 12.1, 8.64;
+// 8 heads 10.4, 9.0; 16 heads, 4096 rows, 32768 tokens 7.31, 5.37.  Three quarters where splits have two or three tiles: 24 heads on 8,
+// 512 rows, 3.04, 3.24).  Many tiles: when the last wave of one-CTA-per-SM would be less than half full, its tiles are split
+// in two (the partial-result buffer holds 2 * kAttnSplitTiles tiles of two splits).
+AttnPlan plan_attn(int64_t tiles, int64_t m) {
+  const int64_t ntot_min = (m + 127) / 128 + 1;
+  int64_t nsp = std::max(std::min(kAttnSplitTiles / tiles, ntot_min / 2), std::min(3 * kAttnSplitTiles / tiles, (ntot_min + 8) / 9));
+  nsp = std::max<int64_t>(1, std::min<int64_t>(nsp, kAttnMaxSplits));
+  if (nsp > 1) return {0, (int)nsp};
+  const int64_t rem = tiles % 148;
+  if (tiles > 148 && rem > 0 && rem <= 2 * kAttnSplitTiles && ntot_min >= 4) return {(int)(tiles - rem), 2};
+  return {(int)tiles, 1};
+}
+
 int launch_attn_tc(State* st, const AttnArgs& a, cudaStream_t s) {
   AttnTcParams p;
   p.q_row0 = a.q_row0; p.t0 = a.t0; p.m = a.m; p.win_row0 = a.win_row0; p.b = a.b; p.out_t0 = a.out_t0;
@@ -569,26 +585,11 @@ int launch_attn_tc(State* st, const AttnArgs& a, cudaStream_t s) {
   if (tell && ++st->foldNo == 0) ++st->foldNo;   // (0 says nothing)
   p.fold_seen = st->foldSeen; p.fold_no = st->foldNo;
   p.out_vec = (reinterpret_cast<uintptr_t>(a.out) % 16 == 0 && a.so[0] % 8 == 0 && a.so[1] % 8 == 0 && a.so[2] % 8 == 0) ? 1 : 0;
-  // key splits when there are few query tiles: up to a quarter of the GPU (the folds of the block before run beside this kernel and
-  // are usually the longer chain), at least two key tiles per split; up to three quarters where a split still has nine or so, for
-  // there the attention is the longer chain (ms, a quarter and as chosen: 16 heads on 4, 65536 tokens 12.1, 8.64; 8 heads 10.4, 9.0; 16
-  // heads, 4096 rows, 32768 tokens 7.31, 5.37.  Three quarters where splits have two or three tiles: 24 heads on 8, 512 rows, 3.04, 3.24)
   const int qtiles = (a.nq + 127) / 128;
-  const int ctas = qtiles * st->B * st->Hq;
-  const int ntot_min = (int)((a.m + 127) / 128) + 1;
-  int nsp = std::max(std::min(kAttnSplitTiles / ctas, ntot_min / 2), std::min(3 * kAttnSplitTiles / ctas, (ntot_min + 8) / 9));
-  nsp = std::max(1, std::min(nsp, kAttnMaxSplits));
-  // Many tiles: when the last wave of one-CTA-per-SM would be less than half full, its tiles are split
-  // in two (the partial-result buffer holds 2 * kAttnSplitTiles tiles of two splits).
   const int tiles = qtiles * st->B * st->Hq;
-  int n_whole = nsp > 1 ? 0 : tiles, nsp_rest = nsp;
-  if (nsp == 1 && tiles > 148) {
-    const int rem = tiles % 148;
-    const int ntot_min2 = (int)((a.m + 127) / 128) + 1;
-    if (rem > 0 && rem <= 2 * kAttnSplitTiles && ntot_min2 >= 4) { n_whole = tiles - rem; nsp_rest = 2; }
-  }
-  p.qtiles = qtiles; p.n_whole = n_whole; p.nsp_rest = nsp_rest;
-  dim3 grid(n_whole + (tiles - n_whole) * nsp_rest);
+  const AttnPlan pl = plan_attn(tiles, a.m);
+  p.qtiles = qtiles; p.n_whole = pl.n_whole; p.nsp_rest = pl.nsp_rest;
+  dim3 grid(pl.n_whole + (tiles - pl.n_whole) * pl.nsp_rest);
   const CUtensorMap* tm = reinterpret_cast<const CUtensorMap*>(st->tmaps);
   const int ks = (st->nfolds & 1) ? 6 : 1, vs = (st->nfolds & 1) ? 7 : 2;   // readout copy of the current version
   // where every kernel has the GPU to itself this one's CTAs start as the kernel before leaves the SMs

@@ -741,14 +741,16 @@ static bool launch_decode_step(const DecodeParams& p, int ncta, bool early, cuda
 // warps have all their rows in flight at once, one pass; 8 for 8 to 16 groups of heads, where two steps fit beside each other
 // (16 heads, 600 rows 4.5, 4.3); two passes of 8 splits while those fit (8 heads, 1400 rows 6.7, 5.9; 32 heads 8.6, 8.1; three: 8
 // heads, 2400 rows 8.2, 8.8).  Two query heads of a kv head per CTA, not four: 32 on 8, 900 rows 6.2, 5.4.
-int plan_short(int nQ, int G, int d, int64_t n) {
+DecodeShortPlan plan_decode_short(int nQ, int G, int d, int64_t n) {
   static const int kFit[kDecodeCluster] = {296, 148, 88, 71, 56, 45, 37, 33};
-  const int groups = G % 2 == 0 ? nQ / 2 : nQ;
-  const int64_t pass = 8 * 8 * (256 / d);   // rows of a CTA in one pass
-  if (groups > kFit[0] || n > 2 * kDecodeCluster * pass) return 0;
+  const int heads = G % 2 == 0 ? 2 : 1, groups = nQ / heads;
+  const int rows1 = 256 / d;                // rows that a warp loads at once
+  const int64_t pass = 8 * 8 * rows1;       // rows of a CTA in one pass
+  if (groups > kFit[0] || n > 2 * kDecodeCluster * pass) return {0, 0, 0};
   int ns = (int)((n + pass - 1) / pass);
   if (ns > kDecodeCluster || (groups >= 8 && groups <= 16)) ns = kDecodeCluster;
-  return groups <= kFit[ns - 1] ? ns : 0;
+  if (groups > kFit[ns - 1]) return {0, 0, 0};
+  return {heads, ns, ((int)(n + 8 * ns - 1) / (8 * ns) + rows1 - 1) / rows1 * rows1};
 }
 
 // How a step over n rows is cut.  Query heads per CTA (they share a kv head): the largest of 8, 4, 2, 1 that divides the group
@@ -799,8 +801,6 @@ DecodePlan plan_decode(int nQ, int G, int d, int64_t n) {
 
 int launch_decode(State* st, const DecodeArgs& a, cudaStream_t s) {
   const int nQ = st->B * st->Hq;
-  const DecodePlan pl = plan_decode(nQ, st->G, st->d, a.m + (a.t - a.b + 1));
-  const int GQ = pl.heads;
   DecodeParams p;
   p.q = a.q; p.k = a.k; p.v = a.v; p.gate = a.gate; p.inv_freq = st->inv_freq;
   p.lnq_w = st->lnq_w; p.lnq_b = st->lnq_b; p.lnk_w = st->lnk_w; p.lnk_b = st->lnk_b; p.qk_ln_eps = st->qk_ln_eps;
@@ -811,24 +811,25 @@ int launch_decode(State* st, const DecodeArgs& a, cudaStream_t s) {
   p.m = (int)a.m; p.n = (int)(a.m + (a.t - a.b + 1));
   p.ringLen = (int)st->ringLen; p.slot_b = (int)(a.b % st->ringLen); p.slot_t = (int)(a.t % st->ringLen);
   p.Hq = st->Hq; p.Hkv = st->Hkv; p.G = st->G; p.r = st->r;
-  p.nsplit = pl.splits; p.nclus = pl.clusters; p.part = st->decPart; p.ticket = st->decTicket;
+  p.part = st->decPart; p.ticket = st->decTicket;
   const bool early = st->prof_hook == nullptr;
   p.seen = st->decSeen; p.no = st->decNo++; p.base = st->decBase; p.status = st->status;
-  const int ns = early ? plan_short(nQ, st->G, st->d, p.n) : 0;   // (with the timing hook on nothing overlaps)
-  if (ns > 0) {
-    const int rows1 = 256 / st->d /* rows that a warp loads at once */, heads = st->G % 2 == 0 ? 2 : 1;
-    p.nsplit = ns;
-    p.rpw = ((p.n + 8 * ns - 1) / (8 * ns) + rows1 - 1) / rows1 * rows1;
-#define KVM_DEC_SHORT(DD, GG, LL)                                                        \
-  if (st->d == DD && heads == GG && st->fusedLn == LL) {                                  \
-    if (p.rpw <= 8 * rows1) launch_decode_short<DD, GG, LL, true>(p, nQ / GG, early, s);  \
-    else launch_decode_short<DD, GG, LL, false>(p, nQ / GG, early, s);                    \
+  const DecodeShortPlan sp = early ? plan_decode_short(nQ, st->G, st->d, p.n) : DecodeShortPlan{0, 0, 0};   // (with the timing hook on nothing overlaps)
+  if (sp.splits > 0) {
+    p.nsplit = sp.splits; p.nclus = 1; p.rpw = sp.rows_per_warp;
+#define KVM_DEC_SHORT(DD, GG, LL)                                                                \
+  if (st->d == DD && sp.heads == GG && st->fusedLn == LL) {                                       \
+    if (p.rpw <= 8 * (256 / DD)) launch_decode_short<DD, GG, LL, true>(p, nQ / GG, early, s);     \
+    else launch_decode_short<DD, GG, LL, false>(p, nQ / GG, early, s);                            \
   }
     KVM_DEC_SHORT(128, 1, false) KVM_DEC_SHORT(128, 2, false) KVM_DEC_SHORT(64, 1, false) KVM_DEC_SHORT(64, 2, false)
     KVM_DEC_SHORT(128, 1, true) KVM_DEC_SHORT(128, 2, true) KVM_DEC_SHORT(64, 1, true) KVM_DEC_SHORT(64, 2, true)
 #undef KVM_DEC_SHORT
     return 1;
   }
+  const DecodePlan pl = plan_decode(nQ, st->G, st->d, p.n);
+  const int GQ = pl.heads;
+  p.nsplit = pl.splits; p.nclus = pl.clusters;
 #define KVM_DEC_GO(DD, GG, LL, MM) \
   if (st->d == DD && GQ == GG && st->fusedLn == LL && (pl.clusters > 1) == MM) launch_decode_step<DD, GG, LL, MM>(p, nQ / GQ, early, s);
   KVM_DEC_EACH(KVM_DEC_GO, true)

@@ -2160,12 +2160,17 @@ __global__ void __launch_bounds__(256) refresh_rows_kernel(RefreshParams p) {
 // 2.14, 2.20; 128 2.49, 2.61; 160 3.19, 3.60; blocks of 64 and 128, 64 to 224 units: one is up to 12 % faster, nowhere more than 1 %
 // slower.  64 channels, 256 rows, blocks of 256: 48 units 1.21, 1.25; 64 1.25, 1.18; 148 2.04, 1.86; 224 2.98, 2.80; of 128: 48 units
 // 0.653, 0.630; 64 0.733, 0.705; 128 1.08, 0.98; 192 1.44, 1.34; of 64: 64 units 0.608, 0.629; 96 0.773, 0.712; 224 1.10, 1.06.
-static bool apply_uses_rows4(const State* st) {
-  const int64_t rows = (int64_t)st->C * st->U;
-  if (st->recomputeK) return true;
-  if (st->d == 64) return st->C > 128 ? rows > 12288 : rows >= 6144;
-  return st->C > 128 && rows > 16384 && st->U < 128;
+// CTAs per unit of the four-rows kernel: one when the units alone fill the GPU's CTA slots (measured at 256 and 2048 units: 1 beats
+// 2, 4 and 8), four where they nearly do (64 channels, 256 rows, one and four: 160 units 2.28, 2.12 ms; 192 2.59, 2.46; 224
+// 2.85, 2.80), else enough to fill them; at most one per 32 row slots.
+ApplyPlan plan_apply(int64_t units, int d, int C, bool recompute) {
+  const int64_t rows = (int64_t)C * units;
+  const bool four = recompute || (d == 64 ? (C > 128 ? rows > 12288 : rows >= 6144) : C > 128 && rows > 16384 && units < 128);
+  if (!four) return {1, (C + 7) / 8};
+  const int64_t fill = units > 148 && !recompute ? 4 : 2 * 148 / units;
+  return {4, (int)std::max<int64_t>(1, std::min<int64_t>(fill, (C + kApplyRowsPerCta - 1) / kApplyRowsPerCta))};
 }
+static ApplyPlan plan_apply(const State* st) { return plan_apply(st->U, st->d, st->C, st->recomputeK); }
 
 int launch_refresh_rows(State* st, int64_t m, cudaStream_t s) {
   if (m <= 0) return 0;
@@ -2175,7 +2180,7 @@ int launch_refresh_rows(State* st, int64_t m, cudaStream_t s) {
   p.Khat0 = st->KhatBuf[0]; p.Vhat0 = st->VhatBuf[0]; p.Khat1 = st->KhatBuf[1]; p.Vhat1 = st->VhatBuf[1];
   p.Mcap = st->Mcap; p.m = m; p.Hkv = st->Hkv; p.radius_on = (st->flags & KVM_FLAG_NO_RADIUS) ? 0 : 1;
   p.ln_eps = (double)st->ln_eps; p.norm_eps = (double)st->norm_eps;
-  if (apply_uses_rows4(st)) {
+  if (plan_apply(st).rows_per_warp == 4) {
     dim3 grid((unsigned)((m + kApplyRowsPerCta - 1) / kApplyRowsPerCta), st->U);
     if (st->d == 128) refresh_rows_kernel<128, true><<<grid, 256, 0, s>>>(p);
     else refresh_rows_kernel<64, true><<<grid, 256, 0, s>>>(p);
@@ -2362,16 +2367,13 @@ int launch_fold(State* st, const FoldArgs& a, cudaStream_t s) {
   q.ln_eps = (double)st->ln_eps; q.norm_eps = (double)st->norm_eps;
   if (a.before_apply && cudaStreamWaitEvent(s, a.before_apply, 0) != cudaSuccess) return -1000000;
   KernelTimer kt(st, 5, s);
-  if (apply_uses_rows4(st)) {
-    // CTAs per unit: one when the units alone fill the GPU's CTA slots (measured at 256 and 2048 units: 1 beats
-    // 2, 4 and 8), four where they nearly do (64 channels, 256 rows, one and four: 160 units 2.28, 2.12 ms; 192 2.59, 2.46; 224
-    // 2.85, 2.80), else enough to fill them; at most one per 32 row slots
-    const int R = std::max(1, std::min(st->U > 148 && !st->recomputeK ? 4 : 2 * 148 / st->U, (C + kApplyRowsPerCta - 1) / kApplyRowsPerCta));
-    dim3 grid(R, st->U);
+  const ApplyPlan pl = plan_apply(st);
+  if (pl.rows_per_warp == 4) {
+    dim3 grid(pl.ctas, st->U);
     if (D == 128) { if (st->recomputeK) fold_apply_rows4_kernel<128, true><<<grid, 256, 0, s>>>(q); else fold_apply_rows4_kernel<128, false><<<grid, 256, 0, s>>>(q); }
     else { if (st->recomputeK) fold_apply_rows4_kernel<64, true><<<grid, 256, 0, s>>>(q); else fold_apply_rows4_kernel<64, false><<<grid, 256, 0, s>>>(q); }
   } else {
-    dim3 grid((C + 7) / 8, st->U);
+    dim3 grid(pl.ctas, st->U);
     if (D == 128) fold_apply_kernel<128><<<grid, 256, 0, s>>>(q);
     else fold_apply_kernel<64><<<grid, 256, 0, s>>>(q);
   }

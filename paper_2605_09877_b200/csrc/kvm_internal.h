@@ -90,8 +90,8 @@ struct State {
   //      call computes them for up to kbSlots consecutive overflow blocks in one launch; slot g holds
   //      one block's arrays in the layouts below ----
   int kbSlots;
-  bool recomputeK;               // (bound with the block) serial && the four-rows-per-warp apply kernel: kbar64 is not kept,
-                                 // the fold kernels recompute kbar_j from the fp16 key and kbarStat
+  bool recomputeK;               // (bound with the block: recomputes_keys) kbar64 is not kept, the fold kernels recompute kbar_j
+                                 // from the fp16 key and kbarStat (the apply kernel with four rows per warp)
   double2* kbarStat;             // [kbSlots][U, Cmax]  (mean, rstd) of zero_r(k_j)
   double* kbar64;                // [kbSlots][U, Cmax, d]
   __half* kbarH;                 // [kbSlots][U, CbarRows, d]
@@ -166,6 +166,8 @@ struct AttnArgs {
   int64_t so[4];       // out strides
   int64_t out_t0;      // token index inside `out` of the first query
 };
+struct AttnPlan { int n_whole, nsp_rest; };   // (batch, head, query tile) CTAs that run whole, key splits of each of the others
+AttnPlan plan_attn(int64_t tiles, int64_t m);
 int launch_attn_simt(State* st, const AttnArgs& a, cudaStream_t s);
 int launch_attn_tc(State* st, const AttnArgs& a, cudaStream_t s);
 bool setup_attn_tc(State* st);   // encodes the tensor maps, raises the shared-memory limits
@@ -191,6 +193,8 @@ struct FoldArgs {
                               // kernel is not the one that writes those keys
 };
 int launch_fold(State* st, const FoldArgs& a, cudaStream_t s);
+struct ApplyPlan { int rows_per_warp, ctas; };   // one or four touched rows per warp, CTAs per unit
+ApplyPlan plan_apply(int64_t units, int d, int C, bool recompute);
 // Memory keys of nblk consecutive blocks (C rows each, starting at ok within every unit) into slots
 // slot0 .. slot0 + nblk - 1.
 int launch_kbar(State* st, const __half* ok, int64_t unit_stride, int nblk, int slot0, bool want_gram, cudaStream_t s);
@@ -212,6 +216,8 @@ struct DecodeArgs {
 int launch_decode(State* st, const DecodeArgs& a, cudaStream_t s);
 struct DecodePlan { int heads, splits, clusters; };   // query heads per CTA, CTAs per cluster, clusters per group of heads
 DecodePlan plan_decode(int n_q, int group, int d, int64_t n_rows);
+struct DecodeShortPlan { int heads, splits, rows_per_warp; };   // a step that fetches its rows ahead; splits == 0: plan_decode
+DecodeShortPlan plan_decode_short(int n_q, int group, int d, int64_t n_rows);
 
 // Self test of the bounded waits: one thread waits `spins` iterations on a barrier nobody arrives at and
 // records KVM_ERR_TIMEOUT in the status word.

@@ -27,7 +27,8 @@ EXPORTS = ["kvm_plan_capacity", "kvm_state_create", "kvm_prefill", "kvm_decode_s
            "kvm_debug_assignments", "kvm_launch_count", "kvm_status_string", "kvm_state_reset",
            "kvm_profile_enable", "kvm_profile_read", "kvm_debug_counters", "kvm_attend_rows_noalloc", "kvm_merge_gate", "kvm_head_layernorm",
            "kvm_state_snapshot_info", "kvm_state_export_window", "kvm_state_import", "kvm_debug_expire_wait",
-           "kvm_debug_decode_plan", "kvm_debug_drop_exchange"]
+           "kvm_debug_decode_plan", "kvm_debug_decode_ahead", "kvm_debug_apply_plan", "kvm_debug_attention_plan",
+           "kvm_debug_drop_exchange"]
 
 
 class KVMError(RuntimeError):
@@ -111,6 +112,12 @@ def _load():
     L.kvm_debug_drop_exchange.argtypes = [vp, C.c_int32]
     L.kvm_debug_decode_plan.restype = C.c_int
     L.kvm_debug_decode_plan.argtypes = [C.c_int32, C.c_int32, C.c_int32, C.c_int32, C.c_int64, C.POINTER(C.c_int32)]
+    L.kvm_debug_decode_ahead.restype = C.c_int
+    L.kvm_debug_decode_ahead.argtypes = [C.c_int32, C.c_int32, C.c_int32, C.c_int32, C.c_int64, C.POINTER(C.c_int32)]
+    L.kvm_debug_apply_plan.restype = C.c_int
+    L.kvm_debug_apply_plan.argtypes = [C.c_int64, C.c_int32, C.c_int32, C.c_int32, C.POINTER(C.c_int32)]
+    L.kvm_debug_attention_plan.restype = C.c_int
+    L.kvm_debug_attention_plan.argtypes = [C.c_int32, C.c_int32, C.c_int32, C.c_int64, C.POINTER(C.c_int32)]
     L.kvm_debug_expire_wait.restype = C.c_int
     L.kvm_debug_expire_wait.argtypes = [vp, C.c_int32, vp]
     L.kvm_head_layernorm.restype = C.c_int
@@ -170,14 +177,34 @@ def head_layernorm(x: "torch.Tensor", weight=None, bias=None, eps: float = 1e-5,
     return x
 
 
-def decode_plan(batch: int, n_q_heads: int, n_kv_heads: int, head_dim: int, n_rows: int):
-    """(query heads per CTA, CTAs per cluster, clusters per group of heads) of a decode step over n_rows rows, where it runs the
-    kernel that loops over them (few heads over few rows are cut otherwise)."""
-    out = (C.c_int32 * 3)()
-    rc = lib.kvm_debug_decode_plan(batch, n_q_heads, n_kv_heads, head_dim, n_rows, out)
+def _plan(fn, n, *args):
+    out = (C.c_int32 * n)()
+    rc = getattr(lib, fn)(*args, out)
     if rc != KVM_OK:
-        raise KVMError(rc, "kvm_debug_decode_plan")
+        raise KVMError(rc, fn)
     return tuple(out)
+
+
+def decode_plan(batch: int, n_q_heads: int, n_kv_heads: int, head_dim: int, n_rows: int):
+    """(query heads per CTA, CTAs per cluster, clusters per group of heads) of a decode step over n_rows rows in the kernel that
+    loops over them (decode_ahead says whether the step runs that one)."""
+    return _plan("kvm_debug_decode_plan", 3, batch, n_q_heads, n_kv_heads, head_dim, n_rows)
+
+
+def decode_ahead(batch: int, n_q_heads: int, n_kv_heads: int, head_dim: int, n_rows: int):
+    """(CTAs per group of query heads, query heads per CTA, rows per warp) of a decode step over n_rows rows in the kernel that
+    fetches its rows ahead; (0, 0, 0): the step runs the kernel that loops over them."""
+    return _plan("kvm_debug_decode_ahead", 3, batch, n_q_heads, n_kv_heads, head_dim, n_rows)
+
+
+def apply_plan(n_units: int, head_dim: int, block: int, serial: bool = False):
+    """(rows per warp, CTAs per unit) of the kernel that writes the rows a fold touches."""
+    return _plan("kvm_debug_apply_plan", 2, n_units, head_dim, block, 1 if serial else 0)
+
+
+def attention_plan(batch: int, n_q_heads: int, n_queries: int, n_slots: int):
+    """(CTAs that run whole, key splits of each of the others) of the attention of n_queries tokens over n_slots rows."""
+    return _plan("kvm_debug_attention_plan", 2, batch, n_q_heads, n_queries, n_slots)
 
 
 def kvm_plan_capacity(block: int, n_bswa_chunks: int, g: Growth, seq_len: int) -> int:

@@ -1,5 +1,5 @@
-"""How a decode step is cut into CTAs (host arithmetic, no GPU): splits that fill the GPU where a few heads meet many rows,
-no empty split inside a single cluster, and merge scratch that holds every plan."""
+"""How a decode step, the rows of a fold and an attention launch are cut into CTAs (host arithmetic, no GPU): splits that fill the GPU
+where a few heads meet many rows, no empty split inside a single cluster, and merge scratch that holds every plan."""
 import pytest
 
 from paper_2605_09877_b200 import kvm
@@ -39,7 +39,57 @@ def test_plans_over_the_range():
                         assert d % (heads * d // splits) == 0
 
 
+def test_steps_that_fetch_ahead_cover_their_rows():
+    """The warps of the cluster cover every row, in one pass or two, and a CTA takes one head, or two of the same group."""
+    for d in (64, 128):
+        rows1 = 256 // d
+        for G in (1, 2, 3, 4, 6, 8):
+            for units in (1, 2, 7, 8, 12, 16, 17, 31, 33, 53, 90, 148, 296, 300):
+                for n in list(range(1, 200, 13)) + [256, 257, 500, 800, 1023, 1024, 1025, 1500, 2048, 2049, 3000, 4096, 4097]:
+                    splits, heads, rpw = kvm.decode_ahead(units, G, 1, d, n)
+                    if splits == 0:
+                        assert (heads, rpw) == (0, 0)
+                        continue
+                    assert 1 <= splits <= 8 and heads == (2 if G % 2 == 0 else 1) and rpw % rows1 == 0
+                    assert rpw * 8 * splits >= n and rpw <= 2 * 8 * rows1
+
+
+def test_key_splits_of_the_attention_have_keys_and_a_place_in_the_scratch():
+    """37 * 8 partial results of a tile, 2 * 37 tickets, and a split has a key tile of the state or the window."""
+    for tiles in list(range(1, 600)) + [1000, 4096]:
+        for m in (0, 64, 128, 256, 300, 512, 1000, 1152, 1280, 2048, 2304, 2560, 4096, 50000):
+            whole, splits = kvm.attention_plan(1, tiles, 128, m)
+            rest = tiles - whole
+            assert 1 <= splits <= 8 and 0 <= whole <= tiles
+            if splits > 1:
+                assert 0 < rest <= 2 * 37 and rest * splits <= 37 * 8 and splits <= (m + 127) // 128 + 1
+            else:
+                assert rest == 0
+    assert kvm.attention_plan(2, 5, 200, 700) == kvm.attention_plan(1, 20, 128, 700)
+
+
+def test_states_without_stored_keys_take_four_rows_per_warp():
+    """Only that kernel recomputes the keys, and its CTAs cover the rows of a block."""
+    for units in (1, 16, 31, 32, 63, 64, 100, 148, 149, 200, 255, 256, 257, 2048):
+        for d in (64, 128):
+            for C in (8, 64, 128, 136, 256):
+                for serial in (False, True):
+                    per_warp, ctas = kvm.apply_plan(units, d, C, serial)
+                    assert per_warp in (1, 4) and 1 <= ctas <= (C + 7) // 8
+                    assert per_warp == 4 or ctas == (C + 7) // 8
+                    if (serial or units >= 256) and C * units >= 8192:
+                        assert per_warp == 4
+
+
 def test_plan_refuses_what_a_state_refuses():
     for bad in [(0, 1, 1, 64, 10), (1, 3, 2, 64, 10), (1, 2, 2, 96, 10), (1, 2, 2, 64, 0)]:
         with pytest.raises(kvm.KVMError):
             kvm.decode_plan(*bad)
+        with pytest.raises(kvm.KVMError):
+            kvm.decode_ahead(*bad)
+    for bad in [(0, 64, 64), (1, 96, 64), (1, 64, 60), (1, 64, 264)]:
+        with pytest.raises(kvm.KVMError):
+            kvm.apply_plan(*bad)
+    for bad in [(0, 1, 1, 1), (1, 0, 1, 1), (1, 1, 0, 1), (1, 1, 1, -1)]:
+        with pytest.raises(kvm.KVMError):
+            kvm.attention_plan(*bad)

@@ -450,9 +450,9 @@ def test_crowded_runs_are_compared_pair_by_pair(Hkv, d, C):
 ])
 def test_rows_with_many_members_in_both_apply_kernels(B, Hkv, d, C, slots, rows4):
     """The kernel that a state's folds run to write the touched rows, at rows with none, one and many members, appended rows
-    among them; the state means and readout rows against the oracle, and again after a snapshot's import."""
-    rows = C * B * Hkv
-    assert rows4 == ((rows > 12288 if C > 128 else rows >= 6144) if d == 64 else C > 128 and rows > 16384 and B * Hkv < 128)
+    among them; the state means and readout rows against the oracle."""
+    from paper_2605_09877_b200 import kvm
+    assert (kvm.apply_plan(B * Hkv, d, C)[0] == 4) == rows4
     wl = synth.Workload("t", B, Hkv, Hkv, d, C * 5 + 11, C, "fixed", fixed_slots=slots, r=32, seed=61, kind="mixture")
     params = synth.make_layer_params(wl, trivial=False)
     units = sorted({(0, 0), (B - 1, Hkv - 1)})
@@ -460,27 +460,19 @@ def test_rows_with_many_members_in_both_apply_kernels(B, Hkv, d, C, slots, rows4
     print(stats)
 
 
-@pytest.mark.parametrize("Hq,Hkv,d,blocks", [(8, 8, 128, 21), (16, 4, 128, 22), (24, 8, 64, 23), (3, 3, 128, 25)])
-def test_attention_of_few_heads_over_many_rows_splits_the_keys(Hq, Hkv, d, blocks):
-    """Key splits of launches of 6 to 48 tiles over 10 to 40 key tiles: two to eight splits, ragged last ones."""
+@pytest.mark.parametrize("Hq,Hkv,d,blocks,splits", [
+    (8, 8, 128, 21, {1, 2, 3, 4, 5}), (16, 4, 128, 22, {1, 2, 3}), (24, 8, 64, 23, {1, 2}), (3, 3, 128, 25, {1, 2, 3, 4, 5, 6})])
+def test_attention_of_few_heads_over_many_rows_splits_the_keys(Hq, Hkv, d, blocks, splits):
+    """Key splits of launches of 6 to 48 tiles over 1 to 49 key tiles, ragged last ones."""
+    from paper_2605_09877_b200 import kvm
+    assert {kvm.attention_plan(1, Hq, 256, 256 * max(b - 1, 0))[1] for b in range(blocks + 1)} == splits
     wl = synth.Workload("t", 1, Hq, Hkv, d, 256 * blocks + 70, 256, "unbounded", r=32, seed=62)
     print(_sampled(wl, [(0, 0), (0, Hkv - 1)]))
 
 
-def _short_splits(n_q, group, d, n):
-    """CTAs per cluster of the decode kernel that fetches its rows ahead (0: the step is not one of its)."""
-    groups, cta = (n_q // 2 if group % 2 == 0 else n_q), 64 * (256 // d)
-    fit = (296, 148, 88, 71, 56, 45, 37, 33)
-    if groups > fit[0] or n > 16 * cta:
-        return 0
-    ns = -(-n // cta)
-    ns = 8 if ns > 8 or 8 <= groups <= 16 else ns
-    return ns if groups <= fit[ns - 1] else 0
-
-
 @pytest.mark.parametrize("Hq,Hkv,d,C,slots,r,splits", [
     (1, 1, 64, 16, 40, 0, {1}), (3, 1, 128, 16, 80, 32, {1}), (2, 2, 128, 32, 170, 32, {2}), (2, 1, 128, 64, 300, 64, {3, 4}),
-    (5, 5, 64, 64, 960, 16, {4, 5}), (4, 2, 128, 64, 600, 0, {6}), (3, 3, 128, 64, 700, 32, {6, 7}), (12, 12, 64, 32, 300, 0, {8}),
+    (5, 5, 64, 64, 960, 16, {5}), (4, 2, 128, 64, 600, 0, {6}), (3, 3, 128, 64, 700, 32, {6, 7}), (12, 12, 64, 32, 300, 0, {8}),
     (24, 12, 128, 64, 900, 32, {8}), (33, 33, 128, 64, 930, 0, {8}),
     (2, 2, 128, 64, 1500, 32, {8}), (1, 1, 64, 256, 3500, 0, {8}), (66, 33, 64, 64, 2700, 32, {8}),   # two passes over a warp's rows
 ])
@@ -489,7 +481,8 @@ def test_decode_steps_that_fetch_their_rows_ahead(Hq, Hkv, d, C, slots, r, split
     which each fetches what the ones before leave complete, against the oracle and against steps that are waited for."""
     start = (slots // C + 4) * C - 6
     wl = synth.Workload("short", 1, Hq, Hkv, d, start + 14, C, "fixed", fixed_slots=slots, r=r, seed=400 + slots)
-    assert {_short_splits(Hq, Hq // Hkv, d, _decode_rows(wl, t)) for t in range(start, wl.T)} <= splits
+    from paper_2605_09877_b200 import kvm
+    assert {kvm.decode_ahead(1, Hq, Hkv, d, _decode_rows(wl, t))[0] for t in range(start, wl.T)} == splits
     params = synth.make_layer_params(wl, trivial=False)
     tensors = synth.make_inputs(wl)
     y, st = pu.run_gpu(wl, tensors, params, decode_from=start)
