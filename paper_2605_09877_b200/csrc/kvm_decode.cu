@@ -734,23 +734,37 @@ static bool launch_decode_step(const DecodeParams& p, int ncta, bool early, cuda
   return cudaLaunchKernelEx(&lc, decode_step_kernel<D, GQ, LN, MULTI>, p) == cudaSuccess;
 }
 
-// CTAs per cluster of decode_short_kernel for a step over n rows, 0 where decode_step_kernel is the better one.  kFit: clusters of 1
-// to 8 CTAs that the GPU holds at once at two CTAs per SM: more would be another wave, which costs more than the early loads
-// save (us per step, loop kernel and this: 48 heads, 900 rows in 8 splits 7.4, 12; 128 heads on 32, 600 rows 9.0, 14; 93 heads in 3
-// splits, which fill the GPU to the last cluster, 7.1, 7.9: 88 there).  The fewest splits whose
-// warps have all their rows in flight at once, one pass; 8 for 8 to 16 groups of heads, where two steps fit beside each other
-// (16 heads, 600 rows 4.5, 4.3); two passes of 8 splits while those fit (8 heads, 1400 rows 6.7, 5.9; 32 heads 8.6, 8.1; three: 8
-// heads, 2400 rows 8.2, 8.8).  Two query heads of a kv head per CTA, not four: 32 on 8, 900 rows 6.2, 5.4.
+// CTAs per cluster of decode_short_kernel for a step over n rows, 0 where decode_step_kernel is the better one.  Measured: us per step,
+// the loop and this, steps of a block in a graph (launched one by one the host is the longer side up to 5.8 us).
+// kFit: clusters of 1 to 8 CTAs up to which this is the faster one; the GPU holds 296, 148, 93, 71, 56, 45, 37, 33 at two CTAs per SM, and
+// the last ones cost what the early loads save (single heads, 630 rows in 5 splits: 52 6.59, 5.77; 53 6.60, 6.08; 55 6.61, 6.88; 56
+// 6.60, 7.35; 890 rows in 7: 36 6.68, 6.20; 37 6.67, 6.79; 1020 in 8: 32 6.84, 5.90; 33 6.85, 7.15; 296 in one 5.57, 4.62; 148 in two
+// 6.82, 6.12; 71 in four 6.37, 5.76).  Two heads per CTA, where the loop has no more of 128 channels: 52 in 5 6.88, 7.06; 36 in 7 7.55,
+// 8.12; 32 in 8 6.91, 7.23; 30 6.67, 6.07.
+// The fewest splits whose warps have all their rows in flight at once, one pass; 8 for 8 to 16 groups of heads, where two steps
+// fit beside each other, from the rows on that pay for the exchange (16 heads, 40 rows in one split and in 8: 2.90, 3.55; 90 rows 3.17,
+// 3.55; 240 rows in two 3.88, 3.60; 700 rows in 6 3.97, 3.74; 12 pairs, 60 rows in one 3.3, 4.7; 200 in two 4.2, 4.7).
+// Two passes of 8 splits (8 heads, 1300 rows 6.21, 5.00; 32 heads 8.04, 7.33; three: 8 heads, 2400 rows 8.2, 8.8) up to 32 single heads
+// (1800 rows 9.14, 8.48; 33 9.11, 9.13; 1950 rows, where the loop's last pass is nearly full, 16 heads 7.21, 7.44, 32 9.06, 9.33) and 20
+// pairs (1600 rows 8.93, 8.11; 24 at 1500 7.53, 8.06), but for pairs over 10.5 to 12 passes, the end of the loop's third (20 pairs, 1300
+// rows 8.07, 7.67; 1400 7.37, 7.66; 1500 7.56, 7.99).  Where the loop takes four or eight heads per CTA two are better all along: 32 on 8, 900 rows 6.2,
+// 5.4; 64 on 8, 2000 rows 10.97, 9.31.
 DecodeShortPlan plan_decode_short(int nQ, int G, int d, int64_t n) {
-  static const int kFit[kDecodeCluster] = {296, 148, 88, 71, 56, 45, 37, 33};
+  static const int kFit[2][kDecodeCluster] = {{296, 148, 88, 71, 53, 45, 36, 32}, {296, 148, 88, 71, 51, 45, 35, 30}};
   const int heads = G % 2 == 0 ? 2 : 1, groups = nQ / heads;
+  const bool same = G % 4 != 0;             // the loop has as many heads per CTA
   const int rows1 = 256 / d;                // rows that a warp loads at once
   const int64_t pass = 8 * 8 * rows1;       // rows of a CTA in one pass
-  if (groups > kFit[0] || n > 2 * kDecodeCluster * pass) return {0, 0, 0};
-  int ns = (int)((n + pass - 1) / pass);
-  if (ns > kDecodeCluster || (groups >= 8 && groups <= 16)) ns = kDecodeCluster;
-  if (groups > kFit[ns - 1]) return {0, 0, 0};
-  return {heads, ns, ((int)(n + 8 * ns - 1) / (8 * ns) + rows1 - 1) / rows1 * rows1};
+  int64_t ns = (n + pass - 1) / pass;
+  if (ns > 2 * kDecodeCluster) return {0, 0, 0};
+  if (ns > kDecodeCluster) {
+    if (same && (heads == 1 ? groups > 32 : groups > 20 || (2 * n > 21 * pass && ns <= 12))) return {0, 0, 0};
+    ns = kDecodeCluster;
+  } else if (groups >= 8 && groups <= 16 && ns >= 2 * heads) {
+    ns = kDecodeCluster;
+  }
+  if (groups > kFit[heads == 2 && same && d == 128][ns - 1]) return {0, 0, 0};
+  return {heads, (int)ns, (int)(((n + 8 * ns - 1) / (8 * ns) + rows1 - 1) / rows1 * rows1)};
 }
 
 // How a step over n rows is cut.  Query heads per CTA (they share a kv head): the largest of 8, 4, 2, 1 that divides the group

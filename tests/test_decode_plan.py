@@ -54,6 +54,20 @@ def test_steps_that_fetch_ahead_cover_their_rows():
                     assert rpw * 8 * splits >= n and rpw <= 2 * 8 * rows1
 
 
+@pytest.mark.parametrize("Hq,Hkv,d,n,splits", [
+    # few rows: no more splits than hold them, also for 8 to 16 groups of heads
+    (16, 16, 128, 40, 1), (12, 12, 64, 80, 1), (8, 8, 128, 128, 1), (16, 16, 128, 129, 8), (24, 4, 128, 60, 1), (24, 4, 128, 200, 2),
+    (32, 8, 64, 250, 1), (32, 8, 128, 400, 8), (17, 17, 128, 400, 4),
+    # clusters that would fill the GPU to the last one are the loop's
+    (53, 53, 128, 630, 5), (54, 54, 128, 630, 0), (56, 56, 64, 1260, 0), (36, 36, 128, 890, 7), (37, 37, 128, 890, 0), (32, 32, 128, 1020, 8),
+    (33, 33, 128, 1020, 0), (60, 30, 128, 1010, 8), (64, 32, 128, 1010, 0), (64, 32, 64, 2020, 8), (64, 16, 128, 1010, 8), (72, 36, 128, 880, 0),
+    # two passes
+    (32, 32, 128, 1500, 8), (33, 33, 128, 1500, 0), (40, 20, 128, 1300, 8), (40, 20, 128, 1400, 0), (40, 20, 128, 1500, 0), (40, 20, 128, 1600, 8), (48, 8, 128, 1500, 0), (64, 32, 128, 2000, 0),
+    (64, 8, 128, 2000, 8), (64, 16, 64, 4000, 8), (1, 1, 128, 2048, 8), (1, 1, 128, 2049, 0)])
+def test_steps_that_fetch_ahead_where_that_is_the_faster_kernel(Hq, Hkv, d, n, splits):
+    assert kvm.decode_ahead(1, Hq, Hkv, d, n)[0] == splits
+
+
 def test_key_splits_of_the_attention_have_keys_and_a_place_in_the_scratch():
     """37 * 8 partial results of a tile, 2 * 37 tickets, and a split has a key tile of the state or the window."""
     for tiles in list(range(1, 600)) + [1000, 4096]:

@@ -473,8 +473,9 @@ def test_attention_of_few_heads_over_many_rows_splits_the_keys(Hq, Hkv, d, block
 @pytest.mark.parametrize("Hq,Hkv,d,C,slots,r,splits", [
     (1, 1, 64, 16, 40, 0, {1}), (3, 1, 128, 16, 80, 32, {1}), (2, 2, 128, 32, 170, 32, {2}), (2, 1, 128, 64, 300, 64, {3, 4}),
     (5, 5, 64, 64, 960, 16, {5}), (4, 2, 128, 64, 600, 0, {6}), (3, 3, 128, 64, 700, 32, {6, 7}), (12, 12, 64, 32, 300, 0, {8}),
-    (24, 12, 128, 64, 900, 32, {8}), (33, 33, 128, 64, 930, 0, {8}),
-    (2, 2, 128, 64, 1500, 32, {8}), (1, 1, 64, 256, 3500, 0, {8}), (66, 33, 64, 64, 2700, 32, {8}),   # two passes over a warp's rows
+    (24, 12, 128, 64, 900, 32, {8}), (32, 32, 128, 64, 930, 0, {8}),
+    (16, 16, 128, 16, 60, 32, {1}), (24, 12, 64, 64, 300, 32, {2}),
+    (2, 2, 128, 64, 1500, 32, {8}), (1, 1, 64, 256, 3500, 0, {8}), (40, 20, 64, 64, 2500, 32, {8}),   # two passes over a warp's rows
 ])
 def test_decode_steps_that_fetch_their_rows_ahead(Hq, Hkv, d, C, slots, r, splits):
     """One to eight CTAs per group of heads, one and two passes, warps with few rows or none; steps back to back across a fold, of
