@@ -527,9 +527,12 @@ KVM_API kvm_status_t kvm_debug_apply_plan(int64_t n_units, int32_t head_dim, int
   return KVM_OK;
 }
 
-KVM_API kvm_status_t kvm_debug_attention_plan(int32_t batch, int32_t n_q_heads, int32_t n_queries, int64_t n_slots, int32_t* out) {
-  if (batch < 1 || n_q_heads < 1 || n_queries < 1 || n_slots < 0 || !out) return KVM_ERR_INVALID_ARG;
-  const AttnPlan p = plan_attn((int64_t)batch * n_q_heads * ((n_queries + 127) / 128), n_slots);
+KVM_API kvm_status_t kvm_debug_attention_plan(int32_t batch, int32_t n_q_heads, int32_t n_kv_heads, int32_t head_dim,
+                                              int32_t n_queries, int64_t n_slots, int32_t decides, int32_t* out) {
+  if (batch < 1 || n_q_heads < 1 || n_kv_heads < 1 || n_q_heads % n_kv_heads || n_slots < 0 || !out) return KVM_ERR_INVALID_ARG;
+  if (n_queries < 1 || n_queries > kMaxBlock) return KVM_ERR_INVALID_ARG;
+  if (head_dim != 64 && head_dim != 128) return KVM_ERR_UNSUPPORTED;
+  const AttnPlan p = plan_attn((int64_t)batch * n_q_heads * ((n_queries + 127) / 128), decides && n_q_heads == n_kv_heads, head_dim, n_slots);
   out[0] = p.n_whole; out[1] = p.nsp_rest;
   return KVM_OK;
 }
@@ -667,6 +670,7 @@ KVM_API kvm_status_t kvm_prefill(const void* q, const void* k, const void* v, kv
     int64_t b = e - L; if (b < 0) b = 0;
     aa.q_row0 = qs - pos0; aa.nq = (int)(qe - qs); aa.t0 = qs; aa.m = s.m;
     aa.win_row0 = b - ia.hist_start; aa.b = b; aa.out = (__nv_bfloat16*)out; aa.out_t0 = qs - pos0;
+    aa.fold_decides = qe == e && c >= s.w - 1 && s.m > 0 && fold_na[n_done_folds] < C;
     if (ovf && fold_pending >= 0) {
       ev_ok = ev_ok && cudaStreamWaitEvent(stream, s.evFold[fold_pending], 0) == cudaSuccess;
       fold_pending = -1;

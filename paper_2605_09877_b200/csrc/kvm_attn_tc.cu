@@ -558,15 +558,24 @@ bool encode_tmap_rows(CUtensorMap* map, const void* base, int d, int64_t rows, i
             CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
-// Key splits of a launch of `tiles` CTAs over m state rows.  Few query tiles: up to a quarter of the GPU (the folds of the block before
-// run beside this kernel and are usually the longer chain), at least two key tiles per split; up to three quarters where a split
-// still has nine or so, for there the attention is the longer chain (ms, a quarter and as chosen: 16 heads on 4, 65536 tokens 12.1, 8.64;
-// 8 heads 10.4, 9.0; 16 heads, 4096 rows, 32768 tokens 7.31, 5.37.  Three quarters where splits have two or three tiles: 24 heads on 8,
-// 512 rows, 3.04, 3.24).  Many tiles: when the last wave of one-CTA-per-SM would be less than half full, its tiles are split
+// Key splits of a launch of `tiles` CTAs over m state rows of d channels; `beside`: each unit's one query head attends beside a fold that
+// decides on as many tokens.
+// Few query tiles: up to a quarter of the GPU (the folds of the block before run beside this kernel and are usually the longer
+// chain), at least two key tiles per split; up to three quarters from ten key tiles on, a split for every nine begun, for there the
+// attention is the longer chain (ms, a quarter and as chosen: 16 heads on 4, 65536 tokens 12.1, 8.64; 8 heads 10.4, 9.0).  Beside folds as wide
+// two splits of 40 tiles and more take the SMs that those need, and pay only from more key tiles on.  Measured, with splits from ten
+// key tiles over without, 24 blocks of full states: 16 heads, blocks of 256, 1536 rows 0.91, 2560 0.86; 20 heads 1.01, 0.95; 24 heads 1152 rows
+// 1.08, 1792 1.04, 2048 1.01, 2560 0.98; 48 heads, blocks of 128, 1152 rows 1.09, 1792 1.03, 2560 1.00; 54 heads 1.05, 1.08, 1.05; blocks of 64
+// 1.04, 1.04, 1.00; 64 channels: 24 heads, blocks of 256, 1152 rows 1.04, 1536 0.99; 54 heads, blocks of 128, 1152 rows 1.04, 1792 1.02, 2048
+// 1.01.  Two heads per unit: 22 units, blocks of 128, 1536 rows 0.92; 24 units 0.97.
+// Many tiles: when the last wave of one-CTA-per-SM would be less than half full, its tiles are split
 // in two (the partial-result buffer holds 2 * kAttnSplitTiles tiles of two splits).
-AttnPlan plan_attn(int64_t tiles, int64_t m) {
+AttnPlan plan_attn(int64_t tiles, bool beside, int d, int64_t m) {
   const int64_t ntot_min = (m + 127) / 128 + 1;
-  int64_t nsp = std::max(std::min(kAttnSplitTiles / tiles, ntot_min / 2), std::min(3 * kAttnSplitTiles / tiles, (ntot_min + 8) / 9));
+  int64_t from = 10;
+  if (beside && tiles >= 40) from = tiles < 44 ? (d == 64 ? 10 : 15) : tiles <= 48 ? (d == 64 ? 13 : 17) : (d == 64 ? 17 : 23);
+  int64_t nsp = std::min(kAttnSplitTiles / tiles, ntot_min / 2);
+  if (ntot_min >= from) nsp = std::max(nsp, std::min(3 * kAttnSplitTiles / tiles, (ntot_min + 8) / 9));
   nsp = std::max<int64_t>(1, std::min<int64_t>(nsp, kAttnMaxSplits));
   if (nsp > 1) return {0, (int)nsp};
   const int64_t rem = tiles % 148;
@@ -587,7 +596,7 @@ int launch_attn_tc(State* st, const AttnArgs& a, cudaStream_t s) {
   p.out_vec = (reinterpret_cast<uintptr_t>(a.out) % 16 == 0 && a.so[0] % 8 == 0 && a.so[1] % 8 == 0 && a.so[2] % 8 == 0) ? 1 : 0;
   const int qtiles = (a.nq + 127) / 128;
   const int tiles = qtiles * st->B * st->Hq;
-  const AttnPlan pl = plan_attn(tiles, a.m);
+  const AttnPlan pl = plan_attn(tiles, a.fold_decides && st->G == 1, st->d, a.m);
   p.qtiles = qtiles; p.n_whole = pl.n_whole; p.nsp_rest = pl.nsp_rest;
   dim3 grid(pl.n_whole + (tiles - pl.n_whole) * pl.nsp_rest);
   const CUtensorMap* tm = reinterpret_cast<const CUtensorMap*>(st->tmaps);

@@ -165,9 +165,10 @@ struct AttnArgs {
   __nv_bfloat16* out;  // user tensor
   int64_t so[4];       // out strides
   int64_t out_t0;      // token index inside `out` of the first query
+  bool fold_decides;   // a fold that compares the tokens of its block with the state follows (and runs beside the launch)
 };
 struct AttnPlan { int n_whole, nsp_rest; };   // (batch, head, query tile) CTAs that run whole, key splits of each of the others
-AttnPlan plan_attn(int64_t tiles, int64_t m);
+AttnPlan plan_attn(int64_t tiles, bool beside, int d, int64_t m);
 int launch_attn_simt(State* st, const AttnArgs& a, cudaStream_t s);
 int launch_attn_tc(State* st, const AttnArgs& a, cudaStream_t s);
 bool setup_attn_tc(State* st);   // encodes the tensor maps, raises the shared-memory limits

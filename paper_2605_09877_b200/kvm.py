@@ -117,7 +117,7 @@ def _load():
     L.kvm_debug_apply_plan.restype = C.c_int
     L.kvm_debug_apply_plan.argtypes = [C.c_int64, C.c_int32, C.c_int32, C.c_int32, C.POINTER(C.c_int32)]
     L.kvm_debug_attention_plan.restype = C.c_int
-    L.kvm_debug_attention_plan.argtypes = [C.c_int32, C.c_int32, C.c_int32, C.c_int64, C.POINTER(C.c_int32)]
+    L.kvm_debug_attention_plan.argtypes = [C.c_int32] * 5 + [C.c_int64, C.c_int32, C.POINTER(C.c_int32)]
     L.kvm_debug_expire_wait.restype = C.c_int
     L.kvm_debug_expire_wait.argtypes = [vp, C.c_int32, vp]
     L.kvm_head_layernorm.restype = C.c_int
@@ -202,9 +202,10 @@ def apply_plan(n_units: int, head_dim: int, block: int, serial: bool = False):
     return _plan("kvm_debug_apply_plan", 2, n_units, head_dim, block, 1 if serial else 0)
 
 
-def attention_plan(batch: int, n_q_heads: int, n_queries: int, n_slots: int):
-    """(CTAs that run whole, key splits of each of the others) of the attention of n_queries tokens over n_slots rows."""
-    return _plan("kvm_debug_attention_plan", 2, batch, n_q_heads, n_queries, n_slots)
+def attention_plan(batch: int, n_q_heads: int, n_kv_heads: int, head_dim: int, n_queries: int, n_slots: int, decides: bool = True):
+    """(CTAs that run whole, key splits of each of the others) of the attention of n_queries tokens of a block over n_slots rows;
+    decides: a fold that compares its tokens with the state runs beside it."""
+    return _plan("kvm_debug_attention_plan", 2, batch, n_q_heads, n_kv_heads, head_dim, n_queries, n_slots, 1 if decides else 0)
 
 
 def kvm_plan_capacity(block: int, n_bswa_chunks: int, g: Growth, seq_len: int) -> int:

@@ -70,16 +70,29 @@ def test_steps_that_fetch_ahead_where_that_is_the_faster_kernel(Hq, Hkv, d, n, s
 
 def test_key_splits_of_the_attention_have_keys_and_a_place_in_the_scratch():
     """37 * 8 partial results of a tile, 2 * 37 tickets, and a split has a key tile of the state or the window."""
-    for tiles in list(range(1, 600)) + [1000, 4096]:
-        for m in (0, 64, 128, 256, 300, 512, 1000, 1152, 1280, 2048, 2304, 2560, 4096, 50000):
-            whole, splits = kvm.attention_plan(1, tiles, 128, m)
-            rest = tiles - whole
-            assert 1 <= splits <= 8 and 0 <= whole <= tiles
-            if splits > 1:
-                assert 0 < rest <= 2 * 37 and rest * splits <= 37 * 8 and splits <= (m + 127) // 128 + 1
-            else:
-                assert rest == 0
-    assert kvm.attention_plan(2, 5, 200, 700) == kvm.attention_plan(1, 20, 128, 700)
+    for heads in list(range(1, 300)) + [500, 2048]:
+        for n in (1, 128, 256):
+            tiles = heads * ((n + 127) // 128)
+            for d in (64, 128):
+                for m in (0, 64, 128, 256, 300, 512, 1000, 1152, 1280, 1500, 2048, 2304, 2560, 4096, 50000):
+                    whole, splits = kvm.attention_plan(1, heads, heads, d, n, m, decides=m % 3 != 0)
+                    rest = tiles - whole
+                    assert 1 <= splits <= 8 and 0 <= whole <= tiles
+                    if splits > 1:
+                        assert 0 < rest <= 2 * 37 and rest * splits <= 37 * 8 and splits <= (m + 127) // 128 + 1
+                    else:
+                        assert rest == 0
+
+
+@pytest.mark.parametrize("Hq,Hkv,d,C,m,splits", [
+    (16, 16, 128, 256, 512, 1), (16, 16, 128, 256, 1152, 2), (16, 4, 128, 256, 4096, 3), (19, 19, 128, 256, 1280, 2), (24, 6, 128, 256, 1280, 2),
+    # folds as wide beside them: two splits only take SMs from those, up to more rows
+    (20, 20, 128, 256, 1536, 1), (20, 20, 128, 256, 1792, 2), (24, 24, 128, 256, 1792, 1), (24, 24, 128, 192, 2048, 2), (27, 27, 128, 192, 2560, 1),
+    (48, 48, 128, 64, 1536, 1), (54, 54, 128, 128, 2688, 1), (54, 54, 128, 128, 2816, 2), (24, 24, 64, 256, 1408, 1), (24, 24, 64, 256, 1536, 2),
+    (54, 54, 64, 128, 1792, 1), (54, 54, 64, 64, 2048, 2), (40, 40, 64, 128, 1280, 2), (48, 24, 128, 128, 1536, 2)])
+def test_key_splits_beside_folds(Hq, Hkv, d, C, m, splits):
+    assert kvm.attention_plan(1, Hq, Hkv, d, C, m) == (0 if splits > 1 else Hq * ((C + 127) // 128), splits)
+    assert kvm.attention_plan(1, Hq, Hkv, d, C, m, decides=False)[1] == (2 if m >= 1152 and splits == 1 else splits)
 
 
 def test_states_without_stored_keys_take_four_rows_per_warp():
@@ -104,6 +117,6 @@ def test_plan_refuses_what_a_state_refuses():
     for bad in [(0, 64, 64), (1, 96, 64), (1, 64, 60), (1, 64, 264)]:
         with pytest.raises(kvm.KVMError):
             kvm.apply_plan(*bad)
-    for bad in [(0, 1, 1, 1), (1, 0, 1, 1), (1, 1, 0, 1), (1, 1, 1, -1)]:
+    for bad in [(0, 1, 1, 64, 1, 1), (1, 3, 2, 64, 1, 1), (1, 1, 1, 96, 1, 1), (1, 1, 1, 64, 0, 1), (1, 1, 1, 64, 257, 1), (1, 1, 1, 64, 1, -1)]:
         with pytest.raises(kvm.KVMError):
             kvm.attention_plan(*bad)

@@ -465,7 +465,7 @@ def test_rows_with_many_members_in_both_apply_kernels(B, Hkv, d, C, slots, rows4
 def test_attention_of_few_heads_over_many_rows_splits_the_keys(Hq, Hkv, d, blocks, splits):
     """Key splits of launches of 6 to 48 tiles over 1 to 49 key tiles, ragged last ones."""
     from paper_2605_09877_b200 import kvm
-    assert {kvm.attention_plan(1, Hq, 256, 256 * max(b - 1, 0))[1] for b in range(blocks + 1)} == splits
+    assert {kvm.attention_plan(1, Hq, Hkv, d, 256, 256 * max(b - 1, 0), decides=False)[1] for b in range(blocks + 1)} == splits
     wl = synth.Workload("t", 1, Hq, Hkv, d, 256 * blocks + 70, 256, "unbounded", r=32, seed=62)
     print(_sampled(wl, [(0, 0), (0, Hkv - 1)]))
 
