@@ -7,7 +7,7 @@
 // What bounds it: with many heads HBM (K_hat, V_hat and the window are read once); with few the
 // latency of launch, first loads and merge, and on the host the launch itself, which is why the rotation of the
 // token and the merge are not kernels of their own: 32 heads over 256 + window rows took 1.9 + 7.4 + 3.1 us
-// in three kernels and 18.5 us per step on the host's side; now 7.0 us per step.  64 x 32 heads over 4096 + window
+// in three kernels and 18.5 us per step on the host's side; now 7.0 us per step, 4.5 with the rows fetched ahead (decode_short_kernel).  64 x 32 heads over 4096 + window
 // rows: 763 -> 695 us per step with its share of the block's fold, the set-up of a step under the tail of the one before.
 #include <cooperative_groups.h>
 
@@ -493,8 +493,8 @@ __global__ void __launch_bounds__(256) decode_step_kernel(DecodeParams p) {
 // behind the wait, under the latency of the new token's own loads.  (Numbers from before `base`, or not below this step's own - a
 // replayed graph -, say nothing: then every row is fetched behind the wait.)  The splits of a head, a cluster, send each other
 // their shares of the channels (st.async, bytes counted by the receiver): one exchange instead of two cluster barriers and
-// a round of remote loads.  us per step, with the loop above
-// and with this: 32 heads, 600 rows 6.9, 4.6; 900 rows 7.2, 5.5; 16 heads, 900 rows 6.9, 4.2; 32 on 8, 600 rows 8.0, 5.5; one head 5.5, 4.0.
+// a round of remote loads.  us per step in a graph, with the loop above
+// and with this: 32 heads, 630 rows 6.3, 4.5; 890 rows 6.6, 5.1; 16 heads, 850 rows 6.2, 3.8; 32 on 8, 700 rows 6.9, 4.9; 8 heads, 90 rows 3.9, 3.1.
 // ONE: no warp has more than one pass over rows (with the loop's bookkeeping 0.3 us longer).
 template <int D, int GQ, bool LN, bool ONE>
 __global__ void __launch_bounds__(256, 2) decode_short_kernel(const __grid_constant__ DecodeParams p) {
@@ -827,8 +827,8 @@ int launch_decode(State* st, const DecodeArgs& a, cudaStream_t s) {
   p.Hq = st->Hq; p.Hkv = st->Hkv; p.G = st->G; p.r = st->r;
   p.part = st->decPart; p.ticket = st->decTicket;
   const bool early = st->prof_hook == nullptr;
-  p.seen = st->decSeen; p.no = st->decNo++; p.base = st->decBase; p.status = st->status;
-  const DecodeShortPlan sp = early ? plan_decode_short(nQ, st->G, st->d, p.n) : DecodeShortPlan{0, 0, 0};   // (with the timing hook on nothing overlaps)
+  p.seen = st->decSeen; p.no = st->decNo++; p.base = early ? st->decBase : p.no; p.status = st->status;   // (with the timing hook on nothing overlaps)
+  const DecodeShortPlan sp = plan_decode_short(nQ, st->G, st->d, p.n);
   if (sp.splits > 0) {
     p.nsplit = sp.splits; p.nclus = 1; p.rpw = sp.rows_per_warp;
 #define KVM_DEC_SHORT(DD, GG, LL)                                                                \

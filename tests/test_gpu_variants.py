@@ -268,20 +268,27 @@ def _decode_rows(wl, t):
     return kvm.kvm_plan_capacity(wl.C, wl.w, g, t // wl.C * wl.C) + t + 1 - max(0, (t // wl.C + 1 - wl.w) * wl.C)
 
 
-@pytest.mark.parametrize("B,Hq,Hkv,d,pos,steps,plans", [
-    (1, 1, 1, 64, 40, 30, {(1, 1, 1)}), (1, 2, 1, 128, 900, 20, {(2, 6, 1)}), (3, 32, 4, 64, 1300, 10, {(4, 7, 1)}),
-    (7, 21, 21, 128, 300, 9, {(1, 2, 1)}), (9, 64, 64, 64, 700, 6, {(1, 1, 1)}), (40, 32, 8, 128, 300, 4, {(4, 1, 1)}),
-    (1, 1, 1, 128, 60, 20, {(1, 1, 1), (1, 2, 1)}), (1, 2, 2, 128, 110, 10, {(1, 2, 1)}), (1, 3, 3, 64, 400, 5, {(1, 4, 1)}),
-    (1, 1, 1, 64, 1000, 5, {(1, 6, 1)}), (1, 2, 2, 128, 260, 5, {(1, 5, 1)}),
-    (1, 2, 2, 128, 452, 5, {(1, 8, 1)}), (6, 32, 16, 128, 70, 8, {(2, 2, 1)}), (10, 32, 8, 64, 500, 5, {(4, 2, 1)}),
-    (5, 32, 4, 64, 20, 5, {(8, 1, 1)}), (5, 32, 4, 128, 130, 8, {(8, 3, 1)}), (12, 32, 4, 128, 300, 5, {(8, 2, 1)}),
-    (5, 32, 4, 128, 392, 5, {(8, 4, 1)}), (1, 2, 2, 128, 392, 5, {(1, 7, 1)})])
-def test_decode_row_splits_from_one_to_eight(B, Hq, Hkv, d, pos, steps, plans):
-    """One to eight CTAs in the cluster of a group of heads, one to eight query heads per CTA; every case asserts how its
-    steps are cut (query heads per CTA, CTAs per cluster, clusters)."""
+def _decode_kernels(B, Hq, Hkv, d, rows):
+    """What the decode steps over these numbers of rows run: ("ahead", query heads per CTA, CTAs per cluster) or (query heads per CTA,
+    CTAs per cluster, clusters) of the kernel that loops over its rows."""
     from paper_2605_09877_b200 import kvm
+    ahead = {n: kvm.decode_ahead(B, Hq, Hkv, d, n) for n in rows}
+    return {("ahead", a[1], a[0]) if a[0] else kvm.decode_plan(B, Hq, Hkv, d, n) for n, a in ahead.items()}
+
+
+@pytest.mark.parametrize("B,Hq,Hkv,d,pos,steps,kernels", [
+    (1, 1, 1, 64, 40, 30, {("ahead", 1, 1)}), (1, 2, 1, 128, 900, 20, {("ahead", 2, 6)}), (3, 32, 4, 64, 1300, 10, {("ahead", 2, 4)}),
+    (7, 21, 21, 128, 300, 9, {(1, 2, 1)}), (9, 64, 64, 64, 700, 6, {(1, 1, 1)}), (40, 32, 8, 128, 300, 4, {(4, 1, 1)}),
+    (1, 1, 1, 128, 60, 20, {("ahead", 1, 1)}), (1, 2, 2, 128, 110, 10, {("ahead", 1, 1)}), (1, 3, 3, 64, 400, 5, {("ahead", 1, 2)}),
+    (1, 1, 1, 64, 1000, 5, {("ahead", 1, 3)}), (1, 2, 2, 128, 260, 5, {("ahead", 1, 3)}),
+    (1, 2, 2, 128, 452, 5, {("ahead", 1, 4)}), (6, 32, 16, 128, 70, 8, {("ahead", 2, 1)}), (10, 32, 8, 64, 500, 5, {(4, 2, 1)}),
+    (5, 32, 4, 64, 20, 5, {("ahead", 2, 1)}), (5, 32, 4, 128, 130, 8, {("ahead", 2, 2)}), (12, 32, 4, 128, 300, 5, {(8, 2, 1)}),
+    (5, 32, 4, 128, 392, 5, {(8, 4, 1)}), (1, 2, 2, 128, 392, 5, {("ahead", 1, 4)})])
+def test_decode_row_splits_from_one_to_eight(B, Hq, Hkv, d, pos, steps, kernels):
+    """Steps of both decode kernels over a growing state, one to eight query heads per CTA; every case asserts which kernel its steps
+    run and how they are cut."""
     wl = synth.Workload("dec", B, Hq, Hkv, d, pos + steps, 64, "sqrt", sqrt_coeff=20, r=32, seed=330 + pos)
-    assert {kvm.decode_plan(B, Hq, Hkv, d, _decode_rows(wl, t)) for t in range(pos, pos + steps)} == plans
+    assert _decode_kernels(B, Hq, Hkv, d, {_decode_rows(wl, t) for t in range(pos, pos + steps)}) == kernels
     params = synth.make_layer_params(wl, trivial=False)
     print(_sampled(wl, [(0, 0), (B - 1, Hkv - 1)], params=params, decode_from=pos))
 
@@ -510,19 +517,112 @@ def test_decode_steps_that_fetch_their_rows_ahead(Hq, Hkv, d, C, slots, r, split
     assert torch.equal(outs[0], outs[1]) and torch.equal(outs[0], y[:, :, start:])
 
 
-@pytest.mark.parametrize("B,Hq,Hkv,d,pos,steps,plan", [
-    (1, 1, 1, 64, 40, 30, (1, 1, 1)), (1, 2, 1, 128, 900, 20, (2, 6, 1)), (3, 32, 4, 64, 1300, 10, (4, 7, 1)), (7, 21, 21, 128, 300, 9, (1, 2, 1)),
-    (1, 2, 2, 128, 260, 5, (1, 5, 1)), (1, 2, 2, 128, 452, 5, (1, 8, 1)), (5, 32, 4, 64, 20, 5, (8, 1, 1)), (5, 32, 4, 128, 130, 8, (8, 3, 1))])
-def test_decode_kernel_that_loops_over_rows_at_few_rows(B, Hq, Hkv, d, pos, steps, plan):
-    """With the timing hook on every step runs the kernel that loops over its rows, also where a few rows of a few heads are fetched ahead
-    otherwise: one to eight splits and query heads per CTA."""
-    from paper_2605_09877_b200 import kvm
-    wl = synth.Workload("dec", B, Hq, Hkv, d, pos + steps, 64, "sqrt", sqrt_coeff=20, r=32, seed=330 + pos)
-    assert {kvm.decode_plan(B, Hq, Hkv, d, _decode_rows(wl, t)) for t in range(pos, pos + steps)} == {plan}
+@pytest.mark.parametrize("B,Hq,Hkv,d,C,slots,plan", [
+    (10, 24, 8, 128, 16, 110, (1, 1, 1)), (10, 15, 5, 128, 16, 110, (1, 2, 1)), (10, 9, 9, 128, 32, 220, (1, 3, 1)), (8, 9, 9, 128, 32, 370, (1, 4, 1)),
+    (6, 9, 9, 64, 64, 960, (1, 5, 1)), (3, 11, 11, 128, 32, 1010, (1, 6, 1)), (8, 1, 1, 64, 64, 4120, (1, 7, 1)), (8, 1, 1, 128, 64, 2200, (1, 8, 1)),
+    (10, 30, 5, 128, 16, 110, (2, 1, 1)), (12, 16, 8, 64, 64, 440, (2, 2, 1)), (12, 10, 5, 128, 32, 490, (2, 3, 1)), (2, 22, 11, 128, 32, 1010, (2, 6, 1)),
+    (10, 64, 16, 128, 16, 16, (4, 1, 1)), (10, 16, 4, 128, 32, 370, (4, 4, 1)), (10, 8, 2, 128, 32, 770, (4, 7, 1)), (6, 12, 3, 128, 64, 820, (4, 8, 1)),
+    (10, 64, 8, 64, 16, 16, (8, 1, 1)), (10, 24, 3, 128, 32, 220, (8, 3, 1)), (12, 16, 2, 128, 32, 230, (8, 5, 1)), (6, 24, 3, 128, 64, 620, (8, 6, 1))])
+def test_decode_steps_that_loop_over_their_rows(B, Hq, Hkv, d, C, slots, plan):
+    """One to eight splits and query heads per CTA of the kernel that loops over its rows, each where the library takes it; steps
+    across a fold, behind which some run the other kernel, against the oracle."""
+    start = (slots // C + 4) * C - 4
+    wl = synth.Workload("loop", B, Hq, Hkv, d, start + 8, C, "fixed", fixed_slots=slots, r=32, seed=500 + slots)
+    assert plan in _decode_kernels(B, Hq, Hkv, d, {_decode_rows(wl, t) for t in range(start, wl.T)})
     params = synth.make_layer_params(wl, trivial=False)
-    tensors = synth.make_inputs(wl)
-    units = sorted({(0, 0), (B - 1, Hkv - 1)})
-    y, st = pu.run_gpu(wl, tensors, params, decode_from=pos, timed=True)
-    y_ref, o = pu.run_oracle(wl, tensors, params, units=units)
-    print(pu.compare(wl, y, st, y_ref, o, units=units))
+    print(_sampled(wl, sorted({(0, 0), (B - 1, Hkv - 1)}), params=params, decode_from=start))
+
+
+@pytest.mark.parametrize("B,Hq,Hkv,d,C,slots", [(1, 4, 4, 128, 64, 500), (1, 16, 4, 64, 64, 1200), (2, 4, 2, 128, 64, 1500), (10, 64, 16, 128, 16, 16)])
+def test_timed_decode_steps_run_the_kernels_that_serve(B, Hq, Hkv, d, C, slots):
+    """With the timing hook on no step overlaps the one before it, but it is the same kernel: bit for bit the same outputs."""
+    start = (slots // C + 4) * C - 6
+    wl = synth.Workload("hook", B, Hq, Hkv, d, start + 12, C, "fixed", fixed_slots=slots, r=32, seed=520 + slots)
+    params = synth.make_layer_params(wl, trivial=False)
+    t = {n: x.cuda() for n, x in synth.make_inputs(wl).items() if n in "qkv"}
+    outs = []
+    for hook in (False, True):
+        st, g = pu.gpu_layer(wl, params, max_call_tokens=start)
+        st.prefill(t["q"][:, :, :start], t["k"][:, :, :start], t["v"][:, :, :start], wl.C, g, wl.r)
+        st.profile_enable(hook)
+        outs.append(torch.stack([st.decode_step(*(t[n][:, :, i].contiguous() for n in "qkv")) for i in range(start, wl.T)]).cpu())
+        assert st.check() == 0 and (not hook or st.profile_read()["decode"][1] == wl.T - start)
+        st.free()
+    assert torch.equal(outs[0], outs[1])
+
+
+@pytest.mark.parametrize("Hq,Hkv,d,slots", [(4, 4, 128, 600), (2, 1, 64, 1500), (1, 1, 128, 1300)])
+def test_replayed_steps_fetch_no_rows_of_an_earlier_replay_ahead(Hq, Hkv, d, slots):
+    """A captured run of steps carries the numbers it was captured with.  Replayed behind a prefill of another sequence, and once
+    more behind itself, its steps give what the same steps give one by one."""
+    C, n = 64, 12
+    start = (slots // C + 4) * C + 5
+    wl = synth.Workload("replay", 1, Hq, Hkv, d, start + n, C, "fixed", fixed_slots=slots, r=32, seed=530 + slots)
+    assert {k[0] for k in _decode_kernels(1, Hq, Hkv, d, {_decode_rows(wl, t) for t in range(start, wl.T)})} == {"ahead"}
+    params = synth.make_layer_params(wl, trivial=False)
+    seqs = [{m: x.cuda() for m, x in synth.make_inputs(wl.scaled(seed=530 + slots + i)).items() if m in "qkv"} for i in range(3)]
+
+    def prefill(st, g, t):
+        st.prefill(t["q"][:, :, :start], t["k"][:, :, :start], t["v"][:, :, :start], C, g, wl.r)
+
+    want = []
+    for t in seqs:
+        st, g = pu.gpu_layer(wl, params, max_call_tokens=start)
+        prefill(st, g, t)
+        ys = []
+        for i in range(start, wl.T):
+            ys.append(st.decode_step(*(t[m][:, :, i].contiguous() for m in "qkv")))
+            torch.cuda.synchronize()
+        want.append(torch.stack(ys))
+        st.free()
+    st, g = pu.gpu_layer(wl, params, max_call_tokens=start)
+    prefill(st, g, seqs[0])
+    steps = [[seqs[0][m][:, :, i].clone(memory_format=torch.contiguous_format) for m in "qkv"] for i in range(start, wl.T)]
+    out = torch.empty_like(want[0])
+    torch.cuda.synchronize()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        for s, y in zip(steps, out):
+            st.decode_step(*s, out=y)
+    for t, y_ref in zip(seqs, want):
+        if t is not seqs[0]:
+            st.reset()
+            prefill(st, g, t)
+            for i, s in zip(range(start, wl.T), steps):
+                for m, x in zip("qkv", s):
+                    x.copy_(t[m][:, :, i])
+        for _ in range(2):
+            out.zero_()
+            graph.replay()
+            torch.cuda.synchronize()
+            assert torch.equal(out, y_ref)
+    assert st.check() == 0
+    del graph
     st.free()
+
+
+def test_steps_of_two_states_in_turn_on_one_stream():
+    """The layers of a model: a step is resident under the one of another state, across the folds of both."""
+    wls = [synth.Workload("la", 1, 4, 4, 128, 700 + 40, 64, "fixed", fixed_slots=400, r=32, seed=541),
+           synth.Workload("lb", 1, 8, 2, 64, 690 + 40, 64, "sqrt", sqrt_coeff=16, r=0, seed=542)]
+    starts, outs = (700, 690), []
+    for together in (False, True):
+        made = []
+        for wl, start in zip(wls, starts):
+            t = {n: x.cuda() for n, x in synth.make_inputs(wl).items() if n in "qkv"}
+            st, g = pu.gpu_layer(wl, synth.make_layer_params(wl), max_call_tokens=start)
+            st.prefill(t["q"][:, :, :start], t["k"][:, :, :start], t["v"][:, :, :start], wl.C, g, wl.r)
+            made.append((st, [[t[n][:, :, i].contiguous() for n in "qkv"] for i in range(start, wl.T)]))
+        ys = [[torch.empty_like(s[0]) for s in steps] for _, steps in made]
+        torch.cuda.synchronize()
+        order = [(l, i) for i in range(40) for l in range(2)] if together else [(l, i) for l in range(2) for i in range(40)]
+        for l, i in order:
+            made[l][0].decode_step(*made[l][1][i], out=ys[l][i])
+            if not together:
+                torch.cuda.synchronize()
+        torch.cuda.synchronize()
+        assert all(st.check() == 0 for st, _ in made)
+        outs.append([torch.stack(y) for y in ys])
+        for st, _ in made:
+            st.free()
+    assert torch.equal(outs[0][0], outs[1][0]) and torch.equal(outs[0][1], outs[1][1])
