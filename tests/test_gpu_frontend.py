@@ -86,7 +86,7 @@ def test_fused_qk_layernorm_equals_standalone_kernel_then_plain_calls(d, r, C):
 
 @pytest.mark.parametrize("G", [2, 8])
 def test_decode_grouped_queries_share_a_cta(G):
-    """G query heads per kv head: the decode kernel serves a whole group, or four heads of it, from one pass over the rows."""
+    """G query heads per kv head: two of them share a CTA of the decode kernel and its pass over the rows."""
     wl = synth.Workload("gq", 2, 2 * G, 2, 64 if G == 8 else 128, 300 + 70, 64, "sqrt", sqrt_coeff=7, r=16, seed=63 + G)
     params = synth.make_layer_params(wl, trivial=False)
     tensors = synth.make_inputs(wl)
@@ -94,3 +94,54 @@ def test_decode_grouped_queries_share_a_cta(G):
     y_ref, o = pu.run_oracle(wl, tensors, params)
     print(pu.compare(wl, y_gpu, st, y_ref, o))
     st.free()
+
+
+def _kernel(wl, t):
+    """("ahead", query heads per CTA, passes over the rows) or ("loop", query heads per CTA, one cluster or several per group)."""
+    from paper_2605_09877_b200 import kvm
+    n = wl.fixed_slots + t + 1 - max(0, (t // wl.C + 1 - wl.w) * wl.C)
+    splits, heads, rows = kvm.decode_ahead(wl.B, wl.Hq, wl.Hkv, wl.d, n)
+    if splits:
+        return "ahead", heads, 1 if rows <= 8 * (256 // wl.d) else 2
+    heads, _, clusters = kvm.decode_plan(wl.B, wl.Hq, wl.Hkv, wl.d, n)
+    return "loop", heads, min(clusters, 2)
+
+
+@pytest.mark.parametrize("B,Hq,Hkv,d,C,slots,kernel", [
+    (1, 1, 1, 128, 16, 16, ("ahead", 1, 1)), (1, 3, 1, 128, 64, 1000, ("ahead", 1, 2)), (1, 4, 2, 128, 64, 500, ("ahead", 2, 1)),
+    (1, 2, 1, 128, 64, 1000, ("ahead", 2, 2)), (1, 2, 2, 64, 64, 500, ("ahead", 1, 1)), (1, 1, 1, 64, 64, 2000, ("ahead", 1, 2)),
+    (12, 2, 1, 64, 16, 16, ("ahead", 2, 1)), (1, 4, 1, 64, 64, 2000, ("ahead", 2, 2)),
+    (8, 1, 1, 128, 64, 2000, ("loop", 1, 1)), (8, 2, 1, 128, 64, 2000, ("loop", 2, 1)), (8, 12, 3, 128, 64, 600, ("loop", 4, 1)),
+    (8, 24, 3, 128, 64, 300, ("loop", 8, 1)), (8, 1, 1, 64, 128, 4000, ("loop", 1, 1)), (8, 2, 1, 64, 128, 4000, ("loop", 2, 1)),
+    (3, 36, 9, 64, 64, 1000, ("loop", 4, 1)), (8, 24, 3, 64, 64, 600, ("loop", 8, 1)),
+    (1, 1, 1, 128, 64, 2000, ("loop", 1, 2)), (1, 2, 1, 128, 64, 2000, ("loop", 2, 2)), (1, 4, 1, 128, 64, 2000, ("loop", 4, 2)),
+    (1, 1, 1, 64, 128, 4000, ("loop", 1, 2)), (1, 2, 1, 64, 128, 4000, ("loop", 2, 2)), (1, 4, 1, 64, 128, 4000, ("loop", 4, 2))])
+def test_fused_qk_layernorm_in_every_build_of_the_decode_steps(B, Hq, Hkv, d, C, slots, kernel):
+    """Both decode kernels with LN_q / LN_k, one to eight query heads per CTA, one and two passes, one and several clusters: steps back
+    to back across a fold give the bits of the same steps on tensors that the stand-alone kernel normalised."""
+    from paper_2605_09877_b200 import kvm
+    start = (slots // C + 4) * C - 4
+    wl = synth.Workload("feb", B, Hq, Hkv, d, start + 8, C, "fixed", fixed_slots=slots, r=32, seed=65)
+    assert {_kernel(wl, t) for t in range(start, wl.T)} == {kernel}
+    params = synth.make_layer_params(wl, trivial=False)
+    gen = torch.Generator(device="cuda").manual_seed(66)
+    q = (torch.randn((B, Hq, wl.T, d), generator=gen, device="cuda") * 1.7 + 0.3).to(torch.bfloat16)
+    k = (torch.randn((B, Hkv, wl.T, d), generator=gen, device="cuda") * 0.6 - 0.2).to(torch.bfloat16)
+    v = torch.randn((B, Hkv, wl.T, d), generator=gen, device="cuda").to(torch.bfloat16)
+    wq, bq = 1.0 + 0.2 * torch.randn((Hq, d), generator=gen, device="cuda"), 0.1 * torch.randn((Hq, d), generator=gen, device="cuda")
+    wk = 1.0 + 0.2 * torch.randn((Hkv, d), generator=gen, device="cuda")
+    g = kvm.growth("fixed", slots)
+    outs = []
+    for fused in (False, True):
+        qi, ki = q.clone(), k.clone()
+        if not fused:
+            kvm.head_layernorm(qi, wq, bq, 1e-5)
+            kvm.head_layernorm(ki, wk, None, 1e-5)
+        ln = dict(eps=1e-5, q_weight=wq.cpu().numpy(), q_bias=bq.cpu().numpy(), k_weight=wk.cpu().numpy()) if fused else None
+        st = kvm.KVMState(kvm.LayerConfig(B, Hq, Hkv, d, C, max(slots, C), start), ln_weight=params["ln_w"], ln_bias=params["ln_b"],
+                          tau_state=params["tau_s"], tau_bswa=params["tau_b"], qk_ln=ln)
+        st.prefill(qi[:, :, :start], ki[:, :, :start], v[:, :, :start], C, g, wl.r)
+        outs.append(torch.stack([st.decode_step(*(x[:, :, i].contiguous() for x in (qi, ki, v))) for i in range(start, wl.T)]))
+        assert st.check() == 0
+        st.free()
+    assert torch.isfinite(outs[0].float()).all() and torch.equal(outs[0], outs[1])
