@@ -108,6 +108,15 @@ def test_states_without_stored_keys_take_four_rows_per_warp():
                         assert per_warp == 4
 
 
+@pytest.mark.parametrize("units,d,C,serial,rows", [
+    (72, 128, 256, False, 1), (96, 128, 256, False, 1), (127, 128, 136, False, 1), (148, 128, 256, False, 1), (255, 128, 256, False, 1), (32, 128, 256, True, 4),
+    (256, 128, 32, False, 4), (256, 128, 24, False, 1), (31, 64, 256, False, 1), (32, 64, 256, False, 4), (37, 64, 256, False, 4), (38, 64, 256, False, 1),
+    (48, 64, 256, False, 1), (49, 64, 256, False, 4), (56, 64, 160, False, 4), (60, 64, 136, False, 1), (67, 64, 136, False, 1), (68, 64, 136, False, 4),
+    (47, 64, 128, False, 1), (48, 64, 128, False, 4), (96, 64, 64, False, 4), (95, 64, 64, False, 1)])
+def test_rows_per_warp_of_the_apply_kernel(units, d, C, serial, rows):
+    assert kvm.apply_plan(units, d, C, serial)[0] == rows
+
+
 def test_plan_refuses_what_a_state_refuses():
     for bad in [(0, 1, 1, 64, 10), (1, 3, 2, 64, 10), (1, 2, 2, 96, 10), (1, 2, 2, 64, 0)]:
         with pytest.raises(kvm.KVMError):

@@ -449,8 +449,10 @@ def test_crowded_runs_are_compared_pair_by_pair(Hkv, d, C):
     (1, 3, 128, 256, 64, False),    # one row per warp: four members a row on average, many rows with more than a batch of four
     (1, 2, 64, 200, 24, False),
     (2, 9, 128, 64, 1, False),      # every token of a block joins one of the 64 rows of the first fold
-    (3, 24, 128, 256, 300, True),   # four rows per warp with stored memory keys
-    (2, 25, 64, 256, 256, True),
+    (3, 24, 128, 256, 300, False),
+    (2, 25, 64, 256, 256, True),    # four rows per warp with stored memory keys
+    (1, 36, 64, 256, 256, True),    # (eight CTAs per unit)
+    (2, 34, 64, 136, 100, True),
     (5, 32, 64, 192, 64, True),     # (four CTAs per unit)
     (2, 24, 64, 128, 90, True),
     (1, 47, 64, 128, 300, False),
