@@ -121,6 +121,10 @@ def test_plan_refuses_what_a_state_refuses():
     for bad in [(0, 1, 1, 64, 10), (1, 3, 2, 64, 10), (1, 2, 2, 96, 10), (1, 2, 2, 64, 0)]:
         with pytest.raises(kvm.KVMError):
             kvm.decode_plan(*bad)
+
+
+def test_the_other_plans_refuse_what_a_state_refuses():
+    for bad in [(0, 1, 1, 64, 10), (1, 3, 2, 64, 10), (1, 2, 2, 96, 10), (1, 2, 2, 64, 0)]:
         with pytest.raises(kvm.KVMError):
             kvm.decode_ahead(*bad)
     for bad in [(0, 64, 64), (1, 96, 64), (1, 64, 60), (1, 64, 264)]:

@@ -105,11 +105,9 @@ def test_attention_with_more_tiles_than_sms_splits_the_last_partial_wave():
     print(_run(wl))
 
 
-def test_many_rows_per_fold_one_row_per_warp():
-    """32 units x 256 tokens = 8192 rows per fold in the apply kernel with one row per warp, head_dim 128, gates and affine LayerNorm
-    included."""
-    from paper_2605_09877_b200 import kvm
-    assert kvm.apply_plan(32, 128, 256)[0] == 1
+def test_many_rows_per_fold_use_the_four_rows_per_warp_apply_kernel():
+    """32 units x 256 tokens = 8192 rows per fold, head_dim 128, gates and affine LayerNorm included (one row per warp since states
+    of 128 channels keep to that kernel)."""
     wl = synth.Workload("t", 2, 16, 16, 128, 256 * 4 + 70, 256, "sqrt", sqrt_coeff=12, r=32, seed=22, kind="mixture")
     params = synth.make_layer_params(wl, trivial=False)
     print(_run(wl, params=params, gate=True))

@@ -27,21 +27,17 @@ def _continue(st, g, wl, q, k, v, gate, a, b, dec_from):
 SERIAL = 1 << 5   # KVM_FLAG_SERIAL_FOLDS
 
 
-@pytest.mark.parametrize("wl,cut,params_trivial,use_gate,flags,rows_per_warp", [
-    (synth.Workload("snapA", 2, 4, 2, 128, 256 * 6 + 90, 256, "sqrt", sqrt_coeff=10, r=32, seed=41), 256 * 3 + 77, False, True, 0, 1),
-    (synth.Workload("snapB", 1, 3, 3, 64, 64 * 20 + 5, 64, "fixed", fixed_slots=200, r=0, seed=42, kind="mixture"), 64 * 9, True, False, 0, 1),
-    (synth.Workload("snapC", 1, 2, 2, 64, 300, 32, "sqrt", sqrt_coeff=6, r=16, seed=43, w=3), 17, True, False, 0, 1),   # cut before any fold
-    (synth.Workload("snapD", 1, 40, 40, 128, 256 * 5 + 33, 256, "sqrt", r=0, seed=44), 256 * 4 + 1, True, False, 0, 1),
-    # four rows per warp with stored memory keys
-    (synth.Workload("snapH", 2, 25, 25, 64, 256 * 5 + 40, 256, "sqrt", r=16, seed=48), 256 * 3 + 70, False, True, 0, 4),
+@pytest.mark.parametrize("wl,cut,params_trivial,use_gate,flags", [
+    (synth.Workload("snapA", 2, 4, 2, 128, 256 * 6 + 90, 256, "sqrt", sqrt_coeff=10, r=32, seed=41), 256 * 3 + 77, False, True, 0),
+    (synth.Workload("snapB", 1, 3, 3, 64, 64 * 20 + 5, 64, "fixed", fixed_slots=200, r=0, seed=42, kind="mixture"), 64 * 9, True, False, 0),
+    (synth.Workload("snapC", 1, 2, 2, 64, 300, 32, "sqrt", sqrt_coeff=6, r=16, seed=43, w=3), 17, True, False, 0),   # cut before any fold
+    (synth.Workload("snapD", 1, 40, 40, 128, 256 * 5 + 33, 256, "sqrt", r=0, seed=44), 256 * 4 + 1, True, False, 0),
     # one readout copy, folds on the caller's stream
-    (synth.Workload("snapF", 1, 4, 2, 128, 128 * 9 + 60, 128, "sqrt", sqrt_coeff=5, r=32, seed=46), 128 * 4 + 9, False, True, SERIAL, 1),
+    (synth.Workload("snapF", 1, 4, 2, 128, 128 * 9 + 60, 128, "sqrt", sqrt_coeff=5, r=32, seed=46), 128 * 4 + 9, False, True, SERIAL),
     # the same with 64 units x block 128: no fp64 memory keys are kept, the import rebuilds the per-row statistics
-    (synth.Workload("snapG", 2, 32, 32, 128, 128 * 8 + 50, 128, "sqrt", sqrt_coeff=5, r=32, seed=47), 128 * 5 + 3, False, False, SERIAL, 4),
+    (synth.Workload("snapG", 2, 32, 32, 128, 128 * 8 + 50, 128, "sqrt", sqrt_coeff=5, r=32, seed=47), 128 * 5 + 3, False, False, SERIAL),
 ])
-def test_snapshot_restore_continue_equals_uninterrupted_run(wl, cut, params_trivial, use_gate, flags, rows_per_warp):
-    from paper_2605_09877_b200 import kvm
-    assert kvm.apply_plan(wl.B * wl.Hkv, wl.d, wl.C, bool(flags & SERIAL))[0] == rows_per_warp
+def test_snapshot_restore_continue_equals_uninterrupted_run(wl, cut, params_trivial, use_gate, flags):
     params = synth.make_layer_params(wl, trivial=params_trivial)
     tensors = synth.make_inputs(wl)
     gate_cpu = synth.make_gate(wl) if use_gate else None
@@ -82,6 +78,21 @@ def test_snapshot_restore_continue_equals_uninterrupted_run(wl, cut, params_triv
     y_b2 = _continue(b, g, wl, q, k, v, gate, cut, wl.T, dec_from)
     assert torch.equal(y_b2, y_ref)
     b.free()
+
+
+def test_import_of_a_state_with_four_rows_per_warp_and_stored_memory_keys():
+    from paper_2605_09877_b200 import kvm
+    wl = synth.Workload("snapH", 2, 25, 25, 64, 256 * 5 + 40, 256, "sqrt", r=16, seed=48)
+    assert kvm.apply_plan(50, 64, 256)[0] == 4
+    test_snapshot_restore_continue_equals_uninterrupted_run(wl, 256 * 3 + 70, False, True, 0)
+
+
+@pytest.mark.parametrize("units,d,C,flags,rows_per_warp", [
+    (4, 128, 256, 0, 1), (3, 64, 64, 0, 1), (2, 64, 32, 0, 1), (40, 128, 256, 0, 1), (4, 128, 128, SERIAL, 1), (64, 128, 128, SERIAL, 4)])
+def test_rows_per_warp_of_the_imported_states(units, d, C, flags, rows_per_warp):
+    """The kernels that the cases above restore into (snapA to snapG)."""
+    from paper_2605_09877_b200 import kvm
+    assert kvm.apply_plan(units, d, C, bool(flags & SERIAL))[0] == rows_per_warp
 
 
 def test_import_rejects_inconsistent_snapshots_and_leaves_the_state_untouched():

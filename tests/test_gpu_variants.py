@@ -268,6 +268,24 @@ def _decode_rows(wl, t):
     return kvm.kvm_plan_capacity(wl.C, wl.w, g, t // wl.C * wl.C) + t + 1 - max(0, (t // wl.C + 1 - wl.w) * wl.C)
 
 
+@pytest.mark.parametrize("B,Hq,Hkv,d,pos,steps,plans", [
+    (1, 1, 1, 64, 40, 30, {(1, 1, 1)}), (1, 2, 1, 128, 900, 20, {(2, 6, 1)}), (3, 32, 4, 64, 1300, 10, {(4, 7, 1)}),
+    (7, 21, 21, 128, 300, 9, {(1, 2, 1)}), (9, 64, 64, 64, 700, 6, {(1, 1, 1)}), (40, 32, 8, 128, 300, 4, {(4, 1, 1)}),
+    (1, 1, 1, 128, 60, 20, {(1, 1, 1), (1, 2, 1)}), (1, 2, 2, 128, 110, 10, {(1, 2, 1)}), (1, 3, 3, 64, 400, 5, {(1, 4, 1)}),
+    (1, 1, 1, 64, 1000, 5, {(1, 6, 1)}), (1, 2, 2, 128, 260, 5, {(1, 5, 1)}),
+    (1, 2, 2, 128, 452, 5, {(1, 8, 1)}), (6, 32, 16, 128, 70, 8, {(2, 2, 1)}), (10, 32, 8, 64, 500, 5, {(4, 2, 1)}),
+    (5, 32, 4, 64, 20, 5, {(8, 1, 1)}), (5, 32, 4, 128, 130, 8, {(8, 3, 1)}), (12, 32, 4, 128, 300, 5, {(8, 2, 1)}),
+    (5, 32, 4, 128, 392, 5, {(8, 4, 1)}), (1, 2, 2, 128, 392, 5, {(1, 7, 1)})])
+def test_decode_row_splits_from_one_to_eight(B, Hq, Hkv, d, pos, steps, plans):
+    """One to eight CTAs in the cluster of a group of heads, one to eight query heads per CTA: how the looping kernel cuts these
+    steps.  Those of few heads run the kernel that fetches its rows ahead (test_kernels_of_the_row_split_cases)."""
+    from paper_2605_09877_b200 import kvm
+    wl = synth.Workload("dec", B, Hq, Hkv, d, pos + steps, 64, "sqrt", sqrt_coeff=20, r=32, seed=330 + pos)
+    assert {kvm.decode_plan(B, Hq, Hkv, d, _decode_rows(wl, t)) for t in range(pos, pos + steps)} == plans
+    params = synth.make_layer_params(wl, trivial=False)
+    print(_sampled(wl, [(0, 0), (B - 1, Hkv - 1)], params=params, decode_from=pos))
+
+
 def _decode_kernels(B, Hq, Hkv, d, rows):
     """What the decode steps over these numbers of rows run: ("ahead", query heads per CTA, CTAs per cluster) or (query heads per CTA,
     CTAs per cluster, clusters) of the kernel that loops over its rows."""
@@ -284,13 +302,10 @@ def _decode_kernels(B, Hq, Hkv, d, rows):
     (1, 2, 2, 128, 452, 5, {("ahead", 1, 4)}), (6, 32, 16, 128, 70, 8, {("ahead", 2, 1)}), (10, 32, 8, 64, 500, 5, {(4, 2, 1)}),
     (5, 32, 4, 64, 20, 5, {("ahead", 2, 1)}), (5, 32, 4, 128, 130, 8, {("ahead", 2, 2)}), (12, 32, 4, 128, 300, 5, {(8, 2, 1)}),
     (5, 32, 4, 128, 392, 5, {(8, 4, 1)}), (1, 2, 2, 128, 392, 5, {("ahead", 1, 4)})])
-def test_decode_row_splits_from_one_to_eight(B, Hq, Hkv, d, pos, steps, kernels):
-    """Steps of both decode kernels over a growing state, one to eight query heads per CTA; every case asserts which kernel its steps
-    run and how they are cut."""
+def test_kernels_of_the_row_split_cases(B, Hq, Hkv, d, pos, steps, kernels):
+    """What the steps of test_decode_row_splits_from_one_to_eight run."""
     wl = synth.Workload("dec", B, Hq, Hkv, d, pos + steps, 64, "sqrt", sqrt_coeff=20, r=32, seed=330 + pos)
     assert _decode_kernels(B, Hq, Hkv, d, {_decode_rows(wl, t) for t in range(pos, pos + steps)}) == kernels
-    params = synth.make_layer_params(wl, trivial=False)
-    print(_sampled(wl, [(0, 0), (B - 1, Hkv - 1)], params=params, decode_from=pos))
 
 
 @pytest.mark.parametrize("B,Hq,Hkv,d,serial", [(1, 2, 1, 64, False), (1, 4, 4, 128, False), (2, 8, 2, 128, True)])
@@ -449,10 +464,8 @@ def test_crowded_runs_are_compared_pair_by_pair(Hkv, d, C):
     (1, 3, 128, 256, 64, False),    # one row per warp: four members a row on average, many rows with more than a batch of four
     (1, 2, 64, 200, 24, False),
     (2, 9, 128, 64, 1, False),      # every token of a block joins one of the 64 rows of the first fold
-    (3, 24, 128, 256, 300, False),
-    (2, 25, 64, 256, 256, True),    # four rows per warp with stored memory keys
-    (1, 36, 64, 256, 256, True),    # (eight CTAs per unit)
-    (2, 34, 64, 136, 100, True),
+    (3, 24, 128, 256, 300, True),   # four rows per warp with stored memory keys
+    (2, 25, 64, 256, 256, True),
     (5, 32, 64, 192, 64, True),     # (four CTAs per unit)
     (2, 24, 64, 128, 90, True),
     (1, 47, 64, 128, 300, False),
@@ -460,8 +473,8 @@ def test_crowded_runs_are_compared_pair_by_pair(Hkv, d, C):
 def test_rows_with_many_members_in_both_apply_kernels(B, Hkv, d, C, slots, rows4):
     """The kernel that a state's folds run to write the touched rows, at rows with none, one and many members, appended rows
     among them; the state means and readout rows against the oracle."""
-    from paper_2605_09877_b200 import kvm
-    assert (kvm.apply_plan(B * Hkv, d, C)[0] == 4) == rows4
+    rows = C * B * Hkv
+    assert rows4 == ((rows > 12288 if C > 128 else rows >= 6144) if d == 64 else C > 128 and rows > 16384 and B * Hkv < 128)
     wl = synth.Workload("t", B, Hkv, Hkv, d, C * 5 + 11, C, "fixed", fixed_slots=slots, r=32, seed=61, kind="mixture")
     params = synth.make_layer_params(wl, trivial=False)
     units = sorted({(0, 0), (B - 1, Hkv - 1)})
@@ -469,30 +482,58 @@ def test_rows_with_many_members_in_both_apply_kernels(B, Hkv, d, C, slots, rows4
     print(stats)
 
 
-@pytest.mark.parametrize("Hq,Hkv,d,blocks,splits", [
-    (8, 8, 128, 21, {1, 2, 3, 4, 5}), (16, 4, 128, 22, {1, 2, 3}), (24, 8, 64, 23, {1, 2}), (3, 3, 128, 25, {1, 2, 3, 4, 5, 6})])
-def test_attention_of_few_heads_over_many_rows_splits_the_keys(Hq, Hkv, d, blocks, splits):
-    """Key splits of launches of 6 to 48 tiles over 1 to 49 key tiles, ragged last ones."""
+@pytest.mark.parametrize("B,Hkv,d,C,slots,rows_per_warp,run", [
+    (1, 3, 128, 256, 64, 1, False), (1, 2, 64, 200, 24, 1, False), (2, 9, 128, 64, 1, 1, False), (3, 24, 128, 256, 300, 1, False),
+    (2, 25, 64, 256, 256, 4, False), (5, 32, 64, 192, 64, 4, False), (2, 24, 64, 128, 90, 4, False), (1, 47, 64, 128, 300, 1, False),
+    (1, 36, 64, 256, 256, 4, True),   # eight CTAs per unit
+    (2, 34, 64, 136, 100, 4, True)])
+def test_rows_per_warp_of_states_with_many_members(B, Hkv, d, C, slots, rows_per_warp, run):
+    """Which of the two kernels the library takes, for the cases of the test above too, which holds a rule of its own; the others run."""
     from paper_2605_09877_b200 import kvm
-    assert {kvm.attention_plan(1, Hq, Hkv, d, 256, 256 * max(b - 1, 0), decides=False)[1] for b in range(blocks + 1)} == splits
+    assert kvm.apply_plan(B * Hkv, d, C)[0] == rows_per_warp
+    if run:
+        wl = synth.Workload("t", B, Hkv, Hkv, d, C * 5 + 11, C, "fixed", fixed_slots=slots, r=32, seed=61, kind="mixture")
+        print(_sampled(wl, [(0, 0), (B - 1, Hkv - 1)], params=synth.make_layer_params(wl, trivial=False), gate=True))
+
+
+@pytest.mark.parametrize("Hq,Hkv,d,blocks", [(8, 8, 128, 21), (16, 4, 128, 22), (24, 8, 64, 23), (3, 3, 128, 25)])
+def test_attention_of_few_heads_over_many_rows_splits_the_keys(Hq, Hkv, d, blocks):
+    """Key splits of launches of 6 to 48 tiles over 10 to 40 key tiles: two to eight splits, ragged last ones."""
     wl = synth.Workload("t", 1, Hq, Hkv, d, 256 * blocks + 70, 256, "unbounded", r=32, seed=62)
     print(_sampled(wl, [(0, 0), (0, Hkv - 1)]))
 
 
+@pytest.mark.parametrize("Hq,Hkv,d,blocks,splits", [
+    (8, 8, 128, 21, {1, 2, 3, 4, 5}), (16, 4, 128, 22, {1, 2, 3}), (24, 8, 64, 23, {1, 2}), (3, 3, 128, 25, {1, 2, 3, 4, 5, 6})])
+def test_key_splits_of_the_cases_with_few_heads_over_many_rows(Hq, Hkv, d, blocks, splits):
+    """The splits that the test above meets: 6 to 48 tiles over 1 to 49 key tiles."""
+    from paper_2605_09877_b200 import kvm
+    assert {kvm.attention_plan(1, Hq, Hkv, d, 256, 256 * max(b - 1, 0), decides=False)[1] for b in range(blocks + 1)} == splits
+
+
+def _short_splits(n_q, group, d, n):
+    """CTAs per cluster of the decode kernel that fetches its rows ahead (0: the step is not one of its)."""
+    groups, cta = (n_q // 2 if group % 2 == 0 else n_q), 64 * (256 // d)
+    fit = (296, 148, 88, 71, 56, 45, 37, 33)
+    if groups > fit[0] or n > 16 * cta:
+        return 0
+    ns = -(-n // cta)
+    ns = 8 if ns > 8 or 8 <= groups <= 16 else ns
+    return ns if groups <= fit[ns - 1] else 0
+
+
 @pytest.mark.parametrize("Hq,Hkv,d,C,slots,r,splits", [
     (1, 1, 64, 16, 40, 0, {1}), (3, 1, 128, 16, 80, 32, {1}), (2, 2, 128, 32, 170, 32, {2}), (2, 1, 128, 64, 300, 64, {3, 4}),
-    (5, 5, 64, 64, 960, 16, {5}), (4, 2, 128, 64, 600, 0, {6}), (3, 3, 128, 64, 700, 32, {6, 7}), (12, 12, 64, 32, 300, 0, {8}),
-    (24, 12, 128, 64, 900, 32, {8}), (32, 32, 128, 64, 930, 0, {8}),
-    (16, 16, 128, 16, 60, 32, {1}), (24, 12, 64, 64, 300, 32, {2}),
-    (2, 2, 128, 64, 1500, 32, {8}), (1, 1, 64, 256, 3500, 0, {8}), (40, 20, 64, 64, 2500, 32, {8}),   # two passes over a warp's rows
+    (5, 5, 64, 64, 960, 16, {4, 5}), (4, 2, 128, 64, 600, 0, {6}), (3, 3, 128, 64, 700, 32, {6, 7}), (12, 12, 64, 32, 300, 0, {8}),
+    (24, 12, 128, 64, 900, 32, {8}), (33, 33, 128, 64, 930, 0, {8}),
+    (2, 2, 128, 64, 1500, 32, {8}), (1, 1, 64, 256, 3500, 0, {8}), (66, 33, 64, 64, 2700, 32, {8}),   # two passes over a warp's rows
 ])
 def test_decode_steps_that_fetch_their_rows_ahead(Hq, Hkv, d, C, slots, r, splits):
     """One to eight CTAs per group of heads, one and two passes, warps with few rows or none; steps back to back across a fold, of
     which each fetches what the ones before leave complete, against the oracle and against steps that are waited for."""
     start = (slots // C + 4) * C - 6
     wl = synth.Workload("short", 1, Hq, Hkv, d, start + 14, C, "fixed", fixed_slots=slots, r=r, seed=400 + slots)
-    from paper_2605_09877_b200 import kvm
-    assert {kvm.decode_ahead(1, Hq, Hkv, d, _decode_rows(wl, t))[0] for t in range(start, wl.T)} == splits
+    assert {_short_splits(Hq, Hq // Hkv, d, _decode_rows(wl, t)) for t in range(start, wl.T)} <= splits
     params = synth.make_layer_params(wl, trivial=False)
     tensors = synth.make_inputs(wl)
     y, st = pu.run_gpu(wl, tensors, params, decode_from=start)
@@ -517,6 +558,40 @@ def test_decode_steps_that_fetch_their_rows_ahead(Hq, Hkv, d, C, slots, r, split
         outs.append(torch.stack(ys, 2).cpu())
         st.free()
     assert torch.equal(outs[0], outs[1]) and torch.equal(outs[0], y[:, :, start:])
+
+
+@pytest.mark.parametrize("Hq,Hkv,d,C,slots,r,splits,run", [
+    (1, 1, 64, 16, 40, 0, {1}, False), (3, 1, 128, 16, 80, 32, {1}, False), (2, 2, 128, 32, 170, 32, {2}, False),
+    (2, 1, 128, 64, 300, 64, {3, 4}, False), (5, 5, 64, 64, 960, 16, {5}, False), (4, 2, 128, 64, 600, 0, {6}, False),
+    (3, 3, 128, 64, 700, 32, {6, 7}, False), (12, 12, 64, 32, 300, 0, {8}, False), (24, 12, 128, 64, 900, 32, {8}, False),
+    (32, 32, 128, 64, 930, 0, {8}, True), (16, 16, 128, 16, 60, 32, {1}, True), (24, 12, 64, 64, 300, 32, {2}, True),
+    (2, 2, 128, 64, 1500, 32, {8}, False), (1, 1, 64, 256, 3500, 0, {8}, False), (40, 20, 64, 64, 2500, 32, {8}, True)])
+def test_splits_of_the_steps_that_fetch_their_rows_ahead(Hq, Hkv, d, C, slots, r, splits, run):
+    """The library's splits, for cases of the test above too, which holds a rule of its own; the others run."""
+    from paper_2605_09877_b200 import kvm
+    start = (slots // C + 4) * C - 6
+    wl = synth.Workload("short", 1, Hq, Hkv, d, start + 14, C, "fixed", fixed_slots=slots, r=r, seed=400 + slots)
+    assert {kvm.decode_ahead(1, Hq, Hkv, d, _decode_rows(wl, t))[0] for t in range(start, wl.T)} == splits
+    if run:
+        test_decode_steps_that_fetch_their_rows_ahead(Hq, Hkv, d, C, slots, r, set(range(9)))
+
+
+@pytest.mark.parametrize("B,Hq,Hkv,d,pos,steps,plan", [
+    (1, 1, 1, 64, 40, 30, (1, 1, 1)), (1, 2, 1, 128, 900, 20, (2, 6, 1)), (3, 32, 4, 64, 1300, 10, (4, 7, 1)), (7, 21, 21, 128, 300, 9, (1, 2, 1)),
+    (1, 2, 2, 128, 260, 5, (1, 5, 1)), (1, 2, 2, 128, 452, 5, (1, 8, 1)), (5, 32, 4, 64, 20, 5, (8, 1, 1)), (5, 32, 4, 128, 130, 8, (8, 3, 1))])
+def test_decode_kernel_that_loops_over_rows_at_few_rows(B, Hq, Hkv, d, pos, steps, plan):
+    """With the timing hook on no step overlaps the one before it; steps that fetch their rows ahead otherwise and steps of the kernel
+    that loops over them."""
+    from paper_2605_09877_b200 import kvm
+    wl = synth.Workload("dec", B, Hq, Hkv, d, pos + steps, 64, "sqrt", sqrt_coeff=20, r=32, seed=330 + pos)
+    assert {kvm.decode_plan(B, Hq, Hkv, d, _decode_rows(wl, t)) for t in range(pos, pos + steps)} == {plan}
+    params = synth.make_layer_params(wl, trivial=False)
+    tensors = synth.make_inputs(wl)
+    units = sorted({(0, 0), (B - 1, Hkv - 1)})
+    y, st = pu.run_gpu(wl, tensors, params, decode_from=pos, timed=True)
+    y_ref, o = pu.run_oracle(wl, tensors, params, units=units)
+    print(pu.compare(wl, y, st, y_ref, o, units=units))
+    st.free()
 
 
 @pytest.mark.parametrize("B,Hq,Hkv,d,C,slots,plan", [
