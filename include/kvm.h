@@ -297,8 +297,8 @@ kvm_status_t kvm_debug_drop_exchange(kvm_state_t* state, int32_t unit);
  *   (kvm_debug_decode_plan); out[1] query heads per CTA, out[2] rows per warp.
  * - kvm_debug_decode_plan: the same step in the looping kernel.  out[0] query heads per CTA, out[1] CTAs per cluster (row splits
  *   merged through shared memory), out[2] clusters per group of heads (merged through global memory).
- * - kvm_debug_apply_plan: the kernel that writes the rows a fold touches, for n_units = batch * n_kv_heads; serial: with
- *   KVM_FLAG_SERIAL_FOLDS.  out[0] rows per warp (1 or 4), out[1] CTAs per unit.
+ * - kvm_debug_apply_plan: the kernel that writes the rows a fold touches, for n_units = batch * n_kv_heads of `group` query
+ *   heads; serial: with KVM_FLAG_SERIAL_FOLDS.  out[0] rows per warp (1 or 4), out[1] CTAs per unit.
  * - kvm_debug_attention_plan: the attention of n_queries tokens of a block over n_slots state rows; decides: a fold that compares its
  *   tokens with the state runs beside it.  out[0] (batch, head, query tile) CTAs that run whole, out[1] key splits of each of the
  *   others. */
@@ -306,7 +306,7 @@ kvm_status_t kvm_debug_decode_ahead(int32_t batch, int32_t n_q_heads, int32_t n_
                                     int32_t* out);
 kvm_status_t kvm_debug_decode_plan(int32_t batch, int32_t n_q_heads, int32_t n_kv_heads, int32_t head_dim, int64_t n_rows,
                                    int32_t* out);
-kvm_status_t kvm_debug_apply_plan(int64_t n_units, int32_t head_dim, int32_t block, int32_t serial, int32_t* out);
+kvm_status_t kvm_debug_apply_plan(int64_t n_units, int32_t group, int32_t head_dim, int32_t block, int32_t serial, int32_t* out);
 kvm_status_t kvm_debug_attention_plan(int32_t batch, int32_t n_q_heads, int32_t n_kv_heads, int32_t head_dim,
                                       int32_t n_queries, int64_t n_slots, int32_t decides, int32_t* out);
 

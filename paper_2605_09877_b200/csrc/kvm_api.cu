@@ -519,10 +519,10 @@ KVM_API kvm_status_t kvm_debug_decode_ahead(int32_t batch, int32_t n_q_heads, in
   return KVM_OK;
 }
 
-KVM_API kvm_status_t kvm_debug_apply_plan(int64_t n_units, int32_t head_dim, int32_t block, int32_t serial, int32_t* out) {
-  if (n_units < 1 || block < 8 || block > kMaxBlock || block % 8 || !out) return KVM_ERR_INVALID_ARG;
+KVM_API kvm_status_t kvm_debug_apply_plan(int64_t n_units, int32_t group, int32_t head_dim, int32_t block, int32_t serial, int32_t* out) {
+  if (n_units < 1 || group < 1 || block < 8 || block > kMaxBlock || block % 8 || !out) return KVM_ERR_INVALID_ARG;
   if (head_dim != 64 && head_dim != 128) return KVM_ERR_UNSUPPORTED;
-  const ApplyPlan p = plan_apply(n_units, head_dim, block, recomputes_keys(serial != 0 || n_units >= kSerialUnits, block, n_units));
+  const ApplyPlan p = plan_apply(n_units, group, head_dim, block, recomputes_keys(serial != 0 || n_units >= kSerialUnits, block, n_units));
   out[0] = p.rows_per_warp; out[1] = p.ctas;
   return KVM_OK;
 }

@@ -2154,24 +2154,24 @@ __global__ void __launch_bounds__(256) refresh_rows_kernel(RefreshParams p) {
 
 // Which apply kernel the folds of this state run (fixed per state and block).  Four rows per warp where the keys are recomputed, and for
 // 64 channels, whose rows are half as much to fetch: there in blocks of up to 128 tokens from 6144 rows on, in longer ones from 68
-// units or 12288 rows, and from 8192 rows while every group of 32 rows has a CTA of its own at once (two per SM).  Measured, four rows
-// per warp over one, 32 blocks, states of 256 rows, 512 rows, square root.  128 channels: blocks of 256, 66 units 0.94, 1.04, 1.03; 80
+// units or 12288 rows, and with one query head per unit from 8192 rows while every group of 32 rows has a CTA of its own at once (two per
+// SM); the attention of several heads holds the SMs that those would take.  Measured, four rows per warp over one, 32 blocks, states of 256 rows, 512 rows, square root.  128 channels: blocks of 256, 66 units 0.94, 1.04, 1.03; 80
 // 1.03, 1.00, 0.98; 96 1.06, 1.07, 1.00; 112 1.06, 1.08, 1.07; 148 0.97, 0.99, 1.00; blocks of 192, 96 units 1.04, 1.05, 0.98; 112 1.05, 1.08, 1.08; blocks
 // of 136, 66 units 1.07, 1.11, 1.04; 126 1.13, 1.11, 1.08; blocks of 64 to 128 up to 1.09, nowhere below 0.97.  64 channels: blocks of 256, 36
 // units 0.99, 0.99, 0.98; 40 1.03, 1.05, 1.00; 48 1.03, 1.05, 0.97; 64 1.02, 0.97, 0.96; 72 0.94, 0.95, 0.95; 148 0.92, 0.90, 0.91; 255
-// 0.93, 0.91, 0.93; blocks of 136, 56 units 0.99, 1.00, 0.99; 60 1.05, 1.03, 1.02; 72 0.98, 1.00, 0.97; 88 0.98, 0.98, 0.97.  (ms, one and four:
+// 0.93, 0.91, 0.93; two heads per unit, 34 units 1.04, 1.00, 0.98; 37 1.03, 1.01, 0.94; eight heads 1.02, 1.00, 0.99; 1.01, 1.00, 0.99; blocks of 136, 56 units 0.99, 1.00, 0.99; 60 1.05, 1.03, 1.02; 72 0.98, 1.00, 0.97; 88 0.98, 0.98, 0.97.  (ms, one and four:
 // blocks of 128, 48 units 0.653, 0.630; 64 0.733, 0.705; 128 1.08, 0.98; 192 1.44, 1.34; of 64, 64 units 0.608, 0.629; 96 0.773, 0.712; 224 1.10, 1.06.)
 // CTAs per unit of the four-rows kernel: one when the units alone fill the GPU's CTA slots (measured at 256 and 2048 units: 1 beats
 // 2, 4 and 8), four where they nearly do (64 channels, 256 rows, one and four: 160 units 2.28, 2.12 ms; 192 2.59, 2.46; 224
 // 2.85, 2.80, but in blocks of 160 1.38, 1.42: just over three waves), else enough to fill them; at most one per 32 row slots.
-ApplyPlan plan_apply(int64_t units, int d, int C, bool recompute) {
+ApplyPlan plan_apply(int64_t units, int group, int d, int C, bool recompute) {
   const int64_t rows = (int64_t)C * units, groups = (C + kApplyRowsPerCta - 1) / kApplyRowsPerCta;
-  const bool longer = rows > 12288 || units >= 68 || (rows >= 8192 && units * groups <= 2 * 148);
+  const bool longer = rows > 12288 || units >= 68 || (group == 1 && rows >= 8192 && units * groups <= 2 * 148);
   if (!recompute && (d == 128 || (C > 128 ? !longer : rows < 6144))) return {1, (C + 7) / 8};
   const int64_t fill = units > 148 && !recompute ? 4 : 2 * 148 / units;
   return {4, (int)std::max<int64_t>(1, std::min(fill, groups))};
 }
-static ApplyPlan plan_apply(const State* st) { return plan_apply(st->U, st->d, st->C, st->recomputeK); }
+static ApplyPlan plan_apply(const State* st) { return plan_apply(st->U, st->G, st->d, st->C, st->recomputeK); }
 
 int launch_refresh_rows(State* st, int64_t m, cudaStream_t s) {
   if (m <= 0) return 0;

@@ -195,7 +195,7 @@ struct FoldArgs {
 };
 int launch_fold(State* st, const FoldArgs& a, cudaStream_t s);
 struct ApplyPlan { int rows_per_warp, ctas; };   // one or four touched rows per warp, CTAs per unit
-ApplyPlan plan_apply(int64_t units, int d, int C, bool recompute);
+ApplyPlan plan_apply(int64_t units, int group, int d, int C, bool recompute);
 // Memory keys of nblk consecutive blocks (C rows each, starting at ok within every unit) into slots
 // slot0 .. slot0 + nblk - 1.
 int launch_kbar(State* st, const __half* ok, int64_t unit_stride, int nblk, int slot0, bool want_gram, cudaStream_t s);

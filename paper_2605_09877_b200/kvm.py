@@ -115,7 +115,7 @@ def _load():
     L.kvm_debug_decode_ahead.restype = C.c_int
     L.kvm_debug_decode_ahead.argtypes = [C.c_int32, C.c_int32, C.c_int32, C.c_int32, C.c_int64, C.POINTER(C.c_int32)]
     L.kvm_debug_apply_plan.restype = C.c_int
-    L.kvm_debug_apply_plan.argtypes = [C.c_int64, C.c_int32, C.c_int32, C.c_int32, C.POINTER(C.c_int32)]
+    L.kvm_debug_apply_plan.argtypes = [C.c_int64, C.c_int32, C.c_int32, C.c_int32, C.c_int32, C.POINTER(C.c_int32)]
     L.kvm_debug_attention_plan.restype = C.c_int
     L.kvm_debug_attention_plan.argtypes = [C.c_int32] * 5 + [C.c_int64, C.c_int32, C.POINTER(C.c_int32)]
     L.kvm_debug_expire_wait.restype = C.c_int
@@ -197,9 +197,9 @@ def decode_ahead(batch: int, n_q_heads: int, n_kv_heads: int, head_dim: int, n_r
     return _plan("kvm_debug_decode_ahead", 3, batch, n_q_heads, n_kv_heads, head_dim, n_rows)
 
 
-def apply_plan(n_units: int, head_dim: int, block: int, serial: bool = False):
-    """(rows per warp, CTAs per unit) of the kernel that writes the rows a fold touches."""
-    return _plan("kvm_debug_apply_plan", 2, n_units, head_dim, block, 1 if serial else 0)
+def apply_plan(n_units: int, head_dim: int, block: int, serial: bool = False, group: int = 1):
+    """(rows per warp, CTAs per unit) of the kernel that writes the rows a fold touches; group: query heads per unit."""
+    return _plan("kvm_debug_apply_plan", 2, n_units, group, head_dim, block, 1 if serial else 0)
 
 
 def attention_plan(batch: int, n_q_heads: int, n_kv_heads: int, head_dim: int, n_queries: int, n_slots: int, decides: bool = True):

@@ -117,6 +117,11 @@ def test_rows_per_warp_of_the_apply_kernel(units, d, C, serial, rows):
     assert kvm.apply_plan(units, d, C, serial)[0] == rows
 
 
+@pytest.mark.parametrize("units,d,C,group,rows", [(34, 64, 256, 1, 4), (34, 64, 256, 2, 1), (37, 64, 256, 8, 1), (48, 64, 256, 8, 1), (49, 64, 256, 8, 4), (68, 64, 136, 8, 4), (48, 64, 128, 2, 4)])
+def test_rows_per_warp_beside_the_attention_of_several_heads(units, d, C, group, rows):
+    assert kvm.apply_plan(units, d, C, group=group)[0] == rows
+
+
 def test_plan_refuses_what_a_state_refuses():
     for bad in [(0, 1, 1, 64, 10), (1, 3, 2, 64, 10), (1, 2, 2, 96, 10), (1, 2, 2, 64, 0)]:
         with pytest.raises(kvm.KVMError):
